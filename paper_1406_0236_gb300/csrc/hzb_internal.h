@@ -130,6 +130,12 @@ struct TargetBlock {
     int excl_hi;
 };
 
+// How the pair-symmetric kernels share one block pair among `nz` CTAs (grid z): each takes
+// `jchunk` sources of the source-side block and 32 / nstep of the rotation steps of a tile.
+struct SymSplit {
+    int jchunk, nstep, nz;
+};
+
 }  // namespace hzb
 
 struct hzb_ctx {
@@ -286,7 +292,8 @@ const float2 *weighted_sigma32(hzb_ctx *c, int R, const double2 *sigma);      //
 hzb_status ensure_sctab(hzb_ctx *c);                                          // nbody.cu: FP64 cos/sin table
 hzb_status interbody64_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y);  // nbody_sym.cu
 hzb_status interbody32_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tp);  // nbody_sym.cu
-hzb_status ensure_block_pairs(hzb_ctx *c);                                    // nbody_sym.cu  // nbody_tc.cu
+hzb_status ensure_block_pairs(hzb_ctx *c);                                    // nbody_sym.cu
+SymSplit sym_split(hzb_ctx *c, int rhs_chunks);      // the split for the context's block pairs (nbody_sym.cu)
 void split_reduce_f2(hzb_ctx *c, size_t n, int nsplit, const float2 *part, double2 *y);
 hzb_status interbody64_cfg(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tpt, int nsplit);
 hzb_status interbody32_cfg(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tpt, int nsplit, bool x2);

@@ -74,12 +74,16 @@ __global__ void __launch_bounds__(DFL_T, 1)
 nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict__ blocks, int R,
                      const float4 *__restrict__ pa, const float4 *__restrict__ pb, const float4 *__restrict__ pc,
                      const double4 *__restrict__ pos64, const double2 *__restrict__ sigma,
-                     const float4 *__restrict__ tab, DflConst K, double2 *__restrict__ y)
+                     const float4 *__restrict__ tab, DflConst K, double2 *__restrict__ y, SymSplit sp)
 {
     __shared__ DflTile<RC> s_tile[2];                     // double-buffered source tiles
     __shared__ float4 s_tab[DFL_TAB];
     const int2 pr = pairs[blockIdx.x];
     const TargetBlock bi = blocks[pr.x], bj = blocks[pr.y];
+    // this CTA's sources [jlo, jhi) of J and rotation steps [st0, st1) of each tile
+    const int jlo = (blockIdx.z / sp.nstep) * sp.jchunk, jhi = min(bj.count, jlo + sp.jchunk);
+    const int st0 = (blockIdx.z % sp.nstep) * (DFL_S / sp.nstep), st1 = st0 + DFL_S / sp.nstep;
+    if (jlo >= jhi) return;
     const int r0 = blockIdx.y * RC;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int q = tid; q < DFL_TAB; q += DFL_T) s_tab[q] = tab[q];
@@ -107,7 +111,7 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
     // the first warp loads the next tile's sources into registers while the tile runs
     float4 na, nb, nc, ns[RC];
     auto fetch = [&](int j0) {
-        const int cnt = min(DFL_S, bj.count - j0);
+        const int cnt = min(DFL_S, jhi - j0);
         if (lane < cnt) {
             const int g = bj.start + j0 + lane;
             na = pa[g]; nb = pb[g]; nc = pc[g];
@@ -132,25 +136,25 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
         for (int c = 0; c < RC; ++c) T.sig[lane][c] = ns[c];
     };
     if (warp == 0) {
-        fetch(0);
+        fetch(jlo);
         stage(s_tile[0]);
-        if (DFL_S < bj.count) fetch(DFL_S);
+        if (jlo + DFL_S < jhi) fetch(jlo + DFL_S);
     }
     const bool warp_live = warp * 32 < bi.count;
     int buf = 0;
-    for (int j0 = 0; j0 < bj.count; j0 += DFL_S, buf ^= 1) {
-        const int cnt = min(DFL_S, bj.count - j0);
+    for (int j0 = jlo; j0 < jhi; j0 += DFL_S, buf ^= 1) {
+        const int cnt = min(DFL_S, jhi - j0);
         __syncthreads();                                   // tile j0 staged; the other buffer is free
-        if (warp == 0 && j0 + DFL_S < bj.count) {
+        if (warp == 0 && j0 + DFL_S < jhi) {
             stage(s_tile[buf ^ 1]);
-            if (j0 + 2 * DFL_S < bj.count) fetch(j0 + 2 * DFL_S);
+            if (j0 + 2 * DFL_S < jhi) fetch(j0 + 2 * DFL_S);
         }
         if (!warp_live) continue;
         const DflTile<RC> &T = s_tile[buf];
         dd asr[RC], asi[RC];
 #pragma unroll
         for (int c = 0; c < RC; ++c) asr[c] = asi[c] = {0.f, 0.f};
-        for (int s = 0; s < DFL_S; ++s) {
+        for (int s = st0; s < st1; ++s) {
             const int q = (lane + s) & (DFL_S - 1);
             const float4 A4 = T.a[q], B4 = T.b[q], C4 = T.c[q];
             // d = x_i - x_j
@@ -209,12 +213,14 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
         }
 #pragma unroll
         for (int c = 0; c < RC; ++c) { atr[c] = norm(atr[c]); ati[c] = norm(ati[c]); }
-        // after 32 steps lane l holds this warp's sum for source l: straight into y
-        if (lane < cnt) {
+        // after the last step lane l holds this warp's sum for source (l + st1) mod 32:
+        // straight into y
+        const int src = (lane + st1) & (DFL_S - 1);
+        if (src < cnt) {
 #pragma unroll
             for (int c = 0; c < RC; ++c)
                 if (r0 + c < R) {
-                    double2 *o = y + (size_t)(bj.start + j0 + lane) * R + r0 + c;
+                    double2 *o = y + (size_t)(bj.start + j0 + src) * R + r0 + c;
                     atomicAdd(&o->x, (double)asr[c].h + (double)asr[c].l);
                     atomicAdd(&o->y, (double)asi[c].h + (double)asi[c].l);
                 }
@@ -464,15 +470,16 @@ hzb_status interbody_dfl_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y
     const DflConst K = dfl_constants(c);
     const int slot = prof_begin(c, 2);
     const int rc = (R == 1) ? 1 : 2;
-    dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, 1);
+    const SymSplit sp = sym_split(c, (R + rc - 1) / rc);
+    dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, sp.nz);
     if (rc == 1)
         nbody_dfl_sym_kernel<1><<<g, DFL_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->dfa.ptr,
                                                             c->dfb.ptr, c->dfc.ptr, c->pos64.ptr, sigma,
-                                                            c->dfltab.ptr, K, y);
+                                                            c->dfltab.ptr, K, y, sp);
     else
         nbody_dfl_sym_kernel<2><<<g, DFL_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->dfa.ptr,
                                                             c->dfb.ptr, c->dfc.ptr, c->pos64.ptr, sigma,
-                                                            c->dfltab.ptr, K, y);
+                                                            c->dfltab.ptr, K, y, sp);
     cudaError_t e = cudaGetLastError();
     prof_end(c, slot);
     return check_cuda(c, e, "nbody_dfl_sym_kernel");

@@ -15,7 +15,7 @@
 // own sum and the j <- i term to a rotating sum that then moves to lane l - 1, so each
 // source's partial sum visits every lane once and no two lanes touch the same source
 // at a step.  The warps' partial sums of a tile are added in a fixed order in shared
-// memory.  Both directions reach y through FP64 atomic adds (y is zeroed first), so
+// memory.  On small geometries several CTAs share a block pair (sym_split).  Both directions reach y through FP64 atomic adds (y is zeroed first), so
 // the order of the additions into one y entry varies between runs: the result is
 // reproducible to rounding, not bit for bit.
 #include <algorithm>
@@ -31,12 +31,23 @@ namespace hzb {
 static const int SYM_T = 512;        // targets per CTA = TargetBlock size
 static const int SYM_S = 32;         // sources per tile (one per lane)
 
+// This CTA's part of its block pair (SymSplit): sources [jlo, jhi) of J and rotation
+// steps [st0, st1) of each of their tiles.
+__device__ __forceinline__ void sym_range(const SymSplit &sp, int nj, int &jlo, int &jhi, int &st0, int &st1)
+{
+    const int zj = blockIdx.z / sp.nstep, zs = blockIdx.z % sp.nstep;
+    jlo = zj * sp.jchunk;
+    jhi = min(nj, jlo + sp.jchunk);
+    st0 = zs * (SYM_S / sp.nstep);
+    st1 = st0 + SYM_S / sp.nstep;
+}
+
 template <int RC>
 __global__ void __launch_bounds__(SYM_T, 1)
 nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict__ blocks, int R,
                    const double4 *__restrict__ pos, const double4 *__restrict__ nrm,
                    const double2 *__restrict__ sigma, const double2 *__restrict__ sctab, double k, double eta,
-                   double kt, double2 *__restrict__ y)
+                   double kt, double2 *__restrict__ y, SymSplit sp)
 {
     __shared__ double4 s_p[SYM_S];               // x, y, z, w
     __shared__ double4 s_n[SYM_S];               // nx, ny, nz
@@ -44,6 +55,9 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
     __shared__ double2 s_red[SYM_T / 32][RC][SYM_S];
     const int2 pr = pairs[blockIdx.x];
     const TargetBlock bi = blocks[pr.x], bj = blocks[pr.y];
+    int jlo, jhi, st0, st1;                      // this CTA's sources of J and rotation steps
+    sym_range(sp, bj.count, jlo, jhi, st0, st1);
+    if (jlo >= jhi) return;
     const int r0 = blockIdx.y * RC;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool live = tid < bi.count;
@@ -67,8 +81,8 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
     for (int c = 0; c < RC; ++c) acc_t[c] = make_double2(0.0, 0.0);
     const bool warp_live = warp * 32 < bi.count;
     const double eta_ = eta;
-    for (int j0 = 0; j0 < bj.count; j0 += SYM_S) {
-        const int cnt = min(SYM_S, bj.count - j0);
+    for (int j0 = jlo; j0 < jhi; j0 += SYM_S) {
+        const int cnt = min(SYM_S, jhi - j0);
         __syncthreads();
         if (tid < SYM_S) {
             if (tid < cnt) {
@@ -95,7 +109,7 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
         for (int c = 0; c < RC; ++c) acc_s[c] = make_double2(0.0, 0.0);
         if (warp_live) {
 #pragma unroll 2
-            for (int s = 0; s < SYM_S; ++s) {
+            for (int s = st0; s < st1; ++s) {
                 const int q = (lane + s) & (SYM_S - 1);
                 const double4 p = s_p[q];
                 const double4 n = s_n[q];
@@ -130,9 +144,9 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
                 }
             }
         }
-        // after 32 steps lane l holds the partial sum of source l
+        // after the last step lane l holds the partial sum of source (l + st1) mod 32
 #pragma unroll
-        for (int c = 0; c < RC; ++c) s_red[warp][c][lane] = acc_s[c];
+        for (int c = 0; c < RC; ++c) s_red[warp][c][(lane + st1) & (SYM_S - 1)] = acc_s[c];
         __syncthreads();
         if (tid < SYM_S * RC) {
             const int src = tid & (SYM_S - 1), c = tid / SYM_S;
@@ -173,11 +187,13 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
 // transcendental-unit latency than five at 96 registers, four at 120 or seven at 72 with
 // more spills (36.8 / 37.5 / 38.6 / 39.3 ms on 258,560 unknowns).
 static constexpr int SYM32_MIN_BLOCKS = 6;
-template <int RC, int TP>
+// STEPS = false: all 32 rotation steps, a constant trip count (2 % of the time at 258,560
+// unknowns against the bounds of a split).
+template <int RC, int TP, bool STEPS>
 __global__ void __launch_bounds__(SYM_T / (2 * TP), (RC == 1 && TP == 2) ? SYM32_MIN_BLOCKS : 1)
 nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict__ blocks, int R,
                    const float4 *__restrict__ pos, const float4 *__restrict__ nrm, const float2 *__restrict__ sw,
-                   float k, float eta, float kt, double2 *__restrict__ y)
+                   float k, float eta, float kt, double2 *__restrict__ y, SymSplit sp)
 {
     constexpr int NT = SYM_T / (2 * TP);
     constexpr int NW = NT / 32;
@@ -187,6 +203,10 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
     __shared__ float2 s_red[NW][RC][SYM_S];
     const int2 pr = pairs[blockIdx.x];
     const TargetBlock bi = blocks[pr.x], bj = blocks[pr.y];
+    int jlo, jhi, st0, st1;                      // this CTA's sources of J and rotation steps
+    sym_range(sp, bj.count, jlo, jhi, st0, st1);
+    if (!STEPS) { st0 = 0; st1 = SYM_S; }
+    if (jlo >= jhi) return;
     const int r0 = blockIdx.y * RC;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     f2x tx[TP], ty[TP], tz[TP], mx[TP], my[TP], mz[TP];      // target positions, negated normals
@@ -217,8 +237,8 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
     }
     const bool warp_live = warp * 32 < bi.count;
     const f2x k2 = f2_splat(k), nk2 = f2_splat(-k), eta2 = f2_splat(eta), neta2 = f2_splat(-eta);
-    for (int j0 = 0; j0 < bj.count; j0 += SYM_S) {
-        const int cnt = min(SYM_S, bj.count - j0);
+    for (int j0 = jlo; j0 < jhi; j0 += SYM_S) {
+        const int cnt = min(SYM_S, jhi - j0);
         __syncthreads();
         if (tid < SYM_S) {
             if (tid < cnt) {
@@ -241,7 +261,7 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
         for (int c = 0; c < RC; ++c) asx[c] = asy[c] = 0ull;
         if (warp_live) {
 #pragma unroll 2
-            for (int s = 0; s < SYM_S; ++s) {
+            for (int s = st0; s < st1; ++s) {
                 const int q = (lane + s) & (SYM_S - 1);
                 const float4 g0 = s_g0[q];
                 const float2 g1 = s_g1[q];
@@ -300,7 +320,7 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
             float xa, xb, ya, yb;
             f2_unpack(asx[c], xa, xb);
             f2_unpack(asy[c], ya, yb);
-            s_red[warp][c][lane] = make_float2(xa + xb, ya + yb);
+            s_red[warp][c][(lane + st1) & (SYM_S - 1)] = make_float2(xa + xb, ya + yb);
         }
         __syncthreads();
         if (tid < SYM_S * RC) {
@@ -334,6 +354,26 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
                     atomicAdd(&o->y, (double)(h ? yb : ya));
                 }
         }
+}
+
+// A block pair per CTA leaves most of the chip idle on small geometries (two spheres of
+// 4,100 nodes: 81 CTAs; 216 nodes: one), and a CTA of 512 x 512 pairs is a long last wave on
+// middling ones.  So the source side is cut until there are about 16 CTAs per SM, down to
+// one tile of 32 sources, and below 4 per SM the rotation steps of a tile are shared out
+// too.  Finer pieces cost more than they fill: every CTA adds its 512 target sums to y with
+// FP64 atomics.  Before -> after, one right-hand side (FP64 / double-float / FP32 sums):
+// 432 unknowns 787 / 139 / 61 -> 18 us each (the call itself); 8,200 unknowns 3,814 / 533 /
+// 122 -> 1,672 / 263 / 39 us (at twice as many pieces 1,693 / 295 / 39); 29,280 unknowns
+// 32.31 / 4.47 / 0.523 -> 31.41 / 4.37 / 0.455 ms; from 64,640 unknowns up nothing is cut.
+SymSplit sym_split(hzb_ctx *c, int rhs_chunks)
+{
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->opt.device);
+    const long long have = c->n_blockpairs * rhs_chunks;
+    SymSplit sp = {SYM_T, 1, 1};
+    while (have * sp.nz < 16LL * sms && sp.jchunk > SYM_S) { sp.jchunk /= 2; sp.nz *= 2; }
+    while (have * sp.nz < 4LL * sms && sp.nstep < 16) { sp.nstep *= 2; sp.nz *= 2; }
+    return sp;
 }
 
 // Unordered pairs of target blocks on different bodies, built once per geometry.
@@ -380,28 +420,32 @@ hzb_status interbody64_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     c->launches += 1;
     const int slot = prof_begin(c, 0);
     const int rc = (R == 1) ? 1 : (R == 2 ? 2 : 4);
-    dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, 1);
+    const SymSplit sp = sym_split(c, (R + rc - 1) / rc);
+    dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, sp.nz);
     const double kt = c->k * (SC_N / (2.0 * M_PI));
     if (rc == 1)
         nbody64_sym_kernel<1><<<g, SYM_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos64.ptr,
-                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y);
+                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y, sp);
     else if (rc == 2)
         nbody64_sym_kernel<2><<<g, SYM_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos64.ptr,
-                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y);
+                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y, sp);
     else
         nbody64_sym_kernel<4><<<g, SYM_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos64.ptr,
-                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y);
+                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y, sp);
     cudaError_t e = cudaGetLastError();
     prof_end(c, slot);
     return check_cuda(c, e, "nbody64_sym_kernel");
 }
 
 template <int RC, int TP>
-static void launch_sym32(hzb_ctx *c, dim3 g, int R, const float2 *sw, double2 *y)
+static void launch_sym32(hzb_ctx *c, dim3 g, int R, const float2 *sw, double2 *y, SymSplit sp)
 {
-    nbody32_sym_kernel<RC, TP><<<g, SYM_T / (2 * TP), 0, c->stream>>>(
-        c->blockpairs.ptr, c->tblocks.ptr, R, c->pos32.ptr, c->nrm32.ptr, sw, (float)c->k, (float)c->eta,
-        (float)(c->k / (2.0 * M_PI)), y);
+    auto launch = [&](auto kern) {
+        kern<<<g, SYM_T / (2 * TP), 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos32.ptr, c->nrm32.ptr, sw,
+                                                    (float)c->k, (float)c->eta, (float)(c->k / (2.0 * M_PI)), y, sp);
+    };
+    if (sp.nstep > 1) launch(nbody32_sym_kernel<RC, TP, true>);
+    else launch(nbody32_sym_kernel<RC, TP, false>);
 }
 
 hzb_status interbody32_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tp)
@@ -420,15 +464,16 @@ hzb_status interbody32_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y, 
     if (!sw) return HZB_ENOMEM;
     c->launches += 1;
     const int rc = (R == 1) ? 1 : (R == 2 ? 2 : 4);
-    dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, 1);
+    const SymSplit sp = sym_split(c, (R + rc - 1) / rc);
+    dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, sp.nz);
     if (tp == 2) {
-        if (rc == 1) launch_sym32<1, 2>(c, g, R, sw, y);
-        else if (rc == 2) launch_sym32<2, 2>(c, g, R, sw, y);
-        else launch_sym32<4, 2>(c, g, R, sw, y);
+        if (rc == 1) launch_sym32<1, 2>(c, g, R, sw, y, sp);
+        else if (rc == 2) launch_sym32<2, 2>(c, g, R, sw, y, sp);
+        else launch_sym32<4, 2>(c, g, R, sw, y, sp);
     } else {
-        if (rc == 1) launch_sym32<1, 1>(c, g, R, sw, y);
-        else if (rc == 2) launch_sym32<2, 1>(c, g, R, sw, y);
-        else launch_sym32<4, 1>(c, g, R, sw, y);
+        if (rc == 1) launch_sym32<1, 1>(c, g, R, sw, y, sp);
+        else if (rc == 2) launch_sym32<2, 1>(c, g, R, sw, y, sp);
+        else launch_sym32<4, 1>(c, g, R, sw, y, sp);
     }
     cudaError_t e = cudaGetLastError();
     prof_end(c, slot);
