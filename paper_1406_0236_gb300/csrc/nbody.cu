@@ -553,110 +553,178 @@ hzb_status interbody32(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
 
 // ------------------------------------------------------------------ fields at points
 
-static const int FP_CHUNK = 2048;     // sources per block of the point-field kernels
-
-// Partial sums of u(p_t) = sum_j w_j K(p_t, x_j) sigma_j over one source chunk:
-// grid (chunks, T); block reduce; partial[(t * nchunk + chunk) * R + r].
-__global__ void field_partial_kernel(int N, int R, const double4 *__restrict__ pos,
-                                     const double4 *__restrict__ nrm, const double2 *__restrict__ sigma,
-                                     const double *__restrict__ pts, double k, double eta, double2 *partial)
+// w_j / (4 pi) times the kernel of one point and one source: far = the far-field pattern's
+// e^{-ik xh.x_j} (-ik xh.n_j - i eta) for a unit direction xh, else K(p, x_j) for a point p.
+template <bool FAR>
+__device__ __forceinline__ double2 point_kernel(double px, double py, double pz, double4 p, double4 n, double k,
+                                                double eta)
 {
-    __shared__ double2 red[256];
-    const int chunk = blockIdx.x, t = blockIdx.y, nchunk = gridDim.x;
-    const double px = pts[3 * t], py = pts[3 * t + 1], pz = pts[3 * t + 2];
-    const int j0 = chunk * FP_CHUNK, j1 = min(N, j0 + FP_CHUNK);
-    for (int r = 0; r < R; ++r) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-            double4 p = pos[j], n = nrm[j];
-            double dx = px - p.x, dy = py - p.y, dz = pz - p.z;
-            double r2 = dx * dx + dy * dy + dz * dz, ir = rsqrt(r2), rr = r2 * ir;
-            double nd = n.x * dx + n.y * dy + n.z * dz;
-            double A = nd * ir * ir * ir, B = k * nd * ir * ir + eta * ir;
-            double s, c;
-            sincos(k * rr, &s, &c);
-            double2 g = make_double2((c * A + s * B) * p.w * HZB_INV4PI, (s * A - c * B) * p.w * HZB_INV4PI);
-            cfma(acc, g, sigma[(size_t)j * R + r]);
+    double s, c;
+    if (FAR) {
+        sincos(k * (px * p.x + py * p.y + pz * p.z), &s, &c);
+        const double2 fac = make_double2(0.0, -(k * (px * n.x + py * n.y + pz * n.z) + eta));
+        return cscale(cmul(make_double2(c, -s), fac), p.w * HZB_INV4PI);
+    }
+    const double dx = px - p.x, dy = py - p.y, dz = pz - p.z;
+    const double r2 = dx * dx + dy * dy + dz * dz, ir = rsqrt(r2), rr = r2 * ir;
+    const double nd = n.x * dx + n.y * dy + n.z * dz;
+    const double A = nd * ir * ir * ir, B = k * nd * ir * ir + eta * ir;
+    sincos(k * rr, &s, &c);
+    return make_double2((c * A + s * B) * p.w * HZB_INV4PI, (s * A - c * B) * p.w * HZB_INV4PI);
+}
+
+// Partial sums over one source chunk for few right-hand sides: one block per (point,
+// chunk, RC right-hand sides), each thread forms its sources' kernel values once for the
+// RC columns; partial[(t * nchunk + chunk) * R + r].
+template <int RC, bool FAR>
+__global__ void __launch_bounds__(256)
+point_partial_kernel(int N, int R, int chunk, const double4 *__restrict__ pos, const double4 *__restrict__ nrm,
+                     const double2 *__restrict__ sigma, const double *__restrict__ pts, double k, double eta,
+                     double2 *__restrict__ partial)
+{
+    __shared__ double2 red[8][RC];
+    const int t = blockIdx.x, ch = blockIdx.y, nchunk = gridDim.y, r0 = blockIdx.z * RC;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double px = pts[3 * (size_t)t], py = pts[3 * (size_t)t + 1], pz = pts[3 * (size_t)t + 2];
+    const int j0 = ch * chunk, j1 = min(N, j0 + chunk);
+    double2 acc[RC];
+#pragma unroll
+    for (int c = 0; c < RC; ++c) acc[c] = make_double2(0.0, 0.0);
+    for (int j = j0 + threadIdx.x; j < j1; j += 256) {
+        const double2 g = point_kernel<FAR>(px, py, pz, pos[j], nrm[j], k, eta);
+#pragma unroll
+        for (int c = 0; c < RC; ++c)
+            if (r0 + c < R) cfma(acc[c], g, sigma[(size_t)j * R + r0 + c]);
+    }
+#pragma unroll
+    for (int c = 0; c < RC; ++c) {
+        for (int o = 16; o > 0; o >>= 1) {
+            acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, o);
+            acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, o);
         }
-        red[threadIdx.x] = acc;
-        __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) red[threadIdx.x] = cadd(red[threadIdx.x], red[threadIdx.x + s]);
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) partial[((size_t)t * nchunk + chunk) * R + r] = red[0];
-        __syncthreads();
+        if (lane == 0) red[warp][c] = acc[c];
+    }
+    __syncthreads();
+    if (threadIdx.x < RC && r0 + threadIdx.x < R) {
+        double2 v = red[0][threadIdx.x];
+        for (int w = 1; w < 8; ++w) v = cadd(v, red[w][threadIdx.x]);
+        partial[((size_t)t * nchunk + ch) * R + r0 + threadIdx.x] = v;
     }
 }
 
-// Far-field partial sums: (1/4pi) sum_j w_j e^{-ik xh.x_j} (-ik xh.n_j - i eta) sigma_j.
-__global__ void farfield_partial_kernel(int N, int R, const double4 *__restrict__ pos,
-                                        const double4 *__restrict__ nrm, const double2 *__restrict__ sigma,
-                                        const double *__restrict__ xh, double k, double eta, double2 *partial)
+// The same partial sums for many right-hand sides: a block owns FP_TM points and RN
+// columns; per tile of FP_SK sources its 256 threads form one kernel value each (FP_TM x
+// FP_SK, shared memory) and then multiply them into the densities.  Bound by the FP64
+// pipe: 4 RN fused multiply-adds per (point, source) against about 70 operations for the
+// kernel value, so wide RN repeats the value least, and tiles need no register blocking
+// (a shared load costs nothing beside four FP64 instructions at 1/64 of the FP32 rate).
+static const int FP_TM = 16, FP_SK = 16;
+
+template <int RN, bool FAR>
+__global__ void __launch_bounds__(256)
+point_tile_kernel(int N, int R, int T, int chunk, const double4 *__restrict__ pos, const double4 *__restrict__ nrm,
+                  const double2 *__restrict__ sigma, const double *__restrict__ pts, double k, double eta,
+                  double2 *__restrict__ partial)
 {
-    __shared__ double2 red[256];
-    const int chunk = blockIdx.x, t = blockIdx.y, nchunk = gridDim.x;
-    const double hx = xh[3 * t], hy = xh[3 * t + 1], hz = xh[3 * t + 2];
-    const int j0 = chunk * FP_CHUNK, j1 = min(N, j0 + FP_CHUNK);
-    for (int r = 0; r < R; ++r) {
-        double2 acc = make_double2(0.0, 0.0);
-        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-            double4 p = pos[j], n = nrm[j];
-            double s, c;
-            sincos(k * (hx * p.x + hy * p.y + hz * p.z), &s, &c);
-            double2 ph = make_double2(c, -s);
-            double2 fac = make_double2(0.0, -(k * (hx * n.x + hy * n.y + hz * n.z) + eta));
-            double2 g = cscale(cmul(ph, fac), p.w * HZB_INV4PI);
-            cfma(acc, g, sigma[(size_t)j * R + r]);
+    constexpr int Q = (RN + 15) / 16;                  // columns per thread, 16 apart
+    __shared__ double2 s_g[FP_SK][FP_TM];
+    __shared__ double2 s_s[FP_SK][RN];
+    const int t0 = blockIdx.x * FP_TM, ch = blockIdx.y, nchunk = gridDim.y, r0 = blockIdx.z * RN;
+    const int hi = threadIdx.x >> 4, lo = threadIdx.x & 15;
+    // kernel-value duty: point lo, source hi of the tile; product duty: point hi, columns lo + 16 q
+    const int tg = min(t0 + lo, T - 1);
+    const double px = pts[3 * (size_t)tg], py = pts[3 * (size_t)tg + 1], pz = pts[3 * (size_t)tg + 2];
+    const int j0 = ch * chunk, j1 = min(N, j0 + chunk);
+    double2 acc[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) acc[q] = make_double2(0.0, 0.0);
+    for (int j = j0; j < j1; j += FP_SK) {
+        double2 g = make_double2(0.0, 0.0);
+        if (j + hi < j1) g = point_kernel<FAR>(px, py, pz, pos[j + hi], nrm[j + hi], k, eta);
+        __syncthreads();                               // the previous tile is consumed
+        s_g[hi][lo] = g;
+        for (int e = threadIdx.x; e < FP_SK * RN; e += 256) {
+            const int jj = e / RN, r = e % RN;
+            s_s[jj][r] = (j + jj < j1 && r0 + r < R) ? sigma[(size_t)(j + jj) * R + r0 + r] : make_double2(0.0, 0.0);
         }
-        red[threadIdx.x] = acc;
         __syncthreads();
-        for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-            if (threadIdx.x < s) red[threadIdx.x] = cadd(red[threadIdx.x], red[threadIdx.x + s]);
-            __syncthreads();
+        if (RN >= 16 || lo < RN) {
+            double2 part[Q];                           // summed by tiles: as accurate as a tree
+#pragma unroll
+            for (int q = 0; q < Q; ++q) part[q] = make_double2(0.0, 0.0);
+#pragma unroll 4
+            for (int kk = 0; kk < FP_SK; ++kk) {
+                const double2 gv = s_g[kk][hi];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) cfma(part[q], gv, s_s[kk][lo + 16 * q]);
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) acc[q] = cadd(acc[q], part[q]);
         }
-        if (threadIdx.x == 0) partial[((size_t)t * nchunk + chunk) * R + r] = red[0];
-        __syncthreads();
     }
+    if (t0 + hi >= T || (RN < 16 && lo >= RN)) return;
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        if (r0 + lo + 16 * q < R) partial[((size_t)(t0 + hi) * nchunk + ch) * R + r0 + lo + 16 * q] = acc[q];
 }
 
 __global__ void chunk_reduce_kernel(int T, int nchunk, int R, const double2 *partial, double2 *out)
 {
-    int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= T * R) return;
-    int t = e / R, r = e % R;
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (size_t)T * R) return;
+    const size_t t = e / R, r = e % R;
     double2 s = make_double2(0.0, 0.0);
-    for (int q = 0; q < nchunk; ++q) s = cadd(s, partial[((size_t)t * nchunk + q) * R + r]);
-    out[(size_t)t * R + r] = s;
+    for (int q = 0; q < nchunk; ++q) s = cadd(s, partial[(t * nchunk + q) * R + r]);
+    out[e] = s;
 }
 
-static hzb_status point_sum(hzb_ctx *c, int R, const double2 *sigma, int T, const double *pts, double2 *out,
-                            bool far)
+// Up to four right-hand sides take a block per point; above, the tiles, whose kernel values
+// serve all columns: 64 right-hand sides, 512 directions, 8,200 nodes 24.9 -> 2.2 ms
+// (1.7 ms of it the products at the FP64 pipe's rate).
+// Chunks of at most 2,048 sources, fewer while the grid is short of about eight blocks per SM.
+template <bool FAR>
+static hzb_status point_sum(hzb_ctx *c, int R, const double2 *sigma, int T, const double *pts, double2 *out)
 {
-    int N = (int)c->N;
-    int nchunk = (N + FP_CHUNK - 1) / FP_CHUNK;
-    size_t need = (size_t)T * nchunk * R;
-    if (check_cuda(c, c->w_d.ensure(need), "alloc field partials")) return HZB_ENOMEM;
-    dim3 grid(nchunk, T);
-    if (far)
-        farfield_partial_kernel<<<grid, 256, 0, c->stream>>>(N, R, c->pos64.ptr, c->nrm64.ptr, sigma, pts, c->k,
-                                                             c->eta, c->w_d.ptr);
-    else
-        field_partial_kernel<<<grid, 256, 0, c->stream>>>(N, R, c->pos64.ptr, c->nrm64.ptr, sigma, pts, c->k,
-                                                          c->eta, c->w_d.ptr);
-    chunk_reduce_kernel<<<(T * R + 255) / 256, 256, 0, c->stream>>>(T, nchunk, R, c->w_d.ptr, out);
+    const int N = (int)c->N;
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->opt.device);
+    const int rn = R <= 1 ? 1 : R <= 2 ? 2 : R <= 4 ? 4 : R <= 8 ? 8 : R <= 16 ? 16 : R <= 32 ? 32 : 64;
+    const long long cols = (R + rn - 1) / rn, tiles = rn <= 4 ? T : (T + FP_TM - 1) / FP_TM;
+    int chunk = 2048;
+    while (chunk > 256 && tiles * cols * ((N + chunk - 1) / chunk) < 8LL * sms) chunk /= 2;
+    const int nchunk = (N + chunk - 1) / chunk;
+    if (check_cuda(c, c->w_d.ensure((size_t)T * nchunk * R), "alloc field partials")) return HZB_ENOMEM;
+    const dim3 grid((unsigned)tiles, nchunk, (unsigned)cols);
+    auto few = [&](auto kern) {
+        kern<<<grid, 256, 0, c->stream>>>(N, R, chunk, c->pos64.ptr, c->nrm64.ptr, sigma, pts, c->k, c->eta,
+                                          c->w_d.ptr);
+    };
+    auto many = [&](auto kern) {
+        kern<<<grid, 256, 0, c->stream>>>(N, R, T, chunk, c->pos64.ptr, c->nrm64.ptr, sigma, pts, c->k, c->eta,
+                                          c->w_d.ptr);
+    };
+    switch (rn) {
+    case 1: few(point_partial_kernel<1, FAR>); break;
+    case 2: few(point_partial_kernel<2, FAR>); break;
+    case 4: few(point_partial_kernel<4, FAR>); break;
+    case 8: many(point_tile_kernel<8, FAR>); break;
+    case 16: many(point_tile_kernel<16, FAR>); break;
+    case 32: many(point_tile_kernel<32, FAR>); break;
+    default: many(point_tile_kernel<64, FAR>); break;
+    }
+    chunk_reduce_kernel<<<(unsigned)(((size_t)T * R + 255) / 256), 256, 0, c->stream>>>(T, nchunk, R, c->w_d.ptr, out);
     c->launches += 2;
     return check_cuda(c, cudaGetLastError(), "point fields");
 }
 
 hzb_status field_points64(hzb_ctx *c, int R, const double2 *sigma, int T, const double *pts, double2 *out)
 {
-    return point_sum(c, R, sigma, T, pts, out, false);
+    return point_sum<false>(c, R, sigma, T, pts, out);
 }
 
 hzb_status far_field64(hzb_ctx *c, int R, const double2 *sigma, int n, const double *xhat, double2 *out)
 {
-    return point_sum(c, R, sigma, n, xhat, out, true);
+    return point_sum<true>(c, R, sigma, n, xhat, out);
 }
 
 // v(x_i) = exp(i k d_r . x_i), N x R
