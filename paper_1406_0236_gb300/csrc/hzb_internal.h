@@ -205,7 +205,11 @@ struct hzb_ctx {
     // double-float inter-body kernel: split positions/normals, cos/sin table, launch shape
     hzb::DevBuf<float4> dfa, dfb, dfc, dftab;
     bool df_ready = false;
-    hzb::DevBuf<float4> dfltab;                // lean double-float kernel: cos/sin(2 pi m / 1024)
+    // lean double-float kernels: cos/sin(2 pi m / 1024), scaled split positions and normals,
+    // a call's split densities and their scales
+    hzb::DevBuf<float4> dfltab, dla, dlb, dlc, dlsig;
+    hzb::DevBuf<float2> dlw;
+    hzb::DevBuf<int> dlkey;
     bool dfltab_ready = false;
     int tunedf_tpt = 0, tunedf_split = 0;
     // GMRES execution: steps between host checks (0 = auto) and CUDA graphs (-1 auto, 0 off, 1 on)
@@ -281,8 +285,8 @@ hzb_status interbody64(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
 hzb_status interbody32(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
 hzb_status interbody_df(hzb_ctx *c, int R, const double2 *sigma, double2 *y);   // nbody_df.cu
 hzb_status interbody_dfl_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y);   // nbody_dfl.cu
-hzb_status interbody_dfl(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int nsplit);   // nbody_dfl.cu
-int dfl_default_nsplit(hzb_ctx *c, int R);                                                  // nbody_dfl.cu
+hzb_status interbody_dfl(hzb_ctx *c, int R, const double2 *sigma, double2 *y);       // nbody_dfl.cu
+bool dfl_symmetric(const hzb_ctx *c, int R);                                          // nbody_dfl.cu
 hzb_status interbody_tc(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int nsplit);
 hzb_status modal_gemm_tma(hzb_ctx *c, ShapeDev &sd, int ncols, const float2 *X, float2 *Cout);  // modal_tma.cu
 enum { T5_SPLIT3 = 0, T5_WS = 1, T5_SINGLE = 2 };   // forms of the tcgen05 inter-body kernel

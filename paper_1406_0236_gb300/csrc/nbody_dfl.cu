@@ -3,24 +3,52 @@
 // solve at about the accuracy of FP64 (measured max-norm error against the oracle
 // ~1e-13 of max |y|), without the FP64 pipe (1/64 of the FP32 rate on GB300).
 //
-// Each unordered pair of nodes on different bodies is evaluated once for both
-// directions (the block-pair scheme of nbody_sym.cu: one CTA per pair of TargetBlocks,
-// 32-source tiles met in 32 rotation steps, source-side sums moving one lane per step,
-// FP64 atomic adds into y).  With d = x_i - x_j, r = |d|, E = e^{ikr}/r:
-//     w_j K(x_i, x_j) sigma_j / (4 pi) ... = E [X_1 - i (k r X_1 + eta)] sigma'_j,  X_1 =  n_j.d / r^2,
-//     w_i K(x_j, x_i) sigma_i / (4 pi) ... = E [X_2 - i (k r X_2 + eta)] sigma'_i,  X_2 = -n_i.d / r^2,
-// sigma' = w sigma / (4 pi); E, r and k r are shared by the two directions.
+// Up to two right-hand sides each unordered pair of nodes on different bodies is evaluated
+// once for both directions (the block-pair scheme of nbody_sym.cu: 32-source tiles met in 32
+// rotation steps, source-side sums moving one lane per step, FP64 atomic adds into y);
+// above, a one-directional kernel shares the pair's work among up to 32 right-hand sides.
+//
+// Lengths are in wavelengths (x k / 2 pi, split into hi + lo after scaling; unscaled when
+// k = 0), so that r is the phase in turns and no rounding stands between them.  With
+// d = x_i - x_j, r = |d|, E = e^{2 pi i r} / r, kr = 2 pi r, eta' = 2 pi eta / k:
+//     w_j K(x_i, x_j) = (k / 2 pi)^2 w_j / (4 pi) E [X_1 - i (kr X_1 + eta')],  X_1 =  n_j.d / r^2,
+//     w_i K(x_j, x_i) = (k / 2 pi)^2 w_i / (4 pi) E [X_2 - i (kr X_2 + eta')],  X_2 = -n_i.d / r^2;
+// E, r and kr are shared by the two directions.  The densities come weighted, scaled per
+// right-hand side by a power of two to |sigma'| < 1 (y is scaled back), and split once per
+// call (dfl_sigma_*_kernel).
 //
 // Arithmetic: lean double-float (lean_df.cuh): error-free products and sums left
-// unnormalised, accumulators renormalised once per tile.  1/r: the hardware estimate of
-// 1/sqrt(r^2) and one Halley step (cubic convergence, so the estimate's 2^-23 error falls
-// below 2^-60).
-// e^{i k r}: k r / (2 pi) in turns is reduced to [-1/2, 1/2] and then to the nearest of
-// 1024 table angles (cos, sin in double-float, shared memory); the remainder
-// |delta| <= pi / 1024 enters through cos(delta) - 1 = -delta^2/2 + delta^4/24 and
-// sin(delta) = delta - delta^3/6 + delta^5/120 (truncation below 1e-17) and angle addition.
+// unnormalised.  Sums whose magnitude is bounded beforehand are taken on a fixed grid instead
+// of by two-sums: adding a product to m = 1.5 * 2^E rounds it to a multiple of ulp(m) in the
+// product's own fused multiply-add (s = a b + m), s - m is exact, and so is what is left,
+// fma(a, b, -(s - m)): three operations where a product and a two-sum take eight.  So are
+//   * n.d (bounded by r), kr X + eta' (by 2 pi + |eta'|) and the angle addition (by 1, with
+//     the table on the grid of ulp(3));
+//   * the sums over sources of the one-directional kernel for five and more right-hand sides
+//     (DflGrid): the mantissas of s enter an integer sum (exact), the remainders an FP32 sum
+//     whose whole units are carried over every four sources, and both a running double-float
+//     sum once per tile of 32.  28 issue slots per complex multiply-add instead of 48.  The
+//     remainders have FP32's 24 bits below a grid 22 bits below the largest product, so that
+//     the grid has to be tight: it follows the magnitude of each pair's kernel (weight
+//     included), and the densities are scaled up to one tile by tile.  A short sum (below
+//     DFL_GRID_MIN sources) keeps two-sums: their error grows with the running sum.
+// 1/r: the hardware estimate of 1/sqrt(r^2) and one Halley step (cubic convergence, so the
+// estimate's 2^-23 error falls below 2^-60); r: r^2 / r rounded, and its residual.
+// e^{2 pi i r}: r is reduced to [-1/2, 1/2] turns and then to the nearest of 1024 table
+// angles (shared memory); the remainder |delta| <= pi / 1024 enters through
+// cos(delta) - 1 = -delta^2/2 + delta^4/24 and sin(delta) = delta - delta^3/6 + delta^5/120
+// (truncation below 1e-17) and angle addition.
 // The translation unit is compiled with -fmad=false so that the compiler never fuses
 // the separately rounded operations these transformations depend on.
+//
+// Both kernels are bound by the issue of FP32 instructions (78 % of the issue slots used, the
+// rest lost to register-port conflicts): about 200 for a pair's geometry and phase, 100 more
+// and the sums' 96 for the second direction.  One pass of the earlier form (two-sums
+// throughout, lengths unscaled) and of this one, and the error of each against 64 bits:
+//   29,280 unknowns, k = 6:  R = 1  4.49 -> 4.10 ms, 1.8e-13 -> 1.1e-13;  R = 8  15.5 -> 11.0;
+//                            R = 16  25.6 -> 16.6;  R = 64  98.6 -> 61.0 ms, 2.8e-13 -> 1.2e-13
+//   8,200 unknowns, k = 2:   R = 4  0.68 -> 0.51 ms, 6.0e-14 -> 5.0e-14;
+//                            R = 64  5.62 -> 3.73 ms, 7.6e-14 -> 5.7e-14
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -32,37 +60,362 @@ namespace hzb {
 
 using namespace lean;
 
-static const int DFL_T = 512;          // targets per CTA (= TargetBlock size)
-static const int DFL_S = 32;           // sources per tile (one per lane)
+static const int DFL_T = 512;          // targets of a TargetBlock
+static const int DFL_S = 32;           // sources per tile
 static const int DFL_TAB = 1024;       // table angles 2 pi m / 1024
+static const int DFL_NT = 256;         // threads (targets) per CTA of the one-directional kernel
+// sources of a target from which on the sums run on a grid: at 4,100 sources the grid's error
+// is that of the two-sums it replaces (5.7e-14 against 6e-14), at 216 it would be twice it
+static const int DFL_GRID_MIN = 4096;
 
 struct DflConst {
-    dd k, kt, twopi, eta;              // k, k / (2 pi), 2 pi, eta
+    dd kappa, eta;                     // 2 pi (0 when k = 0), eta'
+    float eta_m, mb;                   // eta' rounded onto the grid of mb, plus mb; mb = 1.5 * 2^E for kr X + eta'
+    float eta_r;                       // eta' minus its grid value (its low part included)
+    float kbound;                      // 2 pi + |eta'|, rounded up
+    int no_phase;                      // k = 0
 };
 
-// e^{2 pi i theta} for theta (turns) with |theta| < 2^21, in double-float
-__device__ __forceinline__ void dfl_cis(dd theta, const float4 *__restrict__ tab, const DflConst &K, dd &cs, dd &sn)
+// a value of magnitude below 2^(e + 1) with e the exponent of `bound` stays inside the
+// binade of this 1.5 * 2^(e + 2) when added to it
+__device__ __forceinline__ float dfl_magic_of(float bound)
+{
+    return __int_as_float((__float_as_int(bound) & 0x7f800000) + 0x01400000);
+}
+
+// ulp of a number 1.5 * 2^E
+__device__ __forceinline__ float dfl_ulp_of(float m)
+{
+    return __int_as_float((__float_as_int(m) & 0x7f800000) - (23 << 23));
+}
+
+// e^{2 pi i theta} for theta (turns) with |theta| < 2^21; high parts on the grid of ulp(3)
+__device__ __forceinline__ void dfl_cis(dd theta, const float4 *__restrict__ tab, dd &cs, dd &sn)
 {
     const float MAGIC = 12582912.0f;                      // 1.5 * 2^23: adding it rounds to an integer
     const float n0 = (theta.h + MAGIC) - MAGIC;
     const float f = theta.h - n0;                         // exact, |f| <= 1/2
-    const float tm = f * (float)DFL_TAB + MAGIC;          // f * 1024 is exact
+    const float tm = fmaf(f, (float)DFL_TAB, MAGIC);
     const float mf = tm - MAGIC;                          // nearest table index, as a float
     const int idx = __float_as_int(tm) & (DFL_TAB - 1);   // its low bits are the integer
     const float g = fmaf(mf, -1.0f / DFL_TAB, f);         // exact: |g| <= 1/2048 turns
-    const dd del = mul(two_sum(g, theta.l), K.twopi);     // remainder in radians, |delta| <= pi/1024
+    // g is zero or a multiple of ulp(theta.h): the fast two-sum is exact
+    const float gs = g + theta.l;
+    const dd twopi = {6.28318548f, -1.74845553e-7f};
+    const dd del = mul({gs, theta.l - (gs - g)}, twopi);  // remainder in radians, |delta| <= pi/1024
     const float q = del.h * del.h;
     const float qe = fmaf(del.h + del.h, del.l, fmaf(del.h, del.h, -q));   // delta^2 = q + qe
     const dd cm = {-0.5f * q, fmaf(q, q * (1.0f / 24.0f), -0.5f * qe)};     // cos(delta) - 1
     const dd sd = {del.h, fmaf(del.h * q, fmaf(q, 1.0f / 120.0f, -1.0f / 6.0f), del.l)};   // sin(delta)
-    const float4 T = tab[idx];
-    const dd C = {T.x, T.y}, S = {T.z, T.w};
-    cs = add(C, sub(mul(C, cm), mul(S, sd)));
-    sn = add(S, add(mul(S, cm), mul(C, sd)));
+    const float4 T = tab[idx];                            // cos + 3, its low part, sin + 3, its low part
+    const float C = T.x - 3.0f, S = T.z - 3.0f;           // exact
+    {
+        const float s1 = fmaf(-S, sd.h, T.x), t1 = s1 - T.x, l1 = fmaf(-S, sd.h, -t1);
+        const float s2 = fmaf(C, cm.h, s1), t2 = s2 - s1, l2 = fmaf(C, cm.h, -t2);
+        float l = l1 + l2;
+        l = fmaf(C, cm.l, l);
+        l = fmaf(T.y, cm.h, l);
+        l = fmaf(-S, sd.l, l);
+        l = fmaf(-T.w, sd.h, l);
+        cs = {s2 - 3.0f, l + T.y};
+    }
+    {
+        const float s1 = fmaf(C, sd.h, T.z), t1 = s1 - T.z, l1 = fmaf(C, sd.h, -t1);
+        const float s2 = fmaf(S, cm.h, s1), t2 = s2 - s1, l2 = fmaf(S, cm.h, -t2);
+        float l = l1 + l2;
+        l = fmaf(S, cm.l, l);
+        l = fmaf(T.w, cm.h, l);
+        l = fmaf(C, sd.l, l);
+        l = fmaf(T.y, sd.h, l);
+        sn = {s2 - 3.0f, l + T.w};
+    }
 }
 
+// What the two directions of a pair share.
+struct DflGeom {
+    dd dx, dy, dz, ir2, kr, Er, Ei;
+    float mr;                          // grid for n.d
+};
+
+// (W: E times the weight w of the source)
+template <bool W>
+__device__ __forceinline__ DflGeom dfl_geom(dd tx, dd ty, dd tz, float4 A4, float4 B4, dd w,
+                                            const float4 *__restrict__ tab, const DflConst &K)
+{
+    DflGeom G;
+    // d = x_i - x_j
+    G.dx = sub(tx, {A4.x, B4.x});
+    G.dy = sub(ty, {A4.y, B4.y});
+    G.dz = sub(tz, {A4.z, B4.z});
+    // r^2 from exact squares; the sums of the positive squares in fast_two_sum order
+    const float px = G.dx.h * G.dx.h, py = G.dy.h * G.dy.h, pz = G.dz.h * G.dz.h;
+    const float ex = fmaf(G.dx.h, G.dx.h, -px), ey = fmaf(G.dy.h, G.dy.h, -py), ez = fmaf(G.dz.h, G.dz.h, -pz);
+    const float cr = fmaf(G.dx.h, G.dx.l, fmaf(G.dy.h, G.dy.l, G.dz.h * G.dz.l));
+    const float m1 = fmaxf(px, py), l1 = fminf(px, py);
+    const float s1 = m1 + l1, e1 = l1 - (s1 - m1);
+    const float m2 = fmaxf(s1, pz), l2 = fminf(s1, pz);
+    const float s2 = m2 + l2, e2 = l2 - (s2 - m2);
+    const dd r2 = norm({s2, fmaf(2.0f, cr, (e1 + e2) + ((ex + ey) + ez))});
+    // 1/r: hardware estimate y0, Halley step y0 (1 + e/2 + 3 e^2/8), e = 1 - r^2 y0^2
+    const float y0 = rsqrtf(r2.h);
+    const float q0 = y0 * y0, q0e = fmaf(y0, y0, -q0);
+    const float u = r2.h * q0;
+    const float ue = fmaf(r2.l, q0, fmaf(r2.h, q0e, fmaf(r2.h, q0, -u)));
+    const float e = (1.0f - u) - ue;
+    const dd ir = norm({y0, y0 * e * fmaf(e, 0.375f, 0.5f)});
+    // r = rh + (r^2 - rh^2) / (2 r): rh is within an ulp of r, so the next term is below 2^-49 r
+    const float rh = r2.h * ir.h;
+    const float rr = fmaf(-rh, rh, r2.h) + r2.l;
+    const dd r = {rh, rr * (0.5f * ir.h)};
+    G.mr = dfl_magic_of(rh);
+    G.ir2 = mul(ir, ir);
+    G.kr = mul(K.kappa, r);
+    dd cs, sn;
+    dfl_cis(K.no_phase ? dd{0.f, 0.f} : r, tab, cs, sn);
+    const dd iw = W ? mul(ir, w) : ir;
+    G.Er = mul(cs, iw);
+    G.Ei = mul(sn, iw);
+    return G;
+}
+
+// X = n.d / r^2 on the grid of r
+__device__ __forceinline__ dd dfl_projection(dd nx, dd ny, dd nz, const DflGeom &G)
+{
+    const float s1 = fmaf(nx.h, G.dx.h, G.mr), t1 = s1 - G.mr, l1 = fmaf(nx.h, G.dx.h, -t1);
+    const float s2 = fmaf(ny.h, G.dy.h, s1), t2 = s2 - s1, l2 = fmaf(ny.h, G.dy.h, -t2);
+    const float s3 = fmaf(nz.h, G.dz.h, s2), t3 = s3 - s2, l3 = fmaf(nz.h, G.dz.h, -t3);
+    float l = (l1 + l2) + l3;
+    l = fmaf(nx.h, G.dx.l, l);
+    l = fmaf(nx.l, G.dx.h, l);
+    l = fmaf(ny.h, G.dy.l, l);
+    l = fmaf(ny.l, G.dy.h, l);
+    l = fmaf(nz.h, G.dz.l, l);
+    l = fmaf(nz.l, G.dz.h, l);
+    const dd nd = {s3 - G.mr, l};
+    dd X = mul(nd, G.ir2);
+    X.l = fmaf(nd.l, G.ir2.l, X.l);
+    return X;
+}
+
+// G = E [X - i (kr X + eta')]
+__device__ __forceinline__ void dfl_kernel_value(const DflGeom &G, dd X, const DflConst &K, dd &gr, dd &gi)
+{
+    const float s = fmaf(G.kr.h, X.h, K.eta_m), t = s - K.eta_m;
+    float l = fmaf(G.kr.h, X.h, -t) + K.eta_r;
+    l = fmaf(G.kr.h, X.l, l);
+    l = fmaf(G.kr.l, X.h, l);
+    const dd B = norm({s - K.mb, l});                      // its products with E's low part count
+    gr = add(mul(G.Er, X), mul(G.Ei, B));
+    gi = sub(mul(G.Ei, X), mul(G.Er, B));
+}
+
+// A sum over a tile: integers in units of the tile's finest grid, and the remainders.
+struct DflAcc {
+    int v;
+    float l;
+};
+
+// The grids of a tile: a pair of kernel magnitude |G| rounds its products to the multiples of
+// ulp(m), m = dfl_magic_of(max(|Re G|, |Im G|)) (|sigma'| < 1 / sqrt 2, so |G sigma'| stays in
+// m's binade), but to none finer than `fine`, three binades below the tile's bound of |G|;
+// its mantissas enter the integer sums times mult = ulp(m) / ulp(fine).
+struct DflGrid {
+    float m;
+    int mult;
+};
+
+__device__ __forceinline__ float dfl_fine(float rmin, float kbound, float wmax)
+{
+    const float u = 1.0f / rmin;                           // |G| <= w (1/r) (1/r + 2 pi + |eta'|)
+    return __int_as_float(__float_as_int(dfl_magic_of(1.0001f * wmax * u * (u + kbound))) - (3 << 23));
+}
+
+__device__ __forceinline__ DflGrid dfl_grid(float g, float fine)
+{
+    const int fb = __float_as_int(fine);
+    const int mb = max((__float_as_int(g) & 0x7f800000) + 0x01400000, fb);
+    return {__int_as_float(mb), 1 << ((mb - fb) >> 23)};
+}
+
+// acc += a b + c d on the grid of one pair.  v collects the mantissas of s with those of m in
+// them: the caller subtracts the sum of m's mantissas once for all accumulators (dfl_flush).
+__device__ __forceinline__ void dfl_mac2(DflAcc &acc, dd a, dd b, dd c, dd d, DflGrid g)
+{
+    const float s1 = fmaf(a.h, b.h, g.m), t1 = s1 - g.m, l1 = fmaf(a.h, b.h, -t1);
+    const float s2 = fmaf(c.h, d.h, s1), t2 = s2 - s1, l2 = fmaf(c.h, d.h, -t2);
+    float x = a.h * b.l;
+    x = fmaf(a.l, b.h, x);
+    x = fmaf(c.h, d.l, x);
+    x = fmaf(c.l, d.h, x);
+    acc.v = __float_as_int(s2) * g.mult + acc.v;
+    acc.l += (l1 + l2) + x;
+}
+
+// whole units of the remainders into the integers (|l| stays about one unit)
+__device__ __forceinline__ void dfl_carry(DflAcc &acc, float fine)
+{
+    const float s = acc.l + fine;
+    acc.v += __float_as_int(s) - __float_as_int(fine);
+    acc.l -= s - fine;
+}
+
+// run += sc acc, the tile's sum (v - corr below 2^31, sc a power of two), normalised; acc = 0
+__device__ __forceinline__ dd dfl_flush(dd run, DflAcc &acc, int corr, float ulp, float sc)
+{
+    const float us = ulp * sc;
+    const int v = acc.v - corr;
+    const dd a = two_sum(run.h, __int2float_rn(v & ~255) * us);
+    const dd b = two_sum(a.h, __int2float_rn(v & 255) * us);
+    const dd r = norm({b.h, run.l + fmaf(acc.l, sc, a.l + b.l)});
+    acc = {0, 0.f};
+    return r;
+}
+
+// the power of two that brings values up to the one with these bits below one (and back)
+__device__ __forceinline__ float dfl_up(int bits)
+{
+    const int e = bits >> 23;                              // 0: all zero; 255: not finite
+    return (e < 1 || e > 252) ? 1.0f : __int_as_float((253 - e) << 23);
+}
+__device__ __forceinline__ float dfl_down(int bits)
+{
+    const int e = bits >> 23;
+    return (e < 1 || e > 252) ? 1.0f : __int_as_float((e + 1) << 23);
+}
+__device__ __forceinline__ int dfl_bits(float4 v)          // of sqrt 2 times the modulus, rounded up
+{
+    return __float_as_int(1.4144f * sqrtf(v.x * v.x + v.z * v.z));
+}
+__device__ __forceinline__ float4 dfl_times(float4 v, float s)
+{
+    return make_float4(v.x * s, v.y * s, v.z * s, v.w * s);
+}
+
+// scale of right-hand side r back from sigma' (a power of two)
+__device__ __forceinline__ int dfl_exponent(int key)
+{
+    return key ? min(960, max(-960, (key >> 20) - 1022)) : 0;
+}
+__device__ __forceinline__ double dfl_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// A ball about a tile's sources (x, y, z, radius), by one warp whose lanes hold them.
+__device__ __forceinline__ float4 dfl_ball(float4 a, bool have, int cnt)
+{
+    float x = have ? a.x : 0.f, y = have ? a.y : 0.f, z = have ? a.z : 0.f;
+    for (int o = 16; o > 0; o >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
+        z += __shfl_xor_sync(0xffffffffu, z, o);
+    }
+    const float ic = 1.0f / cnt;
+    x *= ic; y *= ic; z *= ic;
+    const float dx = a.x - x, dy = a.y - y, dz = a.z - z;
+    float r = have ? sqrtf(dx * dx + dy * dy + dz * dz) : 0.f;
+    for (int o = 16; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
+    // rounding of the centre, the radius and the distances measured from it
+    return make_float4(x, y, z, r * 1.0001f + 1e-6f * (fabsf(x) + fabsf(y) + fabsf(z)));
+}
+
+// Lower bound of the distance from a target to a tile's sources: through the ball, or, where
+// the ball is no use (closer than its own size), over the sources.
+__device__ __forceinline__ float dfl_rmin(dd tx, dd ty, dd tz, float4 ball, const float4 *a, const float4 *b, int cnt)
+{
+    const float dx = tx.h - ball.x, dy = ty.h - ball.y, dz = tz.h - ball.z;
+    const float dist = sqrtf(dx * dx + dy * dy + dz * dz) * 0.9999f - 1e-6f * (fabsf(tx.h) + fabsf(ty.h) + fabsf(tz.h));
+    float rm = dist - ball.w;
+    if (rm < 0.5f * dist) {
+        float r2 = 3.0e38f;
+        for (int j = 0; j < cnt; ++j) {
+            const float x = (tx.h - a[j].x) + (tx.l - b[j].x), y = (ty.h - a[j].y) + (ty.l - b[j].y),
+                        z = (tz.h - a[j].z) + (tz.l - b[j].z);
+            r2 = fminf(r2, x * x + y * y + z * z);
+        }
+        rm = 0.999f * sqrtf(r2);
+    }
+    return rm;
+}
+
+// ---------------------------------------------------------------- densities
+
+static const int DFL_SIG_SMALL = 16384;   // N x R up to which one block does both passes
+
+// key[r] = largest high word of |Re|, |Im| of w_j sigma_{j,r} c0 over the finite ones
+__device__ __forceinline__ int dfl_key(double2 v, double w, double c0)
+{
+    const int hx = __double2hiint(v.x) & 0x7fffffff, hy = __double2hiint(v.y) & 0x7fffffff;
+    const int h = __double2hiint(__hiloint2double(max(hx, hy) | 1, 0) * (w * c0));
+    return h < 0x7ff00000 ? h + 1 : 0;                     // + 1: the low words dropped above
+}
+
+__device__ __forceinline__ float4 dfl_sigma(double2 v, double w, double c0, int key)
+{
+    const double sc = dfl_pow2(-dfl_exponent(key)), wq = w * c0;
+    return csplit(make_double2(v.x * wq * sc, v.y * wq * sc));
+}
+
+// grid (blocks, ceil(R / 256)): 256 threads over up to 256 right-hand sides
+__global__ void __launch_bounds__(256)
+dfl_sigma_max_kernel(long long N, int R, const double4 *__restrict__ pos, const double2 *__restrict__ sigma, double c0,
+                     int weighted, int *__restrict__ key)
+{
+    __shared__ int s_key[256];
+    const int cols = min(R - (int)blockIdx.y * 256, 256), rows = 256 / cols;
+    const int c = threadIdx.x % cols, row = threadIdx.x / cols, r = blockIdx.y * 256 + c;
+    s_key[threadIdx.x] = 0;
+    __syncthreads();
+    int m = 0;
+    if (row < rows)
+        for (long long i = (long long)blockIdx.x * rows + row; i < N; i += (long long)gridDim.x * rows)
+            m = max(m, dfl_key(sigma[i * R + r], weighted ? pos[i].w : 1.0, c0));
+    if (m) atomicMax(&s_key[c], m);
+    __syncthreads();
+    if ((int)threadIdx.x < cols && s_key[threadIdx.x]) atomicMax(&key[blockIdx.y * 256 + threadIdx.x], s_key[threadIdx.x]);
+}
+
+__global__ void dfl_sigma_split_kernel(size_t n, int R, const double4 *__restrict__ pos,
+                                       const double2 *__restrict__ sigma, double c0, int weighted,
+                                       const int *__restrict__ key, float4 *__restrict__ out)
+{
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n) out[e] = dfl_sigma(sigma[e], weighted ? pos[e / R].w : 1.0, c0, key[e % R]);
+}
+
+// both passes in one block (R <= 64)
+__global__ void __launch_bounds__(1024)
+dfl_sigma_small_kernel(int n, int R, const double4 *__restrict__ pos, const double2 *__restrict__ sigma, double c0,
+                       int weighted, int *__restrict__ key, float4 *__restrict__ out)
+{
+    __shared__ int s_key[64];
+    if (threadIdx.x < 64) s_key[threadIdx.x] = 0;
+    __syncthreads();
+    for (int e = threadIdx.x; e < n; e += 1024) 
+        atomicMax(&s_key[e % R], dfl_key(sigma[e], weighted ? pos[e / R].w : 1.0, c0));
+    __syncthreads();
+    if ((int)threadIdx.x < R) key[threadIdx.x] = s_key[threadIdx.x];
+    for (int e = threadIdx.x; e < n; e += 1024)
+        out[e] = dfl_sigma(sigma[e], weighted ? pos[e / R].w : 1.0, c0, s_key[e % R]);
+}
+
+__global__ void dfl_nodes_kernel(long long N, const double4 *__restrict__ pos, const double4 *__restrict__ nrm,
+                                 double3 o, double s, float4 *__restrict__ a, float4 *__restrict__ b,
+                                 float4 *__restrict__ cn, float2 *__restrict__ w)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const double4 p = pos[i], n = nrm[i];
+    const dd x = split((p.x - o.x) * s), y = split((p.y - o.y) * s), z = split((p.z - o.z) * s);
+    const dd nx = split(n.x), ny = split(n.y), nz = split(n.z);
+    a[i] = make_float4(x.h, y.h, z.h, nx.h);
+    b[i] = make_float4(x.l, y.l, z.l, nx.l);
+    cn[i] = make_float4(ny.h, nz.h, ny.l, nz.l);
+    const dd wd = split(p.w);
+    w[i] = make_float2(wd.h, wd.l);
+}
+
+// ---------------------------------------------------------------- pair-symmetric kernel
+
 // Source j of a tile, staged in shared memory: position and normal (hi, lo split as
-// in the double-float node arrays) and sigma'_j for RC right-hand sides.
+// in the node arrays) and sigma'_j for RC right-hand sides.
 template <int RC>
 struct DflTile {
     float4 a[DFL_S], b[DFL_S], c[DFL_S];
@@ -73,8 +426,8 @@ template <int RC>
 __global__ void __launch_bounds__(DFL_T, 1)
 nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict__ blocks, int R,
                      const float4 *__restrict__ pa, const float4 *__restrict__ pb, const float4 *__restrict__ pc,
-                     const double4 *__restrict__ pos64, const double2 *__restrict__ sigma,
-                     const float4 *__restrict__ tab, DflConst K, double2 *__restrict__ y, SymSplit sp)
+                     const float4 *__restrict__ sdd, const int *__restrict__ key, const float4 *__restrict__ tab,
+                     DflConst K, double2 *__restrict__ y, SymSplit sp)
 {
     __shared__ DflTile<RC> s_tile[2];                     // double-buffered source tiles
     __shared__ float4 s_tab[DFL_TAB];
@@ -91,21 +444,23 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
     dd tx = {1e5f + tid, 0.f}, ty = {1e5f, 0.f}, tz = {1e5f, 0.f};
     dd mx = {0.f, 0.f}, my = {0.f, 0.f}, mz = {0.f, 0.f};
     dd wr[RC], wi[RC], atr[RC], ati[RC];
+    double scale[RC];
 #pragma unroll
-    for (int c = 0; c < RC; ++c) { wr[c] = wi[c] = atr[c] = ati[c] = {0.f, 0.f}; }
+    for (int c = 0; c < RC; ++c) {
+        wr[c] = wi[c] = atr[c] = ati[c] = {0.f, 0.f};
+        scale[c] = r0 + c < R ? dfl_pow2(dfl_exponent(key[r0 + c])) : 0.0;
+    }
     if (live) {
         const int g = bi.start + tid;
         const float4 A = pa[g], B = pb[g], C = pc[g];
         tx = {A.x, B.x}; ty = {A.y, B.y}; tz = {A.z, B.z};
-        mx = {A.w, B.w}; my = {C.x, C.z}; mz = {C.y, C.w};
-        const double wq = pos64[g].w * 0.07957747154594767;
+        mx = {-A.w, -B.w}; my = {-C.x, -C.z}; mz = {-C.y, -C.w};      // negated: X_2 = -n_i.d / r^2
 #pragma unroll
         for (int c = 0; c < RC; ++c)
             if (r0 + c < R) {
-                const double2 v = sigma[(size_t)g * R + r0 + c];
-                const double vr = v.x * wq, vi = v.y * wq;
-                wr[c] = {(float)vr, (float)(vr - (double)(float)vr)};
-                wi[c] = {(float)vi, (float)(vi - (double)(float)vi)};
+                const float4 v = sdd[(size_t)g * R + r0 + c];
+                wr[c] = {v.x, v.y};
+                wi[c] = {v.z, v.w};
             }
     }
     // the first warp loads the next tile's sources into registers while the tile runs
@@ -115,14 +470,9 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
         if (lane < cnt) {
             const int g = bj.start + j0 + lane;
             na = pa[g]; nb = pb[g]; nc = pc[g];
-            const double wq = pos64[g].w * 0.07957747154594767;
 #pragma unroll
-            for (int c = 0; c < RC; ++c) {
-                const double2 v = (r0 + c < R) ? sigma[(size_t)g * R + r0 + c] : make_double2(0.0, 0.0);
-                const double vr = v.x * wq, vi = v.y * wq;
-                const float hr = (float)vr, hi = (float)vi;
-                ns[c] = make_float4(hr, (float)(vr - (double)hr), hi, (float)(vi - (double)hi));
-            }
+            for (int c = 0; c < RC; ++c)
+                ns[c] = (r0 + c < R) ? sdd[(size_t)g * R + r0 + c] : make_float4(0.f, 0.f, 0.f, 0.f);
         } else {                                           // far, zero density: contributes 0 both ways
             na = make_float4(-1e5f - lane, -1e5f, -1e5f, 0.f);
             nb = nc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -157,42 +507,12 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
         for (int s = st0; s < st1; ++s) {
             const int q = (lane + s) & (DFL_S - 1);
             const float4 A4 = T.a[q], B4 = T.b[q], C4 = T.c[q];
-            // d = x_i - x_j
-            const dd dx = sub(tx, {A4.x, B4.x}), dy = sub(ty, {A4.y, B4.y}), dz = sub(tz, {A4.z, B4.z});
-            // r^2 from exact squares; the sums of the positive squares in fast_two_sum order
-            const float px = dx.h * dx.h, py = dy.h * dy.h, pz = dz.h * dz.h;
-            const float ex = fmaf(dx.h + dx.h, dx.l, fmaf(dx.h, dx.h, -px));
-            const float ey = fmaf(dy.h + dy.h, dy.l, fmaf(dy.h, dy.h, -py));
-            const float ez = fmaf(dz.h + dz.h, dz.l, fmaf(dz.h, dz.h, -pz));
-            const float m1 = fmaxf(px, py), l1 = fminf(px, py);
-            const float s1 = m1 + l1, e1 = l1 - (s1 - m1);
-            const float m2 = fmaxf(s1, pz), l2 = fminf(s1, pz);
-            const float s2 = m2 + l2, e2 = l2 - (s2 - m2);
-            const dd r2 = {s2, (e1 + e2) + ((ex + ey) + ez)};
-            // 1/r: hardware estimate y0, Halley step y0 (1 + e/2 + 3 e^2/8), e = 1 - r^2 y0^2
-            const float y0 = rsqrtf(r2.h);
-            const float q0 = y0 * y0, q0e = fmaf(y0, y0, -q0);
-            const float u = r2.h * q0;
-            const float ue = fmaf(r2.l, q0, fmaf(r2.h, q0e, fmaf(r2.h, q0, -u)));
-            const float e = (1.0f - u) - ue;
-            const dd ir = {y0, y0 * e * fmaf(e, 0.375f, 0.5f)};
-            const dd r = mul(r2, ir);
-            const dd ir2 = mul(ir, ir);
-            const dd kr = mul(K.k, r);
-            dd cs, sn;
-            dfl_cis(mul(K.kt, r), s_tab, K, cs, sn);
-            // E = e^{ikr} / r; G = E [X - i (k r X + eta)] = X P + Q with
-            // P = E (1 - i k r), Q = -i eta E, shared by both directions
-            const dd Er = mul(cs, ir), Ei = mul(sn, ir);
-            const dd Pr = add(Er, mul(Ei, kr)), Pi = sub(Ei, mul(Er, kr));
-            const dd Qr = mul(K.eta, Ei), Qi = neg(mul(K.eta, Er));
+            const DflGeom G = dfl_geom<false>(tx, ty, tz, A4, B4, dd{0.f, 0.f}, s_tab, K);
+            dd g1r, g1i, g2r, g2i;
             // i <- j: normal of source j
-            const dd nx = {A4.w, B4.w}, ny = {C4.x, C4.z}, nz = {C4.y, C4.w};
-            const dd X1 = mul(add(add(mul(nx, dx), mul(ny, dy)), mul(nz, dz)), ir2);
-            const dd g1r = add(mul(X1, Pr), Qr), g1i = add(mul(X1, Pi), Qi);
+            dfl_kernel_value(G, dfl_projection({A4.w, B4.w}, {C4.x, C4.z}, {C4.y, C4.w}, G), K, g1r, g1i);
             // j <- i: normal of target i, d reversed
-            const dd X2 = neg(mul(add(add(mul(mx, dx), mul(my, dy)), mul(mz, dz)), ir2));
-            const dd g2r = add(mul(X2, Pr), Qr), g2i = add(mul(X2, Pi), Qi);
+            dfl_kernel_value(G, dfl_projection(mx, my, mz, G), K, g2r, g2i);
 #pragma unroll
             for (int c = 0; c < RC; ++c) {
                 const float4 S = T.sig[q][c];
@@ -221,8 +541,8 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
             for (int c = 0; c < RC; ++c)
                 if (r0 + c < R) {
                     double2 *o = y + (size_t)(bj.start + j0 + src) * R + r0 + c;
-                    atomicAdd(&o->x, (double)asr[c].h + (double)asr[c].l);
-                    atomicAdd(&o->y, (double)asi[c].h + (double)asi[c].l);
+                    atomicAdd(&o->x, value(asr[c]) * scale[c]);
+                    atomicAdd(&o->y, value(asi[c]) * scale[c]);
                 }
         }
     }
@@ -231,116 +551,164 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
         for (int c = 0; c < RC; ++c)
             if (r0 + c < R) {
                 double2 *o = y + (size_t)(bi.start + tid) * R + r0 + c;
-                atomicAdd(&o->x, (double)atr[c].h + (double)atr[c].l);
-                atomicAdd(&o->y, (double)ati[c].h + (double)ati[c].l);
+                atomicAdd(&o->x, value(atr[c]) * scale[c]);
+                atomicAdd(&o->y, value(ati[c]) * scale[c]);
             }
     }
 }
 
-// One-directional form for several right-hand sides (the refinement residual of a
-// batched solve): one CTA per (TargetBlock part, chunk of RC right-hand sides, source
-// chunk); a CTA of NT threads owns NT targets of a 512-target block (512 / NT CTAs per
-// block), one per thread; sources in tiles of DFL_OT staged in shared memory.  Per
-// ordered pair the geometry, e^{ikr} and the kernel value
-//     G = E [X - i (k r X + eta)],  E = e^{ikr} / r,  X = n_j.d / r^2
-// are formed once and serve the RC right-hand sides (a double-float complex
-// multiply-add each, ~48 FP32 operations against ~240 for the pair), so wide chunks
-// (RC = 16 with 512 threads, RC = 32 with 256 threads and up to 255 registers) repeat
-// the pair work least.  Source chunks write partial sums that a second kernel adds in a
-// fixed order, so the result is bit-reproducible.
-static const int DFL_OT = 64;
+// ---------------------------------------------------------------- one-directional kernel
 
-template <int RC, int NT>
-__global__ void __launch_bounds__(NT, 1)
+// For several right-hand sides: one CTA per (TargetBlock part, chunk of RC right-hand sides,
+// source chunk); a CTA of DFL_NT threads owns DFL_NT targets of a 512-target block, one per
+// thread, each with a grid of its own per tile.  The source chunks divide the sources outside
+// the block's own body, so all CTAs have equal work.  Per ordered pair the geometry,
+// e^{ikr} and the kernel value are formed once and serve the RC right-hand sides, so wide
+// chunks repeat the pair work least; the tile sums (4 RC registers) leave the running sums
+// no registers: they stay in shared memory and are touched once per tile.  Source chunks
+// write partial sums that a second kernel adds in a fixed order, so the result is
+// bit-reproducible.
+template <int RC, bool GRID>
+__global__ void __launch_bounds__(DFL_NT, RC >= 32 ? 1 : 2)
 nbody_dfl_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chunk, const float4 *__restrict__ pa,
-                 const float4 *__restrict__ pb, const float4 *__restrict__ pc, const double4 *__restrict__ pos64,
-                 const double2 *__restrict__ sigma, const float4 *__restrict__ tab, DflConst K,
-                 double2 *__restrict__ y, size_t split_stride)
+                 const float4 *__restrict__ pb, const float4 *__restrict__ pc, const float2 *__restrict__ pw,
+                 const float4 *__restrict__ sdd,
+                 const int *__restrict__ key, const float4 *__restrict__ tab, DflConst K, double2 *__restrict__ y,
+                 size_t split_stride)
 {
-    constexpr int PARTS = DFL_T / NT;
-    constexpr int OT = RC >= 32 ? DFL_OT / 2 : DFL_OT;   // source tile: static shared memory under 48 KB
-    __shared__ float4 s_a[OT], s_b[OT], s_c[OT];
-    __shared__ float4 s_sig[OT][RC];
-    __shared__ float4 s_tab[DFL_TAB];
+    extern __shared__ float4 dfl_smem[];
+    float4 *s_tab = dfl_smem;                              // DFL_TAB
+    float4 *s_sig = s_tab + DFL_TAB;                       // DFL_S x RC
+    float4 *s_a = s_sig + DFL_S * RC, *s_b = s_a + DFL_S, *s_c = s_b + DFL_S;
+    float4 *s_run = s_c + DFL_S;                           // GRID: RC x DFL_NT running sums (re.hi, re.lo, im.hi, im.lo)
+    __shared__ float2 s_w[DFL_S];
+    __shared__ float s_wmax;
+    __shared__ float4 s_ball;
+    __shared__ int s_bits[2][RC];                          // largest high part of a tile's sigma', per column
+    constexpr int LOADS = (DFL_S * RC + DFL_NT - 1) / DFL_NT;
+    constexpr int PARTS = DFL_T / DFL_NT;
     const TargetBlock tb = blocks[blockIdx.x / PARTS];
-    const int t0 = (blockIdx.x % PARTS) * NT;
+    const int t0 = (blockIdx.x % PARTS) * DFL_NT;
+    if (t0 >= tb.count) return;
     const int r0 = blockIdx.y * RC;
-    const int tid = threadIdx.x;
-    for (int q = tid; q < DFL_TAB; q += NT) s_tab[q] = tab[q];
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int q = tid; q < DFL_TAB; q += DFL_NT) s_tab[q] = tab[q];
     const int g0 = tb.start + min(t0 + tid, tb.count - 1);
     const float4 TA = pa[g0], TB = pb[g0];
     const dd tx = {TA.x, TB.x}, ty = {TA.y, TB.y}, tz = {TA.z, TB.z};
-    dd ar[RC], ai[RC];
+    DflAcc ar[RC], ai[RC];                                 // GRID: the tile's sums
+    dd zr[RC], zi[RC];                                     // else the running sums
 #pragma unroll
-    for (int c = 0; c < RC; ++c) ar[c] = ai[c] = {0.f, 0.f};
-    const int c0 = blockIdx.z * chunk, c1 = min(N, c0 + chunk);
-    for (int range = 0; range < 2; ++range) {
-        const int lo = range ? max(c0, tb.excl_hi) : c0;
-        const int hi = range ? c1 : min(c1, tb.excl_lo);
-        for (int j0 = lo; j0 < hi; j0 += OT) {
-            const int cnt = min(OT, hi - j0);
-            __syncthreads();
-            for (int q = tid; q < cnt; q += NT) {
-                const int g = j0 + q;
-                s_a[q] = pa[g];
-                s_b[q] = pb[g];
-                s_c[q] = pc[g];
-                const double wq = pos64[g].w * 0.07957747154594767;
-#pragma unroll
-                for (int c = 0; c < RC; ++c) {
-                    const double2 v = (r0 + c < R) ? sigma[(size_t)g * R + r0 + c] : make_double2(0.0, 0.0);
-                    const double vr = v.x * wq, vi = v.y * wq;
-                    const float hr = (float)vr, hi2 = (float)vi;
-                    s_sig[q][c] = make_float4(hr, (float)(vr - (double)hr), hi2, (float)(vi - (double)hi2));
+    for (int c = 0; c < RC; ++c) {
+        ar[c] = ai[c] = {0, 0.f};
+        zr[c] = zi[c] = {0.f, 0.f};
+        if (GRID) s_run[c * DFL_NT + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (tid < 2 * RC) s_bits[tid / RC][tid % RC] = 0;
+    // sources outside the own body, counted without it
+    const int own = tb.excl_hi - tb.excl_lo;
+    const int c0 = blockIdx.z * chunk, c1 = min(N - own, c0 + chunk);
+    int buf = 0;
+    for (int j0 = c0; j0 < c1; j0 += DFL_S, buf ^= 1) {
+        const int cnt = min(DFL_S, c1 - j0);
+        __syncthreads();
+        if (tid < 32) {
+            const int j = j0 + lane, g = j < tb.excl_lo ? j : j + own;
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (lane < cnt) {
+                a = pa[g];
+                s_a[lane] = a;
+                s_b[lane] = pb[g];
+                s_c[lane] = pc[g];
+            }
+            if (GRID) {
+                const float2 w = lane < cnt ? pw[g] : make_float2(0.f, 0.f);
+                s_w[lane] = w;
+                const float4 ball = dfl_ball(a, lane < cnt, cnt);
+                const int wm = __reduce_max_sync(0xffffffffu, __float_as_int(w.x));
+                if (lane == 0) {
+                    s_ball = ball;
+                    s_wmax = __int_as_float(wm);
                 }
             }
+        }
+        float4 v[LOADS];
+#pragma unroll
+        for (int u = 0; u < LOADS; ++u) {
+            const int e = tid + u * DFL_NT, q = e / RC, c = e % RC, j = j0 + q, g = j < tb.excl_lo ? j : j + own;
+            v[u] = (q < cnt && r0 + c < R) ? sdd[(size_t)g * R + r0 + c] : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (GRID && q < cnt) atomicMax(&s_bits[buf][c], dfl_bits(v[u]));
+        }
+        if (GRID) {
+            if (tid < RC) s_bits[buf ^ 1][tid] = 0;        // for the next tile
             __syncthreads();
-            for (int jj = 0; jj < cnt; ++jj) {
-                const float4 A4 = s_a[jj], B4 = s_b[jj], C4 = s_c[jj];
-                const dd dx = sub(tx, {A4.x, B4.x}), dy = sub(ty, {A4.y, B4.y}), dz = sub(tz, {A4.z, B4.z});
-                const float px = dx.h * dx.h, py = dy.h * dy.h, pz = dz.h * dz.h;
-                const float ex = fmaf(dx.h + dx.h, dx.l, fmaf(dx.h, dx.h, -px));
-                const float ey = fmaf(dy.h + dy.h, dy.l, fmaf(dy.h, dy.h, -py));
-                const float ez = fmaf(dz.h + dz.h, dz.l, fmaf(dz.h, dz.h, -pz));
-                const float m1 = fmaxf(px, py), l1 = fminf(px, py);
-                const float s1 = m1 + l1, e1 = l1 - (s1 - m1);
-                const float m2 = fmaxf(s1, pz), l2 = fminf(s1, pz);
-                const float s2 = m2 + l2, e2 = l2 - (s2 - m2);
-                const dd r2 = {s2, (e1 + e2) + ((ex + ey) + ez)};
-                const float y0 = rsqrtf(r2.h);
-                const float q0 = y0 * y0, q0e = fmaf(y0, y0, -q0);
-                const float u = r2.h * q0;
-                const float ue = fmaf(r2.l, q0, fmaf(r2.h, q0e, fmaf(r2.h, q0, -u)));
-                const float e = (1.0f - u) - ue;
-                const dd ir = {y0, y0 * e * fmaf(e, 0.375f, 0.5f)};
-                const dd r = mul(r2, ir);
-                const dd kr = mul(K.k, r);
-                dd cs, sn;
-                dfl_cis(mul(K.kt, r), s_tab, K, cs, sn);
-                const dd Er = mul(cs, ir), Ei = mul(sn, ir);
-                const dd nx = {A4.w, B4.w}, ny = {C4.x, C4.z}, nz = {C4.y, C4.w};
-                const dd X = mul(add(add(mul(nx, dx), mul(ny, dy)), mul(nz, dz)), mul(ir, ir));
-                const dd Bv = add(mul(kr, X), K.eta);
-                const dd gr = add(mul(Er, X), mul(Ei, Bv)), gi = sub(mul(Ei, X), mul(Er, Bv));
+        }
+#pragma unroll
+        for (int u = 0; u < LOADS; ++u) {                  // GRID: scaled up to 1, column by column
+            const int e = tid + u * DFL_NT;
+            if (e < cnt * RC) s_sig[e] = GRID ? dfl_times(v[u], dfl_up(s_bits[buf][e % RC])) : v[u];
+        }
+        __syncthreads();
+        const float fine =
+            GRID ? dfl_fine(fmaxf(dfl_rmin(tx, ty, tz, s_ball, s_a, s_b, cnt), 0.f), K.kbound, s_wmax) : 0.f;
+        int corr = 0;                                      // the mantissas of the grids in the sums
+        for (int jj = 0; jj < cnt; ++jj) {
+            const float4 A4 = s_a[jj], B4 = s_b[jj], C4 = s_c[jj];
+            const dd w = GRID ? dd{s_w[jj].x, s_w[jj].y} : dd{0.f, 0.f};
+            const DflGeom G = dfl_geom<GRID>(tx, ty, tz, A4, B4, w, s_tab, K);
+            dd gr, gi;
+            dfl_kernel_value(G, dfl_projection({A4.w, B4.w}, {C4.x, C4.z}, {C4.y, C4.w}, G), K, gr, gi);
+            if (GRID) {
+                const DflGrid grid = dfl_grid(fmaxf(fabsf(gr.h), fabsf(gi.h)), fine);
+                corr += __float_as_int(grid.m) * grid.mult;
 #pragma unroll
                 for (int c = 0; c < RC; ++c) {
-                    const float4 S = s_sig[jj][c];
+                    const float4 S = s_sig[jj * RC + c];
+                    dfl_mac2(ar[c], gr, {S.x, S.y}, neg(gi), {S.z, S.w}, grid);
+                    dfl_mac2(ai[c], gr, {S.z, S.w}, gi, {S.x, S.y}, grid);
+                }
+                if ((jj & 3) == 3) {
+#pragma unroll
+                    for (int c = 0; c < RC; ++c) {
+                        dfl_carry(ar[c], fine);
+                        dfl_carry(ai[c], fine);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < RC; ++c) {
+                    const float4 S = s_sig[jj * RC + c];
                     const dd sr = {S.x, S.y}, si = {S.z, S.w};
-                    ar[c] = add(ar[c], sub(mul(gr, sr), mul(gi, si)));
-                    ai[c] = add(ai[c], add(mul(gr, si), mul(gi, sr)));
+                    zr[c] = add(zr[c], sub(mul(gr, sr), mul(gi, si)));
+                    zi[c] = add(zi[c], add(mul(gr, si), mul(gi, sr)));
                 }
             }
+        }
+        const float ulp = dfl_ulp_of(fine);
 #pragma unroll
-            for (int c = 0; c < RC; ++c) { ar[c] = norm(ar[c]); ai[c] = norm(ai[c]); }
+        for (int c = 0; c < RC; ++c) {
+            if (GRID) {
+                const float4 run = s_run[c * DFL_NT + tid];
+                const float down = dfl_down(s_bits[buf][c]);
+                const dd a = dfl_flush({run.x, run.y}, ar[c], corr, ulp, down),
+                         b = dfl_flush({run.z, run.w}, ai[c], corr, ulp, down);
+                s_run[c * DFL_NT + tid] = make_float4(a.h, a.l, b.h, b.l);
+            } else {
+                zr[c] = norm(zr[c]);
+                zi[c] = norm(zi[c]);
+            }
         }
     }
     if (t0 + tid < tb.count) {
         double2 *yo = y + blockIdx.z * split_stride;
 #pragma unroll
         for (int c = 0; c < RC; ++c)
-            if (r0 + c < R)
+            if (r0 + c < R) {
+                const float4 run = GRID ? s_run[c * DFL_NT + tid] : make_float4(zr[c].h, zr[c].l, zi[c].h, zi[c].l);
+                const double sc = dfl_pow2(dfl_exponent(key[r0 + c]));
                 yo[(size_t)(tb.start + t0 + tid) * R + r0 + c] =
-                    make_double2((double)ar[c].h + (double)ar[c].l, (double)ai[c].h + (double)ai[c].l);
+                    make_double2(((double)run.x + (double)run.y) * sc, ((double)run.z + (double)run.w) * sc);
+            }
     }
 }
 
@@ -358,19 +726,28 @@ __global__ void dfl_split_reduce_kernel(size_t n, int nsplit, const double2 *__r
     y[e] = make_double2(sx, sy);
 }
 
-// cos/sin(2 pi m / 1024) split into double-float, built once per context
-static hzb_status ensure_dfl_table(hzb_ctx *c)
+// scaled node arrays and the table of cos/sin(2 pi m / 1024), high parts plus 3 on the grid of
+// ulp(3), built once per context
+static hzb_status ensure_dfl(hzb_ctx *c)
 {
     if (c->dfltab_ready) return HZB_OK;
-    if (check_cuda(c, c->dfltab.ensure(DFL_TAB), "alloc table")) return HZB_ENOMEM;
+    const size_t N = (size_t)c->N;
+    if (check_cuda(c, c->dfltab.ensure(DFL_TAB), "alloc table") || check_cuda(c, c->dla.ensure(N), "alloc nodes") ||
+        check_cuda(c, c->dlb.ensure(N), "alloc nodes") || check_cuda(c, c->dlc.ensure(N), "alloc nodes") ||
+        check_cuda(c, c->dlw.ensure(N), "alloc nodes"))
+        return HZB_ENOMEM;
     std::vector<float4> tab(DFL_TAB);
     for (int q = 0; q < DFL_TAB; ++q) {
         const long double a = 2.0L * 3.14159265358979323846264338327950288L * q / DFL_TAB;
         const double cv = (double)cosl(a), sv = (double)sinl(a);
-        const float ch = (float)cv, sh = (float)sv;
-        tab[q] = make_float4(ch, (float)(cv - (double)ch), sh, (float)(sv - (double)sh));
+        const float ch = (float)(cv + 3.0), sh = (float)(sv + 3.0);
+        tab[q] = make_float4(ch, (float)(cv - ((double)ch - 3.0)), sh, (float)(sv - ((double)sh - 3.0)));
     }
-    if (check_cuda(c, cudaMemcpyAsync(c->dfltab.ptr, tab.data(), DFL_TAB * sizeof(float4), cudaMemcpyHostToDevice,
+    dfl_nodes_kernel<<<(unsigned)((N + 255) / 256), 256, 0, c->stream>>>(
+        c->N, c->pos64.ptr, c->nrm64.ptr, make_double3(c->center[0], c->center[1], c->center[2]),
+        c->k > 0.0 ? c->k / (2.0 * M_PI) : 1.0, c->dla.ptr, c->dlb.ptr, c->dlc.ptr, c->dlw.ptr);
+    if (check_cuda(c, cudaGetLastError(), "dfl_nodes_kernel") ||
+        check_cuda(c, cudaMemcpyAsync(c->dfltab.ptr, tab.data(), DFL_TAB * sizeof(float4), cudaMemcpyHostToDevice,
                                       c->stream), "copy table") ||
         check_cuda(c, cudaStreamSynchronize(c->stream), "table"))
         return HZB_ECUDA;
@@ -387,40 +764,96 @@ static dd dd_of(double v)
 static DflConst dfl_constants(const hzb_ctx *c)
 {
     DflConst K;
-    K.k = dd_of(c->k);
-    K.kt = dd_of(c->k / (2.0 * M_PI));
-    K.twopi = dd_of(2.0 * M_PI);
-    K.eta = dd_of(c->eta);
+    const double s = c->k > 0.0 ? c->k / (2.0 * M_PI) : 1.0, eta = c->eta / s;
+    K.kappa = dd_of(c->k > 0.0 ? 2.0 * M_PI : 0.0);
+    K.eta = dd_of(eta);
+    K.kbound = (float)((2.0 * M_PI + std::fabs(eta)) * 1.0001);
+    int e;
+    std::frexp(K.kbound, &e);                             // kbound < 2^e
+    K.mb = (float)std::ldexp(1.5, e + 1);
+    K.eta_m = (float)(eta + (double)K.mb);
+    K.eta_r = (float)(eta - ((double)K.eta_m - (double)K.mb));
+    K.no_phase = c->k > 0.0 ? 0 : 1;
     return K;
 }
 
-// right-hand sides per CTA of the one-directional kernel
-int dfl_rc(int R) { return R == 1 ? 1 : (R <= 4 ? 4 : (R <= 8 ? 8 : (R <= 16 ? 16 : 32))); }
+// the densities of a call: weighted, scaled to below one per right-hand side, split
+static hzb_status dfl_densities(hzb_ctx *c, int R, const double2 *sigma, int weighted)
+{
+    const size_t n = (size_t)c->N * R;
+    if (check_cuda(c, c->dlsig.ensure(n), "alloc split densities") || check_cuda(c, c->dlkey.ensure(R), "alloc scales"))
+        return HZB_ENOMEM;
+    const double s = c->k > 0.0 ? c->k / (2.0 * M_PI) : 1.0, c0 = s * s / (4.0 * M_PI);
+    if (n <= DFL_SIG_SMALL && R <= 64) {
+        dfl_sigma_small_kernel<<<1, 1024, 0, c->stream>>>((int)n, R, c->pos64.ptr, sigma, c0, weighted,
+                                                          c->dlkey.ptr, c->dlsig.ptr);
+        c->launches += 1;
+    } else {
+        if (check_cuda(c, cudaMemsetAsync(c->dlkey.ptr, 0, R * sizeof(int), c->stream), "clear scales"))
+            return HZB_ECUDA;
+        const unsigned nb = (unsigned)std::min<size_t>((n + 2047) / 2048, 608);
+        dfl_sigma_max_kernel<<<dim3(nb, (R + 255) / 256), 256, 0, c->stream>>>(c->N, R, c->pos64.ptr, sigma, c0,
+                                                                               weighted, c->dlkey.ptr);
+        dfl_sigma_split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, R, c->pos64.ptr, sigma, c0,
+                                                                                   weighted, c->dlkey.ptr, c->dlsig.ptr);
+        c->launches += 2;
+    }
+    return check_cuda(c, cudaGetLastError(), "dfl_sigma_kernel");
+}
 
-// source chunks of the one-directional kernel: about four CTAs per SM in all (one is
-// resident at a time: 512 threads at <= 128 registers, or 256 at <= 255)
-int dfl_default_nsplit(hzb_ctx *c, int R)
+// right-hand sides per CTA of the one-directional kernel
+static int dfl_rc(int R) { return R == 1 ? 1 : (R <= 4 ? 4 : (R <= 8 ? 8 : (R <= 16 ? 16 : 32))); }
+
+// Source chunks of the one-directional kernel: between six and twelve CTAs per resident
+// place, the number whose last wave is fullest.
+static int dfl_nsplit(hzb_ctx *c, int R, int nb)
 {
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->opt.device);
-    const int rc = dfl_rc(R), nt = rc == 32 ? 256 : 512;
-    const long long ctas = std::max<long long>(1, (long long)c->n_tblocks * (DFL_T / nt) * ((R + rc - 1) / rc));
-    const long long ns = (4LL * sms + ctas - 1) / ctas;
-    return (int)std::min<long long>(64, std::max<long long>(1, ns));
+    const int rc = dfl_rc(R);
+    const long long places = (long long)sms * (rc >= 32 ? 1 : 2);
+    const long long ctas = std::max<long long>(1, (long long)nb * (DFL_T / DFL_NT) * ((R + rc - 1) / rc));
+    const long long lo = std::max<long long>(1, 6 * places / ctas), hi = std::max<long long>(1, 12 * places / ctas);
+    long long best = std::min<long long>(lo, 64);
+    double fill = 0.0;
+    for (long long ns = best; ns <= std::min<long long>(hi, 64); ++ns) {
+        const double waves = (double)(ns * ctas) / places, f = waves / std::ceil(waves);
+        if (f > fill + 0.005) { fill = f; best = ns; }
+    }
+    return (int)best;
 }
 
-// one-directional lean double-float sum (R right-hand sides in chunks of 1, 4, 8, 16 or
-// 32, source chunks for occupancy, added in a fixed order); node arrays as for the
-// symmetric form
-hzb_status interbody_dfl(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int nsplit)
+// the most sources that any target has: those outside the smallest body
+static int dfl_sources(const hzb_ctx *c)
 {
-    hzb_status st = ensure_dfl_table(c);
-    if (st) return st;
+    long long n = 1;
+    for (const BodyRec &b : c->bodies) n = std::max<long long>(n, c->N - b.n_nodes);
+    for (const hzb_ctx::RShape &rs : c->rshapes) n = std::max<long long>(n, c->N - rs.k);
+    return (int)n;
+}
+
+// Up to two right-hand sides the pair-symmetric kernel is the faster (4.10 against 5.44 ms at
+// R = 1, 5.30 against 7.77 at R = 2, 29,280 unknowns), from three on the one-directional one
+// (10.5 against 8.6 ms at R = 4), but for short sums, where the launch counts (432 unknowns,
+// R = 4: 33 against 42 us).
+bool dfl_symmetric(const hzb_ctx *c, int R) { return R <= 2 || (R <= 4 && dfl_sources(c) < DFL_GRID_MIN); }
+
+// one-directional lean double-float sum (R right-hand sides in chunks of 1, 4, 8, 16 or
+// 32, source chunks for occupancy, added in a fixed order)
+hzb_status interbody_dfl(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
+{
     const int N = (int)c->N;
     const int rc = dfl_rc(R);
-    int chunk = (N + nsplit - 1) / nsplit;
-    chunk = ((chunk + DFL_OT - 1) / DFL_OT) * DFL_OT;
-    nsplit = (N + chunk - 1) / chunk;
+    const int nb = c->n_tblocks;
+    const int nsrc = dfl_sources(c);
+    // at R <= 4 the sums are a third of the work and the grid's upkeep eats what it saves
+    const bool grid = nsrc >= DFL_GRID_MIN && rc >= 8;
+    hzb_status st = ensure_dfl(c);
+    if (st || (st = dfl_densities(c, R, sigma, grid ? 0 : 1))) return st;
+    int nsplit = dfl_nsplit(c, R, nb);
+    int chunk = (nsrc + nsplit - 1) / nsplit;
+    chunk = ((chunk + DFL_S - 1) / DFL_S) * DFL_S;
+    nsplit = (nsrc + chunk - 1) / chunk;
     const size_t n = (size_t)N * R;
     double2 *out = y;
     if (nsplit > 1) {
@@ -431,55 +864,55 @@ hzb_status interbody_dfl(hzb_ctx *c, int R, const double2 *sigma, double2 *y, in
     c->interbody_calls++;
     c->launches += (nsplit > 1) ? 2 : 1;
     const int slot = prof_begin(c, 2);
-    const int nb = (c->tune_limit_blocks > 0) ? std::min(c->tune_limit_blocks, c->n_tblocks - c->tblock_off)
-                                              : c->n_tblocks - c->tblock_off;
-    const TargetBlock *tb = c->tblocks.ptr + c->tblock_off;
-    auto launch = [&](auto kern, int nt) {
-        dim3 g((unsigned)(nb * (DFL_T / nt)), (R + rc - 1) / rc, nsplit);
-        kern<<<g, nt, 0, c->stream>>>(tb, N, R, chunk, c->dfa.ptr, c->dfb.ptr, c->dfc.ptr, c->pos64.ptr, sigma,
-                                      c->dfltab.ptr, K, out, n);
+    const size_t smem = sizeof(float4) * ((size_t)DFL_TAB + (grid ? (size_t)rc * DFL_NT : 0) + (size_t)DFL_S * (rc + 3));
+    cudaError_t e = cudaSuccess;
+    auto launch = [&](auto kern) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return;
+        dim3 g((unsigned)(nb * (DFL_T / DFL_NT)), (R + rc - 1) / rc, nsplit);
+        kern<<<g, DFL_NT, smem, c->stream>>>(c->tblocks.ptr, N, R, chunk, c->dla.ptr, c->dlb.ptr, c->dlc.ptr,
+                                             c->dlw.ptr, c->dlsig.ptr, c->dlkey.ptr, c->dfltab.ptr, K, out, n);
+        e = cudaGetLastError();
     };
     switch (rc) {
-    case 1: launch(nbody_dfl_kernel<1, 512>, 512); break;
-    case 4: launch(nbody_dfl_kernel<4, 512>, 512); break;
-    case 8: launch(nbody_dfl_kernel<8, 512>, 512); break;
-    case 16: launch(nbody_dfl_kernel<16, 512>, 512); break;
-    default: launch(nbody_dfl_kernel<32, 256>, 256); break;
+    case 1: launch(nbody_dfl_kernel<1, false>); break;
+    case 4: launch(nbody_dfl_kernel<4, false>); break;
+    case 8: grid ? launch(nbody_dfl_kernel<8, true>) : launch(nbody_dfl_kernel<8, false>); break;
+    case 16: grid ? launch(nbody_dfl_kernel<16, true>) : launch(nbody_dfl_kernel<16, false>); break;
+    default: grid ? launch(nbody_dfl_kernel<32, true>) : launch(nbody_dfl_kernel<32, false>); break;
     }
     if (nsplit > 1) dfl_split_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, nsplit, out, y);
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     prof_end(c, slot);
     return check_cuda(c, e, "nbody_dfl_kernel");
 }
 
-// pair-symmetric lean double-float sum; the split node arrays (dfa, dfb, dfc) come from
-// the double-float set-up of nbody_df.cu (ensure_df), which the caller has run
+// pair-symmetric lean double-float sum
 hzb_status interbody_dfl_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
 {
     if (c->capturing && (c->n_blockpairs == 0 || !c->dfltab_ready))
         return fail(c, HZB_ESTATE, "block pairs or table not built before capture");
     hzb_status st = ensure_block_pairs(c);
     if (st) return st;
-    if ((st = ensure_dfl_table(c))) return st;
+    if ((st = ensure_dfl(c))) return st;
     const size_t n = (size_t)c->N * R;
     if (check_cuda(c, cudaMemsetAsync(y, 0, n * sizeof(double2), c->stream), "zero y")) return HZB_ECUDA;
     c->interbody_calls++;
     if (c->n_blockpairs < 0) return HZB_OK;
     if (c->n_blockpairs > 0x7fffffffLL) return fail(c, HZB_EINVAL, "too many block pairs for one launch");
+    if ((st = dfl_densities(c, R, sigma, 1))) return st;
     c->launches += 1;
     const DflConst K = dfl_constants(c);
     const int slot = prof_begin(c, 2);
     const int rc = (R == 1) ? 1 : 2;
     const SymSplit sp = sym_split(c, (R + rc - 1) / rc);
     dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, sp.nz);
-    if (rc == 1)
-        nbody_dfl_sym_kernel<1><<<g, DFL_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->dfa.ptr,
-                                                            c->dfb.ptr, c->dfc.ptr, c->pos64.ptr, sigma,
-                                                            c->dfltab.ptr, K, y, sp);
-    else
-        nbody_dfl_sym_kernel<2><<<g, DFL_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->dfa.ptr,
-                                                            c->dfb.ptr, c->dfc.ptr, c->pos64.ptr, sigma,
-                                                            c->dfltab.ptr, K, y, sp);
+    auto launch = [&](auto kern) {
+        kern<<<g, DFL_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->dla.ptr, c->dlb.ptr, c->dlc.ptr,
+                                         c->dlsig.ptr, c->dlkey.ptr, c->dfltab.ptr, K, y, sp);
+    };
+    if (rc == 1) launch(nbody_dfl_sym_kernel<1>);
+    else launch(nbody_dfl_sym_kernel<2>);
     cudaError_t e = cudaGetLastError();
     prof_end(c, slot);
     return check_cuda(c, e, "nbody_dfl_sym_kernel");
