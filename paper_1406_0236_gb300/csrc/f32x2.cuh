@@ -39,6 +39,7 @@ __device__ __forceinline__ f2x f2_mul(f2x a, f2x b)
     asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
+__device__ __forceinline__ f2x f2_neg(f2x a) { return a ^ 0x8000000080000000ull; }
 // a * b + c
 __device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c)
 {

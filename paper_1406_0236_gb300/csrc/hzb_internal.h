@@ -189,6 +189,8 @@ struct hzb_ctx {
     hzb::DevBuf<float2> nb_part32;
     hzb::DevBuf<int2> blockpairs;              // unordered TargetBlock pairs on different bodies (nbody_sym.cu)
     long long n_blockpairs = 0;                // 0: not built, -1: none (one body)
+    hzb::DevBuf<float4> symn;                  // FP32 pair-symmetric kernel: N scaled positions, then N normals
+    bool sym32_ready = false;
     int nbody64_engine = -1;                   // FP64/double-float sums: -1 auto (pair-symmetric for R <= 4),
                                                // 0 one-directional, 1 pair-symmetric (double-float: lean forms),
                                                // 2 as -1 with the normalised double-float kernels
@@ -292,7 +294,8 @@ hzb_status modal_gemm_tma(hzb_ctx *c, ShapeDev &sd, int ncols, const float2 *X, 
 enum { T5_SPLIT3 = 0, T5_WS = 1, T5_SINGLE = 2 };   // forms of the tcgen05 inter-body kernel
 hzb_status interbody_tc5(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int nsplit,
                          int mode);  // nbody_tc5.cu
-const float2 *weighted_sigma32(hzb_ctx *c, int R, const double2 *sigma);      // nbody.cu; nullptr on failure
+// nbody.cu; f w_j sigma_j / (4 pi) in FP32; nullptr on failure
+const float2 *weighted_sigma32(hzb_ctx *c, int R, const double2 *sigma, double factor = 1.0);
 hzb_status ensure_sctab(hzb_ctx *c);                                          // nbody.cu: FP64 cos/sin table
 hzb_status interbody64_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y);  // nbody_sym.cu
 hzb_status interbody32_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tp);  // nbody_sym.cu

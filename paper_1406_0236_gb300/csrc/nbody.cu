@@ -309,23 +309,24 @@ nbody32x2_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chunk
     }
 }
 
-// sigma'_{j,r} = w_j sigma_{j,r} / (4 pi), formed in FP64 and rounded once to FP32:
-// the FP32 kernels stage it without per-tile FP64 work.
-__global__ void weight_sigma32_kernel(size_t n, int R, const double4 *__restrict__ pos64,
+// sigma'_{j,r} = f w_j sigma_{j,r} / (4 pi) (f = 1 but for the pair-symmetric kernel), formed in
+// FP64 and rounded once to FP32: the FP32 kernels stage it without per-tile FP64 work.
+__global__ void weight_sigma32_kernel(size_t n, int R, double f, const double4 *__restrict__ pos64,
                                       const double2 *__restrict__ sigma, float2 *__restrict__ out)
 {
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
-    const double wq = pos64[e / R].w * HZB_INV4PI;
+    const double wq = pos64[e / R].w * f;
     const double2 v = sigma[e];
     out[e] = make_float2((float)(v.x * wq), (float)(v.y * wq));
 }
 
-const float2 *weighted_sigma32(hzb_ctx *c, int R, const double2 *sigma)
+const float2 *weighted_sigma32(hzb_ctx *c, int R, const double2 *sigma, double factor)
 {
     const size_t n = (size_t)c->N * R;
     if (check_cuda(c, c->sig32.ensure(n), "alloc weighted densities")) return nullptr;
-    weight_sigma32_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, R, c->pos64.ptr, sigma, c->sig32.ptr);
+    weight_sigma32_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, R, factor * HZB_INV4PI, c->pos64.ptr, sigma,
+                                                                          c->sig32.ptr);
     c->launches++;
     return c->sig32.ptr;
 }

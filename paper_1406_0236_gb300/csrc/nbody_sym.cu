@@ -19,6 +19,7 @@
 // the order of the additions into one y entry varies between runs: the result is
 // reproducible to rounding, not bit for bit.
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "f32x2.cuh"
@@ -31,6 +32,18 @@ namespace hzb {
 static const int SYM_T = 512;        // targets per CTA = TargetBlock size
 static const int SYM_S = 32;         // sources per tile (one per lane)
 
+// Constants of the FP64 kernel: phase in table units, normals times nf, densities times wf.
+struct SymConst {
+    double kt, ik, k, eta, nf, wf;
+};
+
+// Whether eta and k leave the scaled forms of the two kernels in range (else GEN).
+static bool sym_scaled(const hzb_ctx *c)
+{
+    const double q = std::fabs(c->eta) / c->k;
+    return c->k >= 1e-6 && q >= 1e-6 && q <= 1e6;
+}
+
 // This CTA's part of its block pair (SymSplit): sources [jlo, jhi) of J and rotation
 // steps [st0, st1) of each of their tiles.
 __device__ __forceinline__ void sym_range(const SymSplit &sp, int nj, int &jlo, int &jhi, int &st0, int &st1)
@@ -42,12 +55,19 @@ __device__ __forceinline__ void sym_range(const SymSplit &sp, int nj, int &jlo, 
     st1 = st0 + SYM_S / sp.nstep;
 }
 
-template <int RC>
+// With E = e^{ikr} / r = a + i b the pair's two kernel values are, up to the common factor eta,
+//     (n~.d) P + b - i a,   P = (1/r) [(a v + b) + i (b v - a)],  v = 1 / (k r),
+// for the normal n~ = (k / eta) n of the source side: P serves both directions, the single
+// layer's part is E itself, and the factor goes into the densities.  50 FP64 operations per
+// unordered pair with one right-hand side (55 with the two layers formed per direction: 31.4 ->
+// 28.3 ms at 29,280 unknowns), 92 % of the FP64 pipe.  GEN: any k and eta, P and E with
+// their factors (k, eta) in place.
+template <int RC, bool GEN>
 __global__ void __launch_bounds__(SYM_T, 1)
 nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict__ blocks, int R,
                    const double4 *__restrict__ pos, const double4 *__restrict__ nrm,
-                   const double2 *__restrict__ sigma, const double2 *__restrict__ sctab, double k, double eta,
-                   double kt, double2 *__restrict__ y, SymSplit sp)
+                   const double2 *__restrict__ sigma, const double2 *__restrict__ sctab, SymConst K,
+                   double2 *__restrict__ y, SymSplit sp)
 {
     __shared__ double4 s_p[SYM_S];               // x, y, z, w
     __shared__ double4 s_n[SYM_S];               // nx, ny, nz
@@ -66,8 +86,9 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
     double2 wi[RC], acc_t[RC];
     if (live) {
         const double4 p = pos[bi.start + tid], n = nrm[bi.start + tid];
-        tx = p.x; ty = p.y; tz = p.z; mx = n.x; my = n.y; mz = n.z;
-        const double wq = p.w * HZB_INV4PI;
+        tx = p.x; ty = p.y; tz = p.z;
+        mx = -K.nf * n.x; my = -K.nf * n.y; mz = -K.nf * n.z;         // negated: d is reversed for j <- i
+        const double wq = p.w * K.wf;
 #pragma unroll
         for (int c = 0; c < RC; ++c) {
             const double2 v = (r0 + c < R) ? sigma[(size_t)(bi.start + tid) * R + r0 + c] : make_double2(0.0, 0.0);
@@ -80,7 +101,6 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
 #pragma unroll
     for (int c = 0; c < RC; ++c) acc_t[c] = make_double2(0.0, 0.0);
     const bool warp_live = warp * 32 < bi.count;
-    const double eta_ = eta;
     for (int j0 = jlo; j0 < jhi; j0 += SYM_S) {
         const int cnt = min(SYM_S, jhi - j0);
         __syncthreads();
@@ -88,8 +108,9 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
             if (tid < cnt) {
                 const double4 p = pos[bj.start + j0 + tid];
                 s_p[tid] = p;
-                s_n[tid] = nrm[bj.start + j0 + tid];
-                const double wq = p.w * HZB_INV4PI;
+                const double4 n = nrm[bj.start + j0 + tid];
+                s_n[tid] = make_double4(K.nf * n.x, K.nf * n.y, K.nf * n.z, 0.0);
+                const double wq = p.w * K.wf;
 #pragma unroll
                 for (int c = 0; c < RC; ++c) {
                     const double2 v =
@@ -116,25 +137,26 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
                 const double dx = tx - p.x, dy = ty - p.y, dz = tz - p.z;
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
                 const double ir = rsqrt_fp64(r2);
-                const double ir2 = ir * ir, eir = eta_ * ir;
                 double sn, cs;
-                cis_turns((r2 * ir) * kt, sctab, cs, sn);
-                // i <- j: normal of source j
-                const double X1 = fma(n.x, dx, fma(n.y, dy, n.z * dz)) * ir2;
-                const double A1 = X1 * ir, B1 = fma(k, X1, eir);
-                const double g1r = fma(cs, A1, sn * B1), g1i = fma(sn, A1, -cs * B1);
-                // j <- i: normal of target i, d reversed (X2 = -X2p)
-                const double X2p = fma(mx, dx, fma(my, dy, mz * dz)) * ir2;
-                const double A2n = X2p * ir, B2 = fma(-k, X2p, eir);
-                const double g2r = fma(-cs, A2n, sn * B2);            // Re K(x_j, x_i) w
-                const double h = fma(sn, A2n, cs * B2);                 // -Im K(x_j, x_i) w
+                cis_turns((r2 * ir) * K.kt, sctab, cs, sn);
+                const double ea = cs * ir, eb = sn * ir;
+                const double v = GEN ? ir : ir * K.ik;
+                const double pr = ir * fma(ea, v, GEN ? K.k * eb : eb);
+                const double pn = ir * fma(-eb, v, GEN ? K.k * ea : ea);        // -Im P
+                const double qb = GEN ? K.eta * eb : eb, qa = GEN ? K.eta * ea : ea;
+                // i <- j: normal of source j; g1n = -Im
+                const double X1 = fma(n.x, dx, fma(n.y, dy, n.z * dz));
+                const double g1r = fma(X1, pr, qb), g1n = fma(X1, pn, qa);
+                // j <- i: normal of target i, d reversed
+                const double X2 = fma(mx, dx, fma(my, dy, mz * dz));
+                const double g2r = fma(X2, pr, qb), g2n = fma(X2, pn, qa);
 #pragma unroll
                 for (int c = 0; c < RC; ++c) {
                     const double2 wj = s_w[q][c];
-                    acc_t[c].x = fma(g1r, wj.x, fma(-g1i, wj.y, acc_t[c].x));
-                    acc_t[c].y = fma(g1r, wj.y, fma(g1i, wj.x, acc_t[c].y));
-                    acc_s[c].x = fma(g2r, wi[c].x, fma(h, wi[c].y, acc_s[c].x));
-                    acc_s[c].y = fma(g2r, wi[c].y, fma(-h, wi[c].x, acc_s[c].y));
+                    acc_t[c].x = fma(g1r, wj.x, fma(g1n, wj.y, acc_t[c].x));
+                    acc_t[c].y = fma(g1r, wj.y, fma(-g1n, wj.x, acc_t[c].y));
+                    acc_s[c].x = fma(g2r, wi[c].x, fma(g2n, wi[c].y, acc_s[c].x));
+                    acc_s[c].y = fma(g2r, wi[c].y, fma(-g2n, wi[c].x, acc_s[c].y));
                 }
                 // the rotating sum of source (l + s + 1) mod 32 comes from lane l + 1
 #pragma unroll
@@ -178,22 +200,23 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
 // each register pair, and meets one source per step as above, so one f32x2
 // instruction serves two unordered node pairs.  The rotating source sums keep the
 // two halves apart and add them at the end of the tile.  Densities come pre-weighted
-// in FP32 (weighted_sigma32).  With E = e^{ikr}/r, both directions' kernels are
-// G = X P + Q, P = E (1 - ikr), Q = -i eta E (X = n.d / r^2 with the source-side normal),
-// so that P and Q, computed once per node pair, leave two FMAs per direction;
-// e^{ikr} comes straight from the transcendental unit (its own argument scaling).
+// in FP32 (weighted_sigma32), positions times k and normals times k / eta (rounded once from
+// FP64, sym32_nodes_kernel), so that r is the phase and v = 1/r: the form of the FP64 kernel
+// in 32 lane operations per unordered pair and right-hand side one, 36 before (36.9 ->
+// 34.9 ms at 258,560 unknowns); e^{ikr} comes straight from the transcendental unit
+// (its own argument scaling).  GEN as in the FP64 kernel, lengths and normals unscaled.
 // One right-hand side with two packed target pairs per thread is held to 80 registers (a
 // few bytes of spills): six 128-thread CTAs per SM (24 warps) hide more of the FMA and
 // transcendental-unit latency than five at 96 registers, four at 120 or seven at 72 with
-// more spills (36.8 / 37.5 / 38.6 / 39.3 ms on 258,560 unknowns).
+// more spills.
 static constexpr int SYM32_MIN_BLOCKS = 6;
 // STEPS = false: all 32 rotation steps, a constant trip count (2 % of the time at 258,560
 // unknowns against the bounds of a split).
-template <int RC, int TP, bool STEPS>
+template <int RC, int TP, bool STEPS, bool GEN>
 __global__ void __launch_bounds__(SYM_T / (2 * TP), (RC == 1 && TP == 2) ? SYM32_MIN_BLOCKS : 1)
 nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict__ blocks, int R,
                    const float4 *__restrict__ pos, const float4 *__restrict__ nrm, const float2 *__restrict__ sw,
-                   float k, float eta, float kt, double2 *__restrict__ y, SymSplit sp)
+                   float k, float eta, double2 *__restrict__ y, SymSplit sp)
 {
     constexpr int NT = SYM_T / (2 * TP);
     constexpr int NW = NT / 32;
@@ -210,7 +233,7 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
     const int r0 = blockIdx.y * RC;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     f2x tx[TP], ty[TP], tz[TP], mx[TP], my[TP], mz[TP];      // target positions, negated normals
-    f2x wr[TP][RC], wi[TP][RC], nwi[TP][RC], atx[TP][RC], aty[TP][RC];
+    f2x wr[TP][RC], wi[TP][RC], nwr[TP][RC], atx[TP][RC], aty[TP][RC];
 #pragma unroll
     for (int p = 0; p < TP; ++p) {
         float4 P[2], Q[2];
@@ -231,12 +254,12 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
         for (int c = 0; c < RC; ++c) {
             wr[p][c] = f2_pack(V[0][c].x, V[1][c].x);
             wi[p][c] = f2_pack(V[0][c].y, V[1][c].y);
-            nwi[p][c] = f2_pack(-V[0][c].y, -V[1][c].y);
+            nwr[p][c] = f2_pack(-V[0][c].x, -V[1][c].x);
             atx[p][c] = aty[p][c] = 0ull;
         }
     }
     const bool warp_live = warp * 32 < bi.count;
-    const f2x k2 = f2_splat(k), nk2 = f2_splat(-k), eta2 = f2_splat(eta), neta2 = f2_splat(-eta);
+    const f2x k2 = f2_splat(k), eta2 = f2_splat(eta);
     for (int j0 = jlo; j0 < jhi; j0 += SYM_S) {
         const int cnt = min(SYM_S, jhi - j0);
         __syncthreads();
@@ -267,11 +290,11 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
                 const float2 g1 = s_g1[q];
                 const f2x sx = f2_splat(g0.x), sy = f2_splat(g0.y), sz = f2_splat(g0.z);
                 const f2x snx = f2_splat(g0.w), sny = f2_splat(g1.x), snz = f2_splat(g1.y);
-                f2x swr[RC], swi[RC], nswi[RC];
+                f2x swr[RC], swi[RC], nswr[RC];
 #pragma unroll
                 for (int c = 0; c < RC; ++c) {
                     const float2 v = s_w[q][c];
-                    swr[c] = f2_splat(v.x); swi[c] = f2_splat(v.y); nswi[c] = f2_splat(-v.y);
+                    swr[c] = f2_splat(v.x); swi[c] = f2_splat(v.y); nswr[c] = f2_splat(-v.x);
                 }
 #pragma unroll
                 for (int p = 0; p < TP; ++p) {
@@ -280,32 +303,29 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
                     float r2a, r2b;
                     f2_unpack(r2, r2a, r2b);
                     const f2x ir = f2_pack(rsqrtf(r2a), rsqrtf(r2b));
-                    const f2x ir2 = f2_mul(ir, ir);
-                    const f2x r = f2_mul(r2, ir);
-                    const f2x kr = f2_mul(r, k2), nkr = f2_mul(r, nk2);
+                    const f2x kr = GEN ? f2_mul(f2_mul(r2, ir), k2) : f2_mul(r2, ir);
                     // e^{ikr}: the transcendental unit reduces the argument itself (its
                     // scaling to turns rounds like an explicit reduction would)
                     float kra, krb, sa, ca, sb, cb;
                     f2_unpack(kr, kra, krb);
                     __sincosf(kra, &sa, &ca);
                     __sincosf(krb, &sb, &cb);
-                    // E = e^{ikr} / r;  G = E [X - i (k r X + eta)] = X P + Q,
-                    // P = E (1 - i k r), Q = -i eta E: shared by both directions
-                    const f2x Er = f2_mul(f2_pack(ca, cb), ir), Ei = f2_mul(f2_pack(sa, sb), ir);
-                    const f2x Pr = f2_fma(Ei, kr, Er), Pi = f2_fma(Er, nkr, Ei);
-                    const f2x Qr = f2_mul(eta2, Ei), Qi = f2_mul(neta2, Er);
-                    // target <- source q: X1 = n_q.d / r^2
-                    const f2x X1 = f2_mul(f2_fma(snx, dx, f2_fma(sny, dy, f2_mul(snz, dz))), ir2);
-                    const f2x g1r = f2_fma(X1, Pr, Qr), g1i = f2_fma(X1, Pi, Qi);
-                    // source q <- target (d reversed): X2 = -m.d / r^2 (the target normals are stored negated)
-                    const f2x X2 = f2_mul(f2_fma(mx[p], dx, f2_fma(my[p], dy, f2_mul(mz[p], dz))), ir2);
-                    const f2x g2r = f2_fma(X2, Pr, Qr), g2i = f2_fma(X2, Pi, Qi);
+                    const f2x ea = f2_mul(f2_pack(ca, cb), ir), eb = f2_mul(f2_pack(sa, sb), ir);
+                    const f2x pr = f2_mul(ir, f2_fma(ea, ir, GEN ? f2_mul(k2, eb) : eb));
+                    const f2x pn = f2_mul(ir, f2_fma(f2_neg(eb), ir, GEN ? f2_mul(k2, ea) : ea));     // -Im P
+                    const f2x qb = GEN ? f2_mul(eta2, eb) : eb, qa = GEN ? f2_mul(eta2, ea) : ea;
+                    // target <- source q; g1n = -Im
+                    const f2x X1 = f2_fma(snx, dx, f2_fma(sny, dy, f2_mul(snz, dz)));
+                    const f2x g1r = f2_fma(X1, pr, qb), g1n = f2_fma(X1, pn, qa);
+                    // source q <- target, d reversed (the target normals are stored negated)
+                    const f2x X2 = f2_fma(mx[p], dx, f2_fma(my[p], dy, f2_mul(mz[p], dz)));
+                    const f2x g2r = f2_fma(X2, pr, qb), g2n = f2_fma(X2, pn, qa);
 #pragma unroll
                     for (int c = 0; c < RC; ++c) {
-                        atx[p][c] = f2_fma(g1r, swr[c], f2_fma(g1i, nswi[c], atx[p][c]));
-                        aty[p][c] = f2_fma(g1r, swi[c], f2_fma(g1i, swr[c], aty[p][c]));
-                        asx[c] = f2_fma(g2r, wr[p][c], f2_fma(g2i, nwi[p][c], asx[c]));
-                        asy[c] = f2_fma(g2r, wi[p][c], f2_fma(g2i, wr[p][c], asy[c]));
+                        atx[p][c] = f2_fma(g1r, swr[c], f2_fma(g1n, swi[c], atx[p][c]));
+                        aty[p][c] = f2_fma(g1r, swi[c], f2_fma(g1n, nswr[c], aty[p][c]));
+                        asx[c] = f2_fma(g2r, wr[p][c], f2_fma(g2n, wi[p][c], asx[c]));
+                        asy[c] = f2_fma(g2r, wi[p][c], f2_fma(g2n, nwr[p][c], asy[c]));
                     }
                 }
 #pragma unroll
@@ -422,30 +442,56 @@ hzb_status interbody64_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     const int rc = (R == 1) ? 1 : (R == 2 ? 2 : 4);
     const SymSplit sp = sym_split(c, (R + rc - 1) / rc);
     dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, sp.nz);
-    const double kt = c->k * (SC_N / (2.0 * M_PI));
-    if (rc == 1)
-        nbody64_sym_kernel<1><<<g, SYM_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos64.ptr,
-                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y, sp);
-    else if (rc == 2)
-        nbody64_sym_kernel<2><<<g, SYM_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos64.ptr,
-                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y, sp);
-    else
-        nbody64_sym_kernel<4><<<g, SYM_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos64.ptr,
-                                                          c->nrm64.ptr, sigma, c->sctab.ptr, c->k, c->eta, kt, y, sp);
+    const bool gen = !sym_scaled(c);
+    const SymConst K = {c->k * (SC_N / (2.0 * M_PI)), gen ? 0.0 : 1.0 / c->k, c->k, c->eta,
+                        gen ? 1.0 : c->k / c->eta, (gen ? 1.0 : c->eta) * HZB_INV4PI};
+    auto launch = [&](auto kern) {
+        kern<<<g, SYM_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos64.ptr, c->nrm64.ptr, sigma,
+                                         c->sctab.ptr, K, y, sp);
+    };
+    if (rc == 1) gen ? launch(nbody64_sym_kernel<1, true>) : launch(nbody64_sym_kernel<1, false>);
+    else if (rc == 2) gen ? launch(nbody64_sym_kernel<2, true>) : launch(nbody64_sym_kernel<2, false>);
+    else gen ? launch(nbody64_sym_kernel<4, true>) : launch(nbody64_sym_kernel<4, false>);
     cudaError_t e = cudaGetLastError();
     prof_end(c, slot);
     return check_cuda(c, e, "nbody64_sym_kernel");
+}
+
+// positions relative to the centre and normals of the FP32 kernel, scaled (see there)
+__global__ void sym32_nodes_kernel(long long N, const double4 *__restrict__ pos, const double4 *__restrict__ nrm,
+                                   double3 o, double ps, double ns, float4 *__restrict__ p32, float4 *__restrict__ n32)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const double4 p = pos[i], n = nrm[i];
+    p32[i] = make_float4((float)((p.x - o.x) * ps), (float)((p.y - o.y) * ps), (float)((p.z - o.z) * ps), 0.f);
+    n32[i] = make_float4((float)(n.x * ns), (float)(n.y * ns), (float)(n.z * ns), 0.f);
+}
+
+static hzb_status ensure_sym32(hzb_ctx *c)
+{
+    if (c->sym32_ready) return HZB_OK;
+    if (c->capturing) return fail(c, HZB_ESTATE, "scaled nodes not built before capture");
+    if (check_cuda(c, c->symn.ensure(2 * (size_t)c->N), "alloc scaled nodes")) return HZB_ENOMEM;
+    const bool gen = !sym_scaled(c);
+    sym32_nodes_kernel<<<(unsigned)((c->N + 255) / 256), 256, 0, c->stream>>>(
+        c->N, c->pos64.ptr, c->nrm64.ptr, make_double3(c->center[0], c->center[1], c->center[2]), gen ? 1.0 : c->k,
+        gen ? 1.0 : c->k / c->eta, c->symn.ptr, c->symn.ptr + c->N);
+    if (check_cuda(c, cudaGetLastError(), "sym32_nodes_kernel")) return HZB_ECUDA;
+    c->sym32_ready = true;
+    return HZB_OK;
 }
 
 template <int RC, int TP>
 static void launch_sym32(hzb_ctx *c, dim3 g, int R, const float2 *sw, double2 *y, SymSplit sp)
 {
     auto launch = [&](auto kern) {
-        kern<<<g, SYM_T / (2 * TP), 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->pos32.ptr, c->nrm32.ptr, sw,
-                                                    (float)c->k, (float)c->eta, (float)(c->k / (2.0 * M_PI)), y, sp);
+        kern<<<g, SYM_T / (2 * TP), 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->symn.ptr, c->symn.ptr + c->N, sw,
+                                                    (float)c->k, (float)c->eta, y, sp);
     };
-    if (sp.nstep > 1) launch(nbody32_sym_kernel<RC, TP, true>);
-    else launch(nbody32_sym_kernel<RC, TP, false>);
+    const bool gen = !sym_scaled(c);
+    if (sp.nstep > 1) gen ? launch(nbody32_sym_kernel<RC, TP, true, true>) : launch(nbody32_sym_kernel<RC, TP, true, false>);
+    else gen ? launch(nbody32_sym_kernel<RC, TP, false, true>) : launch(nbody32_sym_kernel<RC, TP, false, false>);
 }
 
 hzb_status interbody32_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tp)
@@ -453,14 +499,14 @@ hzb_status interbody32_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y, 
     if (!c->nodes_ready) return fail(c, HZB_ESTATE, "nodes not built");
     if (c->capturing && c->n_blockpairs == 0) return fail(c, HZB_ESTATE, "block pairs not built before capture");
     hzb_status st = ensure_block_pairs(c);
-    if (st) return st;
+    if (st || (st = ensure_sym32(c))) return st;
     const size_t n = (size_t)c->N * R;
     if (check_cuda(c, cudaMemsetAsync(y, 0, n * sizeof(double2), c->stream), "zero y")) return HZB_ECUDA;
     c->interbody_calls++;
     if (c->n_blockpairs < 0) return HZB_OK;
     if (c->n_blockpairs > 0x7fffffffLL) return fail(c, HZB_EINVAL, "too many block pairs for one launch");
     const int slot = prof_begin(c, 1);
-    const float2 *sw = weighted_sigma32(c, R, sigma);
+    const float2 *sw = weighted_sigma32(c, R, sigma, sym_scaled(c) ? c->k * c->eta : 1.0);
     if (!sw) return HZB_ENOMEM;
     c->launches += 1;
     const int rc = (R == 1) ? 1 : (R == 2 ? 2 : 4);

@@ -37,3 +37,20 @@ def test_shared_block_pairs(size, R):
         assert rel_l2(s.interbody(sig, precision=1), ref) < 2e-6
     finally:
         s.set_interbody_engine(-1)
+
+
+@pytest.mark.parametrize("k,eta", [(0.0, 1.5), (2.5, 0.0), (1e-9, 1.0), (3.0, 1e-9), (2.5, -2.5)])
+def test_every_wave_and_coupling(k, eta):
+    """The kernels scale lengths and normals by k and k / eta where both are in range; the
+    others, a static kernel and a pure double layer among them, take the unscaled form."""
+    require_gpu()
+    from oracle import Problem
+    from paper_1406_0236_gb300 import Options, Solver
+    wl = W.two_spheres(n_panels=4, gl_order=7, n_modes=13, k=k, eta=eta)
+    s, P = Solver.from_workload(wl, Options()), Problem(wl)
+    for R in (1, 2, 4):
+        sig = rand_c((P.N, R), 91 + R)
+        ref = P.interbody(sig)
+        s.set_interbody_engine(4)
+        assert np.abs(s.interbody(sig) - ref).max() < 1e-12 * np.abs(ref).max(), R
+        assert rel_l2(s.interbody(sig, precision=1), ref) < 2e-6, R
