@@ -38,7 +38,7 @@ struct SymConst {
 };
 
 // Whether eta and k leave the scaled forms of the two kernels in range (else GEN).
-static bool sym_scaled(const hzb_ctx *c)
+bool sym_scaled(const hzb_ctx *c)
 {
     const double q = std::fabs(c->eta) / c->k;
     return c->k >= 1e-6 && q >= 1e-6 && q <= 1e6;
@@ -203,13 +203,12 @@ nbody64_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
 // in FP32 (weighted_sigma32), positions times k and normals times k / eta (rounded once from
 // FP64, sym32_nodes_kernel), so that r is the phase and v = 1/r: the form of the FP64 kernel
 // in 32 lane operations per unordered pair and right-hand side one, 36 before (36.9 ->
-// 34.9 ms at 258,560 unknowns); e^{ikr} comes straight from the transcendental unit
+// 34.1 ms at 258,560 unknowns); e^{ikr} comes straight from the transcendental unit
 // (its own argument scaling).  GEN as in the FP64 kernel, lengths and normals unscaled.
-// One right-hand side with two packed target pairs per thread is held to 80 registers (a
-// few bytes of spills): six 128-thread CTAs per SM (24 warps) hide more of the FMA and
-// transcendental-unit latency than five at 96 registers, four at 120 or seven at 72 with
-// more spills.
-static constexpr int SYM32_MIN_BLOCKS = 6;
+// One right-hand side with two packed target pairs per thread is held to 96 registers, five
+// 128-thread CTAs per SM, with four steps unrolled: 64,640 unknowns 2.19 ms, against 2.27 for
+// six CTAs at 80 registers and two steps, 2.23 for four CTAs, 2.22 for six and 2.41 for seven.
+static constexpr int SYM32_MIN_BLOCKS = 5;
 // STEPS = false: all 32 rotation steps, a constant trip count (2 % of the time at 258,560
 // unknowns against the bounds of a split).
 template <int RC, int TP, bool STEPS, bool GEN>
@@ -283,7 +282,7 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
 #pragma unroll
         for (int c = 0; c < RC; ++c) asx[c] = asy[c] = 0ull;
         if (warp_live) {
-#pragma unroll 2
+#pragma unroll 4
             for (int s = st0; s < st1; ++s) {
                 const int q = (lane + s) & (SYM_S - 1);
                 const float4 g0 = s_g0[q];
@@ -468,7 +467,7 @@ __global__ void sym32_nodes_kernel(long long N, const double4 *__restrict__ pos,
     n32[i] = make_float4((float)(n.x * ns), (float)(n.y * ns), (float)(n.z * ns), 0.f);
 }
 
-static hzb_status ensure_sym32(hzb_ctx *c)
+hzb_status ensure_sym32(hzb_ctx *c)
 {
     if (c->sym32_ready) return HZB_OK;
     if (c->capturing) return fail(c, HZB_ESTATE, "scaled nodes not built before capture");
