@@ -266,14 +266,17 @@ hzb_status hzb_set_modal_engine(hzb_ctx *ctx, int engine);
  * 2 = CUDA cores, scalar FP32 kernel; 3 = CUDA cores, packed-pair kernel (two sources
  * per f32x2 instruction); 4 = CUDA cores, pair-symmetric packed kernel (each unordered
  * node pair evaluated once for both directions, results added with FP64 atomics: equal
- * to rounding between runs, not bit for bit); 5 = tensor cores through tcgen05 (TF32
- * three-term split, accumulators in tensor memory, 16 or 32 right-hand sides per CTA);
+ * to rounding between runs, not bit for bit); 5 = tensor cores through tcgen05 (FP16
+ * three-term split with scaled operands, the pair kernels and the accumulators in tensor
+ * memory, 16 or 32 right-hand sides per CTA; a TF32 three-term split where the kernels of
+ * the geometry span more than FP16's range, or k or eta is zero);
  * 6 = the same contraction as a warp-specialised pipeline (producer, MMA and epilogue
  * warps synchronised by mbarriers, two operand stages, two accumulators);
- * 7 = engine 5 with single-term TF32 products (no hi/lo split: about 3e-4 relative
- * error in the sum instead of ~3e-6, about 1.4x faster; only ever chosen here, never by
- * the default or the autotuner, for inner solves whose refinement absorbs it);
- * -1 (default) = tcgen05 tensor cores when R >= 16, else as 0, unless hzb_autotune
+ * 7 = the TF32 form with single-term products (no hi/lo split: about 3e-4 relative
+ * error in the sum instead of ~3e-6; only ever chosen here, never by the default or the
+ * autotuner);
+ * -1 (default) = tcgen05 tensor cores from R = 5 on where N^2 R >= 6e8 and from R = 9 on where
+ * N^2 R >= 3e8, else the CUDA cores (pair-symmetric up to R = 4), unless hzb_autotune
  * timed the engines for this R.  Returns HZB_EINVAL for other values. */
 hzb_status hzb_set_interbody_engine(hzb_ctx *ctx, int engine);
 

@@ -142,7 +142,7 @@ hzb_status hzb_destroy(hzb_ctx *c)
     c->red.release(); c->krylov.release(); c->small.release();
     c->sctab.release(); c->nb_part64.release(); c->nb_part32.release(); c->sig32.release(); c->blockpairs.release(); c->kerr.release(); c->Ximg.release();
     c->dfa.release(); c->dfb.release(); c->dfc.release(); c->dftab.release(); c->nodecheck.release();
-    c->dfltab.release(); c->dla.release(); c->dlb.release(); c->dlc.release(); c->symn.release(); c->dlsig.release(); c->dlw.release(); c->dlkey.release();
+    c->dfltab.release(); c->dla.release(); c->dlb.release(); c->dlc.release(); c->symn.release(); c->t5h_tiles.release(); c->t5h_src.release(); c->t5h_img.release(); c->dlsig.release(); c->dlw.release(); c->dlkey.release();
     if (c->host_pinned) cudaFreeHost(c->host_pinned);
     release_graphs(c);
     for (cudaEvent_t e : c->evpool) cudaEventDestroy(e);
@@ -563,14 +563,8 @@ hzb_status hzb_autotune(hzb_ctx *c, int R, int which, double best_ms[2])
 hzb_status hzb_tuned_config(const hzb_ctx *c, int R, int out[6])
 {
     if (!c || !out) return HZB_EINVAL;
-    // the FP32 engine interbody32 takes for R right-hand sides
-    int e = -1;
-    if (c->nbody_engine == 1) e = 1;
-    else if (c->nbody_engine == 5 || c->nbody_engine == 6) e = 2;
-    else if (c->nbody_engine < 0) e = (c->tune32_tc >= 0 && c->tune32_tc_R == R) ? c->tune32_tc : (R >= 16 ? 2 : 0);
-    int v = (c->tune32_x2 >= 0 && c->tune32_R == R) ? c->tune32_x2 : (R <= 2 ? 2 : 1);
-    if (c->nbody_engine >= 2 && c->nbody_engine <= 4) v = c->nbody_engine - 2;
-    out[0] = e == 2 ? 4 : (e == 1 ? 3 : v);
+    const int e = fp32_engine(c, R);          // as interbody32 takes it
+    out[0] = e >= 2 ? 4 : (e == 1 ? 3 : fp32_variant(c, R));
     out[1] = c->tune32_tpt;
     out[2] = c->tune32_split;
     out[3] = (c->nbody64_engine >= 1 || (c->nbody64_engine < 0 && R <= 4)) ? 1 : 0;

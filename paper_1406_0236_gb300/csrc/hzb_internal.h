@@ -191,6 +191,13 @@ struct hzb_ctx {
     long long n_blockpairs = 0;                // 0: not built, -1: none (one body)
     hzb::DevBuf<float4> symn;                  // FP32 pair-symmetric kernel: N scaled positions, then N normals
     bool sym32_ready = false;
+    // FP16 tensor-core form (nbody_t5h.cu): 0 not built, 1 usable, -1 out of FP16's range; tiles of 32
+    // sources of one body, the target blocks' own tiles, the tiles' geometry, operand images of a call
+    int t5h_state = 0, t5h_ntiles = 0, t5h_most = 0, t5h_ctas = 0;
+    double t5h_scale = 0.0;
+    hzb::DevBuf<int2> t5h_tiles;
+    hzb::DevBuf<float> t5h_src;
+    hzb::DevBuf<unsigned char> t5h_img;
     int nbody64_engine = -1;                   // FP64/double-float sums: -1 auto (pair-symmetric for R <= 4),
                                                // 0 one-directional, 1 pair-symmetric (double-float: lean forms),
                                                // 2 as -1 with the normalised double-float kernels
@@ -285,6 +292,8 @@ hzb_status build_shape_matrices(hzb_ctx *c, ShapeDev &s);
 // nbody.cu: y = B sigma; sigma, y device N x R complex FP64 (FP32 path converts internally)
 hzb_status interbody64(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
 hzb_status interbody32(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
+int fp32_engine(const hzb_ctx *c, int R);
+int fp32_variant(const hzb_ctx *c, int R);
 hzb_status interbody_df(hzb_ctx *c, int R, const double2 *sigma, double2 *y);   // nbody_df.cu
 hzb_status interbody_dfl_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y);   // nbody_dfl.cu
 hzb_status interbody_dfl(hzb_ctx *c, int R, const double2 *sigma, double2 *y);       // nbody_dfl.cu
@@ -292,6 +301,15 @@ bool dfl_symmetric(const hzb_ctx *c, int R);                                    
 hzb_status interbody_tc(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int nsplit);
 hzb_status modal_gemm_tma(hzb_ctx *c, ShapeDev &sd, int ncols, const float2 *X, float2 *Cout);  // modal_tma.cu
 enum { T5_SPLIT3 = 0, T5_WS = 1, T5_SINGLE = 2 };   // forms of the tcgen05 inter-body kernel
+// nbody_t5h.cu: FP16 three-term form, where the geometry's kernels fit FP16's range
+bool t5h_usable(hzb_ctx *c, hzb_status *st);
+hzb_status interbody_t5h(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
+// nbody_tc5.cu: the device flag of the tensor-core kernels' bounded waits, around a launch
+hzb_status tc_flag_begin(hzb_ctx *c, bool inject);
+hzb_status tc_flag_end(hzb_ctx *c, const char *kernel);
+hzb_status sigma_keys(hzb_ctx *c, int R, const double2 *sigma, double c0, int weighted, int *key);   // nbody_dfl.cu
+bool sym_scaled(const hzb_ctx *c);              // nbody_sym.cu: k and eta leave the scaled pair kernels in range
+hzb_status ensure_sym32(hzb_ctx *c);            // nbody_sym.cu: symn
 hzb_status interbody_tc5(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int nsplit,
                          int mode);  // nbody_tc5.cu
 // nbody.cu; f w_j sigma_j / (4 pi) in FP32; nullptr on failure

@@ -524,27 +524,48 @@ hzb_status interbody64(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     return interbody64_cfg(c, R, sigma, y, tpt, ns);
 }
 
+// Engine of the FP32 sum: 0 CUDA cores, 1 mma.sync, 2 tcgen05, 3 tcgen05 warp-specialised, 4
+// tcgen05 with single-term TF32 products (opt-in only).  On automatic the tensor cores (FP16
+// form) take five and more right-hand sides once the pair work outweighs their larger
+// set-up, against the packed CUDA-core kernel: R = 8 at 29,280 unknowns 0.96 against 1.42 ms, at
+// 8,200 124 against 120 us; R = 12 at 8,200 127 against 203 us; R = 16 at 432 61 against 33 us.
+int fp32_engine(const hzb_ctx *c, int R)
+{
+    if (c->nbody_engine == 1) return 1;
+    if (c->nbody_engine >= 5 && c->nbody_engine <= 7) return c->nbody_engine - 3;
+    if (c->nbody_engine >= 0) return 0;
+    if (c->tune32_tc >= 0 && c->tune32_tc_R == R) return c->tune32_tc;
+    const double work = (double)c->N * (double)c->N * R;
+    if (R >= 16 && c->t5h_state < 0) return 2;         // TF32 form
+    return c->t5h_state >= 0 && ((R >= 5 && work >= 6e8) || (R >= 9 && work >= 3e8)) ? 2 : 0;
+}
+
+// Kernel of the CUDA-core engine: 0 scalar, 1 packed pairs, 2 pair-symmetric packed (up to four
+// right-hand sides: 0.78 against 0.90 ms at R = 4, 29,280 unknowns).
+int fp32_variant(const hzb_ctx *c, int R)
+{
+    if (c->nbody_engine >= 2 && c->nbody_engine <= 4) return c->nbody_engine - 2;
+    return (c->tune32_x2 >= 0 && c->tune32_R == R) ? c->tune32_x2 : (R <= 4 ? 2 : 1);
+}
+
 hzb_status interbody32(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
 {
-    // many right-hand sides: contraction on the tensor cores, tcgen05 (nbody_tc5.cu) or
-    // mma.sync (nbody_tc.cu); engine choice 0 CUDA cores, 1 mma.sync, 2 tcgen05, 3 tcgen05
-    // warp-specialised, 4 tcgen05 with single-term TF32 products (opt-in only)
-    int e = -1;
-    if (c->nbody_engine == 1) e = 1;
-    else if (c->nbody_engine == 5) e = 2;
-    else if (c->nbody_engine == 6) e = 3;
-    else if (c->nbody_engine == 7) e = 4;
-    else if (c->nbody_engine < 0) e = (c->tune32_tc >= 0 && c->tune32_tc_R == R) ? c->tune32_tc : (R >= 16 ? 2 : 0);
-    if (e >= 2 && e <= 4)
+    const int e = fp32_engine(c, R);
+    if (e == 2) {
+        hzb_status st;
+        if (t5h_usable(c, &st)) return interbody_t5h(c, R, sigma, y);
+        if (st) return st;
+    }
+    // the range of the FP16 form is known only now: few right-hand sides stay on the CUDA cores
+    const bool late = e == 2 && c->nbody_engine < 0 && R < 16 && !(c->tune32_tc >= 0 && c->tune32_tc_R == R);
+    if (e >= 2 && !late)
         return interbody_tc5(c, R, sigma, y, default_nsplit_tc5(c, R),
                              e == 2 ? T5_SPLIT3 : (e == 3 ? T5_WS : T5_SINGLE));
     if (e == 1) {
         int ns = c->tunetc_split > 0 ? c->tunetc_split : default_nsplit_tc(c, R);
         return interbody_tc(c, R, sigma, y, ns);
     }
-    // CUDA cores: variant 0 scalar, 1 packed pairs, 2 pair-symmetric packed
-    int v = (c->tune32_x2 >= 0 && c->tune32_R == R) ? c->tune32_x2 : (R <= 2 ? 2 : 1);
-    if (c->nbody_engine >= 2 && c->nbody_engine <= 4) v = c->nbody_engine - 2;
+    const int v = fp32_variant(c, R);
     if (v == 2) return interbody32_sym(c, R, sigma, y, (c->tune32_x2 == 2 && c->tune32_tpt == 1) ? 1 : 2);
     const bool x2 = v == 1;
     int tpt = c->tune32_tpt > 0 ? c->tune32_tpt : 4;
@@ -848,12 +869,17 @@ hzb_status autotune(hzb_ctx *c, int R, int which, double *best_ms)
             }
             float t5 = 1e30f;
             {
-                if (interbody_tc5(c, R, c->io_in.ptr, c->io_out.ptr, default_nsplit_tc5(c, R), T5_SPLIT3))
-                    return fail(c, HZB_ECUDA, "autotune launch failed");
+                hzb_status st5;
+                const bool half = t5h_usable(c, &st5);
+                if (st5) return st5;
+                auto run5 = [&]() {
+                    return half ? interbody_t5h(c, R, c->io_in.ptr, c->io_out.ptr)
+                                : interbody_tc5(c, R, c->io_in.ptr, c->io_out.ptr, default_nsplit_tc5(c, R), T5_SPLIT3);
+                };
+                if (run5()) return fail(c, HZB_ECUDA, "autotune launch failed");
                 cudaEventRecord(c->ev0, c->stream);
                 for (int q = 0; q < 3; ++q)
-                    if (interbody_tc5(c, R, c->io_in.ptr, c->io_out.ptr, default_nsplit_tc5(c, R), T5_SPLIT3))
-                        return fail(c, HZB_ECUDA, "autotune launch failed");
+                    if (run5()) return fail(c, HZB_ECUDA, "autotune launch failed");
                 cudaEventRecord(c->ev1, c->stream);
                 if (cudaEventSynchronize(c->ev1) != cudaSuccess) return fail(c, HZB_ECUDA, "autotune launch failed");
                 cudaEventElapsedTime(&t5, c->ev0, c->ev1);

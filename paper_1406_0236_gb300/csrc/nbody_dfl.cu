@@ -55,6 +55,7 @@
 
 #include "hzb_internal.h"
 #include "lean_df.cuh"
+#include "sigma_scale.cuh"
 
 namespace hzb {
 
@@ -291,13 +292,6 @@ __device__ __forceinline__ float4 dfl_times(float4 v, float s)
     return make_float4(v.x * s, v.y * s, v.z * s, v.w * s);
 }
 
-// scale of right-hand side r back from sigma' (a power of two)
-__device__ __forceinline__ int dfl_exponent(int key)
-{
-    return key ? min(960, max(-960, (key >> 20) - 1022)) : 0;
-}
-__device__ __forceinline__ double dfl_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-
 // A ball about a tile's sources (x, y, z, radius), by one warp whose lanes hold them.
 __device__ __forceinline__ float4 dfl_ball(float4 a, bool have, int cnt)
 {
@@ -349,7 +343,7 @@ __device__ __forceinline__ int dfl_key(double2 v, double w, double c0)
 
 __device__ __forceinline__ float4 dfl_sigma(double2 v, double w, double c0, int key)
 {
-    const double sc = dfl_pow2(-dfl_exponent(key)), wq = w * c0;
+    const double sc = sigma_pow2(-sigma_exponent(key)), wq = w * c0;
     return csplit(make_double2(v.x * wq * sc, v.y * wq * sc));
 }
 
@@ -448,7 +442,7 @@ nbody_dfl_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restri
 #pragma unroll
     for (int c = 0; c < RC; ++c) {
         wr[c] = wi[c] = atr[c] = ati[c] = {0.f, 0.f};
-        scale[c] = r0 + c < R ? dfl_pow2(dfl_exponent(key[r0 + c])) : 0.0;
+        scale[c] = r0 + c < R ? sigma_pow2(sigma_exponent(key[r0 + c])) : 0.0;
     }
     if (live) {
         const int g = bi.start + tid;
@@ -705,7 +699,7 @@ nbody_dfl_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chunk
         for (int c = 0; c < RC; ++c)
             if (r0 + c < R) {
                 const float4 run = GRID ? s_run[c * DFL_NT + tid] : make_float4(zr[c].h, zr[c].l, zi[c].h, zi[c].l);
-                const double sc = dfl_pow2(dfl_exponent(key[r0 + c]));
+                const double sc = sigma_pow2(sigma_exponent(key[r0 + c]));
                 yo[(size_t)(tb.start + t0 + tid) * R + r0 + c] =
                     make_double2(((double)run.x + (double)run.y) * sc, ((double)run.z + (double)run.w) * sc);
             }
@@ -777,6 +771,18 @@ static DflConst dfl_constants(const hzb_ctx *c)
     return K;
 }
 
+// key[r] of every column (sigma_scale.cuh) of c0 w_j sigma_{j,r} (weighted) or c0 sigma_{j,r}
+hzb_status sigma_keys(hzb_ctx *c, int R, const double2 *sigma, double c0, int weighted, int *key)
+{
+    const size_t n = (size_t)c->N * R;
+    if (check_cuda(c, cudaMemsetAsync(key, 0, R * sizeof(int), c->stream), "clear scales")) return HZB_ECUDA;
+    const unsigned nb = (unsigned)std::min<size_t>((n + 2047) / 2048, 608);
+    dfl_sigma_max_kernel<<<dim3(nb, (R + 255) / 256), 256, 0, c->stream>>>(c->N, R, c->pos64.ptr, sigma, c0, weighted,
+                                                                           key);
+    c->launches++;
+    return check_cuda(c, cudaGetLastError(), "dfl_sigma_max_kernel");
+}
+
 // the densities of a call: weighted, scaled to below one per right-hand side, split
 static hzb_status dfl_densities(hzb_ctx *c, int R, const double2 *sigma, int weighted)
 {
@@ -789,14 +795,11 @@ static hzb_status dfl_densities(hzb_ctx *c, int R, const double2 *sigma, int wei
                                                           c->dlkey.ptr, c->dlsig.ptr);
         c->launches += 1;
     } else {
-        if (check_cuda(c, cudaMemsetAsync(c->dlkey.ptr, 0, R * sizeof(int), c->stream), "clear scales"))
-            return HZB_ECUDA;
-        const unsigned nb = (unsigned)std::min<size_t>((n + 2047) / 2048, 608);
-        dfl_sigma_max_kernel<<<dim3(nb, (R + 255) / 256), 256, 0, c->stream>>>(c->N, R, c->pos64.ptr, sigma, c0,
-                                                                               weighted, c->dlkey.ptr);
+        hzb_status st = sigma_keys(c, R, sigma, c0, weighted, c->dlkey.ptr);
+        if (st) return st;
         dfl_sigma_split_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, R, c->pos64.ptr, sigma, c0,
                                                                                    weighted, c->dlkey.ptr, c->dlsig.ptr);
-        c->launches += 2;
+        c->launches += 1;
     }
     return check_cuda(c, cudaGetLastError(), "dfl_sigma_kernel");
 }

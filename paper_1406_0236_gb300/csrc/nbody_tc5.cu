@@ -521,6 +521,41 @@ nbody_tc5ws_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chu
     if (tid == 0 && s_abort) atomicExch(err, 1);
 }
 
+// The device flag of the bounded waits before a launch; inject: the injected timeout fires here
+// (every CTA finds the flag negative and takes its timeout exit).
+hzb_status tc_flag_begin(hzb_ctx *c, bool inject)
+{
+    if (check_cuda(c, c->kerr.ensure(1), "alloc error flag")) return HZB_ENOMEM;
+    if (!c->kerr_ready) {
+        if (check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0, sizeof(int), c->stream), "clear error flag"))
+            return HZB_ECUDA;
+        c->kerr_ready = true;
+    }
+    if (inject && (c->fault & FAULT_TIMEOUT) && !(c->fault_spent & FAULT_TIMEOUT) && !c->capturing) {
+        c->fault_spent |= FAULT_TIMEOUT;
+        if (check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0xff, sizeof(int), c->stream), "inject timeout"))
+            return HZB_ECUDA;
+    }
+    return HZB_OK;
+}
+
+// and after it: a wait that ran out left NaN outputs (a solve reads the flag once, at its end)
+hzb_status tc_flag_end(hzb_ctx *c, const char *kernel)
+{
+    if (c->capturing || c->in_solve) return HZB_OK;
+    int flag = 0;
+    if (check_cuda(c, cudaMemcpyAsync(&flag, c->kerr.ptr, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
+                   "read error flag") ||
+        check_cuda(c, cudaStreamSynchronize(c->stream), kernel))
+        return HZB_ECUDA;
+    if (flag) {                            // report once; the context stays usable for the next call
+        if (check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0, sizeof(int), c->stream), "clear error flag"))
+            return HZB_ECUDA;
+        return fail(c, HZB_ETIMEOUT, std::string("tensor-core wait timed out in ") + kernel);
+    }
+    return HZB_OK;
+}
+
 // mode: T5_SPLIT3 (three-term TF32 split, FP32-level products), T5_WS (the same, warp-
 // specialised), T5_SINGLE (TF32 products alone: about 3e-4 relative error in the sum, 1.4x
 // faster; for inner solves whose refinement tolerates it)
@@ -538,12 +573,8 @@ hzb_status interbody_tc5(hzb_ctx *c, int R, const double2 *sigma, double2 *y, in
         if (check_cuda(c, c->nb_part32.ensure(n * nsplit), "alloc partial sums")) return HZB_ENOMEM;
         part = c->nb_part32.ptr;
     }
-    if (check_cuda(c, c->kerr.ensure(1), "alloc error flag")) return HZB_ENOMEM;
-    if (!c->kerr_ready) {
-        if (check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0, sizeof(int), c->stream), "clear error flag"))
-            return HZB_ECUDA;
-        c->kerr_ready = true;
-    }
+    hzb_status st = tc_flag_begin(c, !ws);
+    if (st) return st;
     static bool attr_done[64] = {false};
     const int dev = c->opt.device;
     if (dev >= 0 && dev < 64 && !attr_done[dev]) {
@@ -561,11 +592,6 @@ hzb_status interbody_tc5(hzb_ctx *c, int R, const double2 *sigma, double2 *y, in
                                                WS_SMEM), "tcgen05 kernel shared memory"))
             return HZB_ECUDA;
         attr_done[dev] = true;
-    }
-    if ((c->fault & FAULT_TIMEOUT) && !(c->fault_spent & FAULT_TIMEOUT) && !c->capturing && !ws) {
-        c->fault_spent |= FAULT_TIMEOUT;   // injected: every CTA takes the timeout exit (flag -1)
-        if (check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0xff, sizeof(int), c->stream), "inject timeout"))
-            return HZB_ECUDA;
     }
     c->interbody_calls++;
     c->launches += (nsplit > 1) ? 3 : 2;
@@ -596,20 +622,7 @@ hzb_status interbody_tc5(hzb_ctx *c, int R, const double2 *sigma, double2 *y, in
     cudaError_t e = cudaGetLastError();
     prof_end(c, slot);
     if (check_cuda(c, e, "nbody_tc5_kernel")) return HZB_ECUDA;
-    if (!c->capturing && !c->in_solve) {   // a bounded wait that ran out: outputs are NaN (a solve
-                                           // reads the flag once at its end instead)
-        int flag = 0;
-        if (check_cuda(c, cudaMemcpyAsync(&flag, c->kerr.ptr, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
-                       "read error flag") ||
-            check_cuda(c, cudaStreamSynchronize(c->stream), "nbody_tc5_kernel"))
-            return HZB_ECUDA;
-        if (flag) {                    // report once; the context stays usable for the next call
-            if (check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0, sizeof(int), c->stream), "clear error flag"))
-                return HZB_ECUDA;
-            return fail(c, HZB_ETIMEOUT, "tensor-core wait timed out in nbody_tc5_kernel");
-        }
-    }
-    return HZB_OK;
+    return tc_flag_end(c, "nbody_tc5_kernel");
 }
 
 }  // namespace hzb
