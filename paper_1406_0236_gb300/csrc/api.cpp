@@ -129,7 +129,7 @@ hzb_status hzb_destroy(hzb_ctx *c)
     cudaDeviceSynchronize();
     release_compression(c);
     for (ShapeDev *s : c->shapes) {
-        s->ring.release(); s->body_offs.release(); s->A64.release(); s->S64.release(); s->S32.release();
+        s->ring.release(); s->body_offs.release(); s->tw.release(); s->A64.release(); s->S64.release(); s->S32.release();
         s->Sdd.release();
         s->Aimg.release();
         delete s;

@@ -92,6 +92,7 @@ struct ShapeDev {
     std::vector<int> bodies;              // bodies using this shape, in order
     DevBuf<double> ring;                  // NG x 8: r, z, nr, nz, ds, t, (unused)
     DevBuf<long long> body_offs;          // first node of each body of this shape
+    DevBuf<double2> tw;                   // NF: cos, sin(2 pi m / NF)
     DevBuf<double2> A64;                  // (M+1) x NG x NG: A~_p
     DevBuf<double2> S64;                  // (M+1) x NG x NG: S_p = A~_p^{-1}
     DevBuf<float2> S32;                   // FP32 copy of S64

@@ -170,6 +170,16 @@ static bool bodies_disjoint(const hzb_ctx *c, int &p_out, int &q_out)
     return true;
 }
 
+// cos, sin(2 pi m / NF), the azimuthal DFTs' table
+__global__ void twiddle_kernel(int NF, double2 *__restrict__ tw)
+{
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= NF) return;
+    double s, c;
+    sincospi(2.0 * m / NF, &s, &c);
+    tw[m] = make_double2(c, s);
+}
+
 hzb_status make_nodes(hzb_ctx *c)
 {
     if (c->nodes_ready) return HZB_OK;
@@ -205,7 +215,10 @@ hzb_status make_nodes(hzb_ctx *c)
         if (check_cuda(c, sd.ring.ensure(ring.size()), "alloc ring")) return HZB_ENOMEM;
         std::vector<long long> offs;
         for (int b : sd.bodies) offs.push_back(c->bodies[b].offset);
-        if (check_cuda(c, sd.body_offs.ensure(offs.size()), "alloc offsets")) return HZB_ENOMEM;
+        if (check_cuda(c, sd.body_offs.ensure(offs.size()), "alloc offsets") ||
+            check_cuda(c, sd.tw.ensure(g.NF), "alloc twiddles"))
+            return HZB_ENOMEM;
+        twiddle_kernel<<<(g.NF + 127) / 128, 128, 0, c->stream>>>(g.NF, sd.tw.ptr);
         if (check_cuda(c, cudaMemcpyAsync(sd.body_offs.ptr, offs.data(), offs.size() * sizeof(long long),
                                           cudaMemcpyHostToDevice, c->stream), "copy offsets"))
             return HZB_ECUDA;
