@@ -331,7 +331,7 @@ __device__ __forceinline__ float dfl_rmin(dd tx, dd ty, dd tz, float4 ball, cons
 
 // ---------------------------------------------------------------- densities
 
-static const int DFL_SIG_SMALL = 16384;   // N x R up to which one block does both passes
+static const int DFL_SIG_SMALL = 2048;    // N x R up to which one block does both passes
 
 // key[r] = largest high word of |Re|, |Im| of w_j sigma_{j,r} c0 over the finite ones
 __device__ __forceinline__ int dfl_key(double2 v, double w, double c0)

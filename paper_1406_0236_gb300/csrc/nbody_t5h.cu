@@ -23,7 +23,7 @@
 // one another's barriers, MMAs and reads.
 //
 // FP16's range: G' is scaled by the power of two that brings its bound at the smallest
-// distance between two bodies (t5h_gap_kernel, once per geometry) to 2^15, the densities per
+// distance between two bodies (t5h_range_kernel, once per geometry) to 2^15, the densities per
 // right-hand side to 2^14, so that a value down to 2^-17 of the largest keeps 22 bits and no
 // value overflows.  Geometries whose kernels span more than that (or k, eta outside
 // sym_scaled) keep the TF32 form (nbody_tc5.cu).
@@ -38,7 +38,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <cstring>
 #include <vector>
 
 #include "f32x2.cuh"
@@ -307,7 +306,7 @@ __global__ void t5h_source_kernel(int ntiles, const int2 *__restrict__ tiles, co
     }
 #pragma unroll
     for (int a = 0; a < 6; ++a) src[(size_t)tile * TH_SRC + a * TH_S + lane] = v[a];
-    // a ball about the tile, for the gap
+    // a ball about the tile, for the range
     float c[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -321,26 +320,28 @@ __global__ void t5h_source_kernel(int ntiles, const int2 *__restrict__ tiles, co
     if (lane == 0) ball[tile] = make_float4(c[0], c[1], c[2], r * 1.0001f);
 }
 
-// smallest distance between nodes of different bodies (in the scaled lengths, a lower bound
-// within a factor of two): balls first, node by node where the balls are no use.  One warp per
-// tile i against the tiles of later bodies.
-__global__ void t5h_gap_kernel(int ntiles, const int2 *__restrict__ tiles, const int *__restrict__ body_end,
-                               const float *__restrict__ src, const float4 *__restrict__ ball, int *__restrict__ gap)
+// smallest distance between nodes of different bodies (range[0], bits; in the scaled lengths, a
+// lower bound within a factor of two: balls first, node by node where the balls are no use)
+// and an upper bound of the largest (range[1]).  One warp per tile i against the tiles of
+// later bodies.
+__global__ void t5h_range_kernel(int ntiles, const int2 *__restrict__ tiles, const int2 *__restrict__ body_end,
+                                 const float *__restrict__ src, const float4 *__restrict__ ball, int *__restrict__ range)
 {
     const int i = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= ntiles) return;
     const float4 bi = ball[i];
     const float *si = src + (size_t)i * TH_SRC;
-    float best = 3e38f;
-    for (int j0 = body_end[i]; j0 < ntiles; j0 += 32) {
+    float best = 3e38f, far = 0.f;
+    for (int j0 = body_end[i].x; j0 < ntiles; j0 += 32) {
         const int j = j0 + lane;
         bool close = false;
         if (j < ntiles) {
             const float4 bj = ball[j];
             const float dx = bi.x - bj.x, dy = bi.y - bj.y, dz = bi.z - bj.z;
-            const float d = sqrtf(dx * dx + dy * dy + dz * dz) * 0.9999f, b = d - bi.w - bj.w;
+            const float d = sqrtf(dx * dx + dy * dy + dz * dz), b = d * 0.9999f - bi.w - bj.w;
             close = !(b >= 0.5f * d);
             if (!close) best = fminf(best, b);
+            far = fmaxf(far, d * 1.0001f + bi.w + bj.w);
         }
         unsigned m = __ballot_sync(0xffffffffu, close);
         while (m) {
@@ -355,8 +356,14 @@ __global__ void t5h_gap_kernel(int ntiles, const int2 *__restrict__ tiles, const
                 }
         }
     }
-    for (int q = 16; q > 0; q >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, q));
-    if (lane == 0) atomicMin(gap, __float_as_int(fmaxf(best, 0.f)));
+    for (int q = 16; q > 0; q >>= 1) {
+        best = fminf(best, __shfl_xor_sync(0xffffffffu, best, q));
+        far = fmaxf(far, __shfl_xor_sync(0xffffffffu, far, q));
+    }
+    if (lane == 0) {
+        atomicMin(&range[0], __float_as_int(fmaxf(best, 0.f)));
+        atomicMax(&range[1], __float_as_int(far));
+    }
 }
 
 // B images of every tile and chunk of RC right-hand sides, in the swizzled K-major layout the
@@ -447,67 +454,46 @@ static hzb_status ensure_t5h(hzb_ctx *c)
                                       cudaMemcpyDeviceToHost, c->stream), "copy blocks") ||
         check_cuda(c, cudaStreamSynchronize(c->stream), "copy blocks"))
         return HZB_ECUDA;
-    std::vector<int2> tiles, own(tb.size());
-    std::vector<int> end;
+    // one buffer: the tiles, the blocks' own tiles, the end of each tile's body, the range
+    std::vector<int2> tiles, own(tb.size()), end;
     for (size_t b = 0; b < tb.size(); ++b) {
         if (b == 0 || tb[b].excl_lo != tb[b - 1].excl_lo) {    // a new body: its nodes are one range
             const int first = (int)tiles.size();
             for (int s = tb[b].excl_lo; s < tb[b].excl_hi; s += TH_S)
                 tiles.push_back(make_int2(s, std::min(TH_S, tb[b].excl_hi - s)));
-            end.resize(tiles.size(), (int)tiles.size());
+            end.resize(tiles.size(), make_int2((int)tiles.size(), 0));
             own[b] = make_int2(first, (int)tiles.size());
         } else {
             own[b] = own[b - 1];
         }
     }
     const int nt = (int)tiles.size();
-    // one buffer: tiles, the blocks' own tiles, the gap, the end of each tile's body
-    DevBuf<float4> ball;
-    DevBuf<int> bend;
-    int gap = 0x7f7fffff;
-    auto done = [&](hzb_status st) { ball.release(); bend.release(); return st; };
-    if (check_cuda(c, c->t5h_tiles.ensure((size_t)nt + own.size() + 1), "alloc tiles") ||
-        check_cuda(c, c->t5h_src.ensure((size_t)nt * TH_SRC), "alloc tiles") || check_cuda(c, ball.ensure(nt), "alloc") ||
-        check_cuda(c, bend.ensure(nt), "alloc"))
-        return done(HZB_ENOMEM);
-    int *gap_dev = reinterpret_cast<int *>(c->t5h_tiles.ptr + nt + own.size());
-    if (check_cuda(c, cudaMemcpyAsync(c->t5h_tiles.ptr, tiles.data(), nt * sizeof(int2), cudaMemcpyHostToDevice, c->stream),
-                   "copy tiles") ||
-        check_cuda(c, cudaMemcpyAsync(c->t5h_tiles.ptr + nt, own.data(), own.size() * sizeof(int2),
-                                      cudaMemcpyHostToDevice, c->stream), "copy tiles") ||
-        check_cuda(c, cudaMemcpyAsync(bend.ptr, end.data(), nt * sizeof(int), cudaMemcpyHostToDevice, c->stream),
-                   "copy tiles") ||
-        check_cuda(c, cudaMemcpyAsync(gap_dev, &gap, sizeof(int), cudaMemcpyHostToDevice, c->stream), "copy tiles"))
-        return done(HZB_ECUDA);
+    tiles.insert(tiles.end(), own.begin(), own.end());
+    tiles.insert(tiles.end(), end.begin(), end.end());
+    tiles.push_back(make_int2(0x7f7fffff, 0));
+    if (check_cuda(c, c->t5h_tiles.ensure(tiles.size()), "alloc tiles") ||
+        check_cuda(c, c->t5h_src.ensure((size_t)nt * (TH_SRC + 4)), "alloc tiles"))
+        return HZB_ENOMEM;
+    float4 *ball = reinterpret_cast<float4 *>(c->t5h_src.ptr + (size_t)nt * TH_SRC);
+    int2 *const end_dev = c->t5h_tiles.ptr + nt + own.size();
+    int *const range_dev = reinterpret_cast<int *>(end_dev + nt);
+    if (check_cuda(c, cudaMemcpyAsync(c->t5h_tiles.ptr, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice,
+                                      c->stream), "copy tiles"))
+        return HZB_ECUDA;
     t5h_source_kernel<<<(nt + 7) / 8, 256, 0, c->stream>>>(
         nt, c->t5h_tiles.ptr, c->pos64.ptr, c->nrm64.ptr, make_double3(c->center[0], c->center[1], c->center[2]), c->k,
-        c->k / c->eta, c->t5h_src.ptr, ball.ptr);
-    t5h_gap_kernel<<<(nt + 7) / 8, 256, 0, c->stream>>>(nt, c->t5h_tiles.ptr, bend.ptr, c->t5h_src.ptr, ball.ptr,
-                                                        gap_dev);
-    std::vector<float4> hb(nt);
+        c->k / c->eta, c->t5h_src.ptr, ball);
+    t5h_range_kernel<<<(nt + 7) / 8, 256, 0, c->stream>>>(nt, c->t5h_tiles.ptr, end_dev, c->t5h_src.ptr, ball, range_dev);
+    float range[2];
     if (check_cuda(c, cudaGetLastError(), "tiles") ||
-        check_cuda(c, cudaMemcpyAsync(&gap, gap_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "copy gap") ||
-        check_cuda(c, cudaMemcpyAsync(hb.data(), ball.ptr, nt * sizeof(float4), cudaMemcpyDeviceToHost, c->stream),
-                   "copy balls") ||
+        check_cuda(c, cudaMemcpyAsync(range, range_dev, sizeof(range), cudaMemcpyDeviceToHost, c->stream), "copy range") ||
         check_cuda(c, cudaStreamSynchronize(c->stream), "tiles"))
-        return done(HZB_ECUDA);
-    float g;
-    static_assert(sizeof(g) == sizeof(gap), "bits");
-    std::memcpy(&g, &gap, sizeof(g));
+        return HZB_ECUDA;
+    const double g = range[0], diam = range[1];
     // |G'| <= u (1 + (k / |eta|) (1 + u)), u = 1 / (k r); the smallest is about u at the diameter
-    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-    for (const float4 &b : hb) {
-        const double v[3] = {b.x, b.y, b.z};
-        for (int a = 0; a < 3; ++a) {
-            lo[a] = std::min(lo[a], v[a] - b.w);
-            hi[a] = std::max(hi[a], v[a] + b.w);
-        }
-    }
-    const double diam = std::sqrt((hi[0] - lo[0]) * (hi[0] - lo[0]) + (hi[1] - lo[1]) * (hi[1] - lo[1]) +
-                                  (hi[2] - lo[2]) * (hi[2] - lo[2]));
     const double u = 1.0 / g, bound = u * (1.0 + (c->k / std::fabs(c->eta)) * (1.0 + u)) * 1.001;
     c->t5h_state = -1;
-    if (std::isfinite(bound) && g > 0.f && diam > 0.0 && diam < 9e4 && bound * diam < 262144.0) {
+    if (std::isfinite(bound) && g > 0.0 && diam > 0.0 && diam < 9e4 && bound * diam < 262144.0) {
         int e;
         std::frexp(bound, &e);                                 // bound < 2^e
         if (e > -100 && e < 100) {
@@ -520,7 +506,7 @@ static hzb_status ensure_t5h(hzb_ctx *c)
             c->t5h_state = 1;
         }
     }
-    return done(HZB_OK);
+    return HZB_OK;
 }
 
 // whether the context's geometry, k and eta suit this form (-1 in *st: an error)
@@ -536,16 +522,16 @@ hzb_status interbody_t5h(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->opt.device);
     const int rc = R <= 16 ? 16 : 32, nchunk = (R + rc - 1) / rc, nt = c->t5h_ntiles;
     const int most = c->t5h_most;
-    // source chunks: between four and ten CTAs per resident place, the number whose last wave is
-    // fullest, with at least eight tiles to each
+    // Source chunks: the number that gives the shortest sum of the kernel's time (2.5 pairs per
+    // clock and SM, over the fill of its last wave) and of the partial sums' (8 us per 10^6
+    // values written and read), at least eight tiles to each.
     const long long ctas = (long long)c->t5h_ctas * nchunk, places = 3LL * sms;
-    const int cap = std::max(1, std::min(64, most / 8));
+    const double full = (double)ctas * TH_M * TH_S * most / (2.5 * 2.0e3 * sms), part = 8e-6 * (double)c->N * R;
     int nsplit = 1;
-    double fill = 0.0;
-    for (int ns = (int)std::min<long long>(cap, std::max<long long>(1, 4 * places / ctas));
-         ns <= std::min<long long>(cap, std::max<long long>(1, 10 * places / ctas)); ++ns) {
-        const double waves = (double)(ns * ctas) / places, f = waves / std::ceil(waves);
-        if (f > fill + 0.005) { fill = f; nsplit = ns; }
+    double best = 1e300;
+    for (int ns = 1; ns <= std::max(1, std::min(64, most / 8)); ++ns) {
+        const double waves = (double)(ns * ctas) / places, t = full * std::ceil(waves) / waves + part * ns;
+        if (t < best) { best = t; nsplit = ns; }
     }
     const int chunk = (most + nsplit - 1) / nsplit;
     nsplit = (most + chunk - 1) / chunk;
