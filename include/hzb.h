@@ -254,8 +254,8 @@ hzb_status hzb_set_execution(hzb_ctx *ctx, int check_every, int use_graphs);
  * the operands streamed by TMA (embedded, split S_p images built once per shape: about
  * 32 N_G^2 (M+1) bytes; accumulators in tensor memory drained into FP32 registers every
  * 64 of the K = 2 N_G terms); -1 (default) = 2 when a shape's panel has at least 32
- * columns (2 x bodies of the shape x right-hand sides), else 0.  Returns HZB_EINVAL for
- * other values. */
+ * columns (2 x bodies of the shape x right-hand sides) and its contraction (M+1) N_G^2 x
+ * columns >= 6e7 complex multiply-adds, else 0.  Returns HZB_EINVAL for other values. */
 hzb_status hzb_set_modal_engine(hzb_ctx *ctx, int engine);
 
 /* Engine of the FP32 inter-body sum (Sec. 3.3): 0 = CUDA cores (one pair kernel per

@@ -11,6 +11,7 @@
 
 #include "hzb_internal.h"
 #include "kernel_math.cuh"
+#include "modal_gemm.cuh"
 
 namespace hzb {
 
@@ -256,86 +257,12 @@ static void dft_inverse(cudaStream_t st, const ShapeDev &sd, int ms, int R, cons
     else launch(dft_inverse_kernel<T, 1, 1>, 1, 1);
 }
 
-// Batched complex GEMM C[p] = A[p] B[p], A: n x n, B and C: n x nc, row-major.
-// 32 x (16 TB) output tile per block, 256 threads, 2 x TB outputs per thread, K step 16;
-// TB = 1 for panels of at most 16 columns (one body of a shape and R = 1 ... 8 bodies
-// with R = 1 fill 16), so no half of the tile multiplies zeros.
-template <typename T, int TB>
-__global__ void __launch_bounds__(256)
-modal_gemm_kernel(int n, int nc, const typename C2<T>::t *__restrict__ A, const typename C2<T>::t *__restrict__ B,
-                  typename C2<T>::t *__restrict__ C)
-{
-    typedef typename C2<T>::t ct;
-    __shared__ ct As[32][17];
-    __shared__ ct Bs[16][16 * TB + 1];
-    const int p = blockIdx.z;
-    const ct *Ap = A + (size_t)p * n * n;
-    const ct *Bp = B + (size_t)p * n * nc;
-    ct *Cp = C + (size_t)p * n * nc;
-    const int row0 = blockIdx.y * 32, col0 = blockIdx.x * (16 * TB);
-    const int tid = threadIdx.x;
-    const int tr = tid / 16, tc = tid % 16;     // rows tr, tr+16; cols tc (, tc+16)
-    T accr[2][TB], acci[2][TB];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < TB; ++b) accr[a][b] = acci[a][b] = (T)0;
-    for (int k0 = 0; k0 < n; k0 += 16) {
-        for (int e = tid; e < 32 * 16; e += 256) {
-            int r = e / 16, kk = e % 16;
-            int gr = row0 + r, gk = k0 + kk;
-            ct v;
-            v.x = (T)0; v.y = (T)0;
-            if (gr < n && gk < n) v = Ap[(size_t)gr * n + gk];
-            As[r][kk] = v;
-        }
-        for (int e = tid; e < 16 * 16 * TB; e += 256) {
-            int kk = e / (16 * TB), cc = e % (16 * TB);
-            int gk = k0 + kk, gc = col0 + cc;
-            ct v;
-            v.x = (T)0; v.y = (T)0;
-            if (gk < n && gc < nc) v = Bp[(size_t)gk * nc + gc];
-            Bs[kk][cc] = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            const ct a[2] = {As[tr][kk], As[tr + 16][kk]};
-#pragma unroll
-            for (int b = 0; b < TB; ++b) {
-                const ct bb = Bs[kk][tc + 16 * b];
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    accr[q][b] += a[q].x * bb.x - a[q].y * bb.y;
-                    acci[q][b] += a[q].x * bb.y + a[q].y * bb.x;
-                }
-            }
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < TB; ++b) {
-            int gr = row0 + tr + 16 * a, gc = col0 + tc + 16 * b;
-            if (gr < n && gc < nc) {
-                ct v;
-                v.x = accr[a][b];
-                v.y = acci[a][b];
-                Cp[(size_t)gr * nc + gc] = v;
-            }
-        }
-}
-
-template <typename T>
-static void modal_gemm(cudaStream_t st, int n, int nc, int modes, const typename C2<T>::t *A,
-                       const typename C2<T>::t *B, typename C2<T>::t *C)
-{
-    if (nc <= 16)
-        modal_gemm_kernel<T, 1><<<dim3((nc + 15) / 16, (n + 31) / 32, modes), 256, 0, st>>>(n, nc, A, B, C);
-    else
-        modal_gemm_kernel<T, 2><<<dim3((nc + 31) / 32, (n + 31) / 32, modes), 256, 0, st>>>(n, nc, A, B, C);
-}
+// Below this the two launches, the embedding pass and the few blocks of the TMA form cost more
+// than the tensor cores save.  Whole D^{-1}, CUDA cores against TMA (us): N_G = 100, 21 modes,
+// 32 / 64 / 256 columns (7 / 13 / 54e6) 27 / 29 / 66 against 36 / 40 / 73; N_G = 144: 31 / 34 / 82
+// against 38 / 44 / 78 (14 / 28 / 111e6); N_G = 224, 31 modes: 44 / 64 against 48 / 58
+// (50 / 100e6); N_G = 320, 51 modes, 32 columns (167e6): 94 against 88.
+static const double MODAL_TMA_MIN = 6e7;
 
 template <typename T>
 static hzb_status local_inverse_t(hzb_ctx *c, int R, const double2 *y, const double2 *sigma, double alpha,
@@ -367,17 +294,17 @@ static hzb_status local_inverse_t(hzb_ctx *c, int R, const double2 *y, const dou
         const long long *doff = sd.body_offs.ptr;        // first node of each body of the shape
         if (dft_smem<T>(NF, R) > 200 * 1024) return fail(c, HZB_EINVAL, "n_modes * R too large for the modal apply");
         dft_forward<T>(c->stream, sd, ms, R, doff, y, yh);
-        // FP32 path: tensor cores (TF32 x 3) once the panels are wide enough to fill them
-        // FP32 path: tcgen05 fed by TMA (modal_tma.cu) once the panels are wide enough to
-        // fill the tensor cores, or as chosen; mma.sync TF32 x 3 on request
+        // FP32 path: tcgen05 fed by TMA (modal_tma.cu) from 32 columns and MODAL_TMA_MIN complex
+        // multiply-adds on, or as chosen; mma.sync TF32 x 3 on request
         const bool f32 = sizeof(T) == 4;
-        if (f32 && (c->modal_engine == 2 || (c->modal_engine < 0 && ncols >= 32))) {
+        const double macs = (double)(M + 1) * NG * NG * ncols;
+        if (f32 && (c->modal_engine == 2 || (c->modal_engine < 0 && ncols >= 32 && macs >= MODAL_TMA_MIN))) {
             hzb_status st = modal_gemm_tma(c, sd, ncols, (const float2 *)yh, (float2 *)th);
             if (st) return st;
         } else if (f32 && c->modal_engine == 1)
             launch_modal_gemm_tc(c, NG, ncols, M + 1, (const float2 *)S, (const float2 *)yh, (float2 *)th);
         else
-            modal_gemm<T>(c->stream, NG, ncols, M + 1, S, yh, th);
+            modal_gemm<ct, 2, 1>(c->stream, NG, ncols, M + 1, S, yh, th);
         dft_inverse<T>(c->stream, sd, ms, R, doff, th, sigma, alpha, beta, tau);
         c->launches += 3;
         if (check_cuda(c, cudaGetLastError(), "modal apply")) return HZB_ECUDA;
@@ -415,7 +342,7 @@ hzb_status local_inverse64_scratch(hzb_ctx *c, int R, const double2 *y, const do
         if (dft_smem<double>(sd.geom.NF, R) > 200 * 1024)
             return fail(c, HZB_EINVAL, "n_modes * R too large for the modal apply");
         dft_forward<double>(c->stream, sd, ms, R, doff, y, yh);
-        modal_gemm<double>(c->stream, NG, 2 * ms * R, M + 1, sd.S64.ptr, yh, th);
+        modal_gemm<double2, 2, 1>(c->stream, NG, 2 * ms * R, M + 1, sd.S64.ptr, yh, th);
         dft_inverse<double>(c->stream, sd, ms, R, doff, th, sigma, alpha, beta, tau);
         c->launches += 3;
         if (check_cuda(c, cudaGetLastError(), "modal apply")) return HZB_ECUDA;
@@ -436,7 +363,7 @@ hzb_status shape_inverse64(hzb_ctx *c, ShapeDev &sd, int R, const double2 *X, do
     if (check_cuda(c, cudaMemsetAsync(c->zero_off.ptr, 0, sizeof(long long), c->stream), "memset")) return HZB_ECUDA;
     if (dft_smem<double>(NF, R) > 200 * 1024) return fail(c, HZB_EINVAL, "n_modes * R too large for the modal apply");
     dft_forward<double>(c->stream, sd, 1, R, c->zero_off.ptr, X, c->yhat64.ptr);
-    modal_gemm<double>(c->stream, NG, ncols, M + 1, sd.S64.ptr, c->yhat64.ptr, c->that64.ptr);
+    modal_gemm<double2, 2, 1>(c->stream, NG, ncols, M + 1, sd.S64.ptr, c->yhat64.ptr, c->that64.ptr);
     dft_inverse<double>(c->stream, sd, 1, R, c->zero_off.ptr, c->that64.ptr, nullptr, 0.0, 1.0, Y);
     c->launches += 3;
     return check_cuda(c, cudaGetLastError(), "shape inverse");

@@ -15,6 +15,7 @@
 
 #include "hzb_internal.h"
 #include "lean_df.cuh"
+#include "modal_gemm.cuh"
 
 namespace hzb {
 
@@ -150,63 +151,6 @@ __global__ void dfl_dft_inverse_kernel(int NG, int NF, int R, int ncols, const l
     }
 }
 
-// Batched complex GEMM C[p] = A[p] B[p] in double-float: A n x n, B and C n x nc,
-// row-major.  32 x 32 output tile per block of 256 threads, each 2 x 2 outputs
-// (rows tr, tr + 16; columns tc, tc + 16), K step 16.
-__global__ void __launch_bounds__(256)
-dfl_modal_gemm_kernel(int n, int nc, const float4 *__restrict__ A, const float4 *__restrict__ B, float4 *__restrict__ C)
-{
-    __shared__ float4 As[32][17];
-    __shared__ float4 Bs[16][33];
-    const int p = blockIdx.z;
-    const float4 *Ap = A + (size_t)p * n * n;
-    const float4 *Bp = B + (size_t)p * n * nc;
-    float4 *Cp = C + (size_t)p * n * nc;
-    const int row0 = blockIdx.y * 32, col0 = blockIdx.x * 32;
-    const int tid = threadIdx.x, tr = tid / 16, tc = tid % 16;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    dd ar[2][2], ai[2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) ar[a][b] = ai[a][b] = {0.f, 0.f};
-    for (int k0 = 0; k0 < n; k0 += 16) {
-        for (int e = tid; e < 32 * 16; e += 256) {
-            const int r = e / 16, kk = e % 16, gr = row0 + r, gk = k0 + kk;
-            As[r][kk] = (gr < n && gk < n) ? Ap[(size_t)gr * n + gk] : zero;
-        }
-        for (int e = tid; e < 16 * 32; e += 256) {
-            const int kk = e / 32, cc = e % 32, gk = k0 + kk, gc = col0 + cc;
-            Bs[kk][cc] = (gk < n && gc < nc) ? Bp[(size_t)gk * nc + gc] : zero;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < 16; ++kk) {
-            const float4 a0 = As[tr][kk], a1 = As[tr + 16][kk];
-            const float4 b0 = Bs[kk][tc], b1 = Bs[kk][tc + 16];
-            cmac(ar[0][0], ai[0][0], a0, b0);
-            cmac(ar[0][1], ai[0][1], a0, b1);
-            cmac(ar[1][0], ai[1][0], a1, b0);
-            cmac(ar[1][1], ai[1][1], a1, b1);
-        }
-#pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                ar[a][b] = norm(ar[a][b]);
-                ai[a][b] = norm(ai[a][b]);
-            }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int gr = row0 + tr + 16 * a, gc = col0 + tc + 16 * b;
-            if (gr < n && gc < nc) Cp[(size_t)gr * nc + gc] = make_float4(ar[a][b].h, ar[a][b].l, ai[a][b].h, ai[a][b].l);
-        }
-}
-
 // the shape's S_p split into double-float, built on first use after each (re)build
 static hzb_status ensure_sdd(hzb_ctx *c, ShapeDev &sd)
 {
@@ -254,8 +198,7 @@ hzb_status local_inverse_dfl(hzb_ctx *c, int R, const double2 *y, const double2 
         const long long *doff = sd.body_offs.ptr;
         dfl_dft_forward_kernel<<<dim3(NG, ms), DFLM_THREADS, smem, c->stream>>>(NG, NF, R, ncols, doff, y, sd.tw.ptr,
                                                                                 yh);
-        dfl_modal_gemm_kernel<<<dim3((ncols + 31) / 32, (NG + 31) / 32, M + 1), 256, 0, c->stream>>>(
-            NG, ncols, sd.Sdd.ptr, yh, th);
+        modal_gemm<float4, 2, 1>(c->stream, NG, ncols, M + 1, sd.Sdd.ptr, yh, th);
         dfl_dft_inverse_kernel<<<dim3(NG, ms), DFLM_THREADS, smem, c->stream>>>(NG, NF, R, ncols, doff, th, sigma,
                                                                                 sd.tw.ptr, alpha, beta, tau);
         c->launches += 3;
