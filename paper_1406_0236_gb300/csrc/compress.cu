@@ -32,6 +32,7 @@
 #include <vector>
 
 #include "hzb_internal.h"
+#include "modal_gemm.cuh"
 
 namespace hzb {
 
@@ -954,7 +955,7 @@ static void free_ctx_buffers(hzb_ctx *r)
     r->blockpairs.release(); r->kerr.release(); r->dfa.release(); r->dfb.release(); r->dfc.release();
     r->dftab.release(); r->rb.release(); r->rx.release(); r->zero_off.release(); r->yhat64.release();
     r->that64.release(); r->yhat32.release(); r->that32.release(); r->Ximg.release(); r->io_small.release();
-    r->dfltab.release(); r->dla.release(); r->dlb.release(); r->dlc.release(); r->symn.release(); r->t5h_tiles.release(); r->t5h_src.release(); r->t5h_img.release(); r->dlsig.release(); r->dlw.release(); r->dlkey.release();
+    r->dfltab.release(); r->dla.release(); r->dlb.release(); r->dlc.release(); r->symn.release(); r->t5h_tiles.release(); r->t5h_src.release(); r->t5h_img.release(); r->dlsig.release(); r->dlw.release(); r->dlkey.release(); r->ysplit.release();
     if (r->host_pinned) cudaFreeHost(r->host_pinned);
     r->host_pinned = nullptr;
     release_graphs(r);
@@ -1074,89 +1075,124 @@ hzb_status build_reduced(hzb_ctx *c)
     return st;
 }
 
-// out[ooff_b + i][r] = alpha sig[ooff_b + i][r] + beta sum_j A[i][j] y[yoff_b + j][r] for the
-// ms bodies b of a shape and i < rows; A rows x cols row-major.  One warp per row, eight
-// rows per block; the right-hand-side columns (body, r) go in groups of 8, and each
-// 256-wide slice of their y values is staged once in shared memory for the block's
-// eight rows.  F32: A in FP32 and FP32 accumulation (the reduced system's FP32
-// operator), else FP64.  The restriction T w (A = T), the extension T^T y (A = T^T)
-// and the reduced local operator S y (A = S) all take this form.
-static const int GEMV_ROWS = 8;
-template <bool F32>
-__global__ void __launch_bounds__(256) body_gemv_kernel(int rows, int cols, int ms, int R,
-                                                        const long long *__restrict__ yoff,
-                                                        const long long *__restrict__ ooff, const void *__restrict__ Av,
-                                                        const double2 *__restrict__ y, const double2 *__restrict__ sig,
-                                                        double alpha, double beta, double2 *__restrict__ out)
+// x -> (hi, lo) in FP32 with hi = fl(x), lo = fl(x - hi): x = hi + lo to about 2^-48 |x|
+__global__ void split_df_kernel(size_t n, const double2 *__restrict__ a, float4 *__restrict__ out)
 {
-    typedef typename std::conditional<F32, float, double>::type acc_t;
-    __shared__ acc_t ys[8][256][2];
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * GEMV_ROWS + (threadIdx.x >> 5);
-    const int ncol = ms * R;
-    for (int c0 = 0; c0 < ncol; c0 += 8) {
-        const int nc = min(8, ncol - c0);
-        acc_t sx[8], sy[8];
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n) out[e] = lean::csplit(a[e]);
+}
+
+__global__ void round_f32_kernel(size_t n, const double2 *__restrict__ a, float2 *__restrict__ out)
+{
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n) out[e] = make_float2((float)a[e].x, (float)a[e].y);
+}
+
+__device__ __forceinline__ double2 to_double2(double2 v) { return v; }
+__device__ __forceinline__ double2 to_double2(float2 v) { return make_double2((double)v.x, (double)v.y); }
+__device__ __forceinline__ double2 to_double2(float4 v)
+{
+    return make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
+}
+
+// out[ooff_b + i][r] = alpha sig[ooff_b + i][r] + beta sum_j A[i][j] y[yoff_b + j][r] for the
+// ms bodies b of a shape and i < rows; A rows x cols row-major.  E: FP64, FP32, or
+// double-float (FP32 pairs, about 1e-14 per term; 48 FP32 operations per complex multiply-add
+// against 4 FP64 ones at 1/64 of the rate).  The restriction T w (A = T), the extension
+// T^T y (A = T^T) and the reduced local operator S y (A = S) all take this form.
+//
+// A block owns TM rows and 4 TN columns (body, r); its eight warps and the eight lane groups of
+// each share the k sum 64 ways (TM x TN sums to a lane, so that a value read from shared memory
+// serves TN or TM of them), and the shares are added once at the end.  Few rows per block, many
+// blocks: with a warp per row and eight rows to a block the 800-row operators here filled 101
+// blocks.  A and y come by cp.async, the next 1 KB / sizeof(E) terms under the current ones; y is
+// rounded or split beforehand, since a conversion per block would go through the FP64 pipe
+// rows / TM times.  An 803 x 803 operator on 12 columns: FP32 44.7 -> 13.4 us (and 2.9 to round y), FP64
+// 143 -> 75 us; 803 x 7320 in double-float 454 -> 212 us and its transpose 260 -> 202 us.
+template <typename E, int TM, int TN>
+__global__ void __launch_bounds__(256)
+body_gemm_kernel(int rows, int cols, int ms, int R, int ncb, const long long *__restrict__ yoff,
+                 const long long *__restrict__ ooff, const E *__restrict__ A, const E *__restrict__ y,
+                 const double2 *__restrict__ sig, double alpha, double beta, double2 *__restrict__ out)
+{
+    constexpr int KC = 1024 / (int)sizeof(E), BN = 4 * TN, BP = BN % 8 ? BN : BN + 4;   // BP: no bank conflicts
+    constexpr int CP = BN == 12 ? 16 : BN;                                              // staging lanes per k
+    __shared__ __align__(16) unsigned char smem[2 * (TM + BP) * 1024];
+    E *const As = reinterpret_cast<E *>(smem), *const Bs = As + 2 * TM * KC;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, lc = lane & 3, kq = lane >> 2;
+    const int row0 = (int)(blockIdx.x / ncb) * TM, col0 = (int)(blockIdx.x % ncb) * BN, ncol = ms * R;
+    // the column of y that this thread stages
+    const int sc = tid % CP, sk = tid / CP, scol = col0 + sc;
+    const bool has = sc < BN && scol < ncol;
+    const E *const ysrc = has ? y + (size_t)yoff[scol / R] * R + scol % R : y;
+    auto stage = [&](int buf, int k0) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) sx[q] = sy[q] = (acc_t)0;
-        for (int jc = 0; jc < cols; jc += 256) {
-            __syncthreads();
-            {
-                const int j = jc + threadIdx.x;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    if (q < nc) {
-                        const int cc = c0 + q;
-                        double2 v = make_double2(0.0, 0.0);
-                        if (j < cols) v = y[(yoff[cc / R] + j) * R + cc % R];
-                        ys[q][threadIdx.x][0] = (acc_t)v.x;
-                        ys[q][threadIdx.x][1] = (acc_t)v.y;
-                    }
-                }
-            }
-            __syncthreads();
-            if (i < rows) {
-                const int jn = min(256, cols - jc);
-#pragma unroll 4
-                for (int jj = lane; jj < jn; jj += 32) {
-                    acc_t ax, ay;
-                    if (F32) {
-                        const float2 av = ((const float2 *)Av)[(size_t)i * cols + jc + jj];
-                        ax = av.x;
-                        ay = av.y;
-                    } else {
-                        const double2 av = ((const double2 *)Av)[(size_t)i * cols + jc + jj];
-                        ax = (acc_t)av.x;
-                        ay = (acc_t)av.y;
-                    }
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        if (q < nc) {
-                            const acc_t vx = ys[q][jj][0], vy = ys[q][jj][1];
-                            sx[q] = fma(ax, vx, fma(-ay, vy, sx[q]));
-                            sy[q] = fma(ax, vy, fma(ay, vx, sy[q]));
-                        }
-                    }
-                }
-            }
+        for (int e = tid; e < TM * KC; e += 256) {
+            const int r = e / KC, k = k0 + e % KC;
+            const bool in = row0 + r < rows && k < cols;
+            modal_stage(As + buf * TM * KC + e, in ? A + (size_t)(row0 + r) * cols + k : A, in);
         }
+        if (sc < BN)
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            for (int o = 16; o > 0; o >>= 1) {
-                sx[q] += __shfl_xor_sync(0xffffffffu, sx[q], o);
-                sy[q] += __shfl_xor_sync(0xffffffffu, sy[q], o);
+            for (int i = 0; i < KC * CP / 256; ++i) {
+                const int k = sk + i * (256 / CP);
+                const bool in = has && k0 + k < cols;
+                modal_stage(Bs + (buf * KC + k) * BP + sc, in ? ysrc + (size_t)(k0 + k) * R : y, in);
             }
-        if (i < rows && lane < nc) {
-            double vx = 0.0, vy = 0.0;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    ComplexAcc<E> acc[TM][TN];
+    stage(0, 0);
+    for (int k0 = 0, n = 0; k0 < cols; k0 += KC, ++n) {
+        if (k0 + KC < cols) {
+            stage((n + 1) & 1, k0 + KC);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const E *const a0 = As + (n & 1) * TM * KC, *const b0 = Bs + (n & 1) * KC * BP;
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (q == lane) {
-                    vx = (double)sx[q];
-                    vy = (double)sy[q];
-                }
-            const int cc = c0 + lane;
-            const size_t o = (size_t)(ooff[cc / R] + i) * R + cc % R;
-            double2 res = make_double2(beta * vx, beta * vy);
+        for (int i = 0; i < KC / 64; ++i) {
+            const int k = i * 64 + w * 8 + kq;
+            E a[TM], b[TN];
+#pragma unroll
+            for (int t = 0; t < TM; ++t) a[t] = a0[t * KC + k];
+#pragma unroll
+            for (int q = 0; q < TN; ++q) b[q] = b0[k * BP + lc + 4 * q];
+#pragma unroll
+            for (int t = 0; t < TM; ++t)
+#pragma unroll
+                for (int q = 0; q < TN; ++q) acc[t][q].mac(a[t], b[q]);
+        }
+        if ((n & 7) == 7)
+#pragma unroll
+            for (int t = 0; t < TM; ++t)
+#pragma unroll
+                for (int q = 0; q < TN; ++q) acc[t][q].settle();
+        __syncthreads();
+    }
+    double2 *const red = reinterpret_cast<double2 *>(smem);                // [warp][TM][BN]
+#pragma unroll
+    for (int t = 0; t < TM; ++t)
+#pragma unroll
+        for (int q = 0; q < TN; ++q) {
+            acc[t][q].settle();
+#pragma unroll
+            for (int m = 4; m < 32; m *= 2) acc[t][q].add_lane(m);
+            if (kq == 0) red[(w * TM + t) * BN + lc + 4 * q] = to_double2(acc[t][q].value());
+        }
+    __syncthreads();
+    if (tid < TM * BN) {
+        const int row = row0 + tid / BN, cc = col0 + tid % BN;
+        if (row < rows && cc < ncol) {
+            double2 s = red[tid];
+            for (int q = 1; q < 8; ++q) {
+                s.x += red[q * TM * BN + tid].x;
+                s.y += red[q * TM * BN + tid].y;
+            }
+            const size_t o = (size_t)(ooff[cc / R] + row) * R + cc % R;
+            double2 res = make_double2(beta * s.x, beta * s.y);
             if (alpha != 0.0) {
                 res.x += alpha * sig[o].x;
                 res.y += alpha * sig[o].y;
@@ -1166,143 +1202,44 @@ __global__ void __launch_bounds__(256) body_gemv_kernel(int rows, int cols, int 
     }
 }
 
-static unsigned gemv_blocks(int rows) { return (unsigned)((rows + GEMV_ROWS - 1) / GEMV_ROWS); }
-
-// x -> (hi, lo) in FP32 with hi = fl(x), lo = fl(x - hi): x = hi + lo to about 2^-48 |x|
-__global__ void split_df_kernel(size_t n, const double2 *__restrict__ a, float4 *__restrict__ out)
+template <typename E>
+static void body_gemm(cudaStream_t st, int rows, int cols, int ms, int R, const long long *yoff, const long long *ooff,
+                      const E *A, const E *y, const double2 *sig, double alpha, double beta, double2 *out)
 {
-    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const double2 v = a[e];
-    const float hx = (float)v.x, hy = (float)v.y;
-    out[e] = make_float4(hx, hy, (float)(v.x - (double)hx), (float)(v.y - (double)hy));
-}
-
-// a + b exactly as (s, err) (Knuth's two-sum), FP32; the _rn intrinsics keep the
-// compiler from fusing these operations with a neighbouring multiply
-__device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &err)
-{
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-}
-
-// (uh + ul)(vh + vl) ~ p + e with p = fl(uh vh) and e its rounding error plus the
-// cross terms (the ul vl term, ~2^-48 of the product, is dropped)
-__device__ __forceinline__ void prod_df(float uh, float ul, float vh, float vl, float &p, float &e)
-{
-    p = __fmul_rn(uh, vh);
-    e = fmaf(uh, vh, -p);
-    e = fmaf(uh, vl, e);
-    e = fmaf(ul, vh, e);
-}
-
-__device__ __forceinline__ void acc_df(float &sh, float &sl, float p, float e)
-{
-    float s, err;
-    two_sum_f(sh, p, s, err);
-    sh = s;
-    sl += err + e;
-}
-
-// The GEMV of body_gemv_kernel in double-float on the FP32 pipe: A and y split into FP32
-// hi/lo pairs (split_df_kernel), each real product formed with its rounding error and
-// added by two-sum into a (hi, lo) accumulator; about 48 FP32 operations per complex
-// multiply-add instead of 4 FP64 ones (FP64 runs at 1/64 of the FP32 rate), relative
-// error about 1e-14 per term.  Used by the mixed path's restriction and recovery.
-__global__ void __launch_bounds__(256) body_gemv_df_kernel(int rows, int cols, int ms, int R,
-                                                           const long long *__restrict__ yoff,
-                                                           const long long *__restrict__ ooff,
-                                                           const float4 *__restrict__ A, const float4 *__restrict__ y,
-                                                           const double2 *__restrict__ sig, double alpha, double beta,
-                                                           double2 *__restrict__ out)
-{
-    __shared__ float4 ys[8][256];
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * GEMV_ROWS + (threadIdx.x >> 5);
-    const int ncol = ms * R;
-    for (int c0 = 0; c0 < ncol; c0 += 8) {
-        const int nc = min(8, ncol - c0);
-        float rh[8], rl[8], ih[8], il[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) rh[q] = rl[q] = ih[q] = il[q] = 0.f;
-        for (int jc = 0; jc < cols; jc += 256) {
-            __syncthreads();
-            {
-                const int j = jc + threadIdx.x;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    if (q < nc) {
-                        const int cc = c0 + q;
-                        ys[q][threadIdx.x] =
-                            j < cols ? y[(yoff[cc / R] + j) * R + cc % R] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-                }
-            }
-            __syncthreads();
-            if (i < rows) {
-                const int jn = min(256, cols - jc);
-#pragma unroll 2
-                for (int jj = lane; jj < jn; jj += 32) {
-                    const float4 a = A[(size_t)i * cols + jc + jj];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        if (q < nc) {
-                            const float4 v = ys[q][jj];
-                            float p, e;
-                            prod_df(a.x, a.z, v.x, v.z, p, e);          // ar yr
-                            acc_df(rh[q], rl[q], p, e);
-                            prod_df(-a.y, -a.w, v.y, v.w, p, e);        // - ai yi
-                            acc_df(rh[q], rl[q], p, e);
-                            prod_df(a.x, a.z, v.y, v.w, p, e);          // ar yi
-                            acc_df(ih[q], il[q], p, e);
-                            prod_df(a.y, a.w, v.x, v.z, p, e);          // ai yr
-                            acc_df(ih[q], il[q], p, e);
-                        }
-                    }
-                }
-            }
-        }
-        double sx[8], sy[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            sx[q] = (double)rh[q] + (double)rl[q];
-            sy[q] = (double)ih[q] + (double)il[q];
-            for (int o = 16; o > 0; o >>= 1) {
-                sx[q] += __shfl_xor_sync(0xffffffffu, sx[q], o);
-                sy[q] += __shfl_xor_sync(0xffffffffu, sy[q], o);
-            }
-        }
-        if (i < rows && lane < nc) {
-            double vx = 0.0, vy = 0.0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                if (q == lane) {
-                    vx = sx[q];
-                    vy = sy[q];
-                }
-            const int cc = c0 + lane;
-            const size_t o = (size_t)(ooff[cc / R] + i) * R + cc % R;
-            double2 res = make_double2(beta * vx, beta * vy);
-            if (alpha != 0.0) {
-                res.x += alpha * sig[o].x;
-                res.y += alpha * sig[o].y;
-            }
-            out[o] = res;
-        }
+    const int ncol = ms * R, tn = std::min(4, (ncol + 3) / 4), ncb = (ncol + 4 * tn - 1) / (4 * tn);
+    // two rows to a block until that is eight blocks per SM, then four (half the reads of y)
+    const int tm = (long long)rows * ncb >= 2 * 8 * 152 ? 4 : 2;
+    auto run = [&](auto kern) {
+        kern<<<(unsigned)((rows + tm - 1) / tm) * (unsigned)ncb, 256, 0, st>>>(rows, cols, ms, R, ncb, yoff, ooff, A, y,
+                                                                             sig, alpha, beta, out);
+    };
+    if (tm == 4) {
+        if (tn == 1) run(body_gemm_kernel<E, 4, 1>);
+        else if (tn == 2) run(body_gemm_kernel<E, 4, 2>);
+        else if (tn == 3) run(body_gemm_kernel<E, 4, 3>);
+        else run(body_gemm_kernel<E, 4, 4>);
+    } else {
+        if (tn == 1) run(body_gemm_kernel<E, 2, 1>);
+        else if (tn == 2) run(body_gemm_kernel<E, 2, 2>);
+        else if (tn == 3) run(body_gemm_kernel<E, 2, 3>);
+        else run(body_gemm_kernel<E, 2, 4>);
     }
 }
 
 hzb_status reduced_local(hzb_ctx *c, int R, const double2 *y, const double2 *sigma, double alpha, double beta,
                          double2 *tau, bool fp32)
 {
+    float2 *y32 = nullptr;
+    if (fp32) {
+        const size_t n = (size_t)c->N * R;
+        if (check_cuda(c, c->ysplit.ensure((n + 1) / 2), "alloc")) return HZB_ENOMEM;
+        y32 = reinterpret_cast<float2 *>(c->ysplit.ptr);
+        round_f32_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, y, y32);
+        c->launches++;
+    }
     for (const hzb_ctx::RShape &rs : c->rshapes) {
-        if (fp32)
-            body_gemv_kernel<true><<<gemv_blocks(rs.k), 256, 0, c->stream>>>(rs.k, rs.k, rs.ms, R, rs.offs, rs.offs, rs.S32, y,
-                                                                sigma, alpha, beta, tau);
-        else
-            body_gemv_kernel<false><<<gemv_blocks(rs.k), 256, 0, c->stream>>>(rs.k, rs.k, rs.ms, R, rs.offs, rs.offs, rs.S64, y,
-                                                                 sigma, alpha, beta, tau);
+        if (fp32) body_gemm<float2>(c->stream, rs.k, rs.k, rs.ms, R, rs.offs, rs.offs, rs.S32, y32, sigma, alpha, beta, tau);
+        else body_gemm<double2>(c->stream, rs.k, rs.k, rs.ms, R, rs.offs, rs.offs, rs.S64, y, sigma, alpha, beta, tau);
         c->launches++;
     }
     return check_cuda(c, cudaGetLastError(), "reduced local operator");
@@ -1322,13 +1259,11 @@ static hzb_status restrict_all(hzb_ctx *c, int R, const double2 *w, double s, do
         ShapeDev &sd = *sp;
         const int n = sd.geom.NG * sd.geom.NF;
         if (df)
-            body_gemv_df_kernel<<<gemv_blocks(sd.skel_k), 256, 0, c->stream>>>(
-                sd.skel_k, n, (int)sd.bodies.size(), R, sd.body_offs.ptr, sd.red_offs.ptr, sd.Tdf.ptr, c->ysplit.ptr,
-                nullptr, 0.0, s, out);
+            body_gemm<float4>(c->stream, sd.skel_k, n, (int)sd.bodies.size(), R, sd.body_offs.ptr, sd.red_offs.ptr,
+                              sd.Tdf.ptr, c->ysplit.ptr, nullptr, 0.0, s, out);
         else
-            body_gemv_kernel<false><<<gemv_blocks(sd.skel_k), 256, 0, c->stream>>>(
-                sd.skel_k, n, (int)sd.bodies.size(), R, sd.body_offs.ptr, sd.red_offs.ptr, sd.T64.ptr, w, nullptr,
-                0.0, s, out);
+            body_gemm<double2>(c->stream, sd.skel_k, n, (int)sd.bodies.size(), R, sd.body_offs.ptr, sd.red_offs.ptr,
+                               sd.T64.ptr, w, nullptr, 0.0, s, out);
         c->launches++;
     }
     return check_cuda(c, cudaGetLastError(), "restrict");
@@ -1381,13 +1316,11 @@ hzb_status solve_reduced(hzb_ctx *c, int R, const double2 *v, const double2 *x0,
         ShapeDev &sd = *sp;
         const int n = sd.geom.NG * sd.geom.NF;
         if (df)
-            body_gemv_df_kernel<<<gemv_blocks(n), 256, 0, c->stream>>>(n, sd.skel_k, (int)sd.bodies.size(), R,
-                                                                      sd.red_offs.ptr, sd.body_offs.ptr, sd.Udf.ptr,
-                                                                      c->ysplit.ptr, v, -1.0, -1.0, c->w_b.ptr);
+            body_gemm<float4>(c->stream, n, sd.skel_k, (int)sd.bodies.size(), R, sd.red_offs.ptr, sd.body_offs.ptr,
+                              sd.Udf.ptr, c->ysplit.ptr, v, -1.0, -1.0, c->w_b.ptr);
         else
-            body_gemv_kernel<false><<<gemv_blocks(n), 256, 0, c->stream>>>(n, sd.skel_k, (int)sd.bodies.size(), R,
-                                                                          sd.red_offs.ptr, sd.body_offs.ptr, sd.U64.ptr,
-                                                                          r->s_r.ptr, v, -1.0, -1.0, c->w_b.ptr);
+            body_gemm<double2>(c->stream, n, sd.skel_k, (int)sd.bodies.size(), R, sd.red_offs.ptr, sd.body_offs.ptr,
+                               sd.U64.ptr, r->s_r.ptr, v, -1.0, -1.0, c->w_b.ptr);
         c->launches++;
     }
     if (check_cuda(c, cudaGetLastError(), "extend")) return HZB_ECUDA;
