@@ -136,7 +136,7 @@ hzb_status hzb_destroy(hzb_ctx *c)
     }
     c->pos64.release(); c->nrm64.release(); c->pos32.release(); c->nrm32.release(); c->body_of.release();
     c->tblocks.release(); c->body_xf.release(); c->w_a.release(); c->w_b.release(); c->w_c.release();
-    c->w_d.release(); c->f_a.release(); c->f_b.release(); c->yhat64.release(); c->that64.release();
+    c->w_d.release(); c->red_count.release(); c->f_a.release(); c->f_b.release(); c->yhat64.release(); c->that64.release();
     c->yhat32.release(); c->that32.release(); c->s_b.release(); c->s_r.release(); c->s_d.release();
     c->io_in.release(); c->io_out.release(); c->io_small.release(); c->tiny.release(); c->sol.release();
     c->red.release(); c->krylov.release(); c->small.release();

@@ -948,7 +948,7 @@ __global__ void gather_nodes_kernel(long long nr, const long long *__restrict__ 
 static void free_ctx_buffers(hzb_ctx *r)
 {
     r->pos64.release(); r->nrm64.release(); r->pos32.release(); r->nrm32.release(); r->body_of.release();
-    r->tblocks.release(); r->w_a.release(); r->w_b.release(); r->w_c.release(); r->w_d.release();
+    r->tblocks.release(); r->w_a.release(); r->w_b.release(); r->w_c.release(); r->w_d.release(); r->red_count.release();
     r->f_a.release(); r->f_b.release(); r->s_b.release(); r->s_r.release(); r->s_d.release(); r->io_in.release();
     r->io_out.release(); r->tiny.release(); r->sol.release(); r->red.release(); r->krylov.release();
     r->small.release(); r->sctab.release(); r->nb_part64.release(); r->nb_part32.release(); r->sig32.release();

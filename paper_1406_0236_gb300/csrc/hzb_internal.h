@@ -166,6 +166,7 @@ struct hzb_ctx {
 
     // workspaces
     hzb::DevBuf<double2> w_a, w_b, w_c, w_d;   // N x R
+    hzb::DevBuf<unsigned> red_count;           // blocks that have arrived, per dot product (krylov.cu)
     hzb::DevBuf<float2> f_a, f_b;              // N x R (FP32)
     hzb::DevBuf<double2> yhat64;               // modal workspace FP64
     hzb::DevBuf<double2> that64;

@@ -21,52 +21,101 @@
 
 namespace hzb {
 
-static const int RED_THREADS = 256;
+// Vectors are N x R; a block of 256 threads takes up to 32 right-hand sides (blockIdx.z) by a
+// power of two of node slots, so that a warp reads whole rows and a thread keeps to one right-hand
+// side.  R = 64 against one right-hand side per block (reads 16 bytes out of every 1,024): six dot
+// products of 525,000 values 42 -> 33 us, at the FP64 pipe's four FMAs per value; 9,636 values
+// with R = 4 in one block each 8.7 + 3.0 -> 7.5 us, and update, norm and rotation 25.6 -> 15 us in one launch.
+static const int RED_THREADS = 256, RED_COLS = 32, RED_BLOCKS = 608;
 
-// partial[(v * R + r) * nblk + blk] = sum over this block's nodes of conj(V_v) w
-__global__ void cdot_partial_kernel(long long N, int R, const double2 *__restrict__ V, long long vstride,
-                                    const double2 *__restrict__ w, double2 *partial)
+struct RedShape {
+    int cols, slots, chunks;        // right-hand sides per block, node slots, blocks over R
+};
+static RedShape red_shape(int R)
 {
-    __shared__ double2 red[RED_THREADS];
-    const int v = blockIdx.y, r = blockIdx.z, nblk = gridDim.x;
-    const double2 *Vv = V + v * vstride;
-    double2 acc = make_double2(0.0, 0.0);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)nblk * blockDim.x) {
-        double2 a = Vv[i * R + r], b = w[i * R + r];
-        acc.x = fma(a.x, b.x, fma(a.y, b.y, acc.x));
-        acc.y = fma(a.x, b.y, fma(-a.y, b.x, acc.y));
-    }
-    red[threadIdx.x] = acc;
+    RedShape q{std::min(R, RED_COLS), 1, (R + RED_COLS - 1) / RED_COLS};
+    while (2 * q.slots * q.cols <= RED_THREADS) q.slots *= 2;
+    return q;
+}
+// blocks over the nodes for nv vectors at once: about four per SM in all
+static int red_blocks(long long N, int R, int nv)
+{
+    const RedShape q = red_shape(R);
+    const long long most = std::max(1, RED_BLOCKS / (nv * q.chunks));
+    return (int)std::max<long long>(1, std::min<long long>({(N + q.slots - 1) / q.slots, most, 152}));
+}
+// values of partial sums for up to nv vectors (the products with nv = 1 use the most blocks)
+static size_t red_partials(long long N, int R, int nv)
+{
+    const RedShape q = red_shape(R);
+    size_t most = 0;
+    for (int v = 1; v <= nv; ++v) most = std::max(most, (size_t)v * q.chunks * q.cols * red_blocks(N, R, v));
+    return most;
+}
+
+// sum of v over the node slots, in slot 0's threads; every thread of the block calls it
+__device__ __forceinline__ double2 slot_sum(double2 v, double2 *red, int cols, int slots)
+{
+    const int t = threadIdx.x;
+    red[t] = v;
     __syncthreads();
-    for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] = cadd(red[threadIdx.x], red[threadIdx.x + s]);
+    for (int h = slots / 2; h > 0; h >>= 1) {
+        if (t < h * cols) red[t] = cadd(red[t], red[t + h * cols]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) partial[((size_t)v * R + r) * nblk + blockIdx.x] = red[0];
+    return red[t];
 }
 
-__global__ void cdot_final_kernel(int nvr, int nblk, const double2 *partial, double2 *out)
+// Adds the blocks' sums v (slot 0's threads) over blockIdx.x: the block that arrives last returns
+// true with the total in *total (slot 0's threads), the partial sums taken in a fixed order.  The
+// counter wraps to zero.
+__device__ __forceinline__ bool last_block_sum(double2 v, double2 *partial, unsigned *count, int group, int cols, int slots,
+                                               double2 *red, double2 *total)
 {
-    int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nvr) return;
-    double2 s = make_double2(0.0, 0.0);
-    for (int b = 0; b < nblk; ++b) s = cadd(s, partial[(size_t)e * nblk + b]);
-    out[e] = s;
-}
-
-// w[i][r] -= sum_{v < nv} V_v[i][r] h[v][r]
-__global__ void caxpy_multi_kernel(long long N, int R, int nv, const double2 *__restrict__ V, long long vstride,
-                                   const double2 *__restrict__ h, double2 *w)
-{
-    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= N * R) return;
-    int r = (int)(e % R);
-    double2 acc = w[e];
-    for (int v = 0; v < nv; ++v) {
-        double2 hv = h[v * R + r];
-        cfma(acc, make_double2(-hv.x, -hv.y), V[v * vstride + e]);
+    __shared__ bool last;
+    const int t = threadIdx.x, nblk = gridDim.x;
+    double2 *const mine = partial + (size_t)group * nblk * cols;
+    if (t < cols) {
+        mine[(size_t)blockIdx.x * cols + t] = v;
+        __threadfence();
     }
-    w[e] = acc;
+    __syncthreads();
+    if (t == 0) {
+        __threadfence();
+        last = atomicInc(&count[group], (unsigned)nblk - 1) == (unsigned)nblk - 1;
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    double2 s = make_double2(0.0, 0.0);
+    if (t < cols * slots)
+        for (int b = t / cols; b < nblk; b += slots) s = cadd(s, __ldcg(&mine[(size_t)b * cols + t % cols]));
+    *total = slot_sum(s, red, cols, slots);
+    return true;
+}
+
+// out[v * R + r] = sum_i conj(V_v[i][r]) w[i][r], v = blockIdx.y
+__global__ void __launch_bounds__(RED_THREADS)
+cdot_kernel(long long N, int R, int cols, int slots, const double2 *__restrict__ V, long long vstride,
+            const double2 *__restrict__ w, double2 *partial, unsigned *count, double2 *__restrict__ out)
+{
+    __shared__ double2 red[RED_THREADS];
+    const int v = blockIdx.y, t = threadIdx.x, slot = t / cols, r = blockIdx.z * RED_COLS + t % cols;
+    const double2 *const Vv = V + v * vstride;
+    double2 acc = make_double2(0.0, 0.0);
+    if (slot < slots && r < R) {
+        const long long step = (long long)gridDim.x * slots;
+#pragma unroll 4
+        for (long long i = (long long)blockIdx.x * slots + slot; i < N; i += step) {
+            const double2 a = Vv[i * R + r], b = w[i * R + r];
+            acc.x = fma(a.x, b.x, fma(a.y, b.y, acc.x));
+            acc.y = fma(a.x, b.y, fma(-a.y, b.x, acc.y));
+        }
+    }
+    acc = slot_sum(acc, red, cols, slots);
+    double2 total;
+    if (last_block_sum(acc, partial, count, blockIdx.z * gridDim.y + v, cols, slots, red, &total) && t < cols && r < R)
+        out[(size_t)v * R + r] = total;
 }
 
 // x[i][r] += sum_{v < jdone[r]} V_v[i][r] y[v][r]
@@ -134,35 +183,31 @@ __global__ void cycle_start_kernel(int R, int m, GmresState s, double tol, int f
 
 // Arnoldi column j: h = h1 + h2 (CGS2), h_{j+1,j} = ||w||; apply the previous
 // rotations, form the one that zeroes h_{j+1,j}, update g and the residual.
-__global__ void givens_kernel(int R, int m, int j, GmresState s, double tol)
+// column j of the Hessenberg matrix for right-hand side r from h1 + h2 and |w|^2: the rotations so
+// far, the new one, the residual estimate.  The column runs through registers; h1, h2, cs and sn
+// up to j come from earlier launches.
+__device__ void givens_column(int R, int m, int j, const GmresState &s, double tol, int r, double nrm2)
 {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
     if (!s.active[r]) {
         s.inv[r] = 0.0;
         return;
     }
-    if (!isfinite(s.nrm2[r].x)) {          // non-finite basis vector: report, do not treat as breakdown
+    if (!isfinite(nrm2)) {                 // non-finite basis vector: report, do not treat as breakdown
         s.res[r] = __longlong_as_double(0x7ff8000000000000ll);
         s.inv[r] = 0.0;
         s.active[r] = 0;
         return;
     }
-    double hn = sqrt(fmax(s.nrm2[r].x, 0.0));
-    for (int i = 0; i <= j; ++i) {
-        double2 v = cadd(s.h1[i * R + r], s.h2[i * R + r]);
-        s.H[((size_t)i * m + j) * R + r] = v;
-    }
+    const double hn = sqrt(fmax(nrm2, 0.0));
+    double2 a = cadd(__ldg(&s.h1[r]), __ldg(&s.h2[r]));
+#pragma unroll 4
     for (int i = 0; i < j; ++i) {
-        double2 a = s.H[((size_t)i * m + j) * R + r], b = s.H[((size_t)(i + 1) * m + j) * R + r];
-        double2 c = s.cs[i * R + r], sn = s.sn[i * R + r];
-        double2 t = cadd(cmul(c, a), cmul(sn, b));
-        double2 u = csub(cmul(cconj(c), b), cmul(cconj(sn), a));
-        s.H[((size_t)i * m + j) * R + r] = t;
-        s.H[((size_t)(i + 1) * m + j) * R + r] = u;
+        const double2 b = cadd(__ldg(&s.h1[(i + 1) * R + r]), __ldg(&s.h2[(i + 1) * R + r]));
+        const double2 c = __ldg(&s.cs[i * R + r]), sn = __ldg(&s.sn[i * R + r]);
+        s.H[((size_t)i * m + j) * R + r] = cadd(cmul(c, a), cmul(sn, b));
+        a = csub(cmul(cconj(c), b), cmul(cconj(sn), a));
     }
-    double2 a = s.H[((size_t)j * m + j) * R + r];
-    double den = sqrt(a.x * a.x + a.y * a.y + hn * hn);
+    const double den = sqrt(a.x * a.x + a.y * a.y + hn * hn);
     double2 c, sn;
     if (den > 0.0) {
         c = make_double2(a.x / den, -a.y / den);      // conj(a) / den
@@ -174,31 +219,69 @@ __global__ void givens_kernel(int R, int m, int j, GmresState s, double tol)
     s.cs[j * R + r] = c;
     s.sn[j * R + r] = sn;
     s.H[((size_t)j * m + j) * R + r] = make_double2(den, 0.0);
-    double2 gj = s.g[j * R + r];
-    s.g[(j + 1) * R + r] = cscale(cmul(cconj(sn), gj), -1.0);
+    const double2 gj = s.g[j * R + r], gn = cscale(cmul(cconj(sn), gj), -1.0);
+    s.g[(j + 1) * R + r] = gn;
     s.g[j * R + r] = cmul(c, gj);
-    double2 gn = s.g[(j + 1) * R + r];
-    double rel = sqrt(gn.x * gn.x + gn.y * gn.y) / s.bnorm[r];
+    const double rel = sqrt(gn.x * gn.x + gn.y * gn.y) / s.bnorm[r];
     s.res[r] = rel;
     s.jdone[r] = j + 1;
-    bool done = !(rel > tol) || !(hn > 1e-300) || !isfinite(rel);
+    const bool done = !(rel > tol) || !(hn > 1e-300) || !isfinite(rel);
     s.inv[r] = done ? 0.0 : 1.0 / hn;
     if (done) s.active[r] = 0;
 }
 
-// y = H^{-1} g on the leading jdone x jdone upper triangle.
-__global__ void backsolve_kernel(int R, int m, GmresState s, double2 *y)
+// w[i][r] -= sum_{v < nv} V_v[i][r] h[v][r]; STEP: then |w|^2 per right-hand side and, in the block
+// that arrives last, column nv - 1 of the Hessenberg matrix
+template <bool STEP>
+__global__ void __launch_bounds__(RED_THREADS)
+caxpy_kernel(long long N, int R, int cols, int slots, int nv, const double2 *__restrict__ V, long long vstride,
+             const double2 *__restrict__ h, double2 *__restrict__ w, double2 *partial, unsigned *count, int m, GmresState s,
+             double tol)
 {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    int n = s.jdone[r];
-    for (int i = n - 1; i >= 0; --i) {
-        double2 acc = s.g[i * R + r];
-        for (int q = i + 1; q < n; ++q) cfma(acc, make_double2(-1.0, 0.0), cmul(s.H[((size_t)i * m + q) * R + r], y[q * R + r]));
-        double2 d = s.H[((size_t)i * m + i) * R + r];
-        double dd = d.x * d.x + d.y * d.y;
-        y[i * R + r] = dd > 0.0 ? make_double2((acc.x * d.x + acc.y * d.y) / dd, (acc.y * d.x - acc.x * d.y) / dd)
-                                : make_double2(0.0, 0.0);
+    __shared__ double2 red[RED_THREADS];
+    const int t = threadIdx.x, slot = t / cols, r = blockIdx.z * RED_COLS + t % cols;
+    double2 sum = make_double2(0.0, 0.0);
+    if (slot < slots && r < R) {
+        const long long step = (long long)gridDim.x * slots;
+        for (long long i = (long long)blockIdx.x * slots + slot; i < N; i += step) {
+            const long long e = i * R + r;
+            double2 acc = w[e];
+#pragma unroll 4
+            for (int v = 0; v < nv; ++v) {
+                const double2 hv = h[(size_t)v * R + r];
+                cfma(acc, make_double2(-hv.x, -hv.y), V[v * vstride + e]);
+            }
+            w[e] = acc;
+            sum.x = fma(acc.x, acc.x, fma(acc.y, acc.y, sum.x));
+        }
+    }
+    if (!STEP) return;
+    sum = slot_sum(sum, red, cols, slots);
+    double2 total;
+    if (last_block_sum(sum, partial, count, blockIdx.z, cols, slots, red, &total) && t < cols && r < R)
+        givens_column(R, m, nv - 1, s, tol, r, total.x);
+}
+
+// y = H^{-1} g on the leading jdone x jdone upper triangle: a warp per right-hand side, the lanes
+// over the rows above the current one (lane = row mod 32 owns the row's g, which is overwritten).
+__global__ void __launch_bounds__(32) backsolve_kernel(int R, int m, GmresState s, double2 *__restrict__ y)
+{
+    const int r = blockIdx.x, lane = threadIdx.x, n = s.jdone[r];
+    for (int q = n - 1; q >= 0; --q) {
+        double2 yq = make_double2(0.0, 0.0);
+        if (lane == (q & 31)) {
+            const double2 acc = s.g[q * R + r], d = s.H[((size_t)q * m + q) * R + r];
+            const double dd = d.x * d.x + d.y * d.y;
+            if (dd > 0.0) yq = make_double2((acc.x * d.x + acc.y * d.y) / dd, (acc.y * d.x - acc.x * d.y) / dd);
+            y[q * R + r] = yq;
+        }
+        yq.x = __shfl_sync(0xffffffffu, yq.x, q & 31);
+        yq.y = __shfl_sync(0xffffffffu, yq.y, q & 31);
+        for (int i = lane; i < q; i += 32) {
+            double2 acc = s.g[i * R + r];
+            const double2 u = cmul(s.H[((size_t)i * m + q) * R + r], yq);
+            s.g[i * R + r] = csub(acc, u);
+        }
     }
 }
 
@@ -234,17 +317,29 @@ hzb_status vec_zero(hzb_ctx *c, double2 *dst, size_t n)
 
 static unsigned nblocks(long long n, int th = 256) { return (unsigned)((n + th - 1) / th); }
 
+// room for the partial sums and block counters of up to nv vectors
+static hzb_status ensure_red(hzb_ctx *c, int R, int nv)
+{
+    const size_t groups = (size_t)nv * red_shape(R).chunks;
+    if (check_cuda(c, c->w_d.ensure(std::max(red_partials(c->N, R, nv), (size_t)c->N * R)), "alloc partial"))
+        return HZB_ENOMEM;
+    if (groups > c->red_count.n) {
+        if (check_cuda(c, c->red_count.ensure(groups), "alloc counters")) return HZB_ENOMEM;
+        if (check_cuda(c, cudaMemsetAsync(c->red_count.ptr, 0, c->red_count.n * sizeof(unsigned), c->stream), "memset"))
+            return HZB_ECUDA;
+    }
+    return HZB_OK;
+}
+
 // out[v * R + r] = sum_i conj(V_v[i][r]) w[i][r], v < nv
 static hzb_status cdots(hzb_ctx *c, int R, int nv, const double2 *V, long long vstride, const double2 *w,
                         double2 *out)
 {
-    long long N = c->N;
-    int nblk = (int)std::min<long long>(120, std::max<long long>(1, N / (RED_THREADS * 8)));
-    size_t need = (size_t)nv * R * nblk;
-    if (check_cuda(c, c->w_d.ensure(std::max<size_t>(need, (size_t)N * R)), "alloc partial")) return HZB_ENOMEM;
-    cdot_partial_kernel<<<dim3(nblk, nv, R), RED_THREADS, 0, c->stream>>>(N, R, V, vstride, w, c->w_d.ptr);
-    cdot_final_kernel<<<nblocks(nv * R), 256, 0, c->stream>>>(nv * R, nblk, c->w_d.ptr, out);
-    c->launches += 2;
+    if (hzb_status st = ensure_red(c, R, nv)) return st;
+    const RedShape q = red_shape(R);
+    cdot_kernel<<<dim3(red_blocks(c->N, R, nv), nv, q.chunks), RED_THREADS, 0, c->stream>>>(
+        c->N, R, q.cols, q.slots, V, vstride, w, c->w_d.ptr, c->red_count.ptr, out);
+    c->launches++;
     return check_cuda(c, cudaGetLastError(), "cdot");
 }
 
@@ -278,7 +373,7 @@ static hzb_status ensure_pinned(hzb_ctx *c, size_t n)
 
 // Pointers and sizes a captured Arnoldi step depends on: a change invalidates the graphs.
 struct GraphKey {
-    static const int NP = 25;
+    static const int NP = 26;
     const void *p[NP];
     long long N;
     int R, m, precision, tpt32, split32, tpt64, split64, modal_engine, nbody_engine, splittc, tc32, x2, engine64;
@@ -380,13 +475,11 @@ hzb_status gmres_solve(hzb_ctx *c, int R, const double2 *b, double2 *x, int x_is
     double *hres = c->host_pinned;
     int *hact = (int *)(c->host_pinned + R);
     int *hjd = hact + R;
-    // dot-product partial sums sized for the largest step, so that a captured step
-    // never reallocates
-    {
-        int nblk = (int)std::min<long long>(120, std::max<long long>(1, N / (RED_THREADS * 8)));
-        if (check_cuda(c, c->w_d.ensure(std::max<size_t>((size_t)(m + 1) * R * nblk, NR)), "alloc partial"))
-            return HZB_ENOMEM;
-    }
+    // partial sums sized for the largest step, so that a captured step never reallocates
+    if ((st = ensure_red(c, R, m + 1))) return st;
+    const RedShape rq = red_shape(R);
+    const dim3 gaxpy((unsigned)std::max<long long>(1, std::min<long long>((N + rq.slots - 1) / rq.slots, 152 * 8)), 1, rq.chunks);
+    const dim3 gstep(red_blocks(N, R, 1), 1, rq.chunks);
     // CUDA graphs need a capturable (non-legacy) stream; auto = small problems only
     bool graphs = c->use_graphs > 0 || (c->use_graphs < 0 && (long long)NR <= 4000000);
     if (c->stream == nullptr) graphs = false;
@@ -400,7 +493,7 @@ hzb_status gmres_solve(hzb_ctx *c, int R, const double2 *b, double2 *x, int x_is
                                         c->sctab.ptr, (const void *)c->stream, c->tblocks.ptr, c->sig32.ptr,
                                         c->w_a.ptr, c->w_b.ptr, c->f_a.ptr, c->f_b.ptr, c->dfa.ptr,
                                         c->blockpairs.ptr, c->Ximg.ptr, c->t5h_img.ptr, c->dlkey.ptr,
-                                        c->ysplit.ptr};
+                                        c->ysplit.ptr, c->red_count.ptr};
         std::memcpy(graph_key.p, ps, sizeof(ps));
         graph_key.N = N; graph_key.R = R; graph_key.m = m; graph_key.precision = precision;
         graph_key.tpt32 = c->tune32_tpt; graph_key.split32 = c->tune32_split;
@@ -448,12 +541,12 @@ hzb_status gmres_solve(hzb_ctx *c, int R, const double2 *b, double2 *x, int x_is
             double2 *Vj = V + (size_t)jj * NR;
             if ((e2 = apply_op(c, R, Vj, w, precision))) return e2;
             if ((e2 = cdots(c, R, jj + 1, V, (long long)NR, w, s.h1))) return e2;
-            caxpy_multi_kernel<<<gN, 256, 0, c->stream>>>(N, R, jj + 1, V, (long long)NR, s.h1, w);
+            caxpy_kernel<false><<<gaxpy, RED_THREADS, 0, c->stream>>>(N, R, rq.cols, rq.slots, jj + 1, V, (long long)NR, s.h1,
+                                                                     w, nullptr, nullptr, m, s, tol);
             if ((e2 = cdots(c, R, jj + 1, V, (long long)NR, w, s.h2))) return e2;
-            caxpy_multi_kernel<<<gN, 256, 0, c->stream>>>(N, R, jj + 1, V, (long long)NR, s.h2, w);
-            if ((e2 = cdots(c, R, 1, w, 0, w, s.nrm2))) return e2;
-            givens_kernel<<<gR, 64, 0, c->stream>>>(R, m, jj, s, tol);
-            c->launches += 4;                  // two caxpy, givens, scale
+            caxpy_kernel<true><<<gstep, RED_THREADS, 0, c->stream>>>(N, R, rq.cols, rq.slots, jj + 1, V, (long long)NR, s.h2,
+                                                                    w, c->w_d.ptr, c->red_count.ptr, m, s, tol);
+            c->launches += 3;                  // two caxpy (the second with norm and rotation), scale
             scale_kernel<<<gN, 256, 0, c->stream>>>(N, R, w, s.inv, V + (size_t)(jj + 1) * NR);
             return HZB_OK;
         };
@@ -489,7 +582,7 @@ hzb_status gmres_solve(hzb_ctx *c, int R, const double2 *b, double2 *x, int x_is
             for (int r = 0; r < R; ++r) jmax = std::max(jmax, hjd[r]);
             real_iters += jmax;
         }
-        backsolve_kernel<<<gR, 64, 0, c->stream>>>(R, m, s, y);
+        backsolve_kernel<<<(unsigned)R, 32, 0, c->stream>>>(R, m, s, y);
         update_x_kernel<<<gN, 256, 0, c->stream>>>(N, R, m, V, (long long)NR, y, s.jdone, x);
         c->launches += 2;
         if (check_cuda(c, cudaGetLastError(), "gmres update")) return HZB_ECUDA;
