@@ -287,8 +287,11 @@ hzb_status hzb_set_interbody_engine(hzb_ctx *ctx, int engine);
  * shared), about 1.5x fewer operations; both directions are added into y with FP64
  * atomics, so runs agree to rounding but not bit for bit; -1 (default) = 1 for R <= 4
  * right-hand sides, 0 above (the one-directional kernels amortise the pair geometry over
- * up to 8 right-hand sides per CTA; the double-float one, with up to 32, is taken from
- * R = 3 on when a target has 4,096 sources or more); 2 = pair-symmetric, with the double-float sum in its
+ * up to 8 right-hand sides per CTA), except that the double-float sum of R >= 3 right-hand
+ * sides with N^2 R >= 2.4e7 runs on the tensor cores (products of FP16 digits, exact sums;
+ * bit-reproducible; it may return HZB_ETIMEOUT like the FP32 tensor-core sums) unless the
+ * bodies nearly touch or k = 0, and is one-directional from R = 3 on when a target has 4,096
+ * sources or more; 2 = pair-symmetric, with the double-float sum in its
  * earlier form (every double-float operation renormalised; the FP64 sum as for 1).  The
  * pair-symmetric double-float sum of engine 1 leaves its products and sums unnormalised
  * and takes e^{ikr} from a 1024-entry table (about 1.7x fewer FP32 operations).  Returns

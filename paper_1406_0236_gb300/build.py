@@ -22,10 +22,10 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", 
          "--expt-relaxed-constexpr", "-I", INCLUDE]
 
 SOURCES = ["api.cpp", "geometry.cpp", "setup.cu", "nbody.cu", "modal.cu", "krylov.cu", "mlp.cu", "noalloc.cu",
-           "nbody_df.cu", "nbody_tc.cu", "nbody_sym.cu", "nbody_tc5.cu", "nbody_t5h.cu", "persist.cu", "modal_tma.cu", "compress.cu", "nbody_dfl.cu", "peaks.cu", "pod.cu", "modal_dfl.cu"]
+           "nbody_df.cu", "nbody_tc.cu", "nbody_sym.cu", "nbody_tc5.cu", "nbody_t5h.cu", "persist.cu", "modal_tma.cu", "compress.cu", "nbody_dfl.cu", "nbody_dfx.cu", "peaks.cu", "pod.cu", "modal_dfl.cu"]
 # double-float error-free transformations must not be contracted into fused multiply-adds
 # the FP32 inter-body kernel flushes denormals (irrelevant to its values, cheaper intrinsics)
-PER_FILE = {"nbody_df.cu": ["-fmad=false"], "nbody_dfl.cu": ["-fmad=false"], "nbody.cu": ["-ftz=true"], "nbody_tc.cu": ["-ftz=true"], "nbody_sym.cu": ["-ftz=true"], "nbody_tc5.cu": ["-ftz=true"], "nbody_t5h.cu": ["-ftz=true"]}
+PER_FILE = {"nbody_df.cu": ["-fmad=false"], "nbody_dfl.cu": ["-fmad=false"], "nbody_dfx.cu": ["-fmad=false"], "nbody.cu": ["-ftz=true"], "nbody_tc.cu": ["-ftz=true"], "nbody_sym.cu": ["-ftz=true"], "nbody_tc5.cu": ["-ftz=true"], "nbody_t5h.cu": ["-ftz=true"]}
 HEADERS = sorted(f for f in os.listdir(SRC) if f.endswith((".h", ".cuh")))
 
 

@@ -196,11 +196,12 @@ struct hzb_ctx {
     // FP16 tensor-core form (nbody_t5h.cu): 0 not built, 1 usable, -1 out of FP16's range; tiles of 32
     // sources of one body, the target blocks' own tiles, the tiles' geometry, operand images of a call
     int t5h_state = 0, t5h_ntiles = 0, t5h_most = 0, t5h_ctas = 0;
-    double t5h_scale = 0.0;
+    double t5h_scale = 0.0, t5h_span = 0.0;
     hzb::DevBuf<int2> t5h_tiles;
     hzb::DevBuf<float> t5h_src;
     hzb::DevBuf<unsigned char> t5h_img;
-    int nbody64_engine = -1;                   // FP64/double-float sums: -1 auto (pair-symmetric for R <= 4),
+    int nbody64_engine = -1;                   // FP64/double-float sums: -1 auto (pair-symmetric for R <= 4;
+                                               // double-float: nbody_dfx.cu where it applies),
                                                // 0 one-directional, 1 pair-symmetric (double-float: lean forms),
                                                // 2 as -1 with the normalised double-float kernels
     hzb::DevBuf<int> kerr;                     // device error flag of kernels with bounded waits
@@ -304,7 +305,10 @@ hzb_status interbody_tc(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int
 hzb_status modal_gemm_tma(hzb_ctx *c, ShapeDev &sd, int ncols, const float2 *X, float2 *Cout);  // modal_tma.cu
 enum { T5_SPLIT3 = 0, T5_WS = 1, T5_SINGLE = 2 };   // forms of the tcgen05 inter-body kernel
 // nbody_t5h.cu: FP16 three-term form, where the geometry's kernels fit FP16's range
+hzb_status ensure_t5h(hzb_ctx *c);
 bool t5h_usable(hzb_ctx *c, hzb_status *st);
+bool dfx_usable(hzb_ctx *c, int R, hzb_status *st);
+hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
 hzb_status interbody_t5h(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
 // nbody_tc5.cu: the device flag of the tensor-core kernels' bounded waits, around a launch
 hzb_status tc_flag_begin(hzb_ctx *c, bool inject);

@@ -406,11 +406,14 @@ static hzb_status interbody_df_sym(hzb_ctx *c, int R, const double2 *sigma, doub
 hzb_status interbody_df(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
 {
     if (!c->nodes_ready) return fail(c, HZB_ESTATE, "nodes not built");
-    // the lean kernels: pair-symmetric for few right-hand sides, one-directional above
+    // the lean kernels: tensor-core sums where they apply, else pair-symmetric for few right-hand
+    // sides, one-directional above
+    hzb_status st = HZB_OK;
+    if (c->nbody64_engine < 0 && dfx_usable(c, R, &st)) return interbody_dfx(c, R, sigma, y);
+    if (st) return st;
     if (c->nbody64_engine == 1 || (c->nbody64_engine < 0 && dfl_symmetric(c, R))) return interbody_dfl_sym(c, R, sigma, y);
     if (c->nbody64_engine != 2) return interbody_dfl(c, R, sigma, y);
-    hzb_status st = ensure_df(c);
-    if (st) return st;
+    if ((st = ensure_df(c))) return st;
     if (R <= 4) return interbody_df_sym(c, R, sigma, y);
     const int N = (int)c->N;
     const int rc = R == 1 ? 1 : (R <= 4 ? 4 : 8);

@@ -439,7 +439,7 @@ __global__ void t5h_reduce_kernel(size_t n, int R, int nsplit, double f, const i
 // ---------------------------------------------------------------- host
 
 // Tiles, their geometry and the range of the kernel, once per geometry.
-static hzb_status ensure_t5h(hzb_ctx *c)
+hzb_status ensure_t5h(hzb_ctx *c)
 {
     if (c->t5h_state) return HZB_OK;
     if (c->capturing) return fail(c, HZB_ESTATE, "tiles not built before capture");
@@ -491,6 +491,14 @@ static hzb_status ensure_t5h(hzb_ctx *c)
         return HZB_ECUDA;
     const double g = range[0], diam = range[1];
     // |G'| <= u (1 + (k / |eta|) (1 + u)), u = 1 / (k r); the smallest is about u at the diameter
+    c->t5h_ntiles = nt;
+    c->t5h_ctas = 0;
+    for (const TargetBlock &t : tb) c->t5h_ctas += (t.count + TH_M - 1) / TH_M;
+    c->t5h_most = 1;                                           // tiles of the other bodies, at most
+    for (const int2 &o : own) c->t5h_most = std::max(c->t5h_most, nt - (o.y - o.x));
+    // |G| <= u (u + 1 + |eta| / k): its bounds at the smallest and the largest distance (nbody_dfx.cu)
+    const double q = 1.0 + std::fabs(c->eta) / c->k;
+    c->t5h_span = g > 0.0 && diam > 0.0 && diam < 9e4 ? (1.0 / g) * (1.0 / g + q) / ((1.0 / diam) * (1.0 / diam + q)) : 0.0;
     const double u = 1.0 / g, bound = u * (1.0 + (c->k / std::fabs(c->eta)) * (1.0 + u)) * 1.001;
     c->t5h_state = -1;
     if (std::isfinite(bound) && g > 0.0 && diam > 0.0 && diam < 9e4 && bound * diam < 262144.0) {
@@ -498,11 +506,6 @@ static hzb_status ensure_t5h(hzb_ctx *c)
         std::frexp(bound, &e);                                 // bound < 2^e
         if (e > -100 && e < 100) {
             c->t5h_scale = std::ldexp(1.0, 15 - e);
-            c->t5h_ntiles = nt;
-            c->t5h_ctas = 0;
-            for (const TargetBlock &t : tb) c->t5h_ctas += (t.count + TH_M - 1) / TH_M;
-            c->t5h_most = 1;                                   // tiles of the other bodies, at most
-            for (const int2 &o : own) c->t5h_most = std::max(c->t5h_most, nt - (o.y - o.x));
             c->t5h_state = 1;
         }
     }
