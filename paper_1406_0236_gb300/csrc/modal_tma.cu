@@ -149,9 +149,10 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
     const int ng = (nk + MT_FLUSH - 1) / MT_FLUSH;
 
     if (warp == 8) {
-        if (lane == 0) {
-            // ---------------------------------------------- TMA and MMA issue
+        {
+            // ---------------------------------------------- TMA and MMA issue (one elected lane)
             auto issue_tma = [&](int kc) {
+                if (!t5_elect()) return;
                 const int st = kc & 1;
                 const uint32_t sA = base + (uint32_t)st * MT_STAGE;
                 const uint32_t fb = tma_full0 + 8 * st;
@@ -181,6 +182,7 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
                 const uint32_t sA = base + (uint32_t)st * MT_STAGE;
                 const uint32_t as[3] = {sA, sA, sA + MT_A};
                 const uint32_t bs[3] = {sA + 2 * MT_A, sA + 2 * MT_A + MT_B, sA + 2 * MT_A};
+                if (t5_elect()) {
 #pragma unroll
                 for (int ks = 0; ks < MT_K / 8; ++ks)
 #pragma unroll
@@ -194,6 +196,8 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                      acc_full0 + 8 * b)
                                  : "memory");
+                }
+                __syncwarp();
             }
         }
     } else {

@@ -82,14 +82,6 @@ __device__ __forceinline__ void dx_mma(uint32_t d, uint32_t ad, uint32_t bd, uin
         : "memory");
 }
 
-// one lane of a converged warp
-__device__ __forceinline__ bool dx_elect()
-{
-    uint32_t p;
-    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
-    return p != 0;
-}
-
 __device__ __forceinline__ void dx_copy(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar)
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -318,7 +310,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                 ok = t5_wait(bar0 + 32 + 8 * h, (uint32_t)(i & 1)) && !s_fail;
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (dx_elect()) {
+                if (t5_elect()) {
                     // (unrolled: in a loop the address arithmetic of one MMA took this warp 200 cycles)
                     const uint32_t ad = (uint32_t)t5_desc(a0 + 64 * h);
                     const uint32_t bd = (uint32_t)t5_desc(b0 + (uint32_t)((i & 1) * STAGE) + 64 * h);

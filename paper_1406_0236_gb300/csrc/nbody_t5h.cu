@@ -240,7 +240,7 @@ nbody_t5h_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
             ok = false;
             break;
         }
-        if (tid == 0) {
+        if (warp == 0 && t5_elect()) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t desc = t5_desc(base + (uint32_t)((i & 1) * STAGE));
 #pragma unroll

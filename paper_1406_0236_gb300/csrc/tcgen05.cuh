@@ -59,6 +59,14 @@ __device__ __forceinline__ void t5_mma(uint32_t tmem, uint64_t ad, uint64_t bd, 
         : "memory");
 }
 
+// one lane of a converged warp
+__device__ __forceinline__ bool t5_elect()
+{
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ bool t5_wait(uint32_t mbar, uint32_t parity)
 {
     for (int it = 0; it < (1 << 22); ++it) {
