@@ -196,7 +196,7 @@ struct hzb_ctx {
     // FP16 tensor-core form (nbody_t5h.cu): 0 not built, 1 usable, -1 out of FP16's range; tiles of 32
     // sources of one body, the target blocks' own tiles, the tiles' geometry, operand images of a call
     int t5h_state = 0, t5h_ntiles = 0, t5h_most = 0, t5h_ctas = 0;
-    double t5h_scale = 0.0, t5h_span = 0.0;
+    double t5h_scale = 0.0, t5h_span = 0.0, t5h_mean = 1.0;
     hzb::DevBuf<int2> t5h_tiles;
     hzb::DevBuf<float> t5h_src;
     hzb::DevBuf<unsigned char> t5h_img;

@@ -52,7 +52,7 @@ static const int DX_M = 128, DX_FORM = 512, DX_THREADS = DX_FORM + 32, DX_D = 6;
 // and of the one-directional kernel: ratio 45: 4.0e-14, 7.0e-14; 180: 5.6e-14, 7.2e-14; 363:
 // 9.3e-14, 8.8e-14; 8,200: 1.3e-13, 1.0e-13
 static const double DX_SPAN = 128.0;
-static const double DX_START = 0.5;    // a CTA's start, in tiles
+static double dx_start(int rc) { return rc == 8 ? 0.5 : rc == 16 ? 0.8 : 1.2; }    // a CTA's start and end, in tiles
 // N^2 R from which on this form is the faster one (us, here / one-directional): 900 unknowns
 // (R = 16: 1.3e7) 74 / 74, 1,764 (R = 8: 2.5e7) 81 / 79, (R = 16) 85 / 117, 3,968 (R = 5) 163 / 206
 static const double DX_WORK = 2.4e7;
@@ -139,7 +139,7 @@ __device__ __forceinline__ uint32_t dx_pack(float a, float b)
 template <int RC>
 __global__ void __launch_bounds__(DX_THREADS, 1)
 nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict__ own_tiles,
-                 const int2 *__restrict__ tiles, const float4 *__restrict__ ball, int ntiles, int chunk, int R,
+                 const int2 *__restrict__ tiles, const float4 *__restrict__ ball, int ntiles, int R,
                  const float4 *__restrict__ pa, const float4 *__restrict__ pb, const float4 *__restrict__ pc,
                  const unsigned char *__restrict__ img, const int *__restrict__ key, const float4 *__restrict__ tab,
                  DflConst K, double2 *__restrict__ out, size_t split_stride, int *__restrict__ err)
@@ -195,8 +195,8 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     // the tiles of the other bodies, counted without the own body's [own.x, own.y)
     const int2 own = own_tiles[blockIdx.x >> 2];
     const int nown = own.y - own.x;
-    const int i0 = blockIdx.z * chunk, i1 = min(ntiles - nown, i0 + chunk);
-    const int n = max(0, i1 - i0);
+    const int i0 = (int)((long long)(ntiles - nown) * blockIdx.z / gridDim.z);
+    const int n = (int)((long long)(ntiles - nown) * (blockIdx.z + 1) / gridDim.z) - i0;
     auto tile_of = [&](int i) {
         const int q = i0 + i;
         return q < own.x ? q : q + nown;
@@ -484,17 +484,20 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     const int rc = R <= 8 ? 8 : R <= 16 ? 16 : 32, nchunk = (R + rc - 1) / rc, nt = c->t5h_ntiles, most = c->t5h_most;
     hzb_status st = ensure_dfl(c);
     if (st) return st;
-    // Source chunks: the fewest tile times over the waves (a partial sum costs 1e-6 of a tile), at most 256 tiles to a chunk (the sums' 64 bits).
+    // Source chunks: the shortest time, in tiles.  Bodies of one size: whole waves of equal CTAs;
+    // others: the mean load and most of a long CTA's time at the end.  A partial sum costs 1e-6 of a
+    // tile; at most 256 tiles go to a chunk (the sums' 64 bits).
     const long long ctas = (long long)c->t5h_ctas * nchunk;
+    const bool even = c->t5h_mean > 0.97 * most;
     int nsplit = (most + 255) / 256;
     double best = 1e300;
     for (int ns = nsplit; ns <= std::max(nsplit, std::min(64, most)); ++ns) {
-        const double waves = std::ceil((double)(ns * ctas) / sms);
-        const double tt = waves * (std::ceil((double)most / ns) + DX_START) + 1e-6 * (double)c->N * R * ns;
+        const double one = std::ceil((double)most / ns) + dx_start(rc);
+        const double tt = (even ? std::ceil((double)(ns * ctas) / sms) * one
+                                : std::max(one, ctas * (c->t5h_mean + ns * dx_start(rc)) / sms + 0.6 * one)) +
+                          1e-6 * (double)c->N * R * ns;
         if (tt < best) { best = tt; nsplit = ns; }
     }
-    const int chunk = (most + nsplit - 1) / nsplit;
-    nsplit = (most + chunk - 1) / chunk;
     const size_t n = (size_t)c->N * R;
     double2 *out = y;
     if (nsplit > 1) {
@@ -520,7 +523,7 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dx_smem(rc));
         if (e != cudaSuccess) return;
         kern<<<grid, DX_THREADS, dx_smem(rc), c->stream>>>(
-            c->tblocks.ptr, c->t5h_tiles.ptr + nt, c->t5h_tiles.ptr, ball, nt, chunk, R, c->dla.ptr, c->dlb.ptr, c->dlc.ptr,
+            c->tblocks.ptr, c->t5h_tiles.ptr + nt, c->t5h_tiles.ptr, ball, nt, R, c->dla.ptr, c->dlb.ptr, c->dlc.ptr,
             c->t5h_img.ptr, c->dlkey.ptr, c->dfltab.ptr, dfl_constants(c), out, n, c->kerr.ptr);
         e = cudaGetLastError();
     };

