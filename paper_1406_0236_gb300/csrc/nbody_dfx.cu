@@ -17,22 +17,28 @@
 // Per CTA: 128 targets (the M of the MMA), RC right-hand sides (N = 2 RC columns: real and
 // imaginary parts), a chunk of the source tiles.  Sixteen warps form kernels, four sources of each
 // half tile for a thread's target (row): one 16-byte chunk (four sources, real and imaginary part) of
-// each of the six digit images of A in shared memory (K-major, 128-byte swizzle).  A seventeenth
+// each of the six digit images of A in shared memory (K-major, 64-byte swizzle).  A seventeenth
 // warp issues the half tile's 42 MMAs when all have arrived and fetches the digit images of the
 // densities (dfx_density_kernel, one 128-byte row per column and digit) and the sources' nodes two
 // tiles ahead; the sixteen never wait for one another.  Before the first MMA of every second tile
 // they move the levels into the 64-bit sums, which live in tensor memory too (columns 12 RC ..
 // 16 RC).
 //
+// More than 32 right-hand sides (tensor memory holds the levels and sums of 32): two CTAs of a
+// cluster take the same targets and sources with 32 right-hand sides each, form half of every tile
+// each and send it to the other by one bulk copy (stores to the other CTA's shared memory by the
+// forming warps took 4,900 cycles a tile, as long as the forming).  Then the 84 MMAs of a tile (about
+// 60 cycles each: both operands come from shared memory) and the forming take about equally long.
+//
 // Bound by the issue of the pair kernels and digits, about 260 + 55 FP32 operations per pair and
 // RC right-hand sides (77 % of the issue slots at RC = 8); the one-directional kernel of
 // nbody_dfl.cu spends another 28 slots per pair and right-hand side on the sums.  Against it, and
 // the error of each against 64 bits:
-//   29,280 unknowns, k = 6:  R = 4  8.70 -> 7.19 ms;  R = 8  10.9 -> 7.2;  R = 16  16.6 -> 7.4;
-//                            R = 64  61.0 -> 15.1 ms, 1.2e-13 -> 1.1e-13
-//   8,200 unknowns, k = 2:   R = 8  0.65 -> 0.49 ms;  R = 64  3.73 -> 0.99 ms, 5.6e-14 -> 3.4e-14
-// A barrier of all warps per half tile took 1.50 ms for the last, levels moved every tile 1.44, the
-// MMAs issued from a loop (200 cycles each for the address arithmetic) 1.38.
+//   29,280 unknowns, k = 6:  R = 4  8.70 -> 7.26 ms;  R = 8  10.9 -> 7.3;  R = 16  16.6 -> 7.4;
+//                            R = 64  61.0 -> 11.8 ms, 1.2e-13 -> 1.1e-13
+//   8,200 unknowns, k = 2:   R = 8  0.65 -> 0.49 ms;  R = 64  3.73 -> 0.77 ms, 5.6e-14 -> 3.5e-14
+// (R = 64 without the pairs of CTAs 0.97 ms; there a barrier of all warps per half tile took 1.50 ms,
+// levels moved every tile 1.44, the MMAs issued from a loop, 200 cycles each, 1.38.)
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -56,12 +62,12 @@ static double dx_start(int rc) { return rc == 8 ? 0.5 : rc == 16 ? 0.8 : 1.2; } 
 // N^2 R from which on this form is the faster one (us, here / one-directional): 900 unknowns
 // (R = 16: 1.3e7) 74 / 74, 1,764 (R = 8: 2.5e7) 81 / 79, (R = 16) 85 / 117, 3,968 (R = 5) 163 / 206
 static const double DX_WORK = 2.4e7;
-static const int DX_AIMG = DX_M * 128;                         // bytes of one digit image of A
+static const int DX_AIMG = DX_M * 64;                          // bytes of one digit image of half a tile of A
 static const int DX_GEO = 3 * DFL_S * 16;                      // bytes of a tile's nodes
 
 __host__ __device__ constexpr int dx_img(int rc) { return 2 * rc * 128; }                 // one digit image of B
 __host__ __device__ constexpr int dx_stage(int rc) { return DX_D * dx_img(rc) + 2048; }    // B images and nodes
-__host__ __device__ constexpr int dx_smem(int rc) { return DX_D * DX_AIMG + 2 * dx_stage(rc) + DFL_TAB * 16 + 1024; }
+__host__ __device__ constexpr int dx_smem(int rc) { return 2 * DX_D * DX_AIMG + 2 * dx_stage(rc) + DFL_TAB * 16 + 1024; }
 // tensor memory: six levels of 2 RC columns, then low and high words of the sums
 __host__ __device__ constexpr int dx_cols(int rc) { return 16 * rc; }
 static_assert(DX_GEO <= 2048 && dx_smem(32) <= 227 * 1024 && dx_cols(32) <= 512, "sizes");
@@ -72,13 +78,18 @@ __host__ __device__ constexpr uint32_t dx_idesc(int n)
     return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(DX_M >> 4) << 24);
 }
 
-// (descriptors: the low words given, the high words those of t5_desc)
+// A's half tiles: K-major, 64-byte rows and swizzle (chunk c of 16 bytes of row r)
+__device__ __forceinline__ uint32_t dx_chunk_off(int r, int c) { return (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4)); }
+// high words of the descriptors: A 512 bytes between 8-row groups, 64-byte swizzle; B as t5_desc
+static const uint32_t DX_ADESC = (512u >> 4) | (1u << 14) | (4u << 29), DX_BDESC = (1024u >> 4) | (1u << 14) | (2u << 29);
+
+// (descriptors: the low words given)
 __device__ __forceinline__ void dx_mma(uint32_t d, uint32_t ad, uint32_t bd, uint32_t idesc, uint32_t acc)
 {
     asm volatile(
-        "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %5};\n"
+        "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %6};\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}\n" ::"r"(d),
-        "r"(ad), "r"(bd), "r"(idesc), "r"(acc), "r"((uint32_t)(t5_desc(0) >> 32))
+        "r"(ad), "r"(bd), "r"(idesc), "r"(acc), "r"(DX_ADESC), "r"(DX_BDESC)
         : "memory");
 }
 
@@ -87,6 +98,36 @@ __device__ __forceinline__ void dx_copy(uint32_t dst, const void *src, uint32_t 
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(mbar)
                  : "memory");
+}
+
+// the same shared-memory address in the CTA of rank r of the cluster
+__device__ __forceinline__ uint32_t dx_peer(uint32_t addr, uint32_t r)
+{
+    uint32_t d;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(r));
+    return d;
+}
+__device__ __forceinline__ void dx_cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// t5_wait; CL = 2: for arrivals from both CTAs of the cluster
+template <int CL>
+__device__ __forceinline__ bool dx_wait(uint32_t mbar, uint32_t parity)
+{
+    if (CL == 1) return t5_wait(mbar, parity);
+    for (int it = 0; it < (1 << 22); ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(mbar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
 }
 
 // four columns of this warp's 32 lanes, without the wait
@@ -136,7 +177,7 @@ __device__ __forceinline__ uint32_t dx_pack(float a, float b)
     return r;
 }
 
-template <int RC>
+template <int RC, int CL>
 __global__ void __launch_bounds__(DX_THREADS, 1)
 nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict__ own_tiles,
                  const int2 *__restrict__ tiles, const float4 *__restrict__ ball, int ntiles, int R,
@@ -146,7 +187,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
 {
     extern __shared__ __align__(1024) unsigned char dx_raw[];
     __shared__ uint32_t s_taddr;
-    __shared__ __align__(8) unsigned long long s_bar[6];       // full[2]; per half tile: mma[2], formed[2]
+    __shared__ __align__(8) unsigned long long s_bar[8];       // full[2]; per half tile: mma[2], formed[2]; moved, own
     __shared__ int s_rmin;
     __shared__ volatile int s_fail;
     const TargetBlock tb = blocks[blockIdx.x >> 2];
@@ -155,8 +196,8 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     constexpr int IMG = dx_img(RC), STAGE = dx_stage(RC), N = 2 * RC, CW = N / 4;   // CW: columns of a warp
     const uint32_t base = ((uint32_t)__cvta_generic_to_shared(dx_raw) + 1023u) & ~1023u;
     unsigned char *const gbase = dx_raw + (base - (uint32_t)__cvta_generic_to_shared(dx_raw));
-    const uint32_t a0 = base, b0 = base + DX_D * DX_AIMG;
-    unsigned char *const gb0 = gbase + DX_D * DX_AIMG;
+    const uint32_t a0 = base, b0 = base + 2 * DX_D * DX_AIMG;
+    unsigned char *const gb0 = gbase + 2 * DX_D * DX_AIMG;
     float4 *const s_tab = reinterpret_cast<float4 *>(gb0 + 2 * STAGE);
     const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(&s_bar[0]);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -170,8 +211,9 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int q = 0; q < 6; ++q)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 8 * q), "r"(q < 4 ? 1 : DX_FORM / 32)
+        for (int q = 0; q < 8; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 8 * q),
+                         "r"(q < 2 || q == 7 ? 1 : q < 4 ? CL : CL == 2 && q - 4 == (int)(1 - blockIdx.y % 2) ? 1 : DX_FORM / 32)
                          : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -181,6 +223,8 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (CL == 2) dx_cluster_sync();                            // the barriers of both CTAs stand
+    const uint32_t rank = blockIdx.y % CL, peer = rank ^ 1;
     const uint32_t tmem = s_taddr;
     // this warp's lanes and columns of level 0, and of the sums' words
     const uint32_t drow = tmem + ((uint32_t)(32 * quarter) << 16) + CW * q4;
@@ -299,22 +343,38 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         int halves = 0;
         for (int i = 0; i < n && ok; ++i) {
             if (i > 0) {
-                ok = t5_wait(bar0 + 24, (uint32_t)((i - 1) & 1));
+                ok = (CL == 1 || dx_wait<CL>(bar0 + 16, (uint32_t)((i - 1) & 1))) && dx_wait<CL>(bar0 + 24, (uint32_t)((i - 1) & 1));
                 if (ok && i + 1 < n) {
                     if (lane == 0) issue(i + 1);
                     issued = i + 2;
                 }
             }
+            if (CL == 2 && ok && lane == 0)                    // the other half comes from the other CTA
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar0 + 32 + 8 * peer),
+                             "r"(DX_D * DX_AIMG)
+                             : "memory");
+            // (CL = 1: the warps that form the halves have waited for the images)
+            if (CL == 2) ok = ok && t5_wait(bar0 + 8 * (i & 1), (uint32_t)((i >> 1) & 1));
 #pragma unroll 1
-            for (int h = 0; h < 2 && ok; ++h) {
-                ok = t5_wait(bar0 + 32 + 8 * h, (uint32_t)(i & 1)) && !s_fail;
+            for (int hh = 0; hh < 2 && ok; ++hh) {
+                const int h = CL == 2 ? (int)rank ^ hh : hh;   // CL = 2: the own half first
+                ok = dx_wait<CL>(bar0 + 32 + 8 * h, (uint32_t)(i & 1)) && !s_fail;
+                if (CL == 2 && ok && hh == 0 && lane == 0)
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                            dx_peer(a0 + rank * (DX_D * DX_AIMG), peer)),
+                        "r"(a0 + rank * (DX_D * DX_AIMG)), "r"(DX_D * DX_AIMG), "r"(dx_peer(bar0 + 32 + 8 * rank, peer))
+                        : "memory");
+                // (CL = 1: the warps that formed the half have moved the levels)
+                if (CL == 2 && ok && hh == 0 && i > 0 && !(i & 1)) ok = t5_wait(bar0 + 48, (uint32_t)(((i >> 1) - 1) & 1));
                 if (!ok) break;
+                __syncwarp();
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 if (t5_elect()) {
                     // (unrolled: in a loop the address arithmetic of one MMA took this warp 200 cycles)
-                    const uint32_t ad = (uint32_t)t5_desc(a0 + 64 * h);
+                    const uint32_t ad = ((a0 + h * (DX_D * DX_AIMG)) & 0x3FFFF) >> 4 | (1u << 16);
                     const uint32_t bd = (uint32_t)t5_desc(b0 + (uint32_t)((i & 1) * STAGE) + 64 * h);
-                    const uint32_t more = (i & 1) | h;
+                    const uint32_t more = (i & 1) | hh;
 #pragma unroll
                     for (int l = 0; l < DX_D; ++l)
 #pragma unroll
@@ -323,9 +383,15 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                             for (int ks = 0; ks < 2; ++ks)
                                 dx_mma(tmem + l * N, ad + ((a * DX_AIMG + 32 * ks) >> 4), bd + (((l - a) * IMG + 32 * ks) >> 4),
                                        dx_idesc(N), a | ks ? 1u : more);
-                    asm volatile(
-                        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 16 + 8 * h)
-                        : "memory");
+                    if (CL == 1)
+                        asm volatile(
+                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 16 + 8 * h)
+                            : "memory");
+                    else
+                        asm volatile(
+                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
+                            "[%0], %1;" ::"r"(bar0 + 16 + 8 * h), "h"((unsigned short)3)
+                            : "memory");
                 }
                 __syncwarp();
                 ++halves;
@@ -333,8 +399,13 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         }
         if (!ok) s_fail = 1;
         // what is in flight (after a timeout: once more)
-        if (halves > 0) ok &= t5_wait(bar0 + 16, (uint32_t)(((halves - 1) >> 1) & 1));
-        if (halves > 1) ok &= t5_wait(bar0 + 24, (uint32_t)(((halves >> 1) - 1) & 1));
+        if (halves > 0) {
+            if (t5_elect())
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 56)
+                             : "memory");
+            __syncwarp();
+            ok &= t5_wait(bar0 + 56, 0u);
+        }
         for (int i = max(0, issued - 2); i < issued; ++i) ok &= t5_wait(bar0 + 8 * (i & 1), (uint32_t)((i >> 1) & 1));
     } else {
         int next = n > 0 ? tiles[tile_of(0)].y : 0;
@@ -344,7 +415,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
             ok = t5_wait(bar0 + 8 * (i & 1), (uint32_t)((i >> 1) & 1));
             const float4 *const S = reinterpret_cast<const float4 *>(gb0 + (i & 1) * STAGE + DX_D * IMG);
 #pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
+            for (int h = CL == 2 ? (int)rank : 0; h < (CL == 2 ? (int)rank + 1 : 2); ++h) {
                 uint32_t dig[DX_D][4];
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
@@ -364,16 +435,23 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                         for (int l = 0; l < DX_D; ++l) dig[l][v] = 0u;
                     }
                 }
-                if (i > 0) ok &= t5_wait(bar0 + 16 + 8 * h, (uint32_t)((i - 1) & 1));   // A's half is free
-                if (h == 0 && i > 0 && !(i & 1)) {             // the last two tiles are through: their levels
-                    ok &= t5_wait(bar0 + 24, (uint32_t)((i - 1) & 1));
+                if (i > 0) ok &= dx_wait<CL>(bar0 + 16 + 8 * h, (uint32_t)((i - 1) & 1));   // A's half is free
+                // (CL = 2: both halves every tile, so that no phase of a barrier goes by unseen)
+                if (i > 0 && (CL == 2 || (h == 0 && !(i & 1))))
+                    ok &= dx_wait<CL>(bar0 + 16 + 8 * (h ^ 1), (uint32_t)((i - 1) & 1));
+                if ((CL == 2 || h == 0) && i > 0 && !(i & 1)) {   // the last two tiles are through: their levels
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     __syncwarp();
                     drain();
+                    if (CL == 2) {
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar0 + 48) : "memory");
+                    }
                 }
+                const uint32_t at = a0 + h * (DX_D * DX_AIMG) + dx_chunk_off(row, q4);
 #pragma unroll
-                for (int l = 0; l < DX_D; ++l)
-                    t5_st4(a0 + l * DX_AIMG + t5_chunk_off(row, 4 * h + q4), dig[l][0], dig[l][1], dig[l][2], dig[l][3]);
+                for (int l = 0; l < DX_D; ++l) t5_st4(at + l * DX_AIMG, dig[l][0], dig[l][1], dig[l][2], dig[l][3]);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 if (__any_sync(0xffffffffu, !ok)) s_fail = 1;  // ends the MMAs, and below the loop
@@ -387,8 +465,8 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
             }
         }
         if (n > 0 && ok) {                                     // the last tile
-            ok &= t5_wait(bar0 + 16, (uint32_t)((n - 1) & 1));
-            ok &= t5_wait(bar0 + 24, (uint32_t)((n - 1) & 1));
+            ok &= dx_wait<CL>(bar0 + 16, (uint32_t)((n - 1) & 1));
+            ok &= dx_wait<CL>(bar0 + 24, (uint32_t)((n - 1) & 1));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             __syncwarp();
             drain();
@@ -420,6 +498,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(dx_cols(RC)) : "memory");
+    if (CL == 2) dx_cluster_sync();                            // no stores or arrivals into a CTA that has ended
     if (failed && tid == 0) atomicExch(err, 1);
 }
 
@@ -481,7 +560,8 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
 {
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->opt.device);
-    const int rc = R <= 8 ? 8 : R <= 16 ? 16 : 32, nchunk = (R + rc - 1) / rc, nt = c->t5h_ntiles, most = c->t5h_most;
+    const int rc = R <= 8 ? 8 : R <= 16 ? 16 : 32, nt = c->t5h_ntiles, most = c->t5h_most;
+    const int cl = R > 32 ? 2 : 1, nchunk = ((R + rc - 1) / rc + cl - 1) / cl * cl;
     hzb_status st = ensure_dfl(c);
     if (st) return st;
     // Source chunks: the shortest time, in tiles.  Bodies of one size: whole waves of equal CTAs;
@@ -522,14 +602,30 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     auto launch = [&](auto kern) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dx_smem(rc));
         if (e != cudaSuccess) return;
-        kern<<<grid, DX_THREADS, dx_smem(rc), c->stream>>>(
-            c->tblocks.ptr, c->t5h_tiles.ptr + nt, c->t5h_tiles.ptr, ball, nt, R, c->dla.ptr, c->dlb.ptr, c->dlc.ptr,
-            c->t5h_img.ptr, c->dlkey.ptr, c->dfltab.ptr, dfl_constants(c), out, n, c->kerr.ptr);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = dim3(DX_THREADS);
+        cfg.dynamicSmemBytes = dx_smem(rc);
+        cfg.stream = c->stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 1;
+        at[0].val.clusterDim.y = cl;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = cl > 1 ? 1 : 0;
+        e = cudaLaunchKernelEx(&cfg, kern, (const TargetBlock *)c->tblocks.ptr, (const int2 *)(c->t5h_tiles.ptr + nt),
+                               (const int2 *)c->t5h_tiles.ptr, ball, nt, R, (const float4 *)c->dla.ptr,
+                               (const float4 *)c->dlb.ptr, (const float4 *)c->dlc.ptr,
+                               (const unsigned char *)c->t5h_img.ptr, (const int *)c->dlkey.ptr,
+                               (const float4 *)c->dfltab.ptr, dfl_constants(c), out, n, c->kerr.ptr);
+        if (e != cudaSuccess) return;
         e = cudaGetLastError();
     };
-    if (rc == 8) launch(nbody_dfx_kernel<8>);
-    else if (rc == 16) launch(nbody_dfx_kernel<16>);
-    else launch(nbody_dfx_kernel<32>);
+    if (rc == 8) launch(nbody_dfx_kernel<8, 1>);
+    else if (rc == 16) launch(nbody_dfx_kernel<16, 1>);
+    else if (cl == 1) launch(nbody_dfx_kernel<32, 1>);
+    else launch(nbody_dfx_kernel<32, 2>);
     c->launches += 2;
     if (check_cuda(c, e, "nbody_dfx_kernel")) return HZB_ECUDA;
     if (nsplit > 1) {
