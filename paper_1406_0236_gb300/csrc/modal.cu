@@ -30,8 +30,8 @@ template <typename T> struct alignas(16) Quad { T x, y, z, w; };
 // (N_F is odd, often prime).  A thread owns PB modes of RB right-hand sides: twiddles and index
 // updates are shared by the RB columns, folded values by the PB modes.  The twiddles come from
 // the shape's table (make_nodes); computing them in every block took the FP64 pipe longer than
-// the sums at small N_F.  258,560 unknowns, R = 16, FP32: forward 197 -> 96 us, inverse
-// 188 -> 85 us; 8,200 unknowns, R = 1: 6.4 and 7.0 -> 5.5 and 6.0 us.
+// the sums at small N_F.  258,560 unknowns, R = 16, FP32: forward 197 -> 79 us, inverse
+// 188 -> 72 us; 8,200 unknowns, R = 1: 6.4 and 7.0 -> 5.5 and 6.0 us.
 
 // One block per (body of the shape, ring).  y is N x R (FP64); yh is the shape's panel array
 // (M+1) x NG x ncols in precision T, which is also the arithmetic precision.
@@ -68,7 +68,7 @@ dft_forward_kernel(int NG, int NF, int R, int ncols, const long long *__restrict
     __syncthreads();
     const int nrb = (R + RB - 1) / RB, items = ((M + PB) / PB) * nrb;
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
-        const int p0 = (it / nrb) * PB, r0 = (it % nrb) * RB;
+        const int p0 = (it / nrb) * PB, r0 = it % nrb;
         Quad<T> acc[PB][RB];                         // sum s cos, sum d sin
         int idx[PB];
 #pragma unroll
@@ -81,7 +81,7 @@ dft_forward_kernel(int NG, int NF, int R, int ncols, const long long *__restrict
         for (int l = 0; l < M; ++l) {
             Quad<T> v[RB];
 #pragma unroll
-            for (int u = 0; u < RB; ++u) v[u] = sd[l * R + min(r0 + u, R - 1)];
+            for (int u = 0; u < RB; ++u) v[u] = sd[l * R + min(r0 + nrb * u, R - 1)];
 #pragma unroll
             for (int q = 0; q < PB; ++q) {
                 idx[q] += p0 + q;
@@ -103,15 +103,16 @@ dft_forward_kernel(int NG, int NF, int R, int ncols, const long long *__restrict
             ct *o = yh + ((size_t)p * NG + i) * ncols + 2 * bs * R;
 #pragma unroll
             for (int u = 0; u < RB; ++u) {
-                if (r0 + u >= R) break;
+                const int r = r0 + nrb * u;
+                if (r >= R) break;
                 const Quad<T> A = acc[q][u];
-                const ct z = y0[r0 + u];
+                const ct z = y0[r];
                 const T cx = z.x + A.x, cy = z.y + A.y;
                 ct plus, minus;
                 plus.x = cx + A.w; plus.y = cy - A.z;
                 minus.x = p ? cx - A.w : (T)0; minus.y = p ? cy + A.z : (T)0;     // the -0 columns are zero
-                o[r0 + u] = plus;
-                o[R + r0 + u] = minus;
+                o[r] = plus;
+                o[R + r] = minus;
             }
         }
     }
@@ -152,7 +153,7 @@ dft_inverse_kernel(int NG, int NF, int R, int ncols, const long long *__restrict
     const double sc = beta / NF;
     const int nrb = (R + RB - 1) / RB, items = ((M + PB) / PB) * nrb;
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
-        const int l0 = (it / nrb) * PB, r0 = (it % nrb) * RB;
+        const int l0 = (it / nrb) * PB, r0 = it % nrb;
         Quad<T> acc[PB][RB];
         int idx[PB];
 #pragma unroll
@@ -165,7 +166,7 @@ dft_inverse_kernel(int NG, int NF, int R, int ncols, const long long *__restrict
         for (int p = 0; p < M; ++p) {
             Quad<T> v[RB];
 #pragma unroll
-            for (int u = 0; u < RB; ++u) v[u] = ab[p * R + min(r0 + u, R - 1)];
+            for (int u = 0; u < RB; ++u) v[u] = ab[p * R + min(r0 + nrb * u, R - 1)];
 #pragma unroll
             for (int q = 0; q < PB; ++q) {
                 idx[q] += l0 + q;
@@ -196,18 +197,19 @@ dft_inverse_kernel(int NG, int NF, int R, int ncols, const long long *__restrict
             if (l > M) break;
 #pragma unroll
             for (int u = 0; u < RB; ++u) {
-                if (r0 + u >= R) break;
+                const int r = r0 + nrb * u;
+                if (r >= R) break;
                 const Quad<T> A = acc[q][u];
-                const ct z = t0[r0 + u];
+                const ct z = t0[r];
                 const T cx = z.x + A.x, cy = z.y + A.y;
-                put(l, r0 + u, cx - A.w, cy + A.z);
-                if (l) put(NF - l, r0 + u, cx + A.w, cy - A.z);
+                put(l, r, cx - A.w, cy + A.z);
+                if (l) put(NF - l, r, cx + A.w, cy - A.z);
             }
         }
     }
 }
 
-// One thread per (two modes, four right-hand sides), fewer where the batch is smaller.  The
+// One thread per (two or four modes, four right-hand sides), fewer where the batch is smaller.  The
 // dynamic shared memory limit is raised once beyond the default 48 KB, to the largest size any
 // call uses, and never lowered, so that calls with different sizes (and both D^{-1} entry
 // points) cannot invalidate each other's launches.
@@ -223,6 +225,16 @@ static void dft_limit(K kern, size_t bytes)
     if (bytes > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
+// Four modes to a thread, where that leaves blocks of 48 threads and 16,384 of them in all: the
+// reads from shared memory bound these kernels (258,560 unknowns, FP32: R = 16, 52 threads, 96 -> 79
+// and 85 -> 72 us; R = 8, 26 threads, 3 % slower; 8,200 unknowns: R = 64, 96 threads, whole D^{-1}
+// 66 -> 58, R = 16, 24 threads, 29 -> 38).
+static bool dft_wide(int M, int R, long long blocks)
+{
+    const int threads = (M + 4) / 4 * ((R + 3) / 4);
+    return R >= 4 && threads >= 48 && blocks * threads >= 16384;
+}
+
 static int dft_threads(int items) { return std::min(128, std::max(32, (items + 31) / 32 * 32)); }
 
 template <typename T>
@@ -236,7 +248,8 @@ static void dft_forward(cudaStream_t st, const ShapeDev &sd, int ms, int R, cons
         kern<<<dim3(NG, ms), dft_threads((M + pb) / pb * ((R + rb - 1) / rb)), smem, st>>>(NG, NF, R, ncols, off, y,
                                                                                      sd.tw.ptr, yh);
     };
-    if (R >= 4) launch(dft_forward_kernel<T, 2, 4>, 2, 4);
+    if (dft_wide(M, R, NG * ms)) launch(dft_forward_kernel<T, 4, 4>, 4, 4);
+    else if (R >= 4) launch(dft_forward_kernel<T, 2, 4>, 2, 4);
     else if (R >= 2) launch(dft_forward_kernel<T, 1, 2>, 1, 2);
     else launch(dft_forward_kernel<T, 1, 1>, 1, 1);
 }
@@ -252,7 +265,8 @@ static void dft_inverse(cudaStream_t st, const ShapeDev &sd, int ms, int R, cons
         kern<<<dim3(NG, ms), dft_threads((M + pb) / pb * ((R + rb - 1) / rb)), smem, st>>>(
             NG, NF, R, ncols, off, th, sigma, sd.tw.ptr, alpha, beta, out);
     };
-    if (R >= 4) launch(dft_inverse_kernel<T, 2, 4>, 2, 4);
+    if (dft_wide(M, R, NG * ms)) launch(dft_inverse_kernel<T, 4, 4>, 4, 4);
+    else if (R >= 4) launch(dft_inverse_kernel<T, 2, 4>, 2, 4);
     else if (R >= 2) launch(dft_inverse_kernel<T, 1, 2>, 1, 2);
     else launch(dft_inverse_kernel<T, 1, 1>, 1, 1);
 }
