@@ -5,7 +5,7 @@
 //     w_j K(x_i, x_j) = w_j / (4 pi) e^{ikr} [ n_j.d / r^3 - i (k n_j.d / r^2 + eta / r) ]
 //     w_i K(x_j, x_i) = w_i / (4 pi) e^{ikr} [-n_i.d / r^3 - i (-k n_i.d / r^2 + eta / r) ]
 // share d, r, 1/r and e^{ikr}, which are two thirds of the FP64 work of a pair; the
-// two directions differ only in the normal projection.  About 27.5 FP64 operations
+// two directions differ only in the normal projection.  About 25 FP64 operations
 // per ordered pair instead of 41 for the one-directional kernel (nbody64_kernel).
 //
 // Work: one CTA per unordered pair of TargetBlocks (I, J), I < J, on different
