@@ -55,7 +55,7 @@ ORACLE_ITERS = 16
 DRAM_BYTES_NCU = {"nbody64_sym_kernel": 25.96e6, "nbody32_sym_kernel": 15.73e6, "nbody_dfl_sym_kernel": 30.14e6}
 # FP32-pipe (FMA) thread operations per unordered node pair of the lean double-float kernel,
 # counted by ncu (thread instructions per unordered pair on the four-body case)
-DFL_OPS_PER_UNORDERED_PAIR = 440
+DFL_OPS_PER_UNORDERED_PAIR = 363
 
 
 def dist_env():

@@ -324,7 +324,7 @@ hzb_status ensure_sctab(hzb_ctx *c);                                          //
 hzb_status interbody64_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y);  // nbody_sym.cu
 hzb_status interbody32_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tp);  // nbody_sym.cu
 hzb_status ensure_block_pairs(hzb_ctx *c);                                    // nbody_sym.cu
-SymSplit sym_split(hzb_ctx *c, int rhs_chunks);      // the split for the context's block pairs (nbody_sym.cu)
+SymSplit sym_split(hzb_ctx *c, int rhs_chunks, int steps_below);      // the split for the context's block pairs (nbody_sym.cu)
 void split_reduce_f2(hzb_ctx *c, size_t n, int nsplit, const float2 *part, double2 *y);
 hzb_status interbody64_cfg(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tpt, int nsplit);
 hzb_status interbody32_cfg(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int tpt, int nsplit, bool x2);

@@ -773,7 +773,7 @@ hzb_status interbody_dfl_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y
     const DflConst K = dfl_constants(c);
     const int slot = prof_begin(c, 2);
     const int rc = (R == 1) ? 1 : 2;
-    const SymSplit sp = sym_split(c, (R + rc - 1) / rc);
+    const SymSplit sp = sym_split(c, (R + rc - 1) / rc, 1);
     dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, sp.nz);
     auto launch = [&](auto kern) {
         kern<<<g, DFL_T, 0, c->stream>>>(c->blockpairs.ptr, c->tblocks.ptr, R, c->dla.ptr, c->dlb.ptr, c->dlc.ptr,

@@ -378,20 +378,23 @@ nbody32_sym_kernel(const int2 *__restrict__ pairs, const TargetBlock *__restrict
 // A block pair per CTA leaves most of the chip idle on small geometries (two spheres of
 // 4,100 nodes: 81 CTAs; 216 nodes: one), and a CTA of 512 x 512 pairs is a long last wave on
 // middling ones.  So the source side is cut until there are about 16 CTAs per SM, down to
-// one tile of 32 sources, and below 4 per SM the rotation steps of a tile are shared out
-// too.  Finer pieces cost more than they fill: every CTA adds its 512 target sums to y with
+// one tile of 32 sources, and below `steps_below` per SM the rotation steps of a tile are shared
+// out too.  Finer pieces cost more than they fill: every CTA adds its 512 target sums to y with
 // FP64 atomics.  Before -> after, one right-hand side (FP64 / double-float / FP32 sums):
-// 432 unknowns 787 / 139 / 61 -> 18 us each (the call itself); 8,200 unknowns 3,814 / 533 /
-// 122 -> 1,672 / 263 / 39 us (at twice as many pieces 1,693 / 295 / 39); 29,280 unknowns
+// 432 unknowns 787 / 139 / 61 -> 16 / 19 / 16 us each (the call itself); 8,200 unknowns 3,814 /
+// 533 / 122 -> 1,672 / 263 / 39 us (at twice as many pieces 1,693 / 295 / 39); 29,280 unknowns
 // 32.31 / 4.47 / 0.523 -> 31.41 / 4.37 / 0.455 ms; from 64,640 unknowns up nothing is cut.
-SymSplit sym_split(hzb_ctx *c, int rhs_chunks)
+// steps_below = 4, 2, 1, us: 1,350 unknowns on three bodies, FP64 85, 92, 112, double-float 66, 42,
+// 38, FP32 30, 20, 17; 3,968 on two, R = 4: FP64 591, 648, 636, FP32 52, 36, 29, R = 1 double-float
+// 99, 93, 84; 2,640 on eight: FP64 385, 451, 451, double-float 88, 94, 94, FP32 20, 21, 22.
+SymSplit sym_split(hzb_ctx *c, int rhs_chunks, int steps_below)
 {
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->opt.device);
     const long long have = c->n_blockpairs * rhs_chunks;
     SymSplit sp = {SYM_T, 1, 1};
     while (have * sp.nz < 16LL * sms && sp.jchunk > SYM_S) { sp.jchunk /= 2; sp.nz *= 2; }
-    while (have * sp.nz < 4LL * sms && sp.nstep < 16) { sp.nstep *= 2; sp.nz *= 2; }
+    while (have * sp.nz < (long long)steps_below * sms && sp.nstep < 16) { sp.nstep *= 2; sp.nz *= 2; }
     return sp;
 }
 
@@ -439,7 +442,7 @@ hzb_status interbody64_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     c->launches += 1;
     const int slot = prof_begin(c, 0);
     const int rc = (R == 1) ? 1 : (R == 2 ? 2 : 4);
-    const SymSplit sp = sym_split(c, (R + rc - 1) / rc);
+    const SymSplit sp = sym_split(c, (R + rc - 1) / rc, 4);
     dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, sp.nz);
     const bool gen = !sym_scaled(c);
     const SymConst K = {c->k * (SC_N / (2.0 * M_PI)), gen ? 0.0 : 1.0 / c->k, c->k, c->eta,
@@ -509,7 +512,7 @@ hzb_status interbody32_sym(hzb_ctx *c, int R, const double2 *sigma, double2 *y, 
     if (!sw) return HZB_ENOMEM;
     c->launches += 1;
     const int rc = (R == 1) ? 1 : (R == 2 ? 2 : 4);
-    const SymSplit sp = sym_split(c, (R + rc - 1) / rc);
+    const SymSplit sp = sym_split(c, (R + rc - 1) / rc, 1);
     dim3 g((unsigned)c->n_blockpairs, (R + rc - 1) / rc, sp.nz);
     if (tp == 2) {
         if (rc == 1) launch_sym32<1, 2>(c, g, R, sw, y, sp);
