@@ -14,7 +14,7 @@ static const int DFL_S = 32;           // sources per tile
 static const int DFL_TAB = 1024;       // table angles 2 pi m / 1024
 
 struct DflConst {
-    dd kappa, eta;                     // 2 pi (0 when k = 0), eta'
+    dd kappa;                          // 2 pi (0 when k = 0)
     float eta_m, mb;                   // eta' rounded onto the grid of mb, plus mb; mb = 1.5 * 2^E for kr X + eta'
     float eta_r;                       // eta' minus its grid value (its low part included)
     float kbound;                      // 2 pi + |eta'|, rounded up

@@ -625,7 +625,6 @@ DflConst dfl_constants(const hzb_ctx *c)
     DflConst K;
     const double s = c->k > 0.0 ? c->k / (2.0 * M_PI) : 1.0, eta = c->eta / s;
     K.kappa = dd_of(c->k > 0.0 ? 2.0 * M_PI : 0.0);
-    K.eta = dd_of(eta);
     K.kbound = (float)((2.0 * M_PI + std::fabs(eta)) * 1.0001);
     int e;
     std::frexp(K.kbound, &e);                             // kbound < 2^e

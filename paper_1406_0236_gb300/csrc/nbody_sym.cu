@@ -15,9 +15,9 @@
 // own sum and the j <- i term to a rotating sum that then moves to lane l - 1, so each
 // source's partial sum visits every lane once and no two lanes touch the same source
 // at a step.  The warps' partial sums of a tile are added in a fixed order in shared
-// memory.  On small geometries several CTAs share a block pair (sym_split).  Both directions reach y through FP64 atomic adds (y is zeroed first), so
-// the order of the additions into one y entry varies between runs: the result is
-// reproducible to rounding, not bit for bit.
+// memory.  On small geometries several CTAs share a block pair (sym_split).  Both directions
+// reach y through FP64 atomic adds (y is zeroed first), so the order of the additions into one y
+// entry varies between runs: the result is reproducible to rounding, not bit for bit.
 #include <algorithm>
 #include <cmath>
 #include <vector>
