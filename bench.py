@@ -50,9 +50,8 @@ FLOPS_PER_PAIR = 36
 # gives a density error <= 1e-7 (3.9e-8, measured on GB300); the reference arm's oracle
 # solve is its apply time times this count (a full oracle GMRES would take hours)
 ORACLE_ITERS = 16
-# DRAM bytes (read + write) per launch on this workload from one ncu capture of each kernel
-# (profiles/); None for a kernel without a capture of its current version.
-DRAM_BYTES_NCU = {"nbody64_sym_kernel": 25.96e6, "nbody32_sym_kernel": 15.73e6, "nbody_dfl_sym_kernel": 30.14e6}
+# DRAM bytes (read + write) per launch on this workload from one ncu capture of each kernel; None for a kernel without a capture of its current version.
+DRAM_BYTES_NCU = {"nbody32_sym_kernel": 15.94e6, "nbody_dfl_sym_kernel": 21.87e6}
 # FP32-pipe (FMA) thread operations per unordered node pair of the lean double-float kernel,
 # counted by ncu (thread instructions per unordered pair on the four-body case)
 DFL_OPS_PER_UNORDERED_PAIR = 363
