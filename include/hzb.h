@@ -72,8 +72,10 @@ typedef enum {
  *   nan      the first solve's preconditioned right-hand side gets a NaN (HZB_ENAN);
  *   timeout  the first tcgen05 inter-body launch (FP32 engine 5) finds its error flag
  *            set before it starts and takes its timeout exit before issuing any MMA
- *            (HZB_ETIMEOUT).
- * The last three fire once per context.  Nothing is injected on the GPU itself. */
+ *            (HZB_ETIMEOUT);
+ *   timeout_modal  the first tcgen05 mode GEMM of D^{-1} (modal engine 2) does the same, with
+ *            copies and MMAs in flight (HZB_ETIMEOUT).
+ * All but the first fire once per context.  Nothing is injected on the GPU itself. */
 
 typedef enum {
     HZB_PREC_FP64 = 0,        /* every kernel in FP64 */

@@ -46,6 +46,7 @@ int parse_fault_spec(const char *spec)
         else if (t == "geom") f |= FAULT_GEOM;
         else if (t == "nan") f |= FAULT_NAN;
         else if (t == "timeout") f |= FAULT_TIMEOUT;
+        else if (t == "timeout_modal") f |= FAULT_TIMEOUT_MODAL;
         a = b + 1;
     }
     return f;
@@ -349,6 +350,14 @@ static hzb_status finish_out(hzb_ctx *c, const double2 *dev, double *dst, size_t
     return HZB_OK;
 }
 
+// finish_out of an operator: host data have waited for the stream, so a bounded wait that ran out
+// is reported here
+static hzb_status finish_apply(hzb_ctx *c, const double2 *dev, double *dst, size_t n, int on_device, const char *what)
+{
+    hzb_status st = finish_out(c, dev, dst, n, on_device);
+    return st || on_device ? st : tc_flag_report(c, what);
+}
+
 static hzb_status check_apply_args(hzb_ctx *c, int R, const void *a, const void *b, int precision, bool need_build)
 {
     if (c->state < 2) return fail(c, HZB_ESTATE, "no bodies");
@@ -376,7 +385,7 @@ hzb_status hzb_interbody(hzb_ctx *c, int R, const double *sigma, double *y, int 
     st = (precision == HZB_PREC_FP64) ? interbody64(c, R, s, out)
          : (precision == HZB_PREC_DOUBLE_FLOAT) ? interbody_df(c, R, s, out) : interbody32(c, R, s, out);
     if (st) return st;
-    return finish_out(c, out, y, n, on_device);
+    return finish_apply(c, out, y, n, on_device, "the inter-body sum");
 }
 
 hzb_status hzb_interbody_bodies(hzb_ctx *c, int R, const double *sigma, int body_begin, int body_end, double *y,
@@ -439,7 +448,7 @@ hzb_status hzb_local_inverse(hzb_ctx *c, int R, const double *y, const double *s
          : (precision == HZB_PREC_DOUBLE_FLOAT) ? local_inverse_dfl(c, R, dy, ds, alpha, beta, out)
                                                 : local_inverse64(c, R, dy, ds, alpha, beta, out);
     if (st) return st;
-    return finish_out(c, out, tau, n, on_device);
+    return finish_apply(c, out, tau, n, on_device, "the block-diagonal inverse");
 }
 
 hzb_status hzb_apply(hzb_ctx *c, int R, const double *sigma, double *z, int on_device, int precision)
@@ -456,7 +465,7 @@ hzb_status hzb_apply(hzb_ctx *c, int R, const double *sigma, double *z, int on_d
         out = c->io_out.ptr;
     }
     if ((st = apply_op(c, R, s, out, precision))) return st;
-    return finish_out(c, out, z, n, on_device);
+    return finish_apply(c, out, z, n, on_device, "the operator");
 }
 
 hzb_status hzb_solve_plane_waves(hzb_ctx *c, int R, const double *dirs, hzb_stats *stats)

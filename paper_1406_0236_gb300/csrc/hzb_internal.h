@@ -57,8 +57,10 @@ enum {
     FAULT_ALLOC = 1,     // "alloc": every device allocation of the context fails (HZB_ENOMEM)
     FAULT_GEOM = 2,      // "geom": the first node generation writes a NaN weight (HZB_EINVAL)
     FAULT_NAN = 4,       // "nan": the first solve's preconditioned right-hand side gets a NaN (HZB_ENAN)
-    FAULT_TIMEOUT = 8    // "timeout": the first tcgen05 inter-body launch takes its bounded-wait
+    FAULT_TIMEOUT = 8,   // "timeout": the first tcgen05 inter-body launch takes its bounded-wait
                          // exit before any MMA is issued (HZB_ETIMEOUT)
+    FAULT_TIMEOUT_MODAL = 16   // "timeout_modal": the first tcgen05 mode GEMM takes its exit, with
+                               // copies and MMAs in flight (HZB_ETIMEOUT)
 };
 int parse_fault_spec(const char *spec);
 // set by every ABI entry from its context: DevBuf::ensure fails while it is true
@@ -264,6 +266,7 @@ struct hzb_ctx {
     // host fault injection (FAULT_* bits from HZB_FAULT) and the one-shot faults already fired
     int fault = 0;
     int fault_spent = 0;
+    bool fault_flag = false;                   // the flag of the next launch is an injected one
     hzb::DevBuf<int> nodecheck;                // node validation: [bad count, first bad node]
 };
 
@@ -311,7 +314,9 @@ bool dfx_usable(hzb_ctx *c, int R, hzb_status *st);
 hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
 hzb_status interbody_t5h(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
 // nbody_tc5.cu: the device flag of the tensor-core kernels' bounded waits, around a launch
-hzb_status tc_flag_begin(hzb_ctx *c, bool inject);
+hzb_status tc_flag_begin(hzb_ctx *c, int fault);
+hzb_status tc_flag_launched(hzb_ctx *c);
+hzb_status tc_flag_report(hzb_ctx *c, const char *kernel);
 hzb_status tc_flag_end(hzb_ctx *c, const char *kernel);
 hzb_status sigma_keys(hzb_ctx *c, int R, const double2 *sigma, double c0, int weighted, int *key);   // nbody_dfl.cu
 bool sym_scaled(const hzb_ctx *c);              // nbody_sym.cu: k and eta leave the scaled pair kernels in range

@@ -16,8 +16,11 @@
 //     accumulators; warps 0-7 drain an accumulator (tcgen05.ld, 32 lanes x 32 columns
 //     per warp) into FP32 registers every two chunks, so no chain of tensor-core
 //     accumulations is longer than 24 MMAs.  Stages, accumulators and drains hand over
-//     through mbarriers; every wait is bounded and a timeout writes NaN and sets the
-//     context's device error flag.
+//     through mbarriers; every wait is bounded, its answer is one for the whole warp
+//     (t5_all), and a timeout writes NaN and sets the context's device error flag once the
+//     copies and MMAs in flight are through.  An injected timeout (a negative flag, set by
+//     the host) has the draining warps raise the abort flag at once, so that warp 8 gives
+//     up with copies and MMAs in flight.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -124,8 +127,8 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
 {
     extern __shared__ __align__(1024) unsigned char mt_smem_raw[];
     __shared__ uint32_t s_taddr;
-    __shared__ __align__(8) unsigned long long s_bar[8];   // tma_full[2], mma_done[2], acc_full[2], acc_free[2]
-    __shared__ int s_abort;
+    __shared__ __align__(8) unsigned long long s_bar[9];   // tma_full[2], mma_done[2], acc_full[2], acc_free[2], own
+    __shared__ int s_abort, s_forced;
     const uint32_t raw = (uint32_t)__cvta_generic_to_shared(mt_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(&s_bar[0]);
@@ -147,7 +150,9 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(acc_full0 + 8 * q), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(acc_free0 + 8 * q), "r"(256) : "memory");
         }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 64), "r"(1) : "memory");
         s_abort = 0;
+        s_forced = *(volatile int *)err < 0 ? 1 : 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -172,21 +177,24 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
                 mt_tma3(sA + 2 * MT_A, &tmB, kc * MT_K, c0, 2 * p, fb);
                 mt_tma3(sA + 2 * MT_A + MT_B, &tmB, kc * MT_K, c0, 2 * p + 1, fb);
             };
-            bool ok = true;
-            if (nk > 0) issue_tma(0);
-            for (int kc = 0; kc < nk && ok; ++kc) {
+            auto wait = [&](uint32_t mbar, int phase) {
+                return t5_all(mt_wait(mbar, (uint32_t)(phase & 1), abort_flag));
+            };
+            int issued = 0, landed = 0, done = 0;      // chunks copied, seen complete, multiplied
+            if (nk > 0) { issue_tma(0); issued = 1; }
+            for (int kc = 0; kc < nk; ++kc) {
                 if (kc + 1 < nk) {
                     // stage of chunk kc + 1 was read by the MMAs of chunk kc - 1
-                    if (kc >= 1 && !mt_wait(mma_done0 + 8 * ((kc + 1) & 1), (uint32_t)(((kc - 1) >> 1) & 1),
-                                            abort_flag)) { ok = false; break; }
+                    if (kc >= 1 && !wait(mma_done0 + 8 * ((kc + 1) & 1), (kc - 1) >> 1)) break;
                     issue_tma(kc + 1);
+                    issued = kc + 2;
                 }
                 const int st = kc & 1;
-                if (!mt_wait(tma_full0 + 8 * st, (uint32_t)((kc >> 1) & 1), abort_flag)) { ok = false; break; }
+                if (!wait(tma_full0 + 8 * st, kc >> 1)) break;
+                landed = kc + 1;
                 const int g = kc / MT_FLUSH, b = g & 1;
                 const bool first = (kc % MT_FLUSH) == 0;
-                if (first && g >= 2 &&
-                    !mt_wait(acc_free0 + 8 * b, (uint32_t)(((g >> 1) - 1) & 1), abort_flag)) { ok = false; break; }
+                if (first && g >= 2 && !wait(acc_free0 + 8 * b, (g >> 1) - 1)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t sA = base + (uint32_t)st * MT_STAGE;
                 const uint32_t as[3] = {sA, sA, sA + MT_A};
@@ -207,6 +215,19 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
                                  : "memory");
                 }
                 __syncwarp();
+                done = kc + 1;
+            }
+            // what is in flight, within a limit: copies where a wait ran out, MMAs (the draining warps
+            // may have given up on them)
+            for (int kc = landed; kc < issued; ++kc) t5_wait(tma_full0 + 8 * (kc & 1), (uint32_t)((kc >> 1) & 1));
+            __syncwarp();
+            if (done > 0) {
+                if (t5_elect())
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                     bar0 + 64)
+                                 : "memory");
+                __syncwarp();
+                t5_wait(bar0 + 64, 0u);
             }
         }
     } else {
@@ -215,9 +236,10 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
 #pragma unroll
         for (int q = 0; q < 32; ++q) acc[q] = 0.f;
         const uint32_t tl = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(32 * (warp >> 2));
-        for (int g = 0; g < ng; ++g) {
+        if (s_forced) *abort_flag = 1;
+        for (int g = 0; g < ng && !s_forced; ++g) {
             const int b = g & 1;
-            if (!mt_wait(acc_full0 + 8 * b, (uint32_t)((g >> 1) & 1), abort_flag)) break;
+            if (!t5_all(mt_wait(acc_full0 + 8 * b, (uint32_t)((g >> 1) & 1), abort_flag))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             t5_ld16(tl + MT_N * b, acc);
             t5_ld16(tl + MT_N * b + 16, acc + 16);
@@ -242,7 +264,7 @@ modal_gemm_tma_kernel(int n, int nc, const __grid_constant__ CUtensorMap tmA, co
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * MT_N) : "memory");
-    if (tid == 0 && s_abort) atomicExch(err, 1);
+    if (tid == 0 && s_abort && !s_forced) atomicExch(err, 1);   // (a negative flag stays for all CTAs of the launch)
 }
 
 // ---------------------------------------------------------------- host
@@ -298,12 +320,8 @@ hzb_status modal_gemm_tma(hzb_ctx *c, ShapeDev &sd, int ncols, const float2 *X, 
     embed_split_X_kernel<<<dim3((n + 31) / 32, (ncols + 31) / 32, M1), 256, 0, c->stream>>>(n, KP, ncols, X, c->Ximg.ptr);
     CUtensorMap tmB;
     if (!make_map(&tmB, c->Ximg.ptr, KP, ncols, 2 * M1, MT_N)) return fail(c, HZB_ECUDA, "tensor map of the panel");
-    if (check_cuda(c, c->kerr.ensure(1), "alloc error flag")) return HZB_ENOMEM;
-    if (!c->kerr_ready) {
-        if (check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0, sizeof(int), c->stream), "clear error flag"))
-            return HZB_ECUDA;
-        c->kerr_ready = true;
-    }
+    hzb_status st = tc_flag_begin(c, FAULT_TIMEOUT_MODAL);
+    if (st) return st;
     static bool attr_done[64] = {false};
     const int dev = c->opt.device;
     if (dev >= 0 && dev < 64 && !attr_done[dev]) {
@@ -316,7 +334,8 @@ hzb_status modal_gemm_tma(hzb_ctx *c, ShapeDev &sd, int ncols, const float2 *X, 
     modal_gemm_tma_kernel<<<grid, MT_THREADS, MT_SMEM, c->stream>>>(
         n, ncols, *reinterpret_cast<const CUtensorMap *>(sd.tmA), tmB, Cout, c->kerr.ptr);
     c->launches += 2;
-    return check_cuda(c, cudaGetLastError(), "modal_gemm_tma_kernel");
+    if (check_cuda(c, cudaGetLastError(), "modal_gemm_tma_kernel")) return HZB_ECUDA;
+    return tc_flag_launched(c);
 }
 
 }  // namespace hzb

@@ -556,7 +556,7 @@ hzb_status interbody_t5h(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
         check_cuda(c, c->t5h_img.ensure((size_t)nt * nchunk * th_bytes(rc)), "alloc operand images") ||
         check_cuda(c, c->dlkey.ensure(R), "alloc scales"))
         return HZB_ENOMEM;
-    hzb_status st = tc_flag_begin(c, true);
+    hzb_status st = tc_flag_begin(c, FAULT_TIMEOUT);
     if (st) return st;
     const int smem = th_smem(rc);                              // below the 48 KB that need no attribute
     static_assert(th_smem(32) <= 48 * 1024, "dynamic shared memory");

@@ -334,7 +334,7 @@ nbody_tc5ws_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chu
     constexpr int NC = 2 * RC;                         // accumulator columns: [Re y | Im y]
     extern __shared__ __align__(1024) unsigned char ws_smem_raw[];
     __shared__ uint32_t s_taddr;
-    __shared__ __align__(8) unsigned long long s_bar[8];   // full[2], empty[2], accfull[2], accempty[2]
+    __shared__ __align__(8) unsigned long long s_bar[9];   // full[2], empty[2], accfull[2], accempty[2], own
     __shared__ int s_abort;
     __shared__ __align__(16) float s_src[6][T5_K];
     const uint32_t raw = (uint32_t)__cvta_generic_to_shared(ws_smem_raw);
@@ -363,6 +363,7 @@ nbody_tc5ws_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chu
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(accfull0 + 8 * q), "r"(1) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(accempty0 + 8 * q), "r"(128) : "memory");
         }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 64), "r"(1) : "memory");
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -470,7 +471,7 @@ nbody_tc5ws_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chu
         for (int q = 0; q < NC; ++q) acc[q] = 0.f;
         for (int it = 0; it < ntile; ++it) {
             const int b = it & 1, v = it >> 1;
-            if (!ws_wait(accfull0 + 8 * b, (uint32_t)(v & 1), abort_flag)) break;
+            if (!t5_all(ws_wait(accfull0 + 8 * b, (uint32_t)(v & 1), abort_flag))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
             for (int q = 0; q < NC / 16; ++q) t5_ld16(tl + 64 * b + 16 * q, acc + 16 * q);
@@ -493,6 +494,7 @@ nbody_tc5ws_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chu
     } else if (lane == 0) {
         // ------------------------------------------------ MMA issue
         const int am[6] = {0, 0, 1, 2, 2, 3}, bm[6] = {0, 1, 0, 2, 3, 2};
+        int done = 0;
         for (int it = 0; it < ntile; ++it) {
             const int st = it & 1, u = it >> 1;
             if (!ws_wait(full0 + 8 * st, (uint32_t)(u & 1), abort_flag)) break;
@@ -512,6 +514,13 @@ nbody_tc5ws_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chu
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              accfull0 + 8 * st)
                          : "memory");
+            done = it + 1;
+        }
+        if (done > 0) {                                // the MMAs in flight, within a limit (the epilogue may
+                                                       // have given up on them)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 64)
+                         : "memory");
+            t5_wait(bar0 + 64, 0u);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -521,9 +530,10 @@ nbody_tc5ws_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chu
     if (tid == 0 && s_abort) atomicExch(err, 1);
 }
 
-// The device flag of the bounded waits before a launch; inject: the injected timeout fires here
-// (every CTA finds the flag negative and takes its timeout exit).
-hzb_status tc_flag_begin(hzb_ctx *c, bool inject)
+// The device flag of the bounded waits before a launch; fault: the injected timeout (a bit of
+// HZB_FAULT, 0: none) that fires here: every CTA of the launch finds the flag negative and takes its
+// timeout exit.
+hzb_status tc_flag_begin(hzb_ctx *c, int fault)
 {
     if (check_cuda(c, c->kerr.ensure(1), "alloc error flag")) return HZB_ENOMEM;
     if (!c->kerr_ready) {
@@ -531,18 +541,35 @@ hzb_status tc_flag_begin(hzb_ctx *c, bool inject)
             return HZB_ECUDA;
         c->kerr_ready = true;
     }
-    if (inject && (c->fault & FAULT_TIMEOUT) && !(c->fault_spent & FAULT_TIMEOUT) && !c->capturing) {
-        c->fault_spent |= FAULT_TIMEOUT;
+    if ((c->fault & fault) && !(c->fault_spent & fault) && !c->capturing) {
+        c->fault_spent |= fault;
+        c->fault_flag = true;
         if (check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0xff, sizeof(int), c->stream), "inject timeout"))
             return HZB_ECUDA;
     }
     return HZB_OK;
 }
 
+// right after the launch: an injected flag turns positive, so that later launches run
+hzb_status tc_flag_launched(hzb_ctx *c)
+{
+    if (!c->fault_flag) return HZB_OK;
+    c->fault_flag = false;
+    return check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0x01, sizeof(int), c->stream), "injected timeout");
+}
+
 // and after it: a wait that ran out left NaN outputs (a solve reads the flag once, at its end)
 hzb_status tc_flag_end(hzb_ctx *c, const char *kernel)
 {
-    if (c->capturing || c->in_solve) return HZB_OK;
+    hzb_status st = tc_flag_launched(c);
+    if (st || c->capturing || c->in_solve) return st;
+    return tc_flag_report(c, kernel);
+}
+
+// waits for the stream and reports a set flag, once
+hzb_status tc_flag_report(hzb_ctx *c, const char *kernel)
+{
+    if (!c->kerr_ready) return HZB_OK;
     int flag = 0;
     if (check_cuda(c, cudaMemcpyAsync(&flag, c->kerr.ptr, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
                    "read error flag") ||
@@ -573,7 +600,7 @@ hzb_status interbody_tc5(hzb_ctx *c, int R, const double2 *sigma, double2 *y, in
         if (check_cuda(c, c->nb_part32.ensure(n * nsplit), "alloc partial sums")) return HZB_ENOMEM;
         part = c->nb_part32.ptr;
     }
-    hzb_status st = tc_flag_begin(c, !ws);
+    hzb_status st = tc_flag_begin(c, ws ? 0 : FAULT_TIMEOUT);
     if (st) return st;
     static bool attr_done[64] = {false};
     const int dev = c->opt.device;

@@ -81,6 +81,11 @@ __device__ __forceinline__ bool t5_wait(uint32_t mbar, uint32_t parity)
     return false;
 }
 
+// Every wait gives up on its own lane's count of polls (and, where there is one, its own view of an
+// abort flag).  A warp that goes on to warp-wide instructions (elect.sync, tcgen05.ld, __syncwarp)
+// takes one answer for all its lanes: true where every lane's wait came through.
+__device__ __forceinline__ bool t5_all(bool ok) { return __all_sync(0xffffffffu, ok); }
+
 __device__ __forceinline__ void t5_ld32(uint32_t taddr, float *v)
 {
     uint32_t r[32];
