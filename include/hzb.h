@@ -70,9 +70,9 @@ typedef enum {
  *   alloc    every device allocation of the context fails (HZB_ENOMEM);
  *   geom     the first node generation writes a NaN weight (HZB_EINVAL);
  *   nan      the first solve's preconditioned right-hand side gets a NaN (HZB_ENAN);
- *   timeout  the first tcgen05 inter-body launch (FP32 engine 5) finds its error flag
- *            set before it starts and takes its timeout exit before issuing any MMA
- *            (HZB_ETIMEOUT);
+ *   timeout  the first tcgen05 inter-body launch (FP32 engine 5, or the double-float sum of
+ *            several right-hand sides) finds its error flag set before it starts and takes
+ *            its timeout exit before issuing any MMA (HZB_ETIMEOUT);
  *   timeout_modal  the first tcgen05 mode GEMM of D^{-1} (modal engine 2) does the same, with
  *            copies and MMAs in flight (HZB_ETIMEOUT).
  * All but the first fire once per context.  Nothing is injected on the GPU itself. */

@@ -190,6 +190,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     __shared__ __align__(8) unsigned long long s_bar[8];       // full[2]; per half tile: mma[2], formed[2]; moved, own
     __shared__ int s_rmin;
     __shared__ volatile int s_fail;
+    __shared__ int s_forced;                                   // host-set flag: take the timeout exit
     const TargetBlock tb = blocks[blockIdx.x >> 2];
     const int sub = blockIdx.x & 3;
     if (sub * DX_M >= tb.count) return;                        // whole CTA past the block's end
@@ -219,6 +220,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         s_rmin = 0x7f000000;
         s_fail = 0;
+        s_forced = *(volatile int *)err < 0 ? 1 : 0;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -240,7 +242,8 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     const int2 own = own_tiles[blockIdx.x >> 2];
     const int nown = own.y - own.x;
     const int i0 = (int)((long long)(ntiles - nown) * blockIdx.z / gridDim.z);
-    const int n = (int)((long long)(ntiles - nown) * (blockIdx.z + 1) / gridDim.z) - i0;
+    // an injected fault ends the CTA (both of a cluster) before any copy or MMA is issued
+    const int n = s_forced ? 0 : (int)((long long)(ntiles - nown) * (blockIdx.z + 1) / gridDim.z) - i0;
     auto tile_of = [&](int i) {
         const int q = i0 + i;
         return q < own.x ? q : q + nown;
@@ -337,28 +340,34 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     };
-    bool ok = true;
+    bool ok = s_forced == 0;
     if (q4 == 4) {
-        // the last warp: MMAs of each half tile once all 16 have formed it, copies into free stages
-        int halves = 0;
+        // the last warp: MMAs of each half tile once all 16 have formed it, copies into free stages;
+        // every wait gives one answer to all lanes
+        int halves = 0, armed = 0;                             // MMAs of half tiles issued; other halves announced
+        auto wait = [&](uint32_t mbar, int phase) { return t5_all(dx_wait<CL>(mbar, (uint32_t)(phase & 1))); };
+        auto arm = [&]() {                                     // the other half of a tile comes from the other CTA
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar0 + 32 + 8 * peer),
+                             "r"(DX_D * DX_AIMG)
+                             : "memory");
+            ++armed;
+        };
         for (int i = 0; i < n && ok; ++i) {
             if (i > 0) {
-                ok = (CL == 1 || dx_wait<CL>(bar0 + 16, (uint32_t)((i - 1) & 1))) && dx_wait<CL>(bar0 + 24, (uint32_t)((i - 1) & 1));
+                ok = (CL == 1 || wait(bar0 + 16, i - 1)) && wait(bar0 + 24, i - 1);
                 if (ok && i + 1 < n) {
                     if (lane == 0) issue(i + 1);
                     issued = i + 2;
                 }
             }
-            if (CL == 2 && ok && lane == 0)                    // the other half comes from the other CTA
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar0 + 32 + 8 * peer),
-                             "r"(DX_D * DX_AIMG)
-                             : "memory");
+            if (CL == 2) arm();
             // (CL = 1: the warps that form the halves have waited for the images)
-            if (CL == 2) ok = ok && t5_wait(bar0 + 8 * (i & 1), (uint32_t)((i >> 1) & 1));
+            if (CL == 2) ok = ok && wait(bar0 + 8 * (i & 1), i >> 1);
 #pragma unroll 1
             for (int hh = 0; hh < 2 && ok; ++hh) {
                 const int h = CL == 2 ? (int)rank ^ hh : hh;   // CL = 2: the own half first
-                ok = dx_wait<CL>(bar0 + 32 + 8 * h, (uint32_t)(i & 1)) && !s_fail;
+                ok = wait(bar0 + 32 + 8 * h, i) && !__any_sync(0xffffffffu, s_fail);
                 if (CL == 2 && ok && hh == 0 && lane == 0)
                     asm volatile(
                         "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -366,7 +375,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                         "r"(a0 + rank * (DX_D * DX_AIMG)), "r"(DX_D * DX_AIMG), "r"(dx_peer(bar0 + 32 + 8 * rank, peer))
                         : "memory");
                 // (CL = 1: the warps that formed the half have moved the levels)
-                if (CL == 2 && ok && hh == 0 && i > 0 && !(i & 1)) ok = t5_wait(bar0 + 48, (uint32_t)(((i >> 1) - 1) & 1));
+                if (CL == 2 && ok && hh == 0 && i > 0 && !(i & 1)) ok = wait(bar0 + 48, (i >> 1) - 1);
                 if (!ok) break;
                 __syncwarp();
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -398,7 +407,10 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
             }
         }
         if (!ok) s_fail = 1;
-        // what is in flight (after a timeout: once more)
+        // what is in flight (after a timeout: once more, the other CTA's half among it, which that CTA
+        // may have sent before its own wait ran out)
+        if (CL == 2 && !ok && armed > 0) dx_wait<CL>(bar0 + 32 + 8 * peer, (uint32_t)((armed - 1) & 1));
+        __syncwarp();
         if (halves > 0) {
             if (t5_elect())
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 56)
@@ -499,7 +511,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(dx_cols(RC)) : "memory");
     if (CL == 2) dx_cluster_sync();                            // no stores or arrivals into a CTA that has ended
-    if (failed && tid == 0) atomicExch(err, 1);
+    if (failed && tid == 0 && !s_forced) atomicExch(err, 1);   // (a negative flag stays for all CTAs of the launch)
 }
 
 // Digit images of s = 2^8 w sigma c0, scaled below 2^8 per column (key): for every tile and chunk of
@@ -587,7 +599,7 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     if (check_cuda(c, c->t5h_img.ensure((size_t)nt * nchunk * DX_D * dx_img(rc)), "alloc operand images") ||
         check_cuda(c, c->dlkey.ensure(R), "alloc scales"))
         return HZB_ENOMEM;
-    if ((st = tc_flag_begin(c, false))) return st;
+    if ((st = tc_flag_begin(c, FAULT_TIMEOUT))) return st;
     const double s = c->k / (2.0 * M_PI), c0 = s * s / (4.0 * M_PI);
     c->interbody_calls++;
     const int slot = prof_begin(c, 2);

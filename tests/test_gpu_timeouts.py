@@ -1,6 +1,8 @@
-"""The bounded-wait exit of the mode GEMM of D^{-1}, entered through a flag the host sets before the
-launch: it gives up with copies and MMAs in flight and reports HZB_ETIMEOUT, and the same context
-then gives the right result."""
+"""The bounded-wait exits of the tensor-core kernels that every default call uses, entered through a
+flag the host sets before the launch: the mode GEMM of D^{-1} gives up with copies and MMAs in
+flight, the double-float sum (alone and as pairs of CTAs) before it issues any.  Each reports
+HZB_ETIMEOUT, and the same context then gives the right result."""
+import numpy as np
 import pytest
 
 import workloads as W
@@ -30,3 +32,15 @@ def test_modal_gemm_timeout(monkeypatch, panels, gl, modes, R):
     ref = s.local_inverse(y)
     _times_out(lambda: s.local_inverse(y, precision=1))
     assert rel_l2(s.local_inverse(y, precision=1), ref) < 1e-5
+
+
+@pytest.mark.parametrize("R", [8, 16, 32, 33])
+def test_double_float_sum_timeout(monkeypatch, R):
+    require_gpu()
+    monkeypatch.setenv("HZB_FAULT", "timeout")
+    wl = W.two_spheres(n_panels=7, gl_order=9, n_modes=33)
+    s = gpu_solver(wl)
+    sig = rand_c((s.N, R), 22)
+    ref = s.interbody(sig)
+    _times_out(lambda: s.interbody(sig, precision=2))
+    assert np.abs(s.interbody(sig, precision=2) - ref).max() < 1e-12 * np.abs(ref).max()
