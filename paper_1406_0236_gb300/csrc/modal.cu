@@ -12,6 +12,7 @@
 #include "hzb_internal.h"
 #include "kernel_math.cuh"
 #include "modal_gemm.cuh"
+#include "tcgen05.cuh"
 
 namespace hzb {
 
@@ -476,8 +477,8 @@ modal_gemm_tc_kernel(int n, int nc, const float2 *__restrict__ A, const float2 *
             for (int nt = 0; nt < 4; ++nt) {
                 const int c = wn * 32 + nt * 8 + g;
                 const float v0 = Bs[kk + t][c], v1 = Bs[kk + t + 4][c];
-                uint32_t bh[2] = {to_tf32(v0), to_tf32(v1)};
-                uint32_t bl[2] = {to_tf32(v0 - __uint_as_float(bh[0])), to_tf32(v1 - __uint_as_float(bh[1]))};
+                const uint32_t bh[2] = {t5_tf32(v0), t5_tf32(v1)};       // (keeps a NaN of the panel)
+                const uint32_t bl[2] = {t5_tf32(v0 - __uint_as_float(bh[0])), t5_tf32(v1 - __uint_as_float(bh[1]))};
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt) {
                     mma_tf32(acc[mt][nt], al[mt], bh);

@@ -42,8 +42,8 @@ static inline int kpitch(int n) { return (2 * n + 3) & ~3; }
 
 __device__ __forceinline__ void mt_split(double a, float &hi, float &lo)
 {
-    hi = __uint_as_float(t5_tf32i((float)a));
-    lo = __uint_as_float(t5_tf32i((float)(a - (double)hi)));
+    hi = __uint_as_float(t5_tf32((float)a));
+    lo = __uint_as_float(t5_tf32((float)(a - (double)hi)));
 }
 
 // plane (2p + h), row m, column k of the embedded, split S_p
@@ -69,7 +69,7 @@ __global__ void embed_split_S_kernel(int n, int KP, int M1, const double2 *__res
 
 // plane (2p + h), row = panel column c, column k of [Xr; Xi] split.  A block transposes 32 rows
 // (k) x 32 columns of X through shared memory, so that both sides are read and written in whole
-// lines, and splits in FP32 (x - hi is exact); in FP64 the splitting alone kept its pipe busy for
+// lines, and splits in FP32 (x - hi is exact) by the conversion instruction, which keeps a NaN; in FP64 the splitting alone kept its pipe busy for
 // 40 us at 258,560 unknowns, R = 16 (44 -> 18 us).
 __global__ void __launch_bounds__(256)
 embed_split_X_kernel(int n, int KP, int nc, const float2 *__restrict__ X, float *__restrict__ img)
@@ -87,11 +87,11 @@ embed_split_X_kernel(int n, int KP, int nc, const float2 *__restrict__ X, float 
         if (c >= nc || k >= n) continue;
         const float2 v = s[tx][q];
         float *const hi = img + ((size_t)(2 * p) * nc + c) * KP, *const lo = hi + (size_t)nc * KP;
-        const float hx = __uint_as_float(t5_tf32i(v.x)), hy = __uint_as_float(t5_tf32i(v.y));
+        const float hx = __uint_as_float(t5_tf32(v.x)), hy = __uint_as_float(t5_tf32(v.y));
         hi[k] = hx;
-        lo[k] = __uint_as_float(t5_tf32i(v.x - hx));
+        lo[k] = __uint_as_float(t5_tf32(v.x - hx));
         hi[n + k] = hy;
-        lo[n + k] = __uint_as_float(t5_tf32i(v.y - hy));
+        lo[n + k] = __uint_as_float(t5_tf32(v.y - hy));
         if (k < KP - 2 * n) hi[2 * n + k] = lo[2 * n + k] = 0.f;          // the rows' padding
     }
 }

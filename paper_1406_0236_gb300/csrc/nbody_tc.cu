@@ -17,6 +17,7 @@
 
 #include "hzb_internal.h"
 #include "kernel_math.cuh"
+#include "tcgen05.cuh"
 
 namespace hzb {
 
@@ -25,7 +26,7 @@ static const int TC_CTA_TARGETS = 128;
 static const int TC_S = 32;               // sources per tile
 
 // TF32 operand (round to nearest, ties away, 10 mantissa bits) by two integer operations
-// on the bit pattern: equal to cvt.rna.tf32.f32 for finite x, and faster than it
+// on the bit pattern: equal to cvt.rna.tf32.f32 for finite x, and faster than it (a NaN is lost)
 __device__ __forceinline__ uint32_t tf32_of(float x) { return (__float_as_uint(x) + 0x1000u) & 0xFFFFE000u; }
 
 __device__ __forceinline__ void mma_m16n8k8(float *d, const uint32_t *a, const uint32_t *b)
@@ -126,11 +127,11 @@ nbody_tc_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chunk,
                     sr = v.x;
                     si = v.y;
                 }
-                const uint32_t rh = tf32_of(sr), ih = tf32_of(si);
+                const uint32_t rh = t5_tf32(sr), ih = t5_tf32(si);       // (keeps a NaN)
                 s_rh[r * LD + s] = rh;
-                s_rl[r * LD + s] = tf32_of(sr - __uint_as_float(rh));
+                s_rl[r * LD + s] = t5_tf32(sr - __uint_as_float(rh));
                 s_ih[r * LD + s] = ih;
-                s_il[r * LD + s] = tf32_of(si - __uint_as_float(ih));
+                s_il[r * LD + s] = t5_tf32(si - __uint_as_float(ih));
             }
             __syncthreads();
             if (!active) continue;

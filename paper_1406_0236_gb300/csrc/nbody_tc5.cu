@@ -21,8 +21,9 @@
 //     (tcgen05.ld) and adds them to running FP32 sums in registers: the tensor cores'
 //     internal accumulation is not rounded to nearest, so chaining ~10^4 tiles in tensor
 //     memory would drift.
-// TF32 rounding is done by two integer operations on the bit pattern (t5_tf32i), which
-// measured faster than the conversion instruction.  The next tile's positions and
+// TF32 rounding of the pair kernels is done by two integer operations on the bit pattern
+// (t5_tf32i), which measured faster than the conversion instruction; the densities take the
+// instruction, which keeps a NaN.  The next tile's positions and
 // densities are loaded into registers while the current tile's pair kernels and MMAs run.  Every mbarrier wait is bounded; on a timeout the CTA
 // sets an error flag, writes NaN outputs, frees its tensor memory and returns.
 #include <algorithm>
@@ -182,13 +183,13 @@ nbody_tc5_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chunk
         if (bduty) {   // B operands: rows bn (B1 = Re s', B2 = -Im s') and bn + RC (B1 = Im s', B2 = Re s')
             uint32_t h[4], l[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) { h[q] = t5_tf32i(bv[q].x); l[q] = t5_tf32i(bv[q].x - __uint_as_float(h[q])); }
+            for (int q = 0; q < 4; ++q) { h[q] = t5_tf32(bv[q].x); l[q] = t5_tf32(bv[q].x - __uint_as_float(h[q])); }
             t5_st4(sB + 0 * T5_B_BYTES + t5_chunk_off(bn, bc), h[0], h[1], h[2], h[3]);
             if (TERMS == 3) t5_st4(sB + 1 * T5_B_BYTES + t5_chunk_off(bn, bc), l[0], l[1], l[2], l[3]);
             t5_st4(sB + 2 * T5_B_BYTES + t5_chunk_off(bn + RC, bc), h[0], h[1], h[2], h[3]);
             if (TERMS == 3) t5_st4(sB + 3 * T5_B_BYTES + t5_chunk_off(bn + RC, bc), l[0], l[1], l[2], l[3]);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) { h[q] = t5_tf32i(bv[q].y); l[q] = t5_tf32i(bv[q].y - __uint_as_float(h[q])); }
+            for (int q = 0; q < 4; ++q) { h[q] = t5_tf32(bv[q].y); l[q] = t5_tf32(bv[q].y - __uint_as_float(h[q])); }
             t5_st4(sB + 0 * T5_B_BYTES + t5_chunk_off(bn + RC, bc), h[0], h[1], h[2], h[3]);
             if (TERMS == 3) t5_st4(sB + 1 * T5_B_BYTES + t5_chunk_off(bn + RC, bc), l[0], l[1], l[2], l[3]);
 #pragma unroll
@@ -420,13 +421,13 @@ nbody_tc5ws_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chu
             if (bduty) {
                 uint32_t h[4], l[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) { h[q] = t5_tf32i(bv[q].x); l[q] = t5_tf32i(bv[q].x - __uint_as_float(h[q])); }
+                for (int q = 0; q < 4; ++q) { h[q] = t5_tf32(bv[q].x); l[q] = t5_tf32(bv[q].x - __uint_as_float(h[q])); }
                 t5_st4(sB + 0 * T5_B_BYTES + t5_chunk_off(bn, bc), h[0], h[1], h[2], h[3]);
                 t5_st4(sB + 1 * T5_B_BYTES + t5_chunk_off(bn, bc), l[0], l[1], l[2], l[3]);
                 t5_st4(sB + 2 * T5_B_BYTES + t5_chunk_off(bn + RC, bc), h[0], h[1], h[2], h[3]);
                 t5_st4(sB + 3 * T5_B_BYTES + t5_chunk_off(bn + RC, bc), l[0], l[1], l[2], l[3]);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) { h[q] = t5_tf32i(bv[q].y); l[q] = t5_tf32i(bv[q].y - __uint_as_float(h[q])); }
+                for (int q = 0; q < 4; ++q) { h[q] = t5_tf32(bv[q].y); l[q] = t5_tf32(bv[q].y - __uint_as_float(h[q])); }
                 t5_st4(sB + 0 * T5_B_BYTES + t5_chunk_off(bn + RC, bc), h[0], h[1], h[2], h[3]);
                 t5_st4(sB + 1 * T5_B_BYTES + t5_chunk_off(bn + RC, bc), l[0], l[1], l[2], l[3]);
 #pragma unroll
