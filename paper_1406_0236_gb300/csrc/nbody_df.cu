@@ -409,7 +409,12 @@ hzb_status interbody_df(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     // the lean kernels: tensor-core sums where they apply, else pair-symmetric for few right-hand
     // sides, one-directional above
     hzb_status st = HZB_OK;
-    if (c->nbody64_engine < 0 && dfx_usable(c, R, &st)) return interbody_dfx(c, R, sigma, y);
+    if (c->nbody64_engine < 0 && dfx_usable(c, R, &st)) {
+        st = interbody_dfx(c, R, sigma, y);
+        if (st != HZB_ENOMEM) return st;
+        cudaGetLastError();                                // no room for its images: the kernels that need none
+        st = HZB_OK;
+    }
     if (st) return st;
     if (c->nbody64_engine == 1 || (c->nbody64_engine < 0 && dfl_symmetric(c, R))) return interbody_dfl_sym(c, R, sigma, y);
     if (c->nbody64_engine != 2) return interbody_dfl(c, R, sigma, y);

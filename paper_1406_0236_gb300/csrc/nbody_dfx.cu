@@ -12,7 +12,9 @@
 // of the leading digits) is lost on a sum of 2^23 of them.  The levels 0 ... 5 (21 products) are
 // kept; what is left out is below 2^-50 of the largest product, the digits' own cut 2^-53 of the
 // largest kernel value.  After two tiles the six levels enter 64-bit integers (unit 2^-32): no sum is
-// rounded but there, and the result does not depend on the order of the sources.
+// rounded but there.  The integers hold 256 tiles; a longer chunk adds them to y (or its partial sum)
+// in FP64 that often, so that the number of chunks follows the SMs alone (with a chunk per 256 tiles
+// 258,560 unknowns and R = 64 took 7.4 GB of partial sums, 2.2 million and R = 16 152 GB).
 //
 // Per CTA: 128 targets (the M of the MMA), RC right-hand sides (N = 2 RC columns: real and
 // imaginary parts), a chunk of the source tiles.  Sixteen warps form kernels, four sources of each
@@ -62,6 +64,8 @@ static double dx_start(int rc) { return rc == 8 ? 0.5 : rc == 16 ? 0.8 : 1.2; } 
 // N^2 R from which on this form is the faster one (us, here / one-directional): 900 unknowns
 // (R = 16: 1.3e7) 74 / 74, 1,764 (R = 8: 2.5e7) 81 / 79, (R = 16) 85 / 117, 3,968 (R = 5) 163 / 206
 static const double DX_WORK = 2.4e7;
+static const int DX_RUN = 256;         // tiles after which the 64-bit sums are emptied (at most 2^54 to a tile)
+static_assert(DX_RUN >= 2 && (DX_RUN & (DX_RUN - 1)) == 0, "the levels move every second tile");
 static const int DX_AIMG = DX_M * 64;                          // bytes of one digit image of half a tile of A
 static const int DX_GEO = 3 * DFL_S * 16;                      // bytes of a tile's nodes
 
@@ -307,7 +311,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     const dd scale = {__int_as_float((127 + 8 - e2) << 23), 0.f};
 
     uint32_t bad = 0;                                          // columns that met a NaN
-    // the levels of the last tile into the sums
+    // the levels of the last tiles into the sums
     auto drain = [&]() {
 #pragma unroll
         for (int q = 0; q < CW; q += 4) {
@@ -339,6 +343,38 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
             dx_st4(hirow + q, hi);
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    };
+    // the sums into the output, which holds what earlier ones left (begun); then they start at zero
+    bool begun = false, failed = false;
+    auto emit = [&]() {
+        const double f = 0x1p-40 / (double)scale.h;            // 2^-32 of the unit, 2^-8 of the densities
+#pragma unroll 1
+        for (int q = 0; q < CW; q += 4) {
+            uint32_t lo[4], hi[4];
+            const uint32_t z[4] = {0u, 0u, 0u, 0u};
+            __syncwarp();
+            dx_ld4(lorow + q, lo);
+            dx_ld4(hirow + q, hi);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            dx_keep(lo);
+            dx_keep(hi);
+            dx_st4(lorow + q, z);
+            dx_st4(hirow + q, z);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                // columns CW q4 ..: the first RC are real parts, the others imaginary parts
+                const int col = CW * q4 + q + c, r = blockIdx.y * RC + col % RC;
+                if (!live || r >= R) continue;
+                const long long s = (long long)(((unsigned long long)hi[c] << 32) | lo[c]);
+                double v = (double)s * f * sigma_pow2(sigma_exponent(key[r]));
+                double *o = reinterpret_cast<double *>(out + blockIdx.z * split_stride + (size_t)(tb.start + t) * R + r) + col / RC;
+                if (begun) v += *o;
+                *o = (failed || (bad >> (q + c) & 1)) ? __longlong_as_double(0x7ff8000000000000ll) : v;
+            }
+        }
+        __syncwarp();
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        begun = true;
     };
     bool ok = s_forced == 0;
     if (q4 == 4) {
@@ -455,6 +491,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     __syncwarp();
                     drain();
+                    if ((i & (DX_RUN - 1)) == 0) emit();
                     if (CL == 2) {
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         __syncwarp();
@@ -484,28 +521,8 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
             drain();
         }
     }
-    const bool failed = __syncthreads_or(!ok);
-    // columns CW q4 ..: the first RC are real parts, the others imaginary parts
-    const double f = 0x1p-40 / (double)scale.h;                // 2^-32 of the unit, 2^-8 of the densities
-    if (q4 < 4)
-#pragma unroll
-    for (int q = 0; q < CW; q += 4) {
-        uint32_t lo[4], hi[4];
-        dx_ld4(lorow + q, lo);
-        dx_ld4(hirow + q, hi);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        dx_keep(lo);
-        dx_keep(hi);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int col = CW * q4 + q + c, r = blockIdx.y * RC + col % RC;
-            if (!live || r >= R) continue;
-            const long long s = (long long)(((unsigned long long)hi[c] << 32) | lo[c]);
-            const double v = (double)s * f * sigma_pow2(sigma_exponent(key[r]));
-            double *o = reinterpret_cast<double *>(out + blockIdx.z * split_stride + (size_t)(tb.start + t) * R + r);
-            o[col / RC] = (failed || (bad >> (q + c) & 1)) ? __longlong_as_double(0x7ff8000000000000ll) : v;
-        }
-    }
+    failed = __syncthreads_or(!ok);
+    if (q4 < 4) emit();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
@@ -578,12 +595,13 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     if (st) return st;
     // Source chunks: the shortest time, in tiles.  Bodies of one size: whole waves of equal CTAs;
     // others: the mean load and most of a long CTA's time at the end.  A partial sum costs 1e-6 of a
-    // tile; at most 256 tiles go to a chunk (the sums' 64 bits).
+    // tile.  Beyond 32 waves there is nothing left to fill, and the partial sums stay below 0.4 GB
+    // (128 x 32 values to a CTA).
     const long long ctas = (long long)c->t5h_ctas * nchunk;
     const bool even = c->t5h_mean > 0.97 * most;
-    int nsplit = (most + 255) / 256;
+    int nsplit = 1;
     double best = 1e300;
-    for (int ns = nsplit; ns <= std::max(nsplit, std::min(64, most)); ++ns) {
+    for (int ns = 1; ns <= std::min(64, most) && (ns == 1 || ns * ctas <= 32LL * sms); ++ns) {
         const double one = std::ceil((double)most / ns) + dx_start(rc);
         const double tt = (even ? std::ceil((double)(ns * ctas) / sms) * one
                                 : std::max(one, ctas * (c->t5h_mean + ns * dx_start(rc)) / sms + 0.6 * one)) +
