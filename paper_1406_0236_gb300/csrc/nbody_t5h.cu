@@ -18,15 +18,19 @@
 //   * one thread issues 12 MMAs (M = 128, N = 2 RC, K = 16; high x high, high x low, low x
 //     high for Re G' x [Re s | Im s] and -Im G' x [Im s | -Re s]) and commits them;
 //   * the warps read the accumulator (started from zero in every tile: chained tensor-core
-//     sums are not rounded to nearest and drift) and add it to FP32 sums in registers.
+//     sums are not rounded to nearest and drift) and add it, times the tile's scale, to FP32
+//     sums in registers.
 // One block barrier per tile; three CTAs per SM (128 columns of tensor memory each) overlap
 // one another's barriers, MMAs and reads.
 //
 // FP16's range: G' is scaled by the power of two that brings its bound at the smallest
-// distance between two bodies (t5h_range_kernel, once per geometry) to 2^15, the densities per
-// right-hand side to 2^14, so that a value down to 2^-17 of the largest keeps 22 bits and no
-// value overflows.  Geometries whose kernels span more than that (or k, eta outside
-// sym_scaled) keep the TF32 form (nbody_tc5.cu).
+// distance between two bodies (t5h_range_kernel, once per geometry) to 2^15, the densities by tile
+// and right-hand side to 2^14, so that a value down to 2^-17 of the largest keeps 22 bits and no
+// value overflows.  The tile's power of two, against the column's, goes with its images (one scale
+// per column left 2^-38 of the column's largest value to a body whose densities are small, and
+// the rows of the others nothing else to sum: relative error 4e-4 there at 1e-8; now 1e-6, for
+// 900 -> 913 us at 29,280 unknowns, R = 16).  Geometries whose kernels span more than FP16 (or k, eta
+// outside sym_scaled) keep the TF32 form (nbody_tc5.cu).
 //
 // Bound by the transcendental unit (3 operations per ordered pair: 0.39 ms at 29,280
 // unknowns) and issue (29 instructions per pair, a packed one counting twice at dispatch).  Against the TF32
@@ -55,10 +59,16 @@ static const int TH_SRC = 6 * TH_S;                    // floats of a tile's geo
 static const int TH_COLS = 128;                        // tensor-memory columns: A 64, D 2 RC
 static const int TH_A = 0, TH_D = 64;                  // first columns
 static const int TH_ATILE = TH_S / 2;                  // columns of one A part (two FP16 per column)
+// Exponents below the column's largest value at which a tile's scale stops: 2^-100 of it times a sum
+// of 2^-40 (in units of 2^29 and more) is still in FP32's range
+static const int TH_LOW = 100;
 
 __host__ __device__ constexpr int th_bytes(int rc) { return 2 * 2 * rc * 128; }   // B images of a tile: 2 x 2 RC rows
+__host__ __device__ constexpr int th_image(int rc) { return th_bytes(rc) + 4 * rc; }          // and its scales
 __host__ __device__ constexpr int th_stage(int rc) { return th_bytes(rc) + 1024; }
-__host__ __device__ constexpr int th_smem(int rc) { return 2 * th_stage(rc) + 1024; }
+// two stages and the scales of four tiles: a stage is refilled while slower warps still read the
+// scales of the tile that left it
+__host__ __device__ constexpr int th_smem(int rc) { return 2 * th_stage(rc) + 4 * 4 * rc + 1024; }
 static_assert(TH_SRC * 4 <= 1024, "geometry of a tile in its stage");
 
 // kind::f16 with FP16 A and B, FP32 D
@@ -98,6 +108,31 @@ __device__ __forceinline__ void th_copy(uint32_t dst, const void *src, uint32_t 
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(mbar)
                  : "memory");
+}
+
+// acc += f x NC columns of this warp's lanes
+template <int NC>
+__device__ __forceinline__ void th_add(uint32_t taddr, const float *f, float *acc)
+{
+#pragma unroll
+    for (int q0 = 0; q0 < NC; q0 += 16) {
+        uint32_t r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+            "%15}, [%16];\n"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(taddr + q0));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int q = 0; q < 16; q += 4) {
+            const float4 s = *reinterpret_cast<const float4 *>(f + q0 + q);
+            acc[q0 + q] = fmaf(__uint_as_float(r[q]), s.x, acc[q0 + q]);
+            acc[q0 + q + 1] = fmaf(__uint_as_float(r[q + 1]), s.y, acc[q0 + q + 1]);
+            acc[q0 + q + 2] = fmaf(__uint_as_float(r[q + 2]), s.z, acc[q0 + q + 2]);
+            acc[q0 + q + 3] = fmaf(__uint_as_float(r[q + 3]), s.w, acc[q0 + q + 3]);
+        }
+    }
 }
 
 // FP16 parts of a packed pair: the 11 leading bits, and the rest rounded to 11 bits
@@ -174,10 +209,12 @@ nbody_t5h_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     auto issue = [&](int i) {
         const int q = i0 + i, tile = q < own.x ? q : q + nown;
         const uint32_t st = base + (uint32_t)((i & 1) * STAGE), mb = bar0 + 8 * (i & 1);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(BYTES + TH_SRC * 4)
+        const unsigned char *const im = img + ((size_t)tile * gridDim.y + blockIdx.y) * th_image(RC);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(BYTES + TH_SRC * 4 + 4 * RC)
                      : "memory");
-        th_copy(st, img + ((size_t)tile * gridDim.y + blockIdx.y) * BYTES, BYTES, mb);
+        th_copy(st, im, BYTES, mb);
         th_copy(st + BYTES, src + (size_t)tile * TH_SRC, TH_SRC * 4, mb);
+        th_copy(base + 2 * STAGE + (i & 3) * 4 * RC, im + BYTES, 4 * RC, mb);
     };
     if (tid == 0) {
         if (n > 0) issue(0);
@@ -264,8 +301,7 @@ nbody_t5h_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
             issue(i + 2);
             issued = i + 3;
         }
-        if (RC == 32) t5_ld32(drow, acc);
-        else t5_ld16(drow, acc);
+        th_add<RC>(drow, reinterpret_cast<const float *>(gbase + 2 * STAGE) + (i & 3) * RC, acc);
     }
     if (tid == 0) {                                            // after a timeout: what is in flight, once more
         if (!mma_ok) t5_wait(bar0 + 16, (uint32_t)(last & 1));
@@ -368,8 +404,9 @@ __global__ void t5h_range_kernel(int ntiles, const int2 *__restrict__ tiles, con
 
 // B images of every tile and chunk of RC right-hand sides, in the swizzled K-major layout the
 // MMAs read: rows n < RC and n + RC of B1 = [Re s' ; Im s'] and B2 = [Im s' ; -Re s'], each row
-// the high parts of the 32 sources, then the low parts.  s' = w sigma scaled to 2^14 per column
-// (key).  One thread per (tile, column, eight sources).
+// the high parts of the 32 sources, then the low parts; behind them the scales of the RC columns.
+// s' = w sigma 2^(14 - e), e the exponent of the tile's largest value (at least the column's - TH_LOW);
+// the scale 2^(e - the column's).  A warp takes eight columns, a lane one of them and eight sources.
 __global__ void t5h_density_kernel(int ntiles, int R, int rc, int nchunk, const int2 *__restrict__ tiles,
                                    const double4 *__restrict__ pos, const double2 *__restrict__ sigma,
                                    const int *__restrict__ key, unsigned char *__restrict__ img)
@@ -377,25 +414,37 @@ __global__ void t5h_density_kernel(int ntiles, int R, int rc, int nchunk, const 
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int ncol = rc * nchunk;
     if (e >= (size_t)ntiles * ncol * 4) return;
-    const int col = (int)(e % ncol), g = (int)(e / ncol % 4), tile = (int)(e / ncol / 4);
+    const int lane = threadIdx.x & 31, g = lane >> 3, per = ncol / 8;
+    const int tile = (int)(e / 32 / per), col = (int)(e / 32 % per) * 8 + (lane & 7);
     const int2 tl = tiles[tile];
-    const double sc = col < R ? sigma_pow2(14 - sigma_exponent(key[col])) : 0.0;
+    const int top = col < R ? sigma_exponent(key[col]) : 0;
+    double2 z[8];
+    int big = 0;                                               // largest high word of the finite values
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int s = 8 * g + q;
+        z[q] = make_double2(0.0, 0.0);
+        if (s < tl.y && col < R) {
+            const double wq = pos[tl.x + s].w;
+            z[q] = sigma[(size_t)(tl.x + s) * R + col];
+            z[q].x *= wq;
+            z[q].y *= wq;
+            const int hx = __double2hiint(z[q].x) & 0x7fffffff, hy = __double2hiint(z[q].y) & 0x7fffffff;
+            big = max(big, max(hx < 0x7ff00000 ? hx : 0, hy < 0x7ff00000 ? hy : 0));
+        }
+    }
+    big = max(big, __shfl_xor_sync(0xffffffffu, big, 8));
+    big = max(big, __shfl_xor_sync(0xffffffffu, big, 16));
+    const int own = min(top, max(top - TH_LOW, big ? sigma_exponent(big) : -960));
+    const double sc = sigma_pow2(14 - own);
     uint32_t h[2][4], l[2][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         float v[2][2];
 #pragma unroll
         for (int w = 0; w < 2; ++w) {
-            const int s = 8 * g + 2 * q + w;
-            double2 z = make_double2(0.0, 0.0);
-            if (s < tl.y && col < R) {
-                const double wq = pos[tl.x + s].w * sc;
-                z = sigma[(size_t)(tl.x + s) * R + col];
-                z.x *= wq;
-                z.y *= wq;
-            }
-            v[0][w] = (float)z.x;
-            v[1][w] = (float)z.y;
+            v[0][w] = (float)(z[2 * q + w].x * sc);
+            v[1][w] = (float)(z[2 * q + w].y * sc);
         }
 #pragma unroll
         for (int a = 0; a < 2; ++a) {
@@ -406,7 +455,8 @@ __global__ void t5h_density_kernel(int ntiles, int R, int rc, int nchunk, const 
         }
     }
     const int n = col % rc, bytes = th_bytes(rc);
-    unsigned char *b1 = img + ((size_t)tile * nchunk + col / rc) * bytes, *b2 = b1 + bytes / 2;
+    unsigned char *b1 = img + ((size_t)tile * nchunk + col / rc) * th_image(rc), *b2 = b1 + bytes / 2;
+    if (g == 0) reinterpret_cast<float *>(b1 + bytes)[n] = (float)sigma_pow2(own - top);
     const uint32_t neg = 0x80008000u;
     auto put = [&](unsigned char *b, int row, const uint32_t *hi, const uint32_t *lo, uint32_t flip) {
         *reinterpret_cast<uint4 *>(b + t5_chunk_off(row, g)) =
@@ -553,7 +603,7 @@ hzb_status interbody_t5h(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     nsplit = (most + chunk - 1) / chunk;
     const size_t n = (size_t)c->N * R;
     if (check_cuda(c, c->nb_part32.ensure(n * nsplit), "alloc partial sums") ||
-        check_cuda(c, c->t5h_img.ensure((size_t)nt * nchunk * th_bytes(rc)), "alloc operand images") ||
+        check_cuda(c, c->t5h_img.ensure((size_t)nt * nchunk * th_image(rc)), "alloc operand images") ||
         check_cuda(c, c->dlkey.ensure(R), "alloc scales"))
         return HZB_ENOMEM;
     hzb_status st = tc_flag_begin(c, FAULT_TIMEOUT);
