@@ -553,7 +553,12 @@ hzb_status interbody32(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     const int e = fp32_engine(c, R);
     if (e == 2) {
         hzb_status st;
-        if (t5h_usable(c, &st)) return interbody_t5h(c, R, sigma, y);
+        if (t5h_usable(c, &st)) {
+            st = interbody_t5h(c, R, sigma, y);
+            if (st != HZB_ENOMEM) return st;
+            cudaGetLastError();                            // no room for its images: as outside its range
+            st = HZB_OK;
+        }
         if (st) return st;
     }
     // the range of the FP16 form is known only now: few right-hand sides stay on the CUDA cores
