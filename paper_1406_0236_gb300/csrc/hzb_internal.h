@@ -200,6 +200,8 @@ struct hzb_ctx {
     int t5h_state = 0, t5h_ntiles = 0, t5h_most = 0, t5h_ctas = 0;
     double t5h_scale = 0.0, t5h_span = 0.0, t5h_mean = 1.0;
     hzb::DevBuf<int2> t5h_tiles;
+    hzb::DevBuf<int> t5h_body;                 // per tile its body and place in it (t5h_tile_word)
+    int t5h_nbodies = 0;                       // bodies with nodes
     hzb::DevBuf<float> t5h_src;
     hzb::DevBuf<unsigned char> t5h_img;
     int nbody64_engine = -1;                   // FP64/double-float sums: -1 auto (pair-symmetric for R <= 4;
@@ -307,6 +309,11 @@ bool dfl_symmetric(const hzb_ctx *c, int R);                                    
 hzb_status interbody_tc(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int nsplit);
 hzb_status modal_gemm_tma(hzb_ctx *c, ShapeDev &sd, int ncols, const float2 *X, float2 *Cout);  // modal_tma.cu
 enum { T5_SPLIT3 = 0, T5_WS = 1, T5_SINGLE = 2 };   // forms of the tcgen05 inter-body kernel
+// a tile's body, whether its place in the body is odd, and its number of sources (at most 32)
+__host__ __device__ inline int t5h_tile_word(int body, int odd, int count) { return body << 7 | odd << 6 | count; }
+__host__ __device__ inline int t5h_tile_body(int word) { return word >> 7; }
+__host__ __device__ inline int t5h_tile_odd(int word) { return word >> 6 & 1; }
+__host__ __device__ inline int t5h_tile_count(int word) { return word & 63; }
 // nbody_t5h.cu: FP16 three-term form, where the geometry's kernels fit FP16's range
 hzb_status ensure_t5h(hzb_ctx *c);
 bool t5h_usable(hzb_ctx *c, hzb_status *st);

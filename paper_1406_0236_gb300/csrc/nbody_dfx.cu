@@ -2,8 +2,8 @@
 // cores: pair kernels in lean double-float on the FP32 pipe (dfl_pair.cuh), the sums over sources
 // as exact integer products of FP16 digits (tcgen05, FP32 accumulators).
 //
-// With G = E [X - i (kr X + eta')] (nbody_dfl.cu) and sigma' = w sigma c0 scaled below one per
-// right-hand side, y_i = sum_j G_ij sigma'_j.  Each real number is cut into DX_D = 6 digits of
+// With G = E [X - i (kr X + eta')] (nbody_dfl.cu) and sigma' = w sigma c0 scaled below one per body
+// and right-hand side, y_i = sum_j G_ij sigma'_j.  Each real number is cut into DX_D = 6 digits of
 // base 2^9: x = G 2^E with |x| < 2^8 (E from a bound of |G| over the CTA's pairs) and
 // s = 2^8 sigma' are x = sum_a d_a 2^(-9 a) with integers |d_a| <= 2^8 + 4, exact in FP16.  The
 // products of digits a + b = l add up, over two tiles of 32 sources and real and imaginary parts, to
@@ -11,10 +11,14 @@
 // l = 2, 3 unless nearly every digit is at its limit with one sign, when a unit (2^-18 of a product
 // of the leading digits) is lost on a sum of 2^23 of them.  The levels 0 ... 5 (21 products) are
 // kept; what is left out is below 2^-50 of the largest product, the digits' own cut 2^-53 of the
-// largest kernel value.  After two tiles the six levels enter 64-bit integers (unit 2^-32): no sum is
-// rounded but there.  The integers hold 256 tiles; a longer chunk adds them to y (or its partial sum)
-// in FP64 that often, so that the number of chunks follows the SMs alone (with a chunk per 256 tiles
-// 258,560 unknowns and R = 64 took 7.4 GB of partial sums, 2.2 million and R = 16 152 GB).
+// largest kernel value.  After two tiles of one body the six levels enter 64-bit integers (unit 2^-32),
+// shifted from that body's scale to the largest of those the targets sum, their own body's left out:
+// no sum is rounded but there.  (One scale over all bodies left a body whose densities are 1e-8 of the
+// largest 1e-8 of relative error on the others' rows; the shifts and the levels moved at a body's end
+// cost 3 % at 8,200 unknowns, R = 64, and on three bodies of 9,008 unknowns, R = 8.)  The integers hold 256 tiles; a longer chunk
+// adds them to y (or its partial sum) in FP64 that often, so that the number of chunks follows the SMs
+// alone (with a chunk per 256 tiles 258,560 unknowns and R = 64 took 7.4 GB of partial sums, 2.2 million
+// and R = 16 152 GB).
 //
 // Per CTA: 128 targets (the M of the MMA), RC right-hand sides (N = 2 RC columns: real and
 // imaginary parts), a chunk of the source tiles.  Sixteen warps form kernels, four sources of each
@@ -65,7 +69,7 @@ static double dx_start(int rc) { return rc == 8 ? 0.5 : rc == 16 ? 0.8 : 1.2; } 
 // (R = 16: 1.3e7) 74 / 74, 1,764 (R = 8: 2.5e7) 81 / 79, (R = 16) 85 / 117, 3,968 (R = 5) 163 / 206
 static const double DX_WORK = 2.4e7;
 static const int DX_RUN = 256;         // tiles after which the 64-bit sums are emptied (at most 2^54 to a tile)
-static_assert(DX_RUN >= 2 && (DX_RUN & (DX_RUN - 1)) == 0, "the levels move every second tile");
+static_assert((DX_RUN & (DX_RUN - 1)) == 0, "a power of two");
 static const int DX_AIMG = DX_M * 64;                          // bytes of one digit image of half a tile of A
 static const int DX_GEO = 3 * DFL_S * 16;                      // bytes of a tile's nodes
 
@@ -184,7 +188,8 @@ __device__ __forceinline__ uint32_t dx_pack(float a, float b)
 template <int RC, int CL>
 __global__ void __launch_bounds__(DX_THREADS, 1)
 nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict__ own_tiles,
-                 const int2 *__restrict__ tiles, const float4 *__restrict__ ball, int ntiles, int R,
+                 const int2 *__restrict__ tiles, const int *__restrict__ tile_word, int nbodies,
+                 const float4 *__restrict__ ball, int ntiles, int R,
                  const float4 *__restrict__ pa, const float4 *__restrict__ pb, const float4 *__restrict__ pc,
                  const unsigned char *__restrict__ img, const int *__restrict__ key, const float4 *__restrict__ tab,
                  DflConst K, double2 *__restrict__ out, size_t split_stride, int *__restrict__ err)
@@ -195,6 +200,8 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     __shared__ int s_rmin;
     __shared__ volatile int s_fail;
     __shared__ int s_forced;                                   // host-set flag: take the timeout exit
+    __shared__ int s_exp[RC];                                  // exponents of the columns' sums
+    __shared__ unsigned char s_shift[DX_FORM / 32][RC / 2];    // and of the current body's against them, by warp
     const TargetBlock tb = blocks[blockIdx.x >> 2];
     const int sub = blockIdx.x & 3;
     if (sub * DX_M >= tb.count) return;                        // whole CTA past the block's end
@@ -252,6 +259,8 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         const int q = i0 + i;
         return q < own.x ? q : q + nown;
     };
+    // a tile whose levels start from zero: the first of a run, and every second one of a body
+    auto starts = [&](int i, int word) { return (i & (DX_RUN - 1)) == 0 || !t5h_tile_odd(word); };
     auto issue = [&](int i) {
         const int tile = tile_of(i);
         const int2 tl = tiles[tile];
@@ -268,6 +277,15 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         if (n > 1) issue(1);
     }
     int issued = min(n, 2);                                    // copies issued (the last warp's view)
+    // the largest scale of the other bodies' densities (the last warp: it has no pairs to bound)
+    if (q4 == 4 && lane < RC) {
+        const int r = blockIdx.y * RC + lane, mine = t5h_tile_body(tile_word[own.x]);
+        int k = 0;
+        if (r < R)
+            for (int b = 0; b < nbodies; ++b)
+                if (b != mine) k = max(k, key[(size_t)b * R + r]);
+        s_exp[lane] = sigma_exponent(k);
+    }
     // a bound of |G| over the CTA's pairs: the distance to each tile's ball, or node by node where
     // the ball is no use (lengths of the balls: 2 pi times these)
     {
@@ -294,6 +312,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         for (int o = 16; o > 0; o >>= 1) rm = fminf(rm, __shfl_xor_sync(0xffffffffu, rm, o));
         if (lane == 0) atomicMin(&s_rmin, __float_as_int(rm));
     }
+    const int word0 = n > 0 ? tile_word[tile_of(0)] : 0;
     // the sums start at zero
     if (q4 < 4) {
         const uint32_t z[4] = {0u, 0u, 0u, 0u};
@@ -311,7 +330,17 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     const dd scale = {__int_as_float((127 + 8 - e2) << 23), 0.f};
 
     uint32_t bad = 0;                                          // columns that met a NaN
-    // the levels of the last tiles into the sums
+    // the shifts of a body's sums, for this warp's columns
+    auto shifts = [&](int body) {
+        __syncwarp();
+        if (lane < CW) {
+            const int c = (CW * q4 + lane) % RC, r = blockIdx.y * RC + c;
+            const int e = r < R ? sigma_exponent(key[(size_t)body * R + r]) : 0;
+            s_shift[warp][lane] = (unsigned char)min(max(s_exp[c] - e, 0), 62);
+        }
+        __syncwarp();
+    };
+    // the levels of the last tiles (of one body) into the sums
     auto drain = [&]() {
 #pragma unroll
         for (int q = 0; q < CW; q += 4) {
@@ -331,11 +360,13 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                 const float low = fmaf(__uint_as_float(v[5][c]), 0x1p-13f,
                                        fmaf(__uint_as_float(v[4][c]), 0x1p-4f, 32.f * __uint_as_float(v[3][c])));
                 if (low != low) bad |= 1u << (q + c);
-                long long s = (long long)(((unsigned long long)hi[c] << 32) | lo[c]);
-                s += (long long)__float2int_rn(low);
+                long long s = (long long)__float2int_rn(low);
                 s += (long long)__float2int_rn(__uint_as_float(v[2][c])) * (1 << 14);
                 s += (long long)__float2int_rn(__uint_as_float(v[1][c])) * (1 << 23);
                 s += (long long)((unsigned long long)(unsigned)__float2int_rn(__uint_as_float(v[0][c])) << 32);
+                const int d = s_shift[warp][q + c];
+                s = (s + ((1ll << d) >> 1)) >> d;
+                s += (long long)(((unsigned long long)hi[c] << 32) | lo[c]);
                 lo[c] = (uint32_t)s;
                 hi[c] = (uint32_t)((unsigned long long)s >> 32);
             }
@@ -366,7 +397,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                 const int col = CW * q4 + q + c, r = blockIdx.y * RC + col % RC;
                 if (!live || r >= R) continue;
                 const long long s = (long long)(((unsigned long long)hi[c] << 32) | lo[c]);
-                double v = (double)s * f * sigma_pow2(sigma_exponent(key[r]));
+                double v = (double)s * f * sigma_pow2(s_exp[col % RC]);
                 double *o = reinterpret_cast<double *>(out + blockIdx.z * split_stride + (size_t)(tb.start + t) * R + r) + col / RC;
                 if (begun) v += *o;
                 *o = (failed || (bad >> (q + c) & 1)) ? __longlong_as_double(0x7ff8000000000000ll) : v;
@@ -380,7 +411,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     if (q4 == 4) {
         // the last warp: MMAs of each half tile once all 16 have formed it, copies into free stages;
         // every wait gives one answer to all lanes
-        int halves = 0, armed = 0;                             // MMAs of half tiles issued; other halves announced
+        int halves = 0, armed = 0, moves = 0;                  // half tiles' MMAs issued, other halves announced, drains
         auto wait = [&](uint32_t mbar, int phase) { return t5_all(dx_wait<CL>(mbar, (uint32_t)(phase & 1))); };
         auto arm = [&]() {                                     // the other half of a tile comes from the other CTA
             if (lane == 0)
@@ -389,7 +420,10 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                              : "memory");
             ++armed;
         };
+        int next = word0;
         for (int i = 0; i < n && ok; ++i) {
+            const bool first = starts(i, next);
+            if (i + 1 < n) next = tile_word[tile_of(i + 1)];
             if (i > 0) {
                 ok = (CL == 1 || wait(bar0 + 16, i - 1)) && wait(bar0 + 24, i - 1);
                 if (ok && i + 1 < n) {
@@ -411,7 +445,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                         "r"(a0 + rank * (DX_D * DX_AIMG)), "r"(DX_D * DX_AIMG), "r"(dx_peer(bar0 + 32 + 8 * rank, peer))
                         : "memory");
                 // (CL = 1: the warps that formed the half have moved the levels)
-                if (CL == 2 && ok && hh == 0 && i > 0 && !(i & 1)) ok = wait(bar0 + 48, (i >> 1) - 1);
+                if (CL == 2 && ok && hh == 0 && i > 0 && first) ok = wait(bar0 + 48, moves++);
                 if (!ok) break;
                 __syncwarp();
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -419,7 +453,7 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
                     // (unrolled: in a loop the address arithmetic of one MMA took this warp 200 cycles)
                     const uint32_t ad = ((a0 + h * (DX_D * DX_AIMG)) & 0x3FFFF) >> 4 | (1u << 16);
                     const uint32_t bd = (uint32_t)t5_desc(b0 + (uint32_t)((i & 1) * STAGE) + 64 * h);
-                    const uint32_t more = (i & 1) | hh;
+                    const uint32_t more = first ? hh : 1;
 #pragma unroll
                     for (int l = 0; l < DX_D; ++l)
 #pragma unroll
@@ -456,70 +490,82 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
         }
         for (int i = max(0, issued - 2); i < issued; ++i) ok &= t5_wait(bar0 + 8 * (i & 1), (uint32_t)((i >> 1) & 1));
     } else {
-        int next = n > 0 ? tiles[tile_of(0)].y : 0;
-        for (int i = 0; i < n; ++i) {
-            const int cnt = next;
-            if (i + 1 < n) next = tiles[tile_of(i + 1)].y;
-            ok = t5_wait(bar0 + 8 * (i & 1), (uint32_t)((i >> 1) & 1));
-            const float4 *const S = reinterpret_cast<const float4 *>(gb0 + (i & 1) * STAGE + DX_D * IMG);
-#pragma unroll 1
-            for (int h = CL == 2 ? (int)rank : 0; h < (CL == 2 ? (int)rank + 1 : 2); ++h) {
-                uint32_t dig[DX_D][4];
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const int j = 16 * h + 4 * q4 + v;
-                    if (j < cnt) {
-                        const float4 A4 = S[j], B4 = S[DFL_S + j], C4 = S[2 * DFL_S + j];
-                        const DflGeom G = dfl_geom<2>(tx, ty, tz, A4, B4, scale, s_tab, K);
-                        dd gr, gi;
-                        dfl_kernel_value(G, dfl_projection({A4.w, B4.w}, {C4.x, C4.z}, {C4.y, C4.w}, G), K, gr, gi);
-                        float dr[DX_D], di[DX_D];
-                        dx_digits(gr, dr);
-                        dx_digits(gi, di);
-#pragma unroll
-                        for (int l = 0; l < DX_D; ++l) dig[l][v] = dx_pack(dr[l], di[l]);
-                    } else {
-#pragma unroll
-                        for (int l = 0; l < DX_D; ++l) dig[l][v] = 0u;
-                    }
-                }
-                if (i > 0) ok &= dx_wait<CL>(bar0 + 16 + 8 * h, (uint32_t)((i - 1) & 1));   // A's half is free
-                // (CL = 2: both halves every tile, so that no phase of a barrier goes by unseen)
-                if (i > 0 && (CL == 2 || (h == 0 && !(i & 1))))
-                    ok &= dx_wait<CL>(bar0 + 16 + 8 * (h ^ 1), (uint32_t)((i - 1) & 1));
-                if ((CL == 2 || h == 0) && i > 0 && !(i & 1)) {   // the last two tiles are through: their levels
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    __syncwarp();
-                    drain();
-                    if ((i & (DX_RUN - 1)) == 0) emit();
-                    if (CL == 2) {
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar0 + 48) : "memory");
-                    }
-                }
-                const uint32_t at = a0 + h * (DX_D * DX_AIMG) + dx_chunk_off(row, q4);
-#pragma unroll
-                for (int l = 0; l < DX_D; ++l) t5_st4(at + l * DX_AIMG, dig[l][0], dig[l][1], dig[l][2], dig[l][3]);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                if (__any_sync(0xffffffffu, !ok)) s_fail = 1;  // ends the MMAs, and below the loop
-                __syncwarp();
-                if (lane == 0)
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar0 + 32 + 8 * h) : "memory");
-            }
-            if (__any_sync(0xffffffffu, s_fail)) {
-                ok = false;
-                break;
-            }
-        }
-        if (n > 0 && ok) {                                     // the last tile
-            ok &= dx_wait<CL>(bar0 + 16, (uint32_t)((n - 1) & 1));
-            ok &= dx_wait<CL>(bar0 + 24, (uint32_t)((n - 1) & 1));
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        int next = word0, body = t5h_tile_body(word0);         // body: of the levels
+        if (n > 0) shifts(body);
+        auto moved = [&]() {                                   // the levels are free for the next MMAs
+            if (CL == 1) return;                               // (known from the half that this warp forms next)
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            drain();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar0 + 48) : "memory");
+        };
+        // runs of the tiles that the sums hold
+        for (int run0 = 0; run0 < n && ok; run0 += DX_RUN) {
+            const int run1 = min(n, run0 + DX_RUN);
+            for (int i = run0; i < run1; ++i) {
+                const int word = next, cnt = t5h_tile_count(word);
+                const bool first = starts(i, word);
+                if (i + 1 < n) next = tile_word[tile_of(i + 1)];
+                ok = t5_wait(bar0 + 8 * (i & 1), (uint32_t)((i >> 1) & 1));
+                const float4 *const S = reinterpret_cast<const float4 *>(gb0 + (i & 1) * STAGE + DX_D * IMG);
+#pragma unroll 1
+                for (int h = CL == 2 ? (int)rank : 0; h < (CL == 2 ? (int)rank + 1 : 2); ++h) {
+                    uint32_t dig[DX_D][4];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        const int j = 16 * h + 4 * q4 + v;
+                        if (j < cnt) {
+                            const float4 A4 = S[j], B4 = S[DFL_S + j], C4 = S[2 * DFL_S + j];
+                            const DflGeom G = dfl_geom<2>(tx, ty, tz, A4, B4, scale, s_tab, K);
+                            dd gr, gi;
+                            dfl_kernel_value(G, dfl_projection({A4.w, B4.w}, {C4.x, C4.z}, {C4.y, C4.w}, G), K, gr, gi);
+                            float dr[DX_D], di[DX_D];
+                            dx_digits(gr, dr);
+                            dx_digits(gi, di);
+#pragma unroll
+                            for (int l = 0; l < DX_D; ++l) dig[l][v] = dx_pack(dr[l], di[l]);
+                        } else {
+#pragma unroll
+                            for (int l = 0; l < DX_D; ++l) dig[l][v] = 0u;
+                        }
+                    }
+                    if (i > 0) ok &= dx_wait<CL>(bar0 + 16 + 8 * h, (uint32_t)((i - 1) & 1));   // A's half is free
+                    // (CL = 2: both halves every tile, so that no phase of a barrier goes by unseen)
+                    if (i > 0 && (CL == 2 || (h == 0 && first)))
+                        ok &= dx_wait<CL>(bar0 + 16 + 8 * (h ^ 1), (uint32_t)((i - 1) & 1));
+                    if ((CL == 2 || h == 0) && i > run0 && first) {   // the tiles since the last start are through: their levels
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        drain();
+                        moved();
+                    }
+                    if (body != t5h_tile_body(word)) shifts(body = t5h_tile_body(word));
+                    const uint32_t at = a0 + h * (DX_D * DX_AIMG) + dx_chunk_off(row, q4);
+#pragma unroll
+                    for (int l = 0; l < DX_D; ++l) t5_st4(at + l * DX_AIMG, dig[l][0], dig[l][1], dig[l][2], dig[l][3]);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    if (__any_sync(0xffffffffu, !ok)) s_fail = 1;  // ends the MMAs, and below the loop
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar0 + 32 + 8 * h) : "memory");
+                }
+                if (__any_sync(0xffffffffu, s_fail)) {
+                    ok = false;
+                    break;
+                }
+            }
+            if (ok) {                                              // the run's last tiles
+                ok = t5_all(dx_wait<CL>(bar0 + 16, (uint32_t)((run1 - 1) & 1))) &&
+                     t5_all(dx_wait<CL>(bar0 + 24, (uint32_t)((run1 - 1) & 1)));
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                drain();
+                if (run1 < n) {
+                    emit();
+                    moved();
+                }
+            }
         }
+        if (__any_sync(0xffffffffu, !ok)) s_fail = 1;
     }
     failed = __syncthreads_or(!ok);
     if (q4 < 4) emit();
@@ -531,20 +577,47 @@ nbody_dfx_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
     if (failed && tid == 0 && !s_forced) atomicExch(err, 1);   // (a negative flag stays for all CTAs of the launch)
 }
 
-// Digit images of s = 2^8 w sigma c0, scaled below 2^8 per column (key): for every tile and chunk of
+// key[b R + r]: the largest high word of |Re|, |Im| of w_j sigma_{j,r} c0 over the finite values of
+// body b (rounded up; 0: none), so that these are below 2^sigma_exponent(key).  A warp takes eight
+// columns of a tile, a lane one of them and eight sources.
+__global__ void dfx_key_kernel(int ntiles, int R, int per, const int2 *__restrict__ tiles, const int *__restrict__ tile_word,
+                               const double4 *__restrict__ pos, const double2 *__restrict__ sigma, double c0,
+                               int *__restrict__ key)
+{
+    const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (size_t)ntiles * per * 32) return;
+    const int lane = threadIdx.x & 31, tile = (int)(e / 32 / per), col = (int)(e / 32 % per) * 8 + (lane & 7);
+    const int2 tl = tiles[tile];
+    int big = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int s = 8 * (lane >> 3) + q;
+        if (s < tl.y && col < R) {
+            const double2 v = sigma[(size_t)(tl.x + s) * R + col];
+            const double wq = pos[tl.x + s].w * c0;
+            const int hx = __double2hiint(v.x * wq) & 0x7fffffff, hy = __double2hiint(v.y * wq) & 0x7fffffff;
+            big = max(big, max(hx < 0x7ff00000 ? hx : 0, hy < 0x7ff00000 ? hy : 0));
+        }
+    }
+    big = max(big, __shfl_xor_sync(0xffffffffu, big, 8));
+    big = max(big, __shfl_xor_sync(0xffffffffu, big, 16));
+    if (lane < 8 && col < R && big) atomicMax(&key[(size_t)t5h_tile_body(tile_word[tile]) * R + col], big + 1);
+}
+
+// Digit images of s = 2^8 w sigma c0, scaled below 2^8 per body and column (key): for every tile and chunk of
 // RC right-hand sides DX_D images of 2 RC rows of 128 bytes, the values of the 32 sources along a
 // row: column r (real part of y) holds (Re s, -Im s) per source, column RC + r (Im s, Re s).
 // One thread per (tile, column, four sources).
 __global__ void dfx_density_kernel(int ntiles, int R, int rc, int nchunk, const int2 *__restrict__ tiles,
-                                   const double4 *__restrict__ pos, const double2 *__restrict__ sigma, double c0,
-                                   const int *__restrict__ key, unsigned char *__restrict__ img)
+                                   const int *__restrict__ tile_word, const double4 *__restrict__ pos,
+                                   const double2 *__restrict__ sigma, double c0, const int *__restrict__ key, unsigned char *__restrict__ img)
 {
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int ncol = rc * nchunk;
     if (e >= (size_t)ntiles * ncol * 8) return;
     const int col = (int)(e % ncol), g = (int)(e / ncol % 8), tile = (int)(e / ncol / 8);
     const int2 tl = tiles[tile];
-    const double sc = col < R ? c0 * sigma_pow2(8 - sigma_exponent(key[col])) : 0.0;
+    const double sc = col < R ? c0 * sigma_pow2(8 - sigma_exponent(key[(size_t)t5h_tile_body(tile_word[tile]) * R + col])) : 0.0;
     uint32_t re[DX_D][4], im[DX_D][4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
@@ -615,17 +688,21 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
         out = c->nb_part64.ptr;
     }
     if (check_cuda(c, c->t5h_img.ensure((size_t)nt * nchunk * DX_D * dx_img(rc)), "alloc operand images") ||
-        check_cuda(c, c->dlkey.ensure(R), "alloc scales"))
+        check_cuda(c, c->dlkey.ensure((size_t)c->t5h_nbodies * R), "alloc scales"))
         return HZB_ENOMEM;
     if ((st = tc_flag_begin(c, FAULT_TIMEOUT))) return st;
     const double s = c->k / (2.0 * M_PI), c0 = s * s / (4.0 * M_PI);
     c->interbody_calls++;
     const int slot = prof_begin(c, 2);
-    if ((st = sigma_keys(c, R, sigma, c0, 1, c->dlkey.ptr))) return st;
-    const size_t ne = (size_t)nt * rc * nchunk * 8;
+    if (check_cuda(c, cudaMemsetAsync(c->dlkey.ptr, 0, (size_t)c->t5h_nbodies * R * sizeof(int), c->stream), "clear scales"))
+        return HZB_ECUDA;
+    const int per = (R + 7) / 8;
+    const size_t nk = (size_t)nt * per * 32, ne = (size_t)nt * rc * nchunk * 8;
+    dfx_key_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, c->stream>>>(nt, R, per, c->t5h_tiles.ptr, c->t5h_body.ptr,
+                                                                      c->pos64.ptr, sigma, c0, c->dlkey.ptr);
     dfx_density_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, c->stream>>>(nt, R, rc, nchunk, c->t5h_tiles.ptr,
-                                                                          c->pos64.ptr, sigma, c0, c->dlkey.ptr,
-                                                                          c->t5h_img.ptr);
+                                                                          c->t5h_body.ptr, c->pos64.ptr, sigma, c0,
+                                                                          c->dlkey.ptr, c->t5h_img.ptr);
     const dim3 grid((unsigned)c->n_tblocks * 4, nchunk, nsplit);
     const float4 *ball = reinterpret_cast<const float4 *>(c->t5h_src.ptr + (size_t)nt * 6 * DFL_S);
     cudaError_t e = cudaSuccess;
@@ -645,7 +722,8 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
         cfg.attrs = at;
         cfg.numAttrs = cl > 1 ? 1 : 0;
         e = cudaLaunchKernelEx(&cfg, kern, (const TargetBlock *)c->tblocks.ptr, (const int2 *)(c->t5h_tiles.ptr + nt),
-                               (const int2 *)c->t5h_tiles.ptr, ball, nt, R, (const float4 *)c->dla.ptr,
+                               (const int2 *)c->t5h_tiles.ptr, (const int *)c->t5h_body.ptr, c->t5h_nbodies, ball, nt, R,
+                               (const float4 *)c->dla.ptr,
                                (const float4 *)c->dlb.ptr, (const float4 *)c->dlc.ptr,
                                (const unsigned char *)c->t5h_img.ptr, (const int *)c->dlkey.ptr,
                                (const float4 *)c->dfltab.ptr, dfl_constants(c), out, n, c->kerr.ptr);
@@ -656,7 +734,7 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
     else if (rc == 16) launch(nbody_dfx_kernel<16, 1>);
     else if (cl == 1) launch(nbody_dfx_kernel<32, 1>);
     else launch(nbody_dfx_kernel<32, 2>);
-    c->launches += 2;
+    c->launches += 3;
     if (check_cuda(c, e, "nbody_dfx_kernel")) return HZB_ECUDA;
     if (nsplit > 1) {
         if ((st = dfl_split_reduce(c, n, nsplit, out, y))) return st;

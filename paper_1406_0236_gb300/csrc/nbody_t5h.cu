@@ -516,11 +516,17 @@ hzb_status ensure_t5h(hzb_ctx *c)
         return HZB_ECUDA;
     // one buffer: the tiles, the blocks' own tiles, the end of each tile's body, the range
     std::vector<int2> tiles, own(tb.size()), end;
+    std::vector<int> word;
+    int nbodies = 0;
     for (size_t b = 0; b < tb.size(); ++b) {
         if (b == 0 || tb[b].excl_lo != tb[b - 1].excl_lo) {    // a new body: its nodes are one range
             const int first = (int)tiles.size();
-            for (int s = tb[b].excl_lo; s < tb[b].excl_hi; s += TH_S)
-                tiles.push_back(make_int2(s, std::min(TH_S, tb[b].excl_hi - s)));
+            for (int s = tb[b].excl_lo; s < tb[b].excl_hi; s += TH_S) {
+                const int count = std::min(TH_S, tb[b].excl_hi - s);
+                word.push_back(t5h_tile_word(nbodies, ((int)tiles.size() - first) & 1, count));
+                tiles.push_back(make_int2(s, count));
+            }
+            ++nbodies;
             end.resize(tiles.size(), make_int2((int)tiles.size(), 0));
             own[b] = make_int2(first, (int)tiles.size());
         } else {
@@ -532,13 +538,16 @@ hzb_status ensure_t5h(hzb_ctx *c)
     tiles.insert(tiles.end(), end.begin(), end.end());
     tiles.push_back(make_int2(0x7f7fffff, 0));
     if (check_cuda(c, c->t5h_tiles.ensure(tiles.size()), "alloc tiles") ||
+        check_cuda(c, c->t5h_body.ensure(nt), "alloc tiles") ||
         check_cuda(c, c->t5h_src.ensure((size_t)nt * (TH_SRC + 4)), "alloc tiles"))
         return HZB_ENOMEM;
     float4 *ball = reinterpret_cast<float4 *>(c->t5h_src.ptr + (size_t)nt * TH_SRC);
     int2 *const end_dev = c->t5h_tiles.ptr + nt + own.size();
     int *const range_dev = reinterpret_cast<int *>(end_dev + nt);
     if (check_cuda(c, cudaMemcpyAsync(c->t5h_tiles.ptr, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                                      c->stream), "copy tiles"))
+                                      c->stream), "copy tiles") ||
+        check_cuda(c, cudaMemcpyAsync(c->t5h_body.ptr, word.data(), nt * sizeof(int), cudaMemcpyHostToDevice, c->stream),
+                   "copy tiles"))
         return HZB_ECUDA;
     t5h_source_kernel<<<(nt + 7) / 8, 256, 0, c->stream>>>(
         nt, c->t5h_tiles.ptr, c->pos64.ptr, c->nrm64.ptr, make_double3(c->center[0], c->center[1], c->center[2]), c->k,
@@ -552,6 +561,7 @@ hzb_status ensure_t5h(hzb_ctx *c)
     const double g = range[0], diam = range[1];
     // |G'| <= u (1 + (k / |eta|) (1 + u)), u = 1 / (k r); the smallest is about u at the diameter
     c->t5h_ntiles = nt;
+    c->t5h_nbodies = nbodies;
     c->t5h_ctas = 0;
     for (const TargetBlock &t : tb) c->t5h_ctas += (t.count + TH_M - 1) / TH_M;
     c->t5h_most = 1;                                           // tiles of the other bodies, at most
