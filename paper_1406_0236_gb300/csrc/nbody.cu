@@ -535,9 +535,10 @@ int fp32_engine(const hzb_ctx *c, int R)
     if (c->nbody_engine >= 5 && c->nbody_engine <= 7) return c->nbody_engine - 3;
     if (c->nbody_engine >= 0) return 0;
     if (c->tune32_tc >= 0 && c->tune32_tc_R == R) return c->tune32_tc;
+    // (outside FP16's range the TF32 form from R = 16 on, below the CUDA cores: interbody32, which looks
+    // at the geometry before it chooses, so that no earlier call matters)
     const double work = (double)c->N * (double)c->N * R;
-    if (R >= 16 && c->t5h_state < 0) return 2;         // TF32 form
-    return c->t5h_state >= 0 && ((R >= 5 && work >= 6e8) || (R >= 9 && work >= 3e8)) ? 2 : 0;
+    return ((R >= 5 && work >= 6e8) || (R >= 9 && work >= 3e8)) && (R >= 16 || c->t5h_state >= 0) ? 2 : 0;
 }
 
 // Kernel of the CUDA-core engine: 0 scalar, 1 packed pairs, 2 pair-symmetric packed (up to four
