@@ -25,7 +25,10 @@
  *   - Host pointers are read or written before the call returns; the library
  *     keeps no reference to them.  Device pointers (flag *_on_device = 1) must be
  *     device memory of the context's GPU, and are accessed in stream order on the
- *     context's stream.
+ *     context's stream: operators on device data return with the work queued (after a
+ *     first call of the same kind has allocated, the stream may be under capture), but
+ *     for FP32 sums of 16 and more right-hand sides on the tensor cores and sums on an
+ *     explicit tensor-core engine, which wait for it to read their error flag.
  *   - Every call returns an hzb_status; on failure hzb_last_error() describes it.
  *   - The context owns all device memory it allocates; hzb_destroy frees it.
  *   - A context is used by one host thread at a time.
@@ -61,7 +64,9 @@ typedef enum {
  * tensor memory, writes NaN to its outputs and sets a flag that the call reports as
  * HZB_ETIMEOUT (the flag is then cleared, so the context stays usable); inside a solve
  * the flag is read once, at the end of the solve (no synchronisation per launch), unless
- * the NaN outputs stopped GMRES first (HZB_ENAN).  Geometry is
+ * the NaN outputs stopped GMRES first (HZB_ENAN).  An operator call that returns with its
+ * work queued leaves the flag to the next call on the context that waits: an operator on
+ * host data, an FP32 tensor-core sum that waits, or a solve.  Geometry is
  * checked when the nodes are generated: intersecting bodies and non-finite or
  * degenerate nodes give HZB_EINVAL.
  *

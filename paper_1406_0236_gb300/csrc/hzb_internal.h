@@ -324,7 +324,7 @@ hzb_status interbody_t5h(hzb_ctx *c, int R, const double2 *sigma, double2 *y);
 hzb_status tc_flag_begin(hzb_ctx *c, int fault);
 hzb_status tc_flag_launched(hzb_ctx *c);
 hzb_status tc_flag_report(hzb_ctx *c, const char *kernel);
-hzb_status tc_flag_end(hzb_ctx *c, const char *kernel);
+hzb_status tc_flag_end(hzb_ctx *c, const char *kernel, bool wait);
 hzb_status sigma_keys(hzb_ctx *c, int R, const double2 *sigma, double c0, int weighted, int *key);   // nbody_dfl.cu
 bool sym_scaled(const hzb_ctx *c);              // nbody_sym.cu: k and eta leave the scaled pair kernels in range
 hzb_status ensure_sym32(hzb_ctx *c);            // nbody_sym.cu: symn

@@ -741,7 +741,7 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
         c->launches++;
     }
     prof_end(c, slot);
-    return tc_flag_end(c, "nbody_dfx_kernel");
+    return tc_flag_end(c, "nbody_dfx_kernel", false);      // queued, as the other double-float sums are
 }
 
 }  // namespace hzb

@@ -559,11 +559,13 @@ hzb_status tc_flag_launched(hzb_ctx *c)
     return check_cuda(c, cudaMemsetAsync(c->kerr.ptr, 0x01, sizeof(int), c->stream), "injected timeout");
 }
 
-// and after it: a wait that ran out left NaN outputs (a solve reads the flag once, at its end)
-hzb_status tc_flag_end(hzb_ctx *c, const char *kernel)
+// and after it: a wait that ran out left NaN outputs (a solve reads the flag once, at its end).  wait:
+// for the stream, to report it here; without, the call stays queued (and a caller's stream capture
+// takes it), and the next call that waits reports it.
+hzb_status tc_flag_end(hzb_ctx *c, const char *kernel, bool wait)
 {
     hzb_status st = tc_flag_launched(c);
-    if (st || c->capturing || c->in_solve) return st;
+    if (st || !wait || c->capturing || c->in_solve) return st;
     return tc_flag_report(c, kernel);
 }
 
@@ -650,7 +652,7 @@ hzb_status interbody_tc5(hzb_ctx *c, int R, const double2 *sigma, double2 *y, in
     cudaError_t e = cudaGetLastError();
     prof_end(c, slot);
     if (check_cuda(c, e, "nbody_tc5_kernel")) return HZB_ECUDA;
-    return tc_flag_end(c, "nbody_tc5_kernel");
+    return tc_flag_end(c, "nbody_tc5_kernel", true);
 }
 
 }  // namespace hzb
