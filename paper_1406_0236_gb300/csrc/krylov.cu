@@ -44,11 +44,19 @@ static int red_blocks(long long N, int R, int nv)
     const long long most = std::max(1, RED_BLOCKS / (nv * q.chunks));
     return (int)std::max<long long>(1, std::min<long long>({(N + q.slots - 1) / q.slots, most, 152}));
 }
+// blocks of the update with the norm: a block per SM where the vectors stay in L2, four where they do
+// not (258,560 unknowns, R = 16, six vectors: 369 us with 152 blocks, 216 with 608; the update, norm and rotation of its own 244)
+static int step_blocks(long long N, int R)
+{
+    const RedShape q = red_shape(R);
+    const long long rows = (N + q.slots - 1) / q.slots;
+    return (int)std::max<long long>(red_blocks(N, R, 1), std::min<long long>(RED_BLOCKS / q.chunks, rows / 16));
+}
 // values of partial sums for up to nv vectors (the products with nv = 1 use the most blocks)
 static size_t red_partials(long long N, int R, int nv)
 {
     const RedShape q = red_shape(R);
-    size_t most = 0;
+    size_t most = (size_t)q.chunks * q.cols * step_blocks(N, R);
     for (int v = 1; v <= nv; ++v) most = std::max(most, (size_t)v * q.chunks * q.cols * red_blocks(N, R, v));
     return most;
 }
@@ -246,7 +254,6 @@ caxpy_kernel(long long N, int R, int cols, int slots, int nv, const double2 *__r
         for (long long i = (long long)blockIdx.x * slots + slot; i < N; i += step) {
             const long long e = i * R + r;
             double2 acc = w[e];
-#pragma unroll 4
             for (int v = 0; v < nv; ++v) {
                 const double2 hv = h[(size_t)v * R + r];
                 cfma(acc, make_double2(-hv.x, -hv.y), V[v * vstride + e]);
@@ -478,8 +485,8 @@ hzb_status gmres_solve(hzb_ctx *c, int R, const double2 *b, double2 *x, int x_is
     // partial sums sized for the largest step, so that a captured step never reallocates
     if ((st = ensure_red(c, R, m + 1))) return st;
     const RedShape rq = red_shape(R);
-    const dim3 gaxpy((unsigned)std::max<long long>(1, std::min<long long>((N + rq.slots - 1) / rq.slots, 152 * 8)), 1, rq.chunks);
-    const dim3 gstep(red_blocks(N, R, 1), 1, rq.chunks);
+    const dim3 gaxpy((unsigned)std::max<long long>(1, (N + rq.slots - 1) / rq.slots), 1, rq.chunks);
+    const dim3 gstep(step_blocks(N, R), 1, rq.chunks);
     // CUDA graphs need a capturable (non-legacy) stream; auto = small problems only
     bool graphs = c->use_graphs > 0 || (c->use_graphs < 0 && (long long)NR <= 4000000);
     if (c->stream == nullptr) graphs = false;
