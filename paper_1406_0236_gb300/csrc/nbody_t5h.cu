@@ -15,8 +15,11 @@
 //     leading bits) and the rounded rest, and stores the four parts as columns of its own
 //     row of tensor memory (tcgen05.st): the A operands of the MMAs, which shared memory
 //     never sees;
-//   * one thread issues 12 MMAs (M = 128, N = 2 RC, K = 16; high x high, high x low, low x
-//     high for Re G' x [Re s | Im s] and -Im G' x [Im s | -Re s]) and commits them;
+//   * one thread issues 12 MMAs (M = 128, N = 2 RC, K = 16; high x low, low x high and last high x
+//     high, for Re G' x [Re s | Im s] and -Im G' x [Im s | -Re s]) and commits them.  The accumulator
+//     is truncated at every MMA: with the small products first four of the twelve are at its full
+//     size.  Error at 8,200 unknowns, k = 2, R = 12: 6.4e-7 with the three products of a factor in
+//     turn, 5.0e-7 now, 5.3e-7 in FP32 multiply-adds;
 //   * the warps read the accumulator (started from zero in every tile: chained tensor-core
 //     sums are not rounded to nearest and drift) and add it, times the tile's scale, to FP32
 //     sums in registers.
@@ -281,15 +284,15 @@ nbody_t5h_kernel(const TargetBlock *__restrict__ blocks, const int2 *__restrict_
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t desc = t5_desc(base + (uint32_t)((i & 1) * STAGE));
 #pragma unroll
-            for (int z = 0; z < 2; ++z)                        // Re G' x B1, -Im G' x B2
+            for (int term = 0; term < 3; ++term)               // high x low, low x high, then high x high
 #pragma unroll
-                for (int ks = 0; ks < 2; ++ks) {
-                    const uint32_t ah = tmem + TH_A + 2 * z * TH_ATILE + 8 * ks, al = ah + TH_ATILE;
-                    const uint64_t bh = desc + ((z * (BYTES / 2) + 32 * ks) >> 4), bl = bh + (64 >> 4);
-                    th_mma(tmem + TH_D, ah, bh, th_idesc(2 * RC), (z | ks) ? 1u : 0u);
-                    th_mma(tmem + TH_D, ah, bl, th_idesc(2 * RC), 1u);
-                    th_mma(tmem + TH_D, al, bh, th_idesc(2 * RC), 1u);
-                }
+                for (int z = 0; z < 2; ++z)                    // Re G' x B1, -Im G' x B2
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks) {
+                        const uint32_t a = tmem + TH_A + (2 * z + (term == 1 ? 1 : 0)) * TH_ATILE + 8 * ks;
+                        const uint64_t b = desc + ((z * (BYTES / 2) + 32 * ks + (term == 0 ? 64 : 0)) >> 4);
+                        th_mma(tmem + TH_D, a, b, th_idesc(2 * RC), (term | z | ks) ? 1u : 0u);
+                    }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 16)
                          : "memory");
         }
