@@ -1055,6 +1055,7 @@ hzb_status build_reduced(hzb_ctx *c)
         c->launches++;
         r->n_tblocks = (int)blocks.size();
         r->nodes_ready = true;
+        st = ensure_sym32(r);
         for (size_t s = 0; s < c->shapes.size() && !st; ++s) {
             ShapeDev &sd = *c->shapes[s];
             if (check_cuda(c, sd.red_offs.ensure(offs[s].size()), "alloc")) { st = HZB_ENOMEM; break; }
