@@ -251,6 +251,7 @@ static hzb_status add_body_impl(hzb_ctx *c, const hzb_shape *shape, const std::v
     ShapeDev &sd = *c->shapes[sidx];
     long long n = (long long)sd.geom.NG * sd.geom.NF;
     if (c->N + n > (long long)0x7fffffff) return fail(c, HZB_EINVAL, "too many nodes");
+    drop_nodes(c);
     BodyRec b;
     b.shape = sidx;
     std::memcpy(b.c, cen, sizeof(b.c));

@@ -295,6 +295,7 @@ hzb_status check_cuda(hzb_ctx *c, cudaError_t e, const char *what);
 
 // setup.cu
 hzb_status make_nodes(hzb_ctx *c);
+void drop_nodes(hzb_ctx *c);
 hzb_status build_shape_matrices(hzb_ctx *c, ShapeDev &s);
 
 // nbody.cu: y = B sigma; sigma, y device N x R complex FP64 (FP32 path converts internally)

@@ -180,6 +180,16 @@ __global__ void twiddle_kernel(int NF, double2 *__restrict__ tw)
     tw[m] = make_double2(c, s);
 }
 
+// A body added after the nodes were generated (by a sum or a query before the build): they and what
+// later calls derived from them are made again.
+void drop_nodes(hzb_ctx *c)
+{
+    if (!c->nodes_ready) return;
+    c->nodes_ready = c->sym32_ready = c->df_ready = c->dfltab_ready = false;
+    c->n_blockpairs = 0;
+    c->t5h_state = 0;
+}
+
 hzb_status make_nodes(hzb_ctx *c)
 {
     if (c->nodes_ready) return HZB_OK;
