@@ -69,9 +69,10 @@ static const int DFL_NT = 256;         // threads (targets) per CTA of the one-d
 // is that of the two-sums it replaces (5.7e-14 against 6e-14), at 216 it would be twice it
 static const int DFL_GRID_MIN = 4096;
 
-// A sum over a tile: integers in units of the tile's finest grid, and the remainders.
+// A sum over a tile: integers in units of the tile's finest grid (modulo 2^32: the mantissas of m in
+// them pass that many times), and the remainders.
 struct DflAcc {
-    int v;
+    unsigned v;
     float l;
 };
 
@@ -81,7 +82,7 @@ struct DflAcc {
 // its mantissas enter the integer sums times mult = ulp(m) / ulp(fine).
 struct DflGrid {
     float m;
-    int mult;
+    unsigned mult;
 };
 
 __device__ __forceinline__ float dfl_fine(float rmin, float kbound, float wmax)
@@ -94,7 +95,7 @@ __device__ __forceinline__ DflGrid dfl_grid(float g, float fine)
 {
     const int fb = __float_as_int(fine);
     const int mb = max((__float_as_int(g) & 0x7f800000) + 0x01400000, fb);
-    return {__int_as_float(mb), 1 << ((mb - fb) >> 23)};
+    return {__int_as_float(mb), 1u << ((mb - fb) >> 23)};
 }
 
 // acc += a b + c d on the grid of one pair.  v collects the mantissas of s with those of m in
@@ -107,7 +108,7 @@ __device__ __forceinline__ void dfl_mac2(DflAcc &acc, dd a, dd b, dd c, dd d, Df
     x = fmaf(a.l, b.h, x);
     x = fmaf(c.h, d.l, x);
     x = fmaf(c.l, d.h, x);
-    acc.v = __float_as_int(s2) * g.mult + acc.v;
+    acc.v = __float_as_uint(s2) * g.mult + acc.v;
     acc.l += (l1 + l2) + x;
 }
 
@@ -115,19 +116,19 @@ __device__ __forceinline__ void dfl_mac2(DflAcc &acc, dd a, dd b, dd c, dd d, Df
 __device__ __forceinline__ void dfl_carry(DflAcc &acc, float fine)
 {
     const float s = acc.l + fine;
-    acc.v += __float_as_int(s) - __float_as_int(fine);
+    acc.v += __float_as_uint(s) - __float_as_uint(fine);
     acc.l -= s - fine;
 }
 
 // run += sc acc, the tile's sum (v - corr below 2^31, sc a power of two), normalised; acc = 0
-__device__ __forceinline__ dd dfl_flush(dd run, DflAcc &acc, int corr, float ulp, float sc)
+__device__ __forceinline__ dd dfl_flush(dd run, DflAcc &acc, unsigned corr, float ulp, float sc)
 {
     const float us = ulp * sc;
-    const int v = acc.v - corr;
+    const int v = (int)(acc.v - corr);
     const dd a = two_sum(run.h, __int2float_rn(v & ~255) * us);
     const dd b = two_sum(a.h, __int2float_rn(v & 255) * us);
     const dd r = norm({b.h, run.l + fmaf(acc.l, sc, a.l + b.l)});
-    acc = {0, 0.f};
+    acc = {0u, 0.f};
     return r;
 }
 
@@ -453,7 +454,7 @@ nbody_dfl_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chunk
     dd zr[RC], zi[RC];                                     // else the running sums
 #pragma unroll
     for (int c = 0; c < RC; ++c) {
-        ar[c] = ai[c] = {0, 0.f};
+        ar[c] = ai[c] = {0u, 0.f};
         zr[c] = zi[c] = {0.f, 0.f};
         if (GRID) s_run[c * DFL_NT + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -504,7 +505,7 @@ nbody_dfl_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chunk
         __syncthreads();
         const float fine =
             GRID ? dfl_fine(fmaxf(dfl_rmin(tx, ty, tz, s_ball, s_a, s_b, cnt), 0.f), K.kbound, s_wmax) : 0.f;
-        int corr = 0;                                      // the mantissas of the grids in the sums
+        unsigned corr = 0;                                 // the mantissas of the grids in the sums
         for (int jj = 0; jj < cnt; ++jj) {
             const float4 A4 = s_a[jj], B4 = s_b[jj], C4 = s_c[jj];
             const dd w = GRID ? dd{s_w[jj].x, s_w[jj].y} : dd{0.f, 0.f};
@@ -513,7 +514,7 @@ nbody_dfl_kernel(const TargetBlock *__restrict__ blocks, int N, int R, int chunk
             dfl_kernel_value(G, dfl_projection({A4.w, B4.w}, {C4.x, C4.z}, {C4.y, C4.w}, G), K, gr, gi);
             if (GRID) {
                 const DflGrid grid = dfl_grid(fmaxf(fabsf(gr.h), fabsf(gi.h)), fine);
-                corr += __float_as_int(grid.m) * grid.mult;
+                corr += __float_as_uint(grid.m) * grid.mult;
 #pragma unroll
                 for (int c = 0; c < RC; ++c) {
                     const float4 S = s_sig[jj * RC + c];
