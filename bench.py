@@ -50,10 +50,12 @@ FLOPS_PER_PAIR = 36
 # gives a density error <= 1e-7 (3.9e-8, measured on GB300); the reference arm's oracle
 # solve is its apply time times this count (a full oracle GMRES would take hours)
 ORACLE_ITERS = 16
-# DRAM bytes (read + write) per launch on this workload from one ncu capture of each kernel; None for a kernel without a capture of its current version.
-DRAM_BYTES_NCU = {"nbody32_sym_kernel": 15.94e6, "nbody_dfl_sym_kernel": 21.87e6}
+# DRAM bytes (read + write) per launch on this workload, from an ncu capture of each kernel in its
+# present form (profiles/); None for a kernel without one
+DRAM_BYTES_NCU = {"nbody32_sym_kernel": 15.92e6, "nbody_dfl_sym_kernel": 22.08e6}
 # FP32-pipe (FMA) thread operations per unordered node pair of the lean double-float kernel,
-# counted by ncu (thread instructions per unordered pair on the four-body case)
+# counted by ncu (profiles/: thread instructions of that pipe per unordered
+# pair on the four-body case)
 DFL_OPS_PER_UNORDERED_PAIR = 363
 
 

@@ -257,7 +257,9 @@ class Solver:
         self._check(lib().hzb_set_interbody_engine(self._h, int(engine)))
 
     def set_fp64_interbody_engine(self, engine: int):
-        """FP64/double-float inter-body engine: 0 one-directional, 1 pair-symmetric, -1 auto (1 for R <= 4)."""
+        """FP64/double-float inter-body engine: 0 one-directional, 1 pair-symmetric, 2 as -1 with the
+        normalised double-float kernels, -1 auto (FP64: 1 for R <= 4; double-float: pair-symmetric for
+        R <= 2 and short sums, else tensor cores where they apply, else one-directional)."""
         self._check(lib().hzb_set_fp64_interbody_engine(self._h, int(engine)))
 
     def set_options(self, **kw):
@@ -376,7 +378,8 @@ class Solver:
         self._check(lib().hzb_measure_peak(self._h, self.PEAK_KINDS.index(kind), ctypes.byref(v)))
         return v.value
 
-    FP32_KERNELS = ("nbody32_kernel", "nbody32x2_kernel", "nbody32_sym_kernel", "nbody_tc_kernel", "nbody_tc5_kernel")
+    # (tcgen05: nbody_tc5_kernel outside FP16's range and on the explicit engines 6 and 7)
+    FP32_KERNELS = ("nbody32_kernel", "nbody32x2_kernel", "nbody32_sym_kernel", "nbody_tc_kernel", "nbody_t5h_kernel")
 
     def tuned_config(self, R: int = 1) -> dict:
         """The inter-body kernels this solver launches for R right-hand sides."""

@@ -204,8 +204,9 @@ struct hzb_ctx {
     int t5h_nbodies = 0;                       // bodies with nodes
     hzb::DevBuf<float> t5h_src;
     hzb::DevBuf<unsigned char> t5h_img;
-    int nbody64_engine = -1;                   // FP64/double-float sums: -1 auto (pair-symmetric for R <= 4;
-                                               // double-float: nbody_dfx.cu where it applies),
+    int nbody64_engine = -1;                   // FP64/double-float sums: -1 auto (FP64 pair-symmetric for R <= 4;
+                                               // double-float: nbody_dfx.cu where it applies, else as
+                                               // dfl_symmetric says),
                                                // 0 one-directional, 1 pair-symmetric (double-float: lean forms),
                                                // 2 as -1 with the normalised double-float kernels
     hzb::DevBuf<int> kerr;                     // device error flag of kernels with bounded waits
@@ -215,8 +216,8 @@ struct hzb_ctx {
     int tune64_tpt = 0, tune64_split = 0;      // 0: default
     int tune32_tpt = 0, tune32_split = 0;
     int tune32_R = 0;                          // R the FP32 variant was tuned for
-    int tune32_x2 = -1;                        // FP32 CUDA-core kernel: -1 default (packed), 0 scalar, 1 packed,
-                                               // 2 pair-symmetric packed
+    int tune32_x2 = -1;                        // FP32 CUDA-core kernel: -1 default (pair-symmetric up to R = 4,
+                                               // else packed), 0 scalar, 1 packed, 2 pair-symmetric packed
     int tune_limit_blocks = 0;                 // autotuner: time only the first blocks (0 = all)
     // double-float inter-body kernel: split positions/normals, cos/sin table, launch shape
     hzb::DevBuf<float4> dfa, dfb, dfc, dftab;
@@ -231,12 +232,13 @@ struct hzb_ctx {
     // GMRES execution: steps between host checks (0 = auto) and CUDA graphs (-1 auto, 0 off, 1 on)
     int check_every = 0;
     int use_graphs = -1;
-    int modal_engine = -1;                     // FP32 modal GEMM: -1 auto, 0 CUDA cores, 1 tensor cores
+    int modal_engine = -1;                     // FP32 modal GEMM: -1 auto, 0 CUDA cores, 1 mma.sync, 2 tcgen05
     int nbody_engine = -1;                     // FP32 inter-body sum: -1 auto, 0 CUDA cores, 1 tensor cores,
                                                // 2 CUDA cores scalar kernel, 3 CUDA cores packed-pair kernel,
                                                // 4 CUDA cores pair-symmetric packed kernel,
-                                               // 5 tensor cores with tcgen05 (TMEM accumulators),
-                                               // 6 tcgen05, warp-specialised pipeline
+                                               // 5 tensor cores with tcgen05 (FP16 form, TF32 outside its
+                                               // range), 6 tcgen05 TF32, warp-specialised pipeline,
+                                               // 7 tcgen05 TF32, single-term products
     int tunetc_split = 0;                      // tensor-core inter-body source split (0: default)
     int tune32_tc = -1, tune32_tc_R = 0;       // autotuner's engine choice for R = tune32_tc_R (-1: none)
     std::vector<cudaGraphExec_t> gexec;        // captured Arnoldi step j

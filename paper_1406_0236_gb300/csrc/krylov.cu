@@ -189,11 +189,9 @@ __global__ void cycle_start_kernel(int R, int m, GmresState s, double tol, int f
     s.inv[r] = (act && beta > 0.0) ? 1.0 / beta : 0.0;
 }
 
-// Arnoldi column j: h = h1 + h2 (CGS2), h_{j+1,j} = ||w||; apply the previous
-// rotations, form the one that zeroes h_{j+1,j}, update g and the residual.
-// column j of the Hessenberg matrix for right-hand side r from h1 + h2 and |w|^2: the rotations so
-// far, the new one, the residual estimate.  The column runs through registers; h1, h2, cs and sn
-// up to j come from earlier launches.
+// Arnoldi column j for right-hand side r: h = h1 + h2 (CGS2), h_{j+1,j} = |w|; the previous
+// rotations applied, the one that zeroes h_{j+1,j} formed, g and the residual estimate updated.  The
+// column runs through registers; h1, h2, cs and sn up to j come from earlier launches.
 __device__ void givens_column(int R, int m, int j, const GmresState &s, double tol, int r, double nrm2)
 {
     if (!s.active[r]) {
@@ -558,7 +556,7 @@ hzb_status gmres_solve(hzb_ctx *c, int R, const double2 *b, double2 *x, int x_is
             return HZB_OK;
         };
         // Steps run in chunks of `every` without host synchronisation: a right-hand
-        // side that converges inside a chunk is frozen by givens_kernel (its next basis
+        // side that converges inside a chunk is frozen by givens_column (its next basis
         // vectors are zero and its jdone stays), so the extra steps change nothing.
         // automatic: chunks of 4 where an apply is cheap next to a host round trip; every
         // step where an apply costs milliseconds (a converged chunk's extra steps would

@@ -588,7 +588,7 @@ hzb_status tc_flag_report(hzb_ctx *c, const char *kernel)
 
 // mode: T5_SPLIT3 (three-term TF32 split, FP32-level products), T5_WS (the same, warp-
 // specialised), T5_SINGLE (TF32 products alone: about 3e-4 relative error in the sum, 1.4x
-// faster; for inner solves whose refinement tolerates it)
+// faster than the split; the FP16 form of nbody_t5h.cu is faster than either and as exact as the split)
 hzb_status interbody_tc5(hzb_ctx *c, int R, const double2 *sigma, double2 *y, int nsplit, int mode)
 {
     const bool ws = mode == T5_WS;

@@ -51,6 +51,9 @@ __global__ void __launch_bounds__(PK_THREADS) peak_ffma2_kernel(int iters, float
     if (s == never) out[0] = s;
 }
 
+// (1.67 operations per clock and SM, whatever the number of chains, warps or the kind of operation; the
+// FP64 pair kernel, whose FP64 instructions alternate with others, sustains 1.8 and so reads above
+// this "peak" in operations: the pipe's own rate is two)
 __global__ void __launch_bounds__(PK_THREADS) peak_dfma_kernel(int iters, double a, double b, double never, double *out)
 {
     double v[PK_CHAINS];
