@@ -1278,6 +1278,8 @@ static void sync_settings(hzb_ctx *c, hzb_ctx *r)
     r->nbody64_engine = c->nbody64_engine;
     r->check_every = c->check_every;
     r->use_graphs = c->use_graphs;
+    r->fault = c->fault & FAULT_TIMEOUT;                   // (its sums' kernels; fires once in all)
+    r->fault_spent |= c->fault_spent;
 }
 
 hzb_status solve_reduced(hzb_ctx *c, int R, const double2 *v, const double2 *x0, hzb_stats *stats)
@@ -1307,6 +1309,7 @@ hzb_status solve_reduced(hzb_ctx *c, int R, const double2 *v, const double2 *x0,
     if (check_cuda(c, r->s_r.ensure(RR), "alloc")) return HZB_ENOMEM;
     // FP64 path: FP64; mixed path: double-float (about 1e-13 per term, far below its tolerance)
     st = c->opt.precision == HZB_PREC_FP64 ? interbody64(r, R, sig_t, r->s_r.ptr) : interbody_df(r, R, sig_t, r->s_r.ptr);
+    c->fault_spent |= r->fault_spent;
     if (st) return fail(c, st, r->err);
     if (df) {
         if (check_cuda(c, c->ysplit.ensure(std::max(RR, NR)), "alloc")) return HZB_ENOMEM;
@@ -1329,6 +1332,7 @@ hzb_status solve_reduced(hzb_ctx *c, int R, const double2 *v, const double2 *x0,
     c->sol_R = R;
     cudaEventRecord(c->ev1, c->stream);
     if (check_cuda(c, cudaEventSynchronize(c->ev1), "reduced solve")) return HZB_ECUDA;
+    if ((st = tc_flag_report(r, "the recovery sum"))) return fail(c, st, r->err);
     float ms = 0.f;
     cudaEventElapsedTime(&ms, c->ev0, c->ev1);
     c->launches += r->launches - rl0;
@@ -1482,10 +1486,12 @@ extern "C" hzb_status hzb_apply_reduced(hzb_ctx *c, int R, const double *sig, do
     const long long rl0 = r->launches;
     hzb_status st = apply_op(r, R, c->rb.ptr, c->rx.ptr, precision);
     c->launches += r->launches - rl0;
+    c->fault_spent |= r->fault_spent;
     if (st) return fail(c, st, r->err);
     if (check_cuda(c, cudaMemcpyAsync(out, c->rx.ptr, RR * sizeof(double2), cudaMemcpyDeviceToHost, c->stream), "out") ||
         check_cuda(c, cudaStreamSynchronize(c->stream), "apply reduced"))
         return HZB_ECUDA;
+    if ((st = tc_flag_report(r, "the reduced operator"))) return fail(c, st, r->err);
     return HZB_OK;
 }
 

@@ -55,3 +55,25 @@ def test_timeout_of_a_queued_sum(monkeypatch):
     assert e.value.status == -6
     ref = s.interbody(host, precision=0)
     assert np.abs(s.interbody(host, precision=2) - ref).max() < 1e-12 * np.abs(ref).max()
+
+
+def test_timeout_in_the_reduced_system(monkeypatch):
+    """The accelerated scheme's operator (host data) reports a wait that ran out in its own sums."""
+    require_gpu()
+    from paper_1406_0236_gb300 import HzbError
+    from tests._common import gpu_solver
+    monkeypatch.setenv("HZB_FAULT", "timeout")
+    wl = W.separated_spheroids(spacing=4.0, n_panels=6, gl_order=8, n_modes=9)
+    n, k = wl.bodies[0].shape.n_nodes, 257
+    g = np.random.default_rng(3)
+    J = np.sort(g.choice(n, k, replace=False))
+    T = (g.standard_normal((k, n)) + 1j * g.standard_normal((k, n))) / np.sqrt(n)
+    T[:, J] = np.eye(k)
+    s = gpu_solver(wl)
+    s.set_skeleton(0, J, T)
+    x = rand_c((3 * k, 48), 6)                       # 2.9e7 pairs times right-hand sides
+    with pytest.raises(HzbError) as e:
+        s.apply_reduced(x, precision=2)
+    assert e.value.status == -6
+    ref = s.apply_reduced(x, precision=0)
+    assert np.abs(s.apply_reduced(x, precision=2) - ref).max() < 1e-11 * np.abs(ref).max()
