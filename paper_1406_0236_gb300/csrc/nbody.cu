@@ -527,8 +527,8 @@ hzb_status interbody64(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
 // Engine of the FP32 sum: 0 CUDA cores, 1 mma.sync, 2 tcgen05, 3 tcgen05 warp-specialised, 4
 // tcgen05 with single-term TF32 products (opt-in only).  On automatic the tensor cores (FP16
 // form) take five and more right-hand sides once the pair work outweighs their larger
-// set-up, against the packed CUDA-core kernel: R = 8 at 29,280 unknowns 0.96 against 1.42 ms, at
-// 8,200 124 against 120 us; R = 12 at 8,200 127 against 203 us; R = 16 at 432 61 against 33 us.
+// set-up, against the packed CUDA-core kernel: R = 8 at 29,280 unknowns 0.85 against 1.42 ms, at
+// 8,200 125 against 124 us; R = 12 at 8,200 127 against 203 us; R = 16 at 432 61 against 33 us.
 int fp32_engine(const hzb_ctx *c, int R)
 {
     if (c->nbody_engine == 1) return 1;

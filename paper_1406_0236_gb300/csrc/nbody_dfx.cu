@@ -40,9 +40,10 @@
 // RC right-hand sides (77 % of the issue slots at RC = 8); the one-directional kernel of
 // nbody_dfl.cu spends another 28 slots per pair and right-hand side on the sums.  Against it, and
 // the error of each against 64 bits:
-//   29,280 unknowns, k = 6:  R = 4  8.70 -> 7.26 ms;  R = 8  10.9 -> 7.3;  R = 16  16.6 -> 7.4;
-//                            R = 64  61.0 -> 11.8 ms, 1.2e-13 -> 1.1e-13
-//   8,200 unknowns, k = 2:   R = 8  0.65 -> 0.49 ms;  R = 64  3.73 -> 0.77 ms, 5.6e-14 -> 3.5e-14
+//   29,280 unknowns, k = 6:  R = 4  8.70 -> 7.36 ms;  R = 8  10.9 -> 7.4;  R = 16  16.7 -> 7.7;
+//                            R = 64  61.1 -> 12.3 ms, 1.2e-13 -> 1.1e-13
+//   8,200 unknowns, k = 2:   R = 8  0.66 -> 0.47 ms;  R = 64  3.74 -> 0.78 ms, 5.6e-14 -> 3.4e-14
+//   2,230,272 unknowns, k = 6:  R = 16  161 -> 54.8 s
 // (R = 64 without the pairs of CTAs 0.97 ms; there a barrier of all warps per half tile took 1.50 ms,
 // levels moved every tile 1.44, the MMAs issued from a loop, 200 cycles each, 1.38.)
 #include <cuda_fp16.h>

@@ -38,9 +38,10 @@
 // Bound by the transcendental unit (3 operations per ordered pair: 0.39 ms at 29,280
 // unknowns) and issue (29 instructions per pair, a packed one counting twice at dispatch).  Against the TF32
 // form of nbody_tc5.cu, whose operands went through shared memory: 29,280 unknowns, R = 16 1.74 ->
-// 1.03 ms (error 3.1e-6 -> 2.9e-6); R = 32 1.14 ms; 64,640 unknowns, R = 16 4.69, R = 64 10.8 ms.
-// Two, three and four CTAs per SM measured 5.53, 4.69 and 4.74 ms; forming part of the next
-// tile while the MMAs run gained nothing.
+// 0.91 ms (error 3.1e-6 -> 2.9e-6); R = 32 1.08 ms; 64,640 unknowns, R = 16 4.5, R = 64 10.4 ms;
+// 2,230,272 unknowns, R = 16 9.96 -> 5.59 s.  Two, three and four CTAs per SM measured 5.53, 4.69 and
+// 4.74 ms at 64,640, R = 16 (before the transposed images); forming part of the next tile while the
+// MMAs run gained nothing.
 #include <cuda_fp16.h>
 
 #include <algorithm>
