@@ -32,7 +32,7 @@
 // value overflows.  The tile's power of two, against the column's, goes with its images (one scale
 // per column left 2^-38 of the column's largest value to a body whose densities are small, and
 // the rows of the others nothing else to sum: relative error 4e-4 there at 1e-8; now 1e-6, for
-// 900 -> 913 us at 29,280 unknowns, R = 16).  Geometries whose kernels span more than FP16 (or k, eta
+// 905 -> 915 to 930 us at 29,280 unknowns, R = 16).  Geometries whose kernels span more than FP16 (or k, eta
 // outside sym_scaled) keep the TF32 form (nbody_tc5.cu).
 //
 // Bound by the transcendental unit (3 operations per ordered pair: 0.39 ms at 29,280
