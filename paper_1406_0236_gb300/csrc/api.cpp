@@ -143,7 +143,7 @@ hzb_status hzb_destroy(hzb_ctx *c)
     c->red.release(); c->krylov.release(); c->small.release();
     c->sctab.release(); c->nb_part64.release(); c->nb_part32.release(); c->sig32.release(); c->blockpairs.release(); c->kerr.release(); c->Ximg.release();
     c->dfa.release(); c->dfb.release(); c->dfc.release(); c->dftab.release(); c->nodecheck.release();
-    c->dfltab.release(); c->dla.release(); c->dlb.release(); c->dlc.release(); c->symn.release(); c->t5h_tiles.release(); c->t5h_body.release(); c->t5h_src.release(); c->t5h_img.release(); c->dlsig.release(); c->dlw.release(); c->dlkey.release();
+    c->dfltab.release(); c->dla.release(); c->dlb.release(); c->dlc.release(); c->symn.release(); c->t5h_tiles.release(); c->t5h_src.release(); c->t5h_img.release(); c->dlsig.release(); c->dlw.release(); c->dlkey.release();
     if (c->host_pinned) cudaFreeHost(c->host_pinned);
     release_graphs(c);
     for (cudaEvent_t e : c->evpool) cudaEventDestroy(e);

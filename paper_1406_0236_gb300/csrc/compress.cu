@@ -955,7 +955,7 @@ static void free_ctx_buffers(hzb_ctx *r)
     r->blockpairs.release(); r->kerr.release(); r->dfa.release(); r->dfb.release(); r->dfc.release();
     r->dftab.release(); r->rb.release(); r->rx.release(); r->zero_off.release(); r->yhat64.release();
     r->that64.release(); r->yhat32.release(); r->that32.release(); r->Ximg.release(); r->io_small.release();
-    r->dfltab.release(); r->dla.release(); r->dlb.release(); r->dlc.release(); r->symn.release(); r->t5h_tiles.release(); r->t5h_body.release(); r->t5h_src.release(); r->t5h_img.release(); r->dlsig.release(); r->dlw.release(); r->dlkey.release(); r->ysplit.release();
+    r->dfltab.release(); r->dla.release(); r->dlb.release(); r->dlc.release(); r->symn.release(); r->t5h_tiles.release(); r->t5h_src.release(); r->t5h_img.release(); r->dlsig.release(); r->dlw.release(); r->dlkey.release(); r->ysplit.release();
     if (r->host_pinned) cudaFreeHost(r->host_pinned);
     r->host_pinned = nullptr;
     release_graphs(r);

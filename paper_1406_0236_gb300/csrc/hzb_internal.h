@@ -200,7 +200,7 @@ struct hzb_ctx {
     int t5h_state = 0, t5h_ntiles = 0, t5h_most = 0, t5h_ctas = 0;
     double t5h_scale = 0.0, t5h_span = 0.0, t5h_mean = 1.0;
     hzb::DevBuf<int2> t5h_tiles;
-    hzb::DevBuf<int> t5h_body;                 // per tile its body and place in it (t5h_tile_word)
+    const int *t5h_words = nullptr;            // in the same buffer: every tile's body and place in it (t5h_tile_word)
     int t5h_nbodies = 0;                       // bodies with nodes
     hzb::DevBuf<float> t5h_src;
     hzb::DevBuf<unsigned char> t5h_img;

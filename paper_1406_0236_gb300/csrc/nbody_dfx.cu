@@ -699,10 +699,10 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
         return HZB_ECUDA;
     const int per = (R + 7) / 8;
     const size_t nk = (size_t)nt * per * 32, ne = (size_t)nt * rc * nchunk * 8;
-    dfx_key_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, c->stream>>>(nt, R, per, c->t5h_tiles.ptr, c->t5h_body.ptr,
+    dfx_key_kernel<<<(unsigned)((nk + 255) / 256), 256, 0, c->stream>>>(nt, R, per, c->t5h_tiles.ptr, c->t5h_words,
                                                                       c->pos64.ptr, sigma, c0, c->dlkey.ptr);
     dfx_density_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, c->stream>>>(nt, R, rc, nchunk, c->t5h_tiles.ptr,
-                                                                          c->t5h_body.ptr, c->pos64.ptr, sigma, c0,
+                                                                          c->t5h_words, c->pos64.ptr, sigma, c0,
                                                                           c->dlkey.ptr, c->t5h_img.ptr);
     const dim3 grid((unsigned)c->n_tblocks * 4, nchunk, nsplit);
     const float4 *ball = reinterpret_cast<const float4 *>(c->t5h_src.ptr + (size_t)nt * 6 * DFL_S);
@@ -723,7 +723,7 @@ hzb_status interbody_dfx(hzb_ctx *c, int R, const double2 *sigma, double2 *y)
         cfg.attrs = at;
         cfg.numAttrs = cl > 1 ? 1 : 0;
         e = cudaLaunchKernelEx(&cfg, kern, (const TargetBlock *)c->tblocks.ptr, (const int2 *)(c->t5h_tiles.ptr + nt),
-                               (const int2 *)c->t5h_tiles.ptr, (const int *)c->t5h_body.ptr, c->t5h_nbodies, ball, nt, R,
+                               (const int2 *)c->t5h_tiles.ptr, c->t5h_words, c->t5h_nbodies, ball, nt, R,
                                (const float4 *)c->dla.ptr,
                                (const float4 *)c->dlb.ptr, (const float4 *)c->dlc.ptr,
                                (const unsigned char *)c->t5h_img.ptr, (const int *)c->dlkey.ptr,

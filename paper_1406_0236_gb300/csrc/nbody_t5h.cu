@@ -518,7 +518,7 @@ hzb_status ensure_t5h(hzb_ctx *c)
                                       cudaMemcpyDeviceToHost, c->stream), "copy blocks") ||
         check_cuda(c, cudaStreamSynchronize(c->stream), "copy blocks"))
         return HZB_ECUDA;
-    // one buffer: the tiles, the blocks' own tiles, the end of each tile's body, the range
+    // one buffer: the tiles, the blocks' own tiles, the end of each tile's body, the range, the tiles' words
     std::vector<int2> tiles, own(tb.size()), end;
     std::vector<int> word;
     int nbodies = 0;
@@ -541,17 +541,17 @@ hzb_status ensure_t5h(hzb_ctx *c)
     tiles.insert(tiles.end(), own.begin(), own.end());
     tiles.insert(tiles.end(), end.begin(), end.end());
     tiles.push_back(make_int2(0x7f7fffff, 0));
+    const size_t words = tiles.size();
+    if (nt & 1) word.push_back(0);
+    for (int q = 0; q < nt; q += 2) tiles.push_back(make_int2(word[q], word[q + 1]));
     if (check_cuda(c, c->t5h_tiles.ensure(tiles.size()), "alloc tiles") ||
-        check_cuda(c, c->t5h_body.ensure(nt), "alloc tiles") ||
         check_cuda(c, c->t5h_src.ensure((size_t)nt * (TH_SRC + 4)), "alloc tiles"))
         return HZB_ENOMEM;
     float4 *ball = reinterpret_cast<float4 *>(c->t5h_src.ptr + (size_t)nt * TH_SRC);
     int2 *const end_dev = c->t5h_tiles.ptr + nt + own.size();
     int *const range_dev = reinterpret_cast<int *>(end_dev + nt);
     if (check_cuda(c, cudaMemcpyAsync(c->t5h_tiles.ptr, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                                      c->stream), "copy tiles") ||
-        check_cuda(c, cudaMemcpyAsync(c->t5h_body.ptr, word.data(), nt * sizeof(int), cudaMemcpyHostToDevice, c->stream),
-                   "copy tiles"))
+                                      c->stream), "copy tiles"))
         return HZB_ECUDA;
     t5h_source_kernel<<<(nt + 7) / 8, 256, 0, c->stream>>>(
         nt, c->t5h_tiles.ptr, c->pos64.ptr, c->nrm64.ptr, make_double3(c->center[0], c->center[1], c->center[2]), c->k,
@@ -566,6 +566,7 @@ hzb_status ensure_t5h(hzb_ctx *c)
     // |G'| <= u (1 + (k / |eta|) (1 + u)), u = 1 / (k r); the smallest is about u at the diameter
     c->t5h_ntiles = nt;
     c->t5h_nbodies = nbodies;
+    c->t5h_words = reinterpret_cast<const int *>(c->t5h_tiles.ptr + words);
     c->t5h_ctas = 0;
     for (const TargetBlock &t : tb) c->t5h_ctas += (t.count + TH_M - 1) / TH_M;
     c->t5h_most = 1;                                           // tiles of the other bodies, at most
